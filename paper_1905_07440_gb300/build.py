@@ -44,7 +44,9 @@ def build(verbose=False, extra=(), variant=None):
         s = os.path.join(CSRC, src)
         o = os.path.join(build_dir, src.replace(".cu", ".o"))
         if _stale(o, [s] + headers):
-            jobs.append([nvcc(), *ARCH, *FLAGS, *extra, "-c", s, "-o", o])
+            # the chain kernels are many independent functions: optimise them in parallel
+            par = ["--split-compile=0"] if src == "hq_kernels.cu" else []
+            jobs.append([nvcc(), *ARCH, *FLAGS, *par, *extra, "-c", s, "-o", o])
 
     def run(cmd):
         if verbose:

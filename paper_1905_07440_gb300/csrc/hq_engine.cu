@@ -942,7 +942,7 @@ NNLayout nn_layout(const hq::Dev& d, int max_batch, int max_samples) {
   l.av = take(4 * P);
   l.partials = take(4 * P * hq::kNNTrainCtas);
   l.fcache = take(4 * C * NL);
-  l.fnew = take(4 * C * 5 * d.L);
+  l.fnew = take(4 * C * 6 * d.L);
   l.X0 = take(8 * C * NL);
   l.ld0 = take(8 * C);
   l.F0 = take(8 * C);
@@ -1460,9 +1460,8 @@ int hq_group_create(hq_engine* const* engines, int n_engines, void* device_arena
     const int lm = hq::lmax_class(d.nx, d.ny);
     g->lmax = lm > g->lmax ? lm : g->lmax;
   }
-  // every engine's chains run in the group's class, whose QR may need more shared memory
   for (int e = 0; e < n_engines; ++e) {
-    const size_t sb = hq::smem_bytes_class(engines[e]->d, g->lmax);
+    const size_t sb = hq::smem_bytes(engines[e]->d);
     g->sb = sb > g->sb ? sb : g->sb;
   }
   // task table: every chain, longest estimated sweep first (longest-processing-time order)

@@ -102,7 +102,7 @@ struct NNState {
   float* adam_v;
   float* partials;      // [kNNTrainCtas][padded params] per-CTA gradient partials
   float* fcache;        // [C][L N] f of every patch of the current fields
-  float* fnew;          // [C][5 L] block-move scratch
+  float* fnew;          // [C][6 L] block-move scratch: patch values, inputs of the moved site
   double* X0;           // [C][L N] fields at the start of a cumulative step
   double* ld0;          // [C]
   double* F0;           // [C]
@@ -146,8 +146,6 @@ struct CnnState {
 };
 
 size_t smem_bytes(const Dev& d);
-// shared memory of a chain of d in a kernel of class lmax (group launches: the group's class)
-size_t smem_bytes_class(const Dev& d, int lmax);
 
 // Raise a kernel's dynamic shared memory limit to the device maximum (once per kernel and
 // device) when it needs more than the default 48 KB.

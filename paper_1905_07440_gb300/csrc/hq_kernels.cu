@@ -14,6 +14,7 @@
 #include <utility>
 #include <vector>
 #include "hq_device.cuh"
+#include "hq_oz_linalg.cuh"
 #include "hq_internal.h"
 #include "../../include/holstein_dqmc.h"
 
@@ -35,39 +36,28 @@ int section_cycles(unsigned long long* out, int n) {
 
 struct Smem {
   double *ex, *exi, *ey, *eyi;
-  double *dl, *u2, *xn, *dlt, *es, *dcorr, *tau, *norm2, *rinv, *vs, *dv, *rd;
+  double *dl, *u2, *xn, *dlt, *es, *gd, *norm2, *rinv, *dv;
+  double* tau;  // [16]
   double *red, *scal;
-  double *wv, *ws;  // blocked QR scratch (16-wide class only, else nullptr)
   int *perm, *piv, *sint;
+  OzScratch oz;     // tensor-core products (8- and 16-wide classes)
+  char* kin_mem;    // digit fragments of exp(-+dtau K)
+  OzKin kf, kfi;
 };
 
-static constexpr int kSmemVecs = 13;  // vs takes two
+static constexpr int kSmemVecs = 9;
 
-// Kernel template class of a lattice: the largest side rounded up to 2, 4, 8 or 16.
-static inline int lmax_of(int nx, int ny) {
-  const int m = nx > ny ? nx : ny;
-  return m <= 2 ? 2 : m <= 4 ? 4 : m <= 8 ? 8 : 16;
-}
+// Kernel template class of a lattice: both sides up to 8 (N <= 64, two CTAs per SM), or up to 16.
+static inline int lmax_of(int nx, int ny) { return (nx > ny ? nx : ny) <= 8 ? 8 : 16; }
 
-// doubles of the blocked QR scratch: the panel copy (n rows of kQbLd) and S (kQb x kQb)
-__host__ __device__ inline size_t smem_qr_doubles(bool blocked, int n) {
-  return blocked ? (size_t)n * kQbLd + kQb * kQb : 0;
-}
-
-// Shared memory of one chain's CTA in a kernel instantiated for class LMAX (`blocked` =
-// qr_blocked_class(LMAX)): the layout of carve<LMAX>.
-__host__ __device__ inline size_t smem_layout_bytes(int nx, int ny, int n, bool blocked) {
-  return (size_t)(2 * nx * nx + 2 * ny * ny + kSmemVecs * n + 32 + 16) * sizeof(double) +
-         smem_qr_doubles(blocked, n) * sizeof(double) + (size_t)(2 * n + 8) * sizeof(int);
-}
-
+// Shared memory of one chain's CTA: the layout of carve().
 size_t smem_bytes(const Dev& d) {
-  return smem_layout_bytes(d.nx, d.ny, d.n, qr_blocked_class(lmax_of(d.nx, d.ny)));
+  const int n = d.n;
+  return (size_t)(2 * d.nx * d.nx + 2 * d.ny * d.ny + kSmemVecs * n + 16 + 32 + 16 + 16 * oz_pad(n) + 256) *
+             sizeof(double) +
+         oz_frag_bytes(n) + 2 * kOzKinBytes + (size_t)(4 * oz_pad(n) + 2 * n + 8) * sizeof(int);
 }
 
-size_t smem_bytes_class(const Dev& d, int lmax) { return smem_layout_bytes(d.nx, d.ny, d.n, qr_blocked_class(lmax)); }
-
-template <int LMAX>
 __device__ inline Smem carve(const Dev& d, double* base) {
   Smem s;
   double* p = base;
@@ -81,22 +71,22 @@ __device__ inline Smem carve(const Dev& d, double* base) {
   s.xn = p; p += n;
   s.dlt = p; p += n;
   s.es = p; p += n;
-  s.dcorr = p; p += n;
-  s.tau = p; p += n;
+  s.gd = p; p += n;
   s.norm2 = p; p += n;
   s.rinv = p; p += n;
-  s.vs = p; p += 2 * n;
   s.dv = p; p += n;
-  s.rd = p; p += n;
+  s.tau = p; p += 16;
   s.red = p; p += 32;
   s.scal = p; p += 16;
   // 16-byte aligned: every count above is even (nx, ny and n are even)
-  s.wv = nullptr;
-  s.ws = nullptr;
-  if (qr_blocked_class(LMAX)) {
-    s.wv = p; p += (size_t)n * kQbLd;
-    s.ws = p; p += kQb * kQb;
-  }
+  s.oz.frag = reinterpret_cast<uint2*>(p); p += oz_frag_bytes(n) / sizeof(double);
+  s.kin_mem = reinterpret_cast<char*>(p); p += 2 * kOzKinBytes / sizeof(double);
+  s.oz.tall = p; p += oz_pad(n) * 16;
+  s.oz.ws = p; p += 256;
+  s.oz.er = reinterpret_cast<int*>(p);
+  s.oz.ec = s.oz.er + oz_pad(n);
+  s.oz.ev = s.oz.ec + oz_pad(n);
+  p += 2 * oz_pad(n);
   int* q = reinterpret_cast<int*>(p);
   s.perm = q; q += n;
   s.piv = q; q += n;
@@ -104,10 +94,79 @@ __device__ inline Smem carve(const Dev& d, double* base) {
   return s;
 }
 
-__device__ inline void load_kinetic(const Dev& d, const Smem& s) {
+// Digit fragments of exp(-+dtau K) from the factors in shared memory.
+__device__ inline void build_kin_fragments(const Dev& d, Smem& s) {
+  s.kf = oz_kin_build(s.ex, s.ey, d.nx, d.ny, s.kin_mem);
+  s.kfi = oz_kin_build(s.exi, s.eyi, d.nx, d.ny, s.kin_mem + kOzKinBytes);
+  __syncthreads();
+}
+
+__device__ inline void load_kinetic(const Dev& d, Smem& s) {
   const int a = d.nx * d.nx, b = d.ny * d.ny;
   for (int i = threadIdx.x; i < 2 * a + 2 * b; i += HQ_THREADS) s.ex[i] = d.kin[i];  // contiguous
   __syncthreads();
+  build_kin_fragments(d, s);
+}
+
+// ---- the steps of a stabilised product, by lattice class
+template <int LMAX>
+__device__ __noinline__ double lu_logdet(const Smem& sm, double* A, int n) {
+  return oz_lu<LMAX>(A, n, sm.piv, sm.red, sm.oz.tall, sm.oz.frag, sm.oz.er);
+}
+
+// Y <- A^-1 Y right after lu_logdet(A).
+template <int LMAX>
+__device__ __noinline__ void lu_solve(const Smem& sm, const double* A, int n, double* Y) {
+  oz_lu_solve<LMAX>(A, n, sm.piv, Y, sm.oz.tall, sm.oz.frag, sm.oz.er);
+}
+
+// One restabilisation: P (column-graded product) = U diag(D) T' Pi^T, Tout = T' Pi^T Tprev (T' Pi^T with
+// Tprev == nullptr).  Q is scratch (R); P is overwritten (reflector vectors).
+template <int LMAX>
+__device__ __noinline__ void udv_step(const Smem& sm, double* P, double* Q, int n, double* U, double* D, const double* Tprev,
+                                double* Tout) {
+  const QrScratch qs{sm.tau, sm.rinv, sm.perm};
+  HQ_TIC(pp);
+  prepivot(P, Q, n, n, qs, sm.norm2);
+  HQ_TOC(pp, SEC_PREPIVOT);
+  HQ_TIC(qr);
+  oz_qr<LMAX>(Q, P, n, n, qs, sm.oz);
+  HQ_TOC(qr, SEC_QR);
+  HQ_TIC(fq);
+  oz_form_q<LMAX>(P, n, n, U, sm.oz);
+  HQ_TOC(fq, SEC_FORMQ);
+  HQ_TIC(tu);
+  oz_t_update<LMAX>(Q, n, qs, D, Tprev, Tout, sm.oz);
+  HQ_TOC(tu, SEC_TUPD);
+}
+
+// Diagonals exp(-dtau V) of consecutive slices: the k-th one applied is that of row s0 + k step of the
+// fields X (site `site` shifted by dx), or of the table ev of ready exponentials.
+struct SliceDiag {
+  const double* X;
+  const double* ev;
+  int s0, step, site;
+  double dx;
+  __device__ double operator()(const Dev& d, int k, int r) const {
+    const size_t o = (size_t)(s0 + k * step) * d.n + r;
+    if (ev) return ev[o];
+    double x = X[o];
+    if (r == site) x = x + dx;
+    return exp(-d.dtau * (d.g * x - d.mu));
+  }
+};
+
+// P <- slice matrices times U diag(D) (identity with U == nullptr): `count` slices with the diagonals
+// src.  kAfter: diag(d) E (transposed slices), else E diag(d).
+template <int LMAX, bool kAfter>
+__device__ __noinline__ void slice_product(const Dev& d, const Smem& sm, double* P, const double* U, const double* D,
+                                           int count, SliceDiag src) {
+  const int n = d.n;
+  HQ_TIC(kin);
+  const int cap = (int)(oz_frag_bytes(n) / (sizeof(double) * n));
+  oz_slices<kAfter>(d.nx, d.ny, n, sm.kf, P, U, D, count, [&](int k, int r) { return src(d, k, r); },
+                    reinterpret_cast<double*>(sm.oz.frag), cap);
+  HQ_TOC(kin, SEC_KIN);
 }
 
 __device__ inline double* chain_work(const Dev& d, int c, int slot) {
@@ -121,7 +180,8 @@ __device__ inline void flag_nonfinite(const Dev& d, int c, double v) {
 // log|det(I + U D T)| from the last UDV factors (D in sm.dv):
 // I + U D T = U Db (Db^-1 U^T + Ds T), so log|det| = sum log Db + log|det A|.  With G0,
 // also G_0 = (I + (B_L..B_1)^T)^-T = Y^T with Y = A^-1 Db^-1 U^T.
-__device__ double finish_logdet(const Dev& d, int c, const Smem& sm, const double* U, const double* Tc, double* G0) {
+template <int LMAX>
+__device__ __noinline__ double finish_logdet(const Dev& d, int c, const Smem& sm, const double* U, const double* Tc, double* G0) {
   const int n = d.n;
   HQ_TIC(ld);
   double* A = chain_work(d, c, WK_M1);
@@ -138,10 +198,9 @@ __device__ double finish_logdet(const Dev& d, int c, const Smem& sm, const doubl
   double lsum = 0.0;
   for (int i = threadIdx.x; i < n; i += HQ_THREADS) lsum += log(fmax(sm.dv[i], 1.0));
   const double lb = block_sum(lsum, sm.red);
-  const double la = lu_logdet_blocked(A, n, n, sm.piv, sm.sint, sm.red);
+  const double la = lu_logdet<LMAX>(sm, A, n);
   if (G0) {
-    lu_diag_recip(A, n, n, sm.rd);
-    lu_solve_blocked(A, n, n, sm.piv, sm.rd, Y);
+    lu_solve<LMAX>(sm, A, n, Y);
     for (int idx = threadIdx.x; idx < n * n; idx += HQ_THREADS) {
       const int r = idx % n, col = idx / n;
       G0[(size_t)col * n + r] = Y[(size_t)r * n + col];
@@ -160,7 +219,7 @@ __device__ double finish_logdet(const Dev& d, int c, const Smem& sm, const doubl
 // G0 != nullptr also writes G_0 = (I + B_L..B_1)^-1.  With stop > 0 (a boundary) only the
 // slices above it are taken: the factors end in the stack slot of `stop` and 0 is returned.
 template <int LMAX>
-__device__ double udv_top_down(const Dev& d, int c, const Smem& sm, const double* X, int site, double dx,
+__device__ __noinline__ double udv_top_down(const Dev& d, int c, const Smem& sm, const double* X, int site, double dx,
                                bool store, double* G0, int stop = 0) {
   const int n = d.n, L = d.L, nw = d.n_wrap;
   double* P = chain_work(d, c, WK_P);
@@ -168,38 +227,13 @@ __device__ double udv_top_down(const Dev& d, int c, const Smem& sm, const double
   double* Tc = chain_work(d, c, WK_T);
   double* Tn = chain_work(d, c, WK_T2);
   double* Q = chain_work(d, c, WK_M1);
-  const QrScratch qs{sm.tau, sm.vs, sm.rinv, sm.perm, sm.sint, sm.wv, sm.ws};
   int hi = L, lo = ((L - 1) / nw) * nw;
   bool first = true;
   while (true) {
-    if (first) set_identity(P, n, n);
-    else copy_scale_cols(P, U, n, n, sm.dv);
-    __syncthreads();
-    for (int s = hi - 1; s >= lo; --s) {
-      HQ_TIC(dl);
-      for (int r = threadIdx.x; r < n; r += HQ_THREADS) {
-        double x = X[(size_t)s * n + r];
-        if (r == site) x = x + dx;
-        sm.dl[r] = exp(-d.dtau * (d.g * x - d.mu));
-      }
-      HQ_TOC(dl, SEC_DL);
-      HQ_TIC(kin);
-      // B_s^T P = exp(-dtau V_s) exp(-dtau K) P (the scaling reads dl after kin_rows' barrier)
-      kin_rows<LMAX, KIN_SCALE_AFTER>(P, n, n, sm.ex, sm.ey, d.nx, d.ny, sm.dl);
-      HQ_TOC(kin, SEC_KIN);
-    }
-    HQ_TIC(pp);
-    prepivot<qr_group<LMAX>()>(P, Q, n, n, qs, sm.norm2);
-    HQ_TOC(pp, SEC_PREPIVOT);
-    HQ_TIC(qr);
-    qr_factor<LMAX>(Q, n, n, qs);
-    HQ_TOC(qr, SEC_QR);
-    HQ_TIC(fq);
-    qr_form_q<LMAX>(Q, n, n, U, qs);
-    HQ_TOC(fq, SEC_FORMQ);
-    HQ_TIC(tu);
-    t_update(Q, n, n, qs, sm.dv, first ? nullptr : Tc, Tn, P);
-    HQ_TOC(tu, SEC_TUPD);
+    // B_s^T P = exp(-dtau V_s) exp(-dtau K) P for s = hi - 1 .. lo
+    slice_product<LMAX, true>(d, sm, P, first ? nullptr : U, sm.dv, hi - lo,
+                              SliceDiag{X, nullptr, hi - 1, -1, site, dx});
+    udv_step<LMAX>(sm, P, Q, n, U, sm.dv, first ? nullptr : Tc, Tn);
     double* t = Tc; Tc = Tn; Tn = t;
     if (store && lo > 0) {
       const size_t b = (size_t)c * d.n_bound + (lo / nw - 1);
@@ -214,13 +248,13 @@ __device__ double udv_top_down(const Dev& d, int c, const Smem& sm, const double
     lo -= nw;
   }
   // with stop > 0 the factors of (B_L .. B_{stop+1})^T are in the stack slot of boundary stop
-  return stop > 0 ? 0.0 : finish_logdet(d, c, sm, U, Tc, G0);
+  return stop > 0 ? 0.0 : finish_logdet<LMAX>(d, c, sm, U, Tc, G0);
 }
 
 template <int LMAX>
 __device__ void stack_build_body(const Dev& d, int c, double* smraw) {
   if (!d.active[c]) return;
-  const Smem sm = carve<LMAX>(d, smraw);
+  Smem sm = carve(d, smraw);
   load_kinetic(d, sm);
   const double* X = d.X + (size_t)c * d.L * d.n;
   double* G = d.G + (size_t)c * d.n * d.n;
@@ -232,7 +266,7 @@ __device__ void stack_build_body(const Dev& d, int c, double* smraw) {
 }
 
 template <int LMAX>
-__global__ void __launch_bounds__(HQ_THREADS) stack_build_kernel(Dev d) {
+__global__ void __launch_bounds__(HQ_THREADS) stack_build_kernel(const __grid_constant__ Dev d) {
   extern __shared__ __align__(16) double smraw[];
   stack_build_body<LMAX>(d, blockIdx.x, smraw);
 }
@@ -246,7 +280,7 @@ __global__ void __launch_bounds__(HQ_THREADS) stack_build_kernel(Dev d) {
 // shared out so that the halves never touch the same buffer: the top half uses P, U, T, T2,
 // M1; the bottom half M2, M3 and the chain's G (overwritten by the join anyway).
 template <int LMAX>
-__device__ void udv_bottom_half(const Dev& d, int c, const Smem& sm, int m) {
+__device__ __noinline__ void udv_bottom_half(const Dev& d, int c, const Smem& sm, int m) {
   const int n = d.n, nw = d.n_wrap;
   const double* X = d.X + (size_t)c * d.L * n;
   double* UR = d.UR + (size_t)c * n * n;
@@ -255,35 +289,25 @@ __device__ void udv_bottom_half(const Dev& d, int c, const Smem& sm, int m) {
   double* P = chain_work(d, c, WK_M2);
   double* Q = chain_work(d, c, WK_M3);
   double* T2 = d.G + (size_t)c * n * n;
-  const QrScratch qs{sm.tau, sm.vs, sm.rinv, sm.perm, sm.sint, sm.wv, sm.ws};
   for (int s0 = 0; s0 < m; s0 += nw) {
     const int s1 = s0 + nw < m ? s0 + nw : m;
     const bool first = (s0 == 0);
-    if (first) set_identity(P, n, n);
-    else copy_scale_cols(P, UR, n, n, DR);
-    __syncthreads();
-    for (int s = s0; s < s1; ++s) {
-      for (int r = threadIdx.x; r < n; r += HQ_THREADS) sm.dl[r] = exp(-d.dtau * (d.g * X[(size_t)s * n + r] - d.mu));
-      __syncthreads();
-      // B_s P = exp(-dtau K) exp(-dtau V_s) P
-      kin_rows<LMAX, KIN_SCALE_BEFORE>(P, n, n, sm.ex, sm.ey, d.nx, d.ny, sm.dl);
-    }
-    prepivot<qr_group<LMAX>()>(P, Q, n, n, qs, sm.norm2);
-    qr_factor<LMAX>(Q, n, n, qs);
-    qr_form_q<LMAX>(Q, n, n, UR, qs);
-    t_update(Q, n, n, qs, DR, first ? nullptr : TR, T2, P);
+    // B_s P = exp(-dtau K) exp(-dtau V_s) P for s = s0 .. s1 - 1
+    slice_product<LMAX, false>(d, sm, P, first ? nullptr : UR, DR, s1 - s0,
+                               SliceDiag{X, nullptr, s0, 1, -1, 0.0});
+    udv_step<LMAX>(sm, P, Q, n, UR, DR, first ? nullptr : TR, T2);
     copy_mat(TR, T2, n, n);
     __syncthreads();
   }
 }
 
 template <int LMAX>
-__global__ void __launch_bounds__(HQ_THREADS) split_halves_kernel(Dev d, int m) {
+__global__ void __launch_bounds__(HQ_THREADS) split_halves_kernel(const __grid_constant__ Dev d, int m) {
   extern __shared__ __align__(16) double smraw[];
   const int C = d.n_chains;
   const int c = blockIdx.x % C;
   if (!d.active[c]) return;
-  const Smem sm = carve<LMAX>(d, smraw);
+  Smem sm = carve(d, smraw);
   load_kinetic(d, sm);
   if (blockIdx.x < C) {
     udv_top_down<LMAX>(d, c, sm, d.X + (size_t)c * d.L * d.n, -1, 0.0, true, nullptr, m);
@@ -292,15 +316,16 @@ __global__ void __launch_bounds__(HQ_THREADS) split_halves_kernel(Dev d, int m) 
   }
 }
 
+template <int LMAX>
 __device__ double green_two_sided(const Dev& d, int c, const Smem& sm, int l, double* Gf);
 
 template <int LMAX>
-__global__ void __launch_bounds__(HQ_THREADS) split_join_kernel(Dev d, int m) {
+__global__ void __launch_bounds__(HQ_THREADS) split_join_kernel(const __grid_constant__ Dev d, int m) {
   extern __shared__ __align__(16) double smraw[];
   const int c = blockIdx.x;
   if (!d.active[c]) return;
-  const Smem sm = carve<LMAX>(d, smraw);
-  const double ld = green_two_sided(d, c, sm, m, d.G + (size_t)c * d.n * d.n);
+  const Smem sm = carve(d, smraw);
+  const double ld = green_two_sided<LMAX>(d, c, sm, m, d.G + (size_t)c * d.n * d.n);
   if (threadIdx.x == 0) {
     d.logdet[c] = ld;
     flag_nonfinite(d, c, ld);
@@ -311,7 +336,8 @@ __global__ void __launch_bounds__(HQ_THREADS) split_join_kernel(Dev d, int m) {
 // the left stack ((B_L..B_{l+1})^T = UL DL TL):
 //   G_l = UL DLb^-1 [DRb^-1 UR^T UL DLb^-1 + DRs TR TL^T DLs]^-1 DRb^-1 UR^T.
 // Returns log|det M|; G_l goes to Gf.
-__device__ double green_two_sided(const Dev& d, int c, const Smem& sm, int l, double* Gf) {
+template <int LMAX>
+__device__ __noinline__ double green_two_sided(const Dev& d, int c, const Smem& sm, int l, double* Gf) {
   const int n = d.n;
   const double* UR = d.UR + (size_t)c * n * n;
   const double* TR = d.TR + (size_t)c * n * n;
@@ -333,8 +359,8 @@ __device__ double green_two_sided(const Dev& d, int c, const Smem& sm, int l, do
       rdr[i] = 1.0 / fmax(DR[i], 1.0);
       rdl[i] = 1.0 / fmax(DL[i], 1.0);
     }
-    gemm_nn<true, false>(n, UR, UL, M1, n);   // UR^T UL (ends with a barrier)
-    gemm_nn<false, true>(n, TR, TL, M2, n);   // TR TL^T
+    oz_mm<LMAX, true, false>(n, UR, UL, nullptr, nullptr, M1, sm.oz);   // UR^T UL (ends with a barrier)
+    oz_mm<LMAX, false, true>(n, TR, TL, nullptr, nullptr, M2, sm.oz); // TR TL^T
     for (int idx = threadIdx.x; idx < n * n; idx += HQ_THREADS) {
       const int i = idx % n, j = idx / n;
       const double drs = fmin(DR[i], 1.0), dls = fmin(DL[j], 1.0);
@@ -344,16 +370,10 @@ __device__ double green_two_sided(const Dev& d, int c, const Smem& sm, int l, do
     }
     for (int i = threadIdx.x; i < n; i += HQ_THREADS) lsum += log(fmax(DR[i], 1.0)) + log(fmax(DL[i], 1.0));
     __syncthreads();
-    la = lu_logdet_blocked(M2, n, n, sm.piv, sm.sint, sm.red);
-    lu_diag_recip(M2, n, n, sm.rd);
-    lu_solve_blocked(M2, n, n, sm.piv, sm.rd, M3);
-    // M1 <- UL DLb^-1, Gf = M1 M3
-    for (int idx = threadIdx.x; idx < n * n; idx += HQ_THREADS) {
-      const int j = idx / n;
-      M1[idx] = UL[idx] * rdl[j];
-    }
-    __syncthreads();
-    gemm_nn<false, false>(n, M1, M3, Gf, n);
+    la = lu_logdet<LMAX>(sm, M2, n);
+    lu_solve<LMAX>(sm, M2, n, M3);
+    // Gf = UL DLb^-1 M3
+    oz_mm<LMAX, false, false>(n, UL, M3, rdl, nullptr, Gf, sm.oz);
   } else {
     double* rdr = sm.rinv;
     for (int i = threadIdx.x; i < n; i += HQ_THREADS) rdr[i] = 1.0 / fmax(DR[i], 1.0);
@@ -367,16 +387,15 @@ __device__ double green_two_sided(const Dev& d, int c, const Smem& sm, int l, do
     }
     for (int i = threadIdx.x; i < n; i += HQ_THREADS) lsum += log(fmax(DR[i], 1.0));
     __syncthreads();
-    la = lu_logdet_blocked(M2, n, n, sm.piv, sm.sint, sm.red);
-    lu_diag_recip(M2, n, n, sm.rd);
-    lu_solve_blocked(M2, n, n, sm.piv, sm.rd, Gf);
+    la = lu_logdet<LMAX>(sm, M2, n);
+    lu_solve<LMAX>(sm, M2, n, Gf);
   }
   return block_sum(lsum, sm.red) + la;
 }
 
 // Electronic observables from a fresh G (Wick; both spins share G), added to the chain's
 // per-sweep accumulators.
-__device__ void measure_green(const Dev& d, int c, const Smem& sm, const double* G) {
+__device__ __noinline__ void measure_green(const Dev& d, int c, const Smem& sm, const double* G) {
   const int n = d.n;
   double sm_m = 0.0, sm_m2 = 0.0, sm_sm = 0.0, sm_g = 0.0, conn = 0.0;
   for (int r = threadIdx.x; r < n; r += HQ_THREADS) {
@@ -408,42 +427,11 @@ __device__ void measure_green(const Dev& d, int c, const Smem& sm, const double*
   }
 }
 
-// Flush of the delayed updates: G += A B^T (n x n, rank kk; A, B [kk][n]) as a register-tiled
-// contraction, 4 x 4 entries of G per thread (8 loads per 16 FMAs instead of 2 per FMA); every
-// entry still accumulates its kk products in order m = 0 .. kk-1 onto G, so the result does not
-// depend on the tiling.
-__device__ inline void flush_delayed(double* G, const double* A, const double* B, int n, int kk) {
-  const int tiles = n >> 2;  // n is a multiple of 4
-  for (int t = threadIdx.x; t < tiles * tiles; t += HQ_THREADS) {
-    const int r0 = (t % tiles) * 4, c0 = (t / tiles) * 4;
-    double acc[4][4];
-#pragma unroll
-    for (int b = 0; b < 4; ++b)
-#pragma unroll
-      for (int a = 0; a < 4; ++a) acc[a][b] = G[(size_t)(c0 + b) * n + r0 + a];
-    for (int m = 0; m < kk; ++m) {
-      double av[4], bv[4];
-#pragma unroll
-      for (int a = 0; a < 4; ++a) av[a] = A[m * n + r0 + a];
-#pragma unroll
-      for (int b = 0; b < 4; ++b) bv[b] = B[m * n + c0 + b];
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = fma(av[a], bv[b], acc[a][b]);
-    }
-#pragma unroll
-    for (int b = 0; b < 4; ++b)
-#pragma unroll
-      for (int a = 0; a < 4; ++a) G[(size_t)(c0 + b) * n + r0 + a] = acc[a][b];
-  }
-}
-
 template <int LMAX>
-__device__ void local_chunk_body(const Dev& d, int c, int s0, int s1, int measure, double* smraw) {
+__device__ __noinline__ void local_chunk_body(const Dev& d, int c, int s0, int s1, int measure, double* smraw) {
   if (!d.active[c]) return;
   const int n = d.n, L = d.L, k = d.k;
-  const Smem sm = carve<LMAX>(d, smraw);
+  Smem sm = carve(d, smraw);
   load_kinetic(d, sm);
   double* X = d.X + (size_t)c * L * n;
   double* G = d.G + (size_t)c * n * n;
@@ -474,73 +462,91 @@ __device__ void local_chunk_body(const Dev& d, int c, int s0, int s1, int measur
       sm.xn[i] = xnew;
       sm.dlt[i] = exp(-d.dtau * d.g * dx) - 1.0;
       sm.es[i] = exp(-dS);
-      sm.dcorr[i] = 0.0;
+      sm.gd[i] = G[(size_t)i * n + i];
     }
     __syncthreads();
     HQ_TOC(pp, SEC_PROP_PREP);
     HQ_TIC(seq);
     int kk = 0;
-    // Thread 0 runs the decisions in site order; a rejected proposal changes nothing, so it
-    // walks on to the next accepted site before the CTA meets (one barrier per accepted move
-    // instead of one per proposal).  sm.sint[2 + slot] = the accepted site, n when none is left.
+    const int lp = n <= 32 ? 4 : n <= 64 ? 2 : 1;
+    // Warp 0 decides: a rejected proposal changes nothing, so its lanes evaluate the next 32 sites at
+    // once against the diagonal of the current G (kept in gd with the pending updates) and the first
+    // accepted one is taken; the CTA meets once per accepted move.  sm.sint[2 + slot] = the accepted
+    // site, n when none is left.
     for (int i0 = 0, it = 0; i0 < n; ++it) {
       const int slot = it & 1;
-      if (threadIdx.x == 0) {
+      if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
         int next = n;
-        for (int i = i0; i < n; ++i) {
-          // ratio of one spin: R1 = 1 + delta (1 - G_ii), G_ii including pending updates
-          const double gii = G[(size_t)i * n + i] + sm.dcorr[i];
-          const double delta = sm.dlt[i];
-          const double R1 = 1.0 + delta * (1.0 - gii);
-          const double prob = R1 * R1 * sm.es[i];
-          if (!isfinite(R1)) d.status[c] = HQ_ENAN;
-          if (sm.u2[i] < prob) {
-            X[(size_t)s * n + i] = sm.xn[i];
+        for (int base = i0; base < n && next == n; base += 32) {
+          const int i = base + lane;
+          bool acc = false, bad = false;
+          double R1 = 1.0, delta = 0.0;
+          if (i < n) {
+            // ratio of one spin: R1 = 1 + delta (1 - G_ii), G_ii including pending updates
+            delta = sm.dlt[i];
+            R1 = 1.0 + delta * (1.0 - sm.gd[i]);
+            bad = !isfinite(R1);
+            acc = sm.u2[i] < R1 * R1 * sm.es[i];
+          }
+          const unsigned hit = __ballot_sync(HQ_FULL, acc), bads = __ballot_sync(HQ_FULL, bad);
+          const int first = hit ? __ffs(hit) - 1 : 31;
+          if (lane == 0 && (bads & (0xffffffffu >> (31 - first)))) d.status[c] = HQ_ENAN;
+          if (hit) {
+            next = base + first;
+            if (lane == first) {
+              X[(size_t)s * n + i] = sm.xn[i];
+              sm.scal[slot] = delta * recip_fp64(R1);
+            }
             ++n_acc;
-            sm.scal[slot] = delta / R1;
-            next = i;
-            break;
           }
         }
-        sm.sint[2 + slot] = next;
+        if (lane == 0) sm.sint[2 + slot] = next;
       }
       __syncthreads();
       const int i = sm.sint[2 + slot];
       i0 = i + 1;
       if (i < n) {
         // G' = Gc + a b^T with a = (delta/R1)(Gc[:, i] - e_i), b = Gc[i, :],
-        // Gc = G + sum_m A[:, m] B[:, m]^T (updates not yet flushed).
+        // Gc = G + sum_m A[:, m] B[:, m]^T (updates not yet flushed).  Entry r of both new vectors
+        // belongs to lp neighbouring lanes, which share out the pending terms: the sums are DFMA
+        // chains, and with n <= 64 one lane per entry would leave half of the FP64 pipes idle.
         const double f = sm.scal[slot];
-        // entry r of both new vectors in one thread, so the diagonal correction needs no
-        // barrier of its own
-        for (int r = threadIdx.x; r < n; r += HQ_THREADS) {
-          double va = G[(size_t)i * n + r], vb = G[(size_t)r * n + i];
-          for (int m = 0; m < kk; ++m) {
+        for (int w = threadIdx.x; w < n * lp; w += HQ_THREADS) {
+          const int r = w / lp, p = w % lp;
+          double va = p == 0 ? G[(size_t)i * n + r] - (r == i ? 1.0 : 0.0) : 0.0, vb = p == 0 ? G[(size_t)r * n + i] : 0.0;
+          for (int m = p; m < kk; m += lp) {
             va = fma(A[m * n + r], B[m * n + i], va);
             vb = fma(A[m * n + i], B[m * n + r], vb);
           }
-          if (r == i) va -= 1.0;
-          const double a = f * va;
-          A[kk * n + r] = a;
-          B[kk * n + r] = vb;
-          sm.dcorr[r] = fma(a, vb, sm.dcorr[r]);
+          if (lp > 1) {
+            const int rem = n * lp - (w & ~31);  // lanes of this warp in the range (a multiple of lp)
+            const unsigned on = rem >= 32 ? HQ_FULL : (1u << rem) - 1u;
+            for (int o = 1; o < lp; o <<= 1) {
+              va += __shfl_xor_sync(on, va, o);
+              vb += __shfl_xor_sync(on, vb, o);
+            }
+          }
+          if (p == 0) {
+            const double a = f * va;
+            A[kk * n + r] = a;
+            B[kk * n + r] = vb;
+            sm.gd[r] = fma(a, vb, sm.gd[r]);
+          }
         }
         ++kk;
+        __syncthreads();
         if (kk == k) {
-          __syncthreads();
           HQ_TIC(fl);
-          flush_delayed(G, A, B, n, kk);
+          oz_flush<LMAX>(G, A, B, n, kk, sm.oz);
           HQ_TOC(fl, SEC_FLUSH);
-          __syncthreads();
-          for (int r = threadIdx.x; r < n; r += HQ_THREADS) sm.dcorr[r] = 0.0;
           kk = 0;
         }
-        __syncthreads();
       }
     }
     if (kk > 0) {
       HQ_TIC(fl);
-      flush_delayed(G, A, B, n, kk);
+      oz_flush<LMAX>(G, A, B, n, kk, sm.oz);
       HQ_TOC(fl, SEC_FLUSH);
     }
     HQ_TOC(seq, SEC_PROP_SEQ);
@@ -553,13 +559,7 @@ __device__ void local_chunk_body(const Dev& d, int c, int s0, int s1, int measur
       sm.u2[r] = 1.0 / e;
     }
     __syncthreads();
-    for (int idx = threadIdx.x; idx < n * n; idx += HQ_THREADS) {
-      const int r = idx % n, col = idx / n;
-      G[(size_t)col * n + r] = (sm.dl[r] * G[(size_t)col * n + r]) * sm.u2[col];
-    }
-    __syncthreads();
-    kin_rows<LMAX, KIN_PLAIN>(G, n, n, sm.ex, sm.ey, d.nx, d.ny);
-    kin_cols<LMAX>(G, n, n, sm.exi, sm.eyi, d.nx, d.ny);
+    oz_wrap<LMAX>(d.nx, d.ny, n, sm.kf, sm.kfi, G, sm.dl, sm.u2);
     HQ_TOC(wr, SEC_WRAP);
   }
   if (threadIdx.x == 0) {
@@ -577,28 +577,18 @@ __device__ void local_chunk_body(const Dev& d, int c, int s0, int s1, int measur
   double* Gf = chain_work(d, c, WK_U);
   HQ_TIC(rp);
   const bool first = (s0 == 0);
-  if (first) set_identity(P, n, n);
-  else copy_scale_cols(P, UR, n, n, DR);
-  __syncthreads();
-  for (int s = s0; s < s1; ++s) {
-    for (int r = threadIdx.x; r < n; r += HQ_THREADS) sm.dl[r] = exp(-d.dtau * (d.g * X[(size_t)s * n + r] - d.mu));
-    __syncthreads();
-    // B_s P = exp(-dtau K) exp(-dtau V_s) P
-    kin_rows<LMAX, KIN_SCALE_BEFORE>(P, n, n, sm.ex, sm.ey, d.nx, d.ny, sm.dl);
-  }
+  // B_s P = exp(-dtau K) exp(-dtau V_s) P for s = s0 .. s1 - 1
+  slice_product<LMAX, false>(d, sm, P, first ? nullptr : UR, DR, s1 - s0,
+                             SliceDiag{X, nullptr, s0, 1, -1, 0.0});
   HQ_TOC(rp, SEC_RESTAB_PROD);
   HQ_TIC(rq);
   double* Q = chain_work(d, c, WK_M1);
-  const QrScratch qs{sm.tau, sm.vs, sm.rinv, sm.perm, sm.sint, sm.wv, sm.ws};
-  prepivot<qr_group<LMAX>()>(P, Q, n, n, qs, sm.norm2);
-  qr_factor<LMAX>(Q, n, n, qs);
-  qr_form_q<LMAX>(Q, n, n, UR, qs);
-  t_update(Q, n, n, qs, DR, first ? nullptr : TR, T2, P);
+  udv_step<LMAX>(sm, P, Q, n, UR, DR, first ? nullptr : TR, T2);
   copy_mat(TR, T2, n, n);
   __syncthreads();
   HQ_TOC(rq, SEC_RESTAB_QR);
   HQ_TIC(rg);
-  const double ld = green_two_sided(d, c, sm, s1, Gf);
+  const double ld = green_two_sided<LMAX>(d, c, sm, s1, Gf);
   double err = 0.0, bad = 0.0;
   for (int idx = threadIdx.x; idx < n * n; idx += HQ_THREADS) {
     const double gf = Gf[idx];
@@ -629,7 +619,7 @@ __device__ void local_chunk_body(const Dev& d, int c, int s0, int s1, int measur
 // finished chunk q - 1, so an SM that runs one chain alone takes more chunks than an SM
 // shared by two.  sched = [counter, abort, ..., progress[C] at kSchedHeader], zeroed first.
 template <int LMAX>
-__global__ void __launch_bounds__(HQ_THREADS) local_phase_kernel(Dev d, int measure) {
+__global__ void __launch_bounds__(HQ_THREADS, LMAX <= 8 ? 2 : 1) local_phase_kernel(const __grid_constant__ Dev d, int measure) {
   extern __shared__ __align__(16) double smraw[];
   __shared__ int s_task;
   const int C = d.n_chains, Q = (d.L + d.n_wrap - 1) / d.n_wrap, ntask = Q * C;
@@ -685,7 +675,7 @@ __device__ inline double* chain_corr(const Dev& d, int c) {
 
 // exp(-dtau V) of every slice and the chunk products M_q of chain c (current buffer).
 template <int LMAX>
-__device__ void build_chunks(const Dev& d, const Smem& sm, int c) {
+__device__ __noinline__ void build_chunks(const Dev& d, const Smem& sm, int c) {
   const int n = d.n, L = d.L, nw = d.n_wrap;
   const double* X = d.X + (size_t)c * L * n;
   double* ev = d.expV + (size_t)c * L * n;
@@ -695,10 +685,7 @@ __device__ void build_chunks(const Dev& d, const Smem& sm, int c) {
   for (int q = 0; q < d.n_chunks; ++q) {
     const int lo = q * nw, hi = min(lo + nw, L);
     double* M = chunk_mat(d, c, cur, q);
-    set_identity(M, n, n);
-    __syncthreads();
-    for (int s = hi - 1; s >= lo; --s)
-      kin_rows<LMAX, KIN_SCALE_AFTER>(M, n, n, sm.ex, sm.ey, d.nx, d.ny, ev + (size_t)s * n);
+    slice_product<LMAX, true>(d, sm, M, nullptr, nullptr, hi - lo, SliceDiag{nullptr, ev, hi - 1, -1, -1, 0.0});
   }
 }
 
@@ -766,7 +753,7 @@ __device__ void corr_step(const Dev& d, const Smem& sm, double* W, int step, int
 }
 
 template <int LMAX>
-__device__ double udv_top_down_cm(const Dev& d, int c, const Smem& sm, int site, double dx) {
+__device__ __noinline__ double udv_top_down_cm(const Dev& d, int c, const Smem& sm, int site, double dx) {
   const int n = d.n, L = d.L, nw = d.n_wrap;
   const double* X = d.X + (size_t)c * L * n;
   const double* ev = d.expV + (size_t)c * L * n;
@@ -779,8 +766,6 @@ __device__ double udv_top_down_cm(const Dev& d, int c, const Smem& sm, int site,
   double* Tc = chain_work(d, c, WK_T);
   double* Tn = chain_work(d, c, WK_T2);
   double* Q = chain_work(d, c, WK_M1);
-  double* Y = chain_work(d, c, WK_M2);
-  const QrScratch qs{sm.tau, sm.vs, sm.rinv, sm.perm, sm.sint, sm.wv, sm.ws};
   const double delta = expm1(-d.dtau * d.g * dx);
   HQ_TIC(cv);
   for (int s = threadIdx.x; s < L; s += HQ_THREADS) xs[s] = exp(-d.dtau * (d.g * (X[(size_t)s * n + site] + dx) - d.mu));
@@ -824,28 +809,15 @@ __device__ double udv_top_down_cm(const Dev& d, int c, const Smem& sm, int site,
     if (first) {
       copy_mat(P, Mn, n, n);
     } else {
-      copy_scale_cols(Y, U, n, n, sm.dv);
-      __syncthreads();
-      gemm_nn<false, false>(n, Mn, Y, P, n);
+      oz_mm<LMAX, false, false>(n, Mn, U, nullptr, sm.dv, P, sm.oz);
     }
     __syncthreads();
     HQ_TOC(gm, SEC_KIN);
-    HQ_TIC(pp);
-    prepivot<qr_group<LMAX>()>(P, Q, n, n, qs, sm.norm2);
-    HQ_TOC(pp, SEC_PREPIVOT);
-    HQ_TIC(qr);
-    qr_factor<LMAX>(Q, n, n, qs);
-    HQ_TOC(qr, SEC_QR);
-    HQ_TIC(fq);
-    qr_form_q<LMAX>(Q, n, n, U, qs);
-    HQ_TOC(fq, SEC_FORMQ);
-    HQ_TIC(tu);
-    t_update(Q, n, n, qs, sm.dv, first ? nullptr : Tc, Tn, P);
-    HQ_TOC(tu, SEC_TUPD);
+    udv_step<LMAX>(sm, P, Q, n, U, sm.dv, first ? nullptr : Tc, Tn);
     double* t = Tc; Tc = Tn; Tn = t;
     first = false;
   }
-  return finish_logdet(d, c, sm, U, Tc, nullptr);
+  return finish_logdet<LMAX>(d, c, sm, U, Tc, nullptr);
 }
 
 // Sites visited by a sweep's block moves: all N in index order, or with d.block_sites = S
@@ -869,7 +841,7 @@ __device__ inline int block_move_site(const Dev& d, int c, int k) {
 // One block move X(site, .) += dX of chain c: Philox draw, dtau dS_ph, the full stabilised
 // log|det M(X')| and the Metropolis decision (all threads of the CTA).
 template <int LMAX>
-__device__ void block_move(const Dev& d, const Smem& sm, int c, int site) {
+__device__ __noinline__ void block_move(const Dev& d, const Smem& sm, int c, int site) {
   const int n = d.n, L = d.L;
   double* X = d.X + (size_t)c * L * n;
   HQ_TIC(mv);
@@ -929,10 +901,10 @@ __device__ void block_move(const Dev& d, const Smem& sm, int c, int site) {
 // every worker stops taking tasks.  sched = [counter, abort, ..., progress[C] at
 // kSchedHeader], zeroed before the launch.
 template <int LMAX>
-__global__ void __launch_bounds__(HQ_THREADS, 2) global_phase_kernel(Dev d) {
+__global__ void __launch_bounds__(HQ_THREADS, LMAX <= 8 ? 2 : 1) global_phase_kernel(const __grid_constant__ Dev d) {
   extern __shared__ __align__(16) double smraw[];
   __shared__ int s_task;
-  const Smem sm = carve<LMAX>(d, smraw);
+  Smem sm = carve(d, smraw);
   load_kinetic(d, sm);
   const int C = d.n_chains, ntask = (block_move_count(d) + (d.use_cm ? 1 : 0)) * C;
   int* counter = d.sched;
@@ -1030,7 +1002,7 @@ __device__ void sweep_end_body(const Dev& d, int c, int measured, double* red) {
   }
 }
 
-__global__ void __launch_bounds__(HQ_THREADS) sweep_end_kernel(Dev d, int measured) {
+__global__ void __launch_bounds__(HQ_THREADS) sweep_end_kernel(const __grid_constant__ Dev d, int measured) {
   __shared__ double red[HQ_WARPS];
   sweep_end_body(d, blockIdx.x, measured, red);
 }
@@ -1044,7 +1016,7 @@ __global__ void __launch_bounds__(HQ_THREADS) sweep_end_kernel(Dev d, int measur
 // another.  Kernels are instantiated for the largest lattice side of the group (the separable
 // propagator's arithmetic does not depend on it) and take the largest shared-memory carve.
 template <int LMAX>
-__global__ void __launch_bounds__(HQ_THREADS) group_sweep_kernel(GroupDev g, int flags, int stack) {
+__global__ void __launch_bounds__(HQ_THREADS, LMAX <= 8 ? 2 : 1) group_sweep_kernel(const __grid_constant__ GroupDev g, int flags, int stack) {
   extern __shared__ __align__(16) double smraw[];
   __shared__ int s_task;
   __shared__ Dev sd;
@@ -1062,7 +1034,7 @@ __global__ void __launch_bounds__(HQ_THREADS) group_sweep_kernel(GroupDev g, int
     if (e != cur) {
       if (threadIdx.x == 0) sd = g.devs[e];
       __syncthreads();
-      sm = carve<LMAX>(sd, smraw);
+      sm = carve(sd, smraw);
       load_kinetic(sd, sm);
       cur = e;
     }
@@ -1077,6 +1049,7 @@ __global__ void __launch_bounds__(HQ_THREADS) group_sweep_kernel(GroupDev g, int
       if (sd.use_cm) build_chunks<LMAX>(sd, sm, c);
       for (int k = 0, nb = block_move_count(sd); k < nb; ++k) block_move<LMAX>(sd, sm, c, block_move_site(sd, c, k));
     }
+    __syncthreads();  // the last block move's fields are written before the records read them
     sweep_end_body(sd, c, (meas && do_local) ? 1 : 0, sm.red);
     __syncthreads();
   }
@@ -1084,9 +1057,9 @@ __global__ void __launch_bounds__(HQ_THREADS) group_sweep_kernel(GroupDev g, int
 
 // Electronic observables from G_0 of every chain (after a stack build).
 template <int LMAX>
-__global__ void __launch_bounds__(HQ_THREADS) measure_g0_kernel(Dev d) {
+__global__ void __launch_bounds__(HQ_THREADS) measure_g0_kernel(const __grid_constant__ Dev d) {
   extern __shared__ __align__(16) double smraw[];
-  const Smem sm = carve<LMAX>(d, smraw);
+  const Smem sm = carve(d, smraw);
   const int c = blockIdx.x;
   if (!d.active[c]) return;
   measure_green(d, c, sm, d.G + (size_t)c * d.n * d.n);
@@ -1095,7 +1068,7 @@ __global__ void __launch_bounds__(HQ_THREADS) measure_g0_kernel(Dev d) {
 // Slot control without host memory: a copy from pageable host memory can wait for kernels
 // running on other streams, so identity, activity and the per-slot reset are written by a
 // kernel from its arguments.  slot < 0: every chain c gets chain word first + c (creation).
-__global__ void slot_control_kernel(Dev d, int slot, uint32_t key0, uint32_t key1, uint32_t chain, uint32_t sweep,
+__global__ void slot_control_kernel(const __grid_constant__ Dev d, int slot, uint32_t key0, uint32_t key1, uint32_t chain, uint32_t sweep,
                                     int active, int reset) {
   const int c = slot < 0 ? blockIdx.x : slot;
   const uint32_t word = slot < 0 ? chain + (uint32_t)blockIdx.x : chain;
@@ -1118,13 +1091,13 @@ __global__ void slot_control_kernel(Dev d, int slot, uint32_t key0, uint32_t key
   for (int o = threadIdx.x; o < kCounters; o += blockDim.x) d.counters[(size_t)c * kCounters + o] = 0;
 }
 
-__global__ void reset_acc_kernel(Dev d) {
+__global__ void reset_acc_kernel(const __grid_constant__ Dev d) {
   const int c = blockIdx.x;
   for (int o = threadIdx.x; o < kAccSlots; o += blockDim.x) d.acc[(size_t)c * kAccSlots + o] = 0.0;
 }
 
 // log W = 2 log|det M| - dtau S_ph per chain.
-__global__ void __launch_bounds__(HQ_THREADS) log_weight_kernel(Dev d, double* out) {
+__global__ void __launch_bounds__(HQ_THREADS) log_weight_kernel(const __grid_constant__ Dev d, double* out) {
   __shared__ double red[HQ_WARPS];
   const int c = blockIdx.x;
   const int n = d.n, L = d.L;
@@ -1193,8 +1166,6 @@ static inline void allow_smem(K kernel, size_t bytes) {
   do {                                                                                      \
     const size_t sb = smem_bytes(d);                                                        \
     switch (lmax_of((d).nx, (d).ny)) {                                                      \
-      case 2: allow_smem(KERNEL<2>, sb); KERNEL<2><<<(d).n_chains, HQ_THREADS, sb, stream>>>(__VA_ARGS__); break;   \
-      case 4: allow_smem(KERNEL<4>, sb); KERNEL<4><<<(d).n_chains, HQ_THREADS, sb, stream>>>(__VA_ARGS__); break;   \
       case 8: allow_smem(KERNEL<8>, sb); KERNEL<8><<<(d).n_chains, HQ_THREADS, sb, stream>>>(__VA_ARGS__); break;   \
       default: allow_smem(KERNEL<16>, sb); KERNEL<16><<<(d).n_chains, HQ_THREADS, sb, stream>>>(__VA_ARGS__); break; \
     }                                                                                       \
@@ -1227,11 +1198,12 @@ __device__ inline void ring_propagators_smem(const Dev& d, const Smem& s) {
 }
 
 template <int LMAX>
-__global__ void __launch_bounds__(HQ_THREADS) logdet_noalloc_kernel(Dev d, double* out) {
+__global__ void __launch_bounds__(HQ_THREADS) logdet_noalloc_kernel(const __grid_constant__ Dev d, double* out) {
   extern __shared__ __align__(16) double smraw[];
   const int c = blockIdx.x;
-  const Smem sm = carve<LMAX>(d, smraw);
+  Smem sm = carve(d, smraw);
   ring_propagators_smem(d, sm);
+  build_kin_fragments(d, sm);
   const double* X = d.X + (size_t)c * d.L * d.n;
   const double ld = udv_top_down<LMAX>(d, c, sm, X, -1, 0.0, false, nullptr);
   if (threadIdx.x == 0) out[c] = ld;
@@ -1300,8 +1272,6 @@ static cudaError_t launch_split_t(const Dev& d, int m, int part, cudaStream_t s)
 cudaError_t launch_split_logdet(const Dev& d, int m, int part, cudaStream_t s) {
   if (m <= 0 || m >= d.L || m % d.n_wrap != 0) return cudaErrorInvalidValue;
   switch (lmax_of(d.nx, d.ny)) {
-    case 2: return launch_split_t<2>(d, m, part, s);
-    case 4: return launch_split_t<4>(d, m, part, s);
     case 8: return launch_split_t<8>(d, m, part, s);
     default: return launch_split_t<16>(d, m, part, s);
   }
@@ -1331,8 +1301,6 @@ static cudaError_t launch_local_phase_t(const Dev& d, int measure, cudaStream_t 
 
 cudaError_t launch_local_phase(const Dev& d, int measure, cudaStream_t s) {
   switch (lmax_of(d.nx, d.ny)) {
-    case 2: return launch_local_phase_t<2>(d, measure, s);
-    case 4: return launch_local_phase_t<4>(d, measure, s);
     case 8: return launch_local_phase_t<8>(d, measure, s);
     default: return launch_local_phase_t<16>(d, measure, s);
   }
@@ -1365,8 +1333,6 @@ static cudaError_t launch_phase(const Dev& d, cudaStream_t s) {
 
 cudaError_t launch_global_phase(const Dev& d, cudaStream_t s) {
   switch (lmax_of(d.nx, d.ny)) {
-    case 2: return launch_phase<2>(d, s);
-    case 4: return launch_phase<4>(d, s);
     case 8: return launch_phase<8>(d, s);
     default: return launch_phase<16>(d, s);
   }
@@ -1396,8 +1362,6 @@ static cudaError_t launch_group_t(const GroupDev& g, size_t sb, int n_active, in
 cudaError_t launch_group_sweep(const GroupDev& g, int lmax, size_t sb, int n_active, int flags, int stack,
                                cudaStream_t s) {
   switch (lmax) {
-    case 2: return launch_group_t<2>(g, sb, n_active, flags, stack, s);
-    case 4: return launch_group_t<4>(g, sb, n_active, flags, stack, s);
     case 8: return launch_group_t<8>(g, sb, n_active, flags, stack, s);
     default: return launch_group_t<16>(g, sb, n_active, flags, stack, s);
   }

@@ -1,0 +1,290 @@
+// LU with partial pivoting and its solves: panels of 16 columns in registers, everything else as 16-term products on the tensor cores (hq_oz.cuh).
+//
+// A panel is held by four warps, one per scheduler (see hq_panel.cuh: FP64 instructions are what counts),
+// with one row per thread (two for m > 128) or G = 2, 4 threads per row for m <= 64, 32.  A column step
+// needs one barrier: every warp offers its best remaining row (largest high word, by one REDUX) with that
+// row's entries, and after the barrier all threads take the best offer and update their own rows.  Rows
+// are not moved; each thread tracks the position its rows end at.  The column-by-column form in memory took
+// four barriers and about 5800 cycles per column at n = 64.
+// Triangles: the 16 x 16 diagonal blocks are inverted once (one warp each, 60 dependent FP64
+// instructions), so the triangular solves become products too.
+#pragma once
+#include "hq_device.cuh"
+#include "hq_oz.cuh"
+#include "hq_panel.cuh"
+
+namespace hq {
+
+// 1 / u by a float seed and one third-order step in FP64 (no special cases: 0 and non-finite pivots
+// show up in log|U_jj|).
+__device__ __forceinline__ double recip_fp64(double u) {
+  const int hi = __double2hiint(u), lo = __double2loint(u), e = (hi >> 20) & 0x7ff;
+  const double m = __hiloint2double((hi & 0xfffff) | 0x3ff00000, lo);  // |u| 2^(1023 - e) in [1, 2)
+  const float f = __uint_as_float(((uint32_t)(hi & 0xfffff) << 3) | 0x3f800000u | ((uint32_t)lo >> 29));
+  const double g = float_bits_to_double(__frcp_rn(f));
+  const double r = fma(-m, g, 1.0);
+  const double v = oz_scale(fma(g, fma(r, r, r), g), 1023 - e);
+  return hi < 0 ? -v : v;
+}
+
+struct LuShared {
+  double row[2][kPanelWarps][16];
+  int key[2][kPanelWarps], pos[2][kPanelWarps];
+};
+
+// Columns p0 .. p0 + kb - 1, rows p0 .. n - 1 of A, in place (L below, U on and above the diagonal, rows
+// in pivot order); piv[p0 + j] = the row swapped with p0 + j at step j.  Ends with a barrier.
+template <int LM, int CPT, int RPT>
+__device__ __noinline__ void lu_panel_rows(double* A, int ld, int n, int p0, int kb, int* piv, LuShared* ls) {
+  constexpr int G = 16 / CPT, LG = G == 4 ? 2 : G == 2 ? 1 : 0, kThreads = 32 * kPanelWarps, kRows = kThreads / G;
+  const int m = n - p0, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (warp < kPanelWarps) {
+    const int row0 = tid >> LG, cq = tid & (G - 1);
+    double x[RPT][CPT];
+    int pos[RPT];
+    bool active[RPT];
+#pragma unroll
+    for (int r = 0; r < RPT; ++r) {
+      pos[r] = row0 + r * kRows;
+      active[r] = pos[r] < m;
+#pragma unroll
+      for (int i = 0; i < CPT; ++i) {
+        const int c = i * G + cq;
+        x[r][i] = (active[r] && c < kb) ? A[(size_t)(p0 + c) * ld + p0 + pos[r]] : 0.0;
+      }
+    }
+#pragma unroll 1
+    for (int j = 0; j < kb; ++j) {
+      // x[.][i] holds column ((i + jb) % CPT) G + cq; entries i < CPT - jb are the columns not yet done
+      const int jo = j & (G - 1), jb = j >> LG, left = CPT - jb, b = j & 1;
+      double xj[RPT];
+      uint32_t key = 0;
+      int kr = 0;
+#pragma unroll
+      for (int r = 0; r < RPT; ++r) {
+        xj[r] = G == 1 ? x[r][0] : __shfl_sync(HQ_FULL, x[r][0], (lane & ~(G - 1)) | jo);
+        const uint32_t k = active[r] ? oz_abs_hi(xj[r]) + 1u : 0u;
+        if (k > key) {
+          key = k;
+          kr = r;
+        }
+      }
+      const uint32_t best = __reduce_max_sync(HQ_FULL, key);
+      const int cand = (__ffs(__ballot_sync(HQ_FULL, key == best)) - 1) & ~(G - 1);
+      const bool mine = (lane & ~(G - 1)) == cand;
+      if (mine) {
+#pragma unroll
+        for (int r = 0; r < RPT; ++r)
+          if (r == kr) {
+#pragma unroll
+            for (int i = 0; i < CPT; ++i) ls->row[b][warp][((i + jb) & (CPT - 1)) * G + cq] = x[r][i];
+            if (cq == 0) {
+              ls->key[b][warp] = (int)best;
+              ls->pos[b][warp] = pos[r];
+            }
+          }
+      }
+      bar_warps(kThreads);
+      int win = 0;
+      uint32_t top = (uint32_t)ls->key[b][0];
+#pragma unroll
+      for (int w = 1; w < kPanelWarps; ++w) {
+        const uint32_t k = (uint32_t)ls->key[b][w];
+        if (k > top) {
+          top = k;
+          win = w;
+        }
+      }
+      const double* u = ls->row[b][win];
+      const int from = ls->pos[b][win];
+      if (tid == 0) piv[p0 + j] = p0 + from;
+      const double rp = recip_fp64(u[j]);
+#pragma unroll
+      for (int r = 0; r < RPT; ++r) {
+        if (warp == win && mine && r == kr) {
+          pos[r] = j;
+          active[r] = false;
+        } else if (pos[r] == j) {
+          pos[r] = from;
+        }
+        const double l = xj[r] * rp;
+#pragma unroll
+        for (int i = 0; i < CPT; ++i)
+          if (i < left) {
+            const int c = i * G + jb * G + cq;
+            const double upd = fma(-l, u[c], x[r][i]);
+            if (active[r]) {
+              if (c > j) x[r][i] = upd;
+              else if (c == j) x[r][i] = l;
+            }
+          }
+        if (jo == G - 1) {
+          const double first = x[r][0];
+#pragma unroll
+          for (int i = 0; i + 1 < CPT; ++i) x[r][i] = x[r][i + 1];
+          x[r][CPT - 1] = first;
+        }
+      }
+    }
+    const int jb = kb >> LG;
+#pragma unroll
+    for (int r = 0; r < RPT; ++r)
+      if (row0 + r * kRows < m) {
+#pragma unroll
+        for (int i = 0; i < CPT; ++i) {
+          const int c = ((i + jb) & (CPT - 1)) * G + cq;
+          if (c < kb) A[(size_t)(p0 + c) * ld + p0 + pos[r]] = x[r][i];
+        }
+      }
+  }
+  __syncthreads();
+}
+
+// Inverse of a triangular 16 x 16 block by one warp: M[16][16] row-major in shared memory, read from the
+// kb x kb block at (p0, p0) of A (identity beyond kb).  kUnitLower: unit lower triangle, else upper.
+template <bool kUnitLower>
+__device__ inline void invert_triangle(const double* A, int ld, int p0, int kb, double* M) {
+  const int lane = threadIdx.x & 31;
+  auto a = [&](int r, int c) { return (r < kb && c < kb) ? A[(size_t)(p0 + c) * ld + p0 + r] : 0.0; };
+  if (lane < 16) {
+    const int o = lane & 8, c = lane & 7;
+    double x[8];
+    if (kUnitLower) {
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        double v = r == c ? 1.0 : 0.0;
+#pragma unroll
+        for (int k = 0; k < r; ++k) v = fma(-a(o + r, o + k), x[k], v);
+        x[r] = v;
+      }
+    } else {
+#pragma unroll
+      for (int r = 7; r >= 0; --r) {
+        double v = r == c ? 1.0 : 0.0;
+#pragma unroll
+        for (int k = r + 1; k < 8; ++k) v = fma(-a(o + r, o + k), x[k], v);
+        x[r] = o + r < kb ? v * recip_fp64(a(o + r, o + r)) : v;
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      M[(o + r) * 16 + o + c] = x[r];
+      M[(o + r) * 16 + (8 - o) + c] = 0.0;
+    }
+  }
+  __syncwarp();
+  // off-diagonal block: -B22 A21 B11 (lower), -B11 A12 B22 (upper)
+  const int ro = kUnitLower ? 8 : 0, co = 8 - ro;
+  double y[2];
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int r = (lane >> 3) + 4 * u, c = lane & 7;
+    double v = 0.0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v = fma(a(ro + r, co + k), M[(co + k) * 16 + co + c], v);
+    y[u] = v;
+  }
+  double* X = M + ro * 16 + co;
+#pragma unroll
+  for (int u = 0; u < 2; ++u) X[((lane >> 3) + 4 * u) * 16 + (lane & 7)] = y[u];
+  __syncwarp();
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int r = (lane >> 3) + 4 * u, c = lane & 7;
+    double v = 0.0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v = fma(M[(ro + r) * 16 + ro + k], X[k * 16 + c], v);
+    y[u] = -v;
+  }
+  __syncwarp();
+#pragma unroll
+  for (int u = 0; u < 2; ++u) X[((lane >> 3) + 4 * u) * 16 + (lane & 7)] = y[u];
+  __syncwarp();
+}
+
+// Y(p0 : p0 + kb, c0 : c1) <- M Y(p0 : p0 + kb, c0 : c1).  Ends with a barrier.
+template <int LM>
+__device__ __noinline__ void oz_left16(const double* M, double* Y, int ld, int p0, int kb, int c0, int c1, uint2* frag,
+                                       int* er) {
+  oz_rank16<true>(0, kb, c0, c1, kb, frag, er, [&](int r, int k) { return M[r * 16 + k]; },
+                  [&](int k, int c) { return Y[(size_t)c * ld + p0 + k]; },
+                  [&](int r, int c, double s0, double s1) {
+                    *reinterpret_cast<double2*>(Y + (size_t)c * ld + p0 + r) = make_double2(s0, s1);
+                  });
+}
+
+// C(r0:r1, c0:c1) -= A(r0:r1, k0:k0+kb) B(k0:k0+kb, c0:c1), kb <= 16.  Ends with a barrier.
+template <int LM>
+__device__ __noinline__ void oz_rank_update(double* C, const double* A, const double* B, int ld, int r0, int r1, int c0,
+                                            int c1, int k0, int kb, uint2* frag, int* er) {
+  oz_rank16<false>(r0, r1, c0, c1, kb, frag, er, [&](int r, int k) { return A[(size_t)(k0 + k) * ld + r]; },
+                   [&](int k, int c) { return B[(size_t)c * ld + k0 + k]; },
+                   [&](int r, int c, double s0, double s1) {
+                     double2* p = reinterpret_cast<double2*>(C + (size_t)c * ld + r);
+                     const double2 v = *p;
+                     *p = make_double2(v.x - s0, v.y - s1);
+                   });
+}
+
+// In place LU of A; tri: oz_pad(n) / 16 blocks of 16 x 16, left holding the inverses of L's diagonal
+// blocks.  Returns sum_j log|U_jj| (in every thread).
+template <int LM>
+__device__ inline double oz_lu(double* A, int n, int* piv, double* red, double* tri, uint2* frag, int* er) {
+  const int tid = threadIdx.x;
+  LuShared* ls = reinterpret_cast<LuShared*>(frag);
+  for (int p0 = 0; p0 < n; p0 += 16) {
+    const int kb = min(16, n - p0), p1 = p0 + kb, m = n - p0;
+    if (m <= 32) lu_panel_rows<LM, 4, 1>(A, n, n, p0, kb, piv, ls);
+    else if (LM <= 8 || m <= 64) lu_panel_rows<LM, 8, 1>(A, n, n, p0, kb, piv, ls);  // LM <= 8: n <= 64
+    else if (m <= 128) lu_panel_rows<LM, LM <= 8 ? 8 : 16, 1>(A, n, n, p0, kb, piv, ls);
+    else lu_panel_rows<LM, LM <= 8 ? 8 : 16, LM <= 8 ? 1 : 2>(A, n, n, p0, kb, piv, ls);
+    double* M = tri + (p0 >> 4) * 256;
+    if (tid < 32) invert_triangle<true>(A, n, p0, kb, M);
+    else
+      for (int c = tid - 32; c < n; c += HQ_THREADS - 32) {  // the panel's swaps on the other columns
+        if (c >= p0 && c < p1) continue;
+        double* ac = A + (size_t)c * n;
+        for (int j = p0; j < p1; ++j) {
+          const int p = piv[j];
+          if (p != j) { const double v = ac[j]; ac[j] = ac[p]; ac[p] = v; }
+        }
+      }
+    __syncthreads();
+    if (p1 < n) {
+      oz_left16<LM>(M, A, n, p0, kb, p1, n, frag, er);
+      oz_rank_update<LM>(A, A, A, n, p1, n, p1, n, p0, kb, frag, er);
+    }
+  }
+  double a = 0.0;
+  for (int j = tid; j < n; j += HQ_THREADS) a += log(fabs(A[(size_t)j * n + j]));
+  return block_sum(a, red);
+}
+
+// Y <- A^-1 Y (n right-hand sides) for the factors of oz_lu; tri as oz_lu left it (overwritten).
+template <int LM>
+__device__ inline void oz_lu_solve(const double* A, int n, const int* piv, double* Y, double* tri, uint2* frag,
+                                   int* er) {
+  const int tid = threadIdx.x, warp = tid >> 5;
+  for (int c = tid; c < n; c += HQ_THREADS) {
+    double* y = Y + (size_t)c * n;
+    for (int j = 0; j < n; ++j) {
+      const int p = piv[j];
+      if (p != j) { const double v = y[j]; y[j] = y[p]; y[p] = v; }
+    }
+  }
+  __syncthreads();
+  for (int p0 = 0; p0 < n; p0 += 16) {
+    const int kb = min(16, n - p0), p1 = p0 + kb;
+    oz_left16<LM>(tri + (p0 >> 4) * 256, Y, n, p0, kb, 0, n, frag, er);
+    if (p1 < n) oz_rank_update<LM>(Y, A, Y, n, p1, n, 0, n, p0, kb, frag, er);
+  }
+  for (int b = warp; 16 * b < n; b += HQ_WARPS) invert_triangle<false>(A, n, 16 * b, min(16, n - 16 * b), tri + b * 256);
+  __syncthreads();
+  for (int p0 = ((n - 1) >> 4) << 4; p0 >= 0; p0 -= 16) {
+    const int kb = min(16, n - p0);
+    oz_left16<LM>(tri + (p0 >> 4) * 256, Y, n, p0, kb, 0, n, frag, er);
+    if (p0 > 0) oz_rank_update<LM>(Y, A, Y, n, 0, p0, 0, n, p0, kb, frag, er);
+  }
+}
+
+}  // namespace hq

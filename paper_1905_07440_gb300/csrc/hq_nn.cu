@@ -39,6 +39,8 @@ struct NNSmem {
   float* f25;    // [32] f of the patches of a local move
   float* pxf;    // [n] network inputs of the proposed values (local moves)
   int* nbr;      // [n][5] cross neighbours of every site: self, +x, -x, +y, -y
+  float* part;   // [128] layer-3 chains handed between warps (local moves)
+  volatile int* flag;  // [4] decision of a local move
   double* red;   // [HQ_WARPS]
   double* pu2;   // [n] proposal uniforms (local)
   double* pxn;   // [n] proposed values
@@ -51,7 +53,7 @@ struct NNSmem {
 
 __host__ __device__ inline size_t nn_smem_bytes(int n, bool with_cnn = false) {
   size_t b = sizeof(uint2) * TC_FRAGS + sizeof(double) * (HQ_WARPS + 3 * (size_t)n + NN_GROUPS + 8) +
-             sizeof(float) * (TC_FLOATS + 32 + (size_t)n) + sizeof(int) * 5 * (size_t)n;
+             sizeof(float) * (TC_FLOATS + 32 + 128 + (size_t)n) + sizeof(int) * (4 + 5 * (size_t)n);
   if (with_cnn) b += sizeof(float) * CN_WPAD + sizeof(int) * (4 + 3 * CN_WIN + 2 * (size_t)n);
   return b;
 }
@@ -69,6 +71,8 @@ __device__ inline NNSmem nn_carve(int n, char* base, bool with_cnn = false) {
   float* f = (float*)p;
   s.tcf = f; f += TC_FLOATS;
   s.f25 = f; f += 32;
+  s.part = f; f += 128;
+  s.flag = (volatile int*)f; f += 4;
   s.pxf = f; f += n;
   s.nbr = (int*)f; f += 5 * n;
   s.cw = nullptr;
@@ -82,15 +86,62 @@ __device__ inline NNSmem nn_carve(int n, char* base, bool with_cnn = false) {
   return s;
 }
 
-// Position ll * n + j of input k of the patch centred at (l, i): slice ll = l + dl, site j =
-// cross point c of i (k = 5 (dl + 2) + c; c = 0 the site itself, then +x, -x, +y, -y).
-__device__ __forceinline__ int patch_pos(const Dev& d, int l, int i, int k) {
-  const int L = d.L, x = i % d.nx, y = i / d.nx;
-  const int dl = k / 5 - 2, cidx = k % 5;
-  const int cx_ = (cidx == 1) - (cidx == 2), cy_ = (cidx == 3) - (cidx == 4);
-  const int ll = (l + dl + L) % L;
-  const int j = (x + cx_ + d.nx) % d.nx + d.nx * ((y + cy_ + d.ny) % d.ny);
-  return ll * d.n + j;
+__device__ __forceinline__ void bar_sync(int id, int threads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(int id, int threads) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+// sum over the warp of (double)a - (double)b: a 64-bit integer sum in units of 2^-57 of the largest term
+// (a dependent FP64 instruction takes 64 cycles here, an integer shuffle-and-add about 35).
+__device__ __forceinline__ double warp_sum_diff(float a, float b) {
+  const uint32_t ua = __float_as_uint(a), ub = __float_as_uint(b);
+  const uint32_t top = __reduce_max_sync(HQ_FULL, max(ua & 0x7fffffffu, ub & 0x7fffffffu));
+  const int E = (int)(top >> 23);
+  if (E == 255) return __longlong_as_double(0x7ff8000000000000ll);
+  auto fix = [&](uint32_t u) {
+    const int e = (int)((u >> 23) & 0xffu);
+    const long long m = e ? (long long)((((unsigned long long)((u & 0x7fffffu) | 0x800000u)) << 33) >> min(E - e, 63)) : 0ll;
+    return (int)u < 0 ? -m : m;
+  };
+  long long v = fix(ua) - fix(ub);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(HQ_FULL, v, o);
+  if (v == 0) return 0.0;
+  const double d = (double)v;
+  return __hiloint2double(__double2hiint(d) + (E - 183) * (1 << 20), __double2loint(d));
+}
+
+// u < exp(arg): by a single-precision exponential unless the two are within 1e-4 of each other, whose
+// error (|arg| <= 709 rounded to float, and the function's) is below 5e-5.
+__device__ __forceinline__ int metropolis(double u, double arg) {
+  const float pf = expf((float)arg), uf = (float)u;
+  if (uf > pf * 1.0001f) return 0;
+  if (uf < pf * 0.9999f) return 1;
+  return u < exp(arg);
+}
+
+// Cross neighbours of every site: nbr[5 i + c], c = 0 the site itself, then +x, -x, +y, -y.  No barrier.
+__device__ inline void build_cross(const Dev& d, int* nbr) {
+  for (int r = threadIdx.x; r < d.n; r += HQ_THREADS) {
+    const int x = r % d.nx, y = r / d.nx;
+    nbr[5 * r + 0] = r;
+    nbr[5 * r + 1] = (x + 1) % d.nx + d.nx * y;
+    nbr[5 * r + 2] = (x - 1 + d.nx) % d.nx + d.nx * y;
+    nbr[5 * r + 3] = x + d.nx * ((y + 1) % d.ny);
+    nbr[5 * r + 4] = x + d.nx * ((y - 1 + d.ny) % d.ny);
+  }
+}
+
+__device__ __forceinline__ int wrap_slice(int l, int L) { return l < 0 ? l + L : (l >= L ? l - L : l); }
+
+// Inputs of the patch centred at (l, i), in the lane's order, from the input table xf [L][n].
+__device__ __forceinline__ void patch_inputs(const Dev& d, const NNLane& k, const int* nbr, const float* xf, int l,
+                                             int i, float (&z)[8]) {
+#pragma unroll
+  for (int q = 0; q < 8; ++q)
+    z[q] = k.c[q] < 0 ? 0.f : xf[wrap_slice(l + k.dl[q], d.L) * d.n + nbr[5 * i + k.c[q]]];
 }
 
 // Network input of a field value: the value minus the mean field x0, rounded to float.  Every
@@ -119,12 +170,15 @@ __device__ inline double fc_eval_all(const Dev& d, const NNSmem& s, const NNFrag
   const int n = d.n, NL = d.n * d.L;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, g = lane >> 2, t = lane & 3;
   double part = 0.0;
+  const NNLane kin = nn_lane_inputs();
   for (int base = warp * 16; base < NL; base += HQ_WARPS * 16) {
-    float f0, f1;
-    nn_tile_f(w, [&](int row, int k) {
-      const int r = base + row < NL ? base + row : NL - 1;
-      return xf[patch_pos(d, r / n, r % n, k)];
-    }, f0, f1);
+    float f0, f1, z[2][8];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int r = base + g + 8 * h < NL ? base + g + 8 * h : NL - 1;
+      patch_inputs(d, kin, s.nbr, xf, r / n, r % n, z[h]);
+    }
+    nn_tile_f(w, z, f0, f1);
     if (t == 0) {
       if (base + g < NL) {
         part += (double)f0;
@@ -151,7 +205,8 @@ __global__ void __launch_bounds__(HQ_THREADS) nn_eval_kernel(Dev d, NNState nn, 
   extern __shared__ __align__(16) char nraw[];
   const int c = blockIdx.x, n = d.n, NL = d.n * d.L;
   const NNSmem s = nn_carve(n, nraw);
-  const NNFrags w = nn_build_frags(nn.wbf, s.frag, s.tcf);
+  build_cross(d, s.nbr);
+  const NNFrags w = nn_build_frags(nn.wbf, s.frag, s.tcf);  // (ends with a barrier)
   float* xf = nn.xf + (size_t)c * NL;
   to_inputs(Xall + (size_t)c * NL, nn.x0, xf, NL);
   const double F = fc_eval_all(d, s, w, xf, write_cache ? nn.fcache + (size_t)c * NL : nullptr);
@@ -169,28 +224,22 @@ __global__ void __launch_bounds__(HQ_THREADS) nn_eval_kernel(Dev d, NNState nn, 
 // The caches of the current fields (fc; with use_cnn also the convolutional activations) are
 // valid on entry; with use_cnn each network's cache is rebuilt before its part when the other
 // part has changed the fields.
-__global__ void __launch_bounds__(HQ_THREADS) nn_inner_kernel(Dev d, NNState nn, CnnState cn, int n_inner,
+__global__ void __launch_bounds__(HQ_THREADS, 2) nn_inner_kernel(Dev d, NNState nn, CnnState cn, int n_inner,
                                                               int do_local, int do_block, int use_cnn, int window,
                                                               int site_window) {
   extern __shared__ __align__(16) char nraw[];
   const int c = blockIdx.x, n = d.n, L = d.L, NL = n * L;
   if (!d.active[c]) return;
   const NNSmem s = nn_carve(n, nraw, use_cnn != 0);
-  for (int r = threadIdx.x; r < n; r += HQ_THREADS) {
-    const int x = r % d.nx, y = r / d.nx;
-    s.nbr[5 * r + 0] = r;
-    s.nbr[5 * r + 1] = (x + 1) % d.nx + d.nx * y;
-    s.nbr[5 * r + 2] = (x - 1 + d.nx) % d.nx + d.nx * y;
-    s.nbr[5 * r + 3] = x + d.nx * ((y + 1) % d.ny);
-    s.nbr[5 * r + 4] = x + d.nx * ((y - 1 + d.ny) % d.ny);
-  }
+  build_cross(d, s.nbr);
   const NNFrags w = nn_build_frags(nn.wbf, s.frag, s.tcf);  // (ends with a barrier)
   if (use_cnn) cn_load_weights(cn.wbf, s.cw);
   double* X = d.X + (size_t)c * NL;
   float* xf = nn.xf + (size_t)c * NL;  // inputs of the current fields, kept with X below
   to_inputs(X, nn.x0, xf, NL);
   float* fc = nn.fcache + (size_t)c * NL;
-  float* fnew = nn.fnew + (size_t)c * 5 * L;
+  float* fnew = nn.fnew + (size_t)c * 6 * L;
+  float* xsh = fnew + 5 * L;  // inputs of the moved site's proposed values (block moves)
   float *h1c = nullptr, *h2c = nullptr, *o3c = nullptr, *h1p = nullptr, *h2p = nullptr, *o3p = nullptr;
   if (use_cnn) {
     h1c = cn.h1c + (size_t)c * NL * CN_C;
@@ -205,7 +254,15 @@ __global__ void __launch_bounds__(HQ_THREADS) nn_inner_kernel(Dev d, NNState nn,
   const uint32_t key0 = id[0], key1 = id[1], chain = id[2], step = id[3];
   long long nl_acc = 0, nb_acc = 0;
   double path = 0.0;                   // thread 0
-  int any_local = 0;                   // thread 0: a local move was accepted in this part
+  const NNLane kin = nn_lane_inputs();
+  auto opposite = [](int c5) { return c5 == 0 ? 0 : (c5 & 1) ? c5 + 1 : c5 - 1; };
+  int pdl[2], opp[2];  // local moves: patch row g + 8h of the warp's tile
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int q = min(16 * ((warp >> 1) & 1) + g + 8 * h, 24);
+    pdl[h] = q / 5 - 2;
+    opp[h] = opposite(q % 5);
+  }
   bool fc_stale = false, cn_stale = false;  // uniform over the CTA
   const double kfac = d.mass / (2.0 * d.dtau), pfac = 0.5 * d.dtau * d.mass * (d.omega * d.omega);
   double du1, du2;
@@ -233,7 +290,8 @@ __global__ void __launch_bounds__(HQ_THREADS) nn_inner_kernel(Dev d, NNState nn,
     for (int part = 0; part < 2; ++part) {
     const bool local_part = (part == 0) == fwd;
     if (local_part && do_local) {
-      any_local = 0;
+      double lpath = 0.0;  // warp 1
+      int lacc = 0;
       if (fc_stale) {
         fc_eval_all(d, s, w, xf, fc);
         fc_stale = false;
@@ -253,63 +311,106 @@ __global__ void __launch_bounds__(HQ_THREADS) nn_inner_kernel(Dev d, NNState nn,
           s.pds[i] = kfac * kin + pfac * (xn * xn - xo * xo);
         }
         __syncthreads();
-        // The moves of the slice run in warp 0 alone: a move's 25 patches are two tensor-core
-        // tiles, its change of F a fixed-order warp sum, and the decision, the field and the
-        // patch cache are updated without a CTA barrier (the other warps wait for the slice).
-        if (warp == 0) {
-          for (int i0 = 0; i0 < n; ++i0) {
-            const int i = fwd ? i0 : n - 1 - i0;
-            const double xn = s.pxn[i];
-            // patch q = 5 (dl + 2) + c contains (sl, i): centre slice sl - dl, centre site the
-            // neighbour of i opposite to c (q >= 25: padding rows)
-            auto cslice = [&](int q) {
-              const int v = sl - (q / 5 - 2);
-              return v < 0 ? v + L : (v >= L ? v - L : v);
-            };
-            auto csite = [&](int q) {
-              const int c = q % 5;
-              return s.nbr[5 * i + (c == 0 ? 0 : (c & 1) ? c + 1 : c - 1)];
-            };
-            auto zv = [&](int q, int k) -> float {
-              q = q < 25 ? q : 24;
-              int ll = sl - (q / 5 - 2) + (k / 5 - 2);
-              ll = ll < 0 ? ll + L : (ll >= L ? ll - L : ll);
-              const int site = s.nbr[5 * csite(q) + k % 5];
-              return (ll == sl && site == i) ? s.pxf[i] : xf[(size_t)ll * n + site];
-            };
-            float fv[4];
-            nn_tile_f(w, [&](int row, int k) { return zv(row, k); }, fv[0], fv[1]);
-            nn_tile_f(w, [&](int row, int k) { return zv(16 + row, k); }, fv[2], fv[3]);
-            const int qs[4] = {g, g + 8, 16 + g, 24 + g};
-            double part = 0.0;
-            if (t == 0)
-              for (int a = 0; a < 4; ++a)
-                if (qs[a] < 25) part += (double)fv[a] - (double)fc[(size_t)cslice(qs[a]) * n + csite(qs[a])];
-            const double dF = warp_sum_fixed(part);
-            int acc = 0;
-            if (lane == 0) {
-              const double prob = exp(fmin(2.0 * dF - s.pds[i], 709.0));
-              acc = s.pu2[i] < prob;
-              if (acc) {
-                X[(size_t)sl * n + i] = xn;
-                xf[(size_t)sl * n + i] = s.pxf[i];
-                path += dF;
-                any_local = 1;
+        // The moves of the slice run in warps 0 .. 3 (the others wait for the slice): a move's 25
+        // patches are two tiles of 16, warps 2 tau and 2 tau + 1 take tile tau, both forming layer 1 and
+        // half of layer 2 each; the first hands its part of layer 3's chain to the second.  Warp 1
+        // sums dF and decides.  While it does, the inputs of the next move are already loaded; the one
+        // value that an acceptance changes is replaced after the decision.
+        if (warp < 4) {
+          const int tau = warp >> 1;
+          float z[2][8];
+          int pos[2][8];  // table position of every input of the move in hand
+          auto gather = [&](int i) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              // patch q = 5 (dl + 2) + c contains (sl, i): centre slice sl - dl, centre site the
+              // neighbour of i opposite to c (q >= 25: padding rows)
+              const int centre = s.nbr[5 * i + opp[h]];
+#pragma unroll
+              for (int q = 0; q < 8; ++q) {
+                pos[h][q] = kin.c[q] < 0 ? -1 : wrap_slice(sl - pdl[h] + kin.dl[q], L) * n + s.nbr[5 * centre + kin.c[q]];
+                z[h][q] = pos[h][q] < 0 ? 0.f : xf[pos[h][q]];
               }
-              nl_acc += acc;
             }
-            acc = __shfl_sync(HQ_FULL, acc, 0);
-            if (acc && t == 0)
-              for (int a = 0; a < 4; ++a)
-                if (qs[a] < 25) fc[(size_t)cslice(qs[a]) * n + csite(qs[a])] = fv[a];
-            __syncwarp();
+          };
+          const int ifirst = fwd ? 0 : n - 1, istep = fwd ? 1 : -1;
+          gather(ifirst);
+          for (int i0 = 0; i0 < n; ++i0) {
+            const int i = ifirst + istep * i0, here = sl * n + i;
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+              for (int q = 0; q < 8; ++q)
+                if (pos[h][q] == here) z[h][q] = s.pxf[i];
+            float acc1[8][4], acc2[4][4], o0 = 0.f, o1 = 0.f;
+            nn_layer1(w, z, acc1);
+            if (i0 + 1 < n) gather(i + istep);
+            if (!(warp & 1)) {
+              nn_layer2<0, 4>(w, acc1, acc2);
+              nn_layer3<0, 4>(w, acc2, o0, o1);
+              s.part[64 * tau + lane] = o0;
+              s.part[64 * tau + 32 + lane] = o1;
+              bar_arrive(2 + tau, 64);
+            } else {
+              nn_layer2<4, 4>(w, acc1, acc2);
+              bar_sync(2 + tau, 64);
+              o0 = s.part[64 * tau + lane];
+              o1 = s.part[64 * tau + 32 + lane];
+              nn_layer3<4, 4>(w, acc2, o0, o1);
+              o0 = nn_output(w, o0);
+              o1 = nn_output(w, o1);
+              if (t == 0) {
+                s.f25[16 * tau + g] = o0;
+                s.f25[16 * tau + g + 8] = o1;
+              }
+              if (warp == 3) {
+                bar_arrive(4, 64);
+              } else {
+                // lane q < 25: patch q
+                const bool on = lane < 25;
+                const int ql = lane / 5 - 2, qc = lane % 5;
+                const int at = on ? wrap_slice(sl - ql, L) * n + s.nbr[5 * i + (qc == 0 ? 0 : (qc & 1) ? qc + 1 : qc - 1)] : 0;
+                const float fold = on ? fc[at] : 0.f;
+                bar_sync(4, 64);
+                const float fnow = on ? s.f25[lane] : 0.f;
+                const double dF = warp_sum_diff(fnow, fold);
+                const int acc = metropolis(s.pu2[i], fmin(2.0 * dF - s.pds[i], 709.0));
+                if (acc && on) fc[at] = fnow;
+                if (lane == 0) {
+                  s.flag[0] = acc;
+                  if (acc) {
+                    X[(size_t)here] = s.pxn[i];
+                    xf[here] = s.pxf[i];
+                  }
+                }
+                if (acc) {
+                  lpath += dF;
+                  ++lacc;
+                }
+              }
+            }
+            bar_sync(1, 128);
+            if (s.flag[0] && i0 + 1 < n) {
+#pragma unroll
+              for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+                  if (pos[h][q] == here) z[h][q] = s.pxf[i];
+            }
           }
         }
         __syncthreads();
       }
-      if (threadIdx.x == 0) s.scal[3] = any_local;
+      if (threadIdx.x == 32) {
+        s.scal[3] = (double)lacc;
+        s.scal[4] = lpath;
+      }
       __syncthreads();
       if (s.scal[3] != 0.0) cn_stale = true;
+      if (threadIdx.x == 0) {
+        nl_acc += (long long)s.scal[3];
+        path += s.scal[4];
+      }
       __syncthreads();
     }
     if (!local_part && do_block) {
@@ -331,10 +432,10 @@ __global__ void __launch_bounds__(HQ_THREADS) nn_inner_kernel(Dev d, NNState nn,
         for (int sl = threadIdx.x; sl < L; sl += HQ_THREADS) {
           const double x = X[(size_t)sl * n + i];
           a += (x + dx) * (x + dx) - x * x;
+          xsh[sl] = net_input(x + dx, nn.x0);
         }
         a = block_sum(a, s.red);
         const double dS = pfac * a;
-        const int x = i % d.nx, y = i / d.nx;
         double dF;
         if (use_cnn) {
           cn_build_window(d, i, s.win);
@@ -342,30 +443,33 @@ __global__ void __launch_bounds__(HQ_THREADS) nn_inner_kernel(Dev d, NNState nn,
         } else {
           // the 5 L patches containing site i: patch q has centre (q / 5, i - c), c = q % 5; warp
           // w takes the tiles w, w + 8, ... of 16 patches
-          auto centre = [&](int q) {
-            const int cidx = q % 5, sl = q / 5;
-            const int cx_ = (cidx == 1) - (cidx == 2), cy_ = (cidx == 3) - (cidx == 4);
-            const int j = (x - cx_ + d.nx) % d.nx + d.nx * ((y - cy_ + d.ny) % d.ny);
-            return sl * n + j;
-          };
           double pt = 0.0;
           for (int base = warp * 16; base < 5 * L; base += HQ_WARPS * 16) {
-            float f0, f1;
-            nn_tile_f(w, [&](int row, int k) {
-              const int q = base + row < 5 * L ? base + row : 5 * L - 1;
-              const int r = centre(q);
-              const int pos = patch_pos(d, r / n, r % n, k);
-              return pos % n == i ? net_input(X[pos] + dx, nn.x0) : xf[pos];
-            }, f0, f1);
+            float f0, f1, z[2][8];
+            int at[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const int q = min(base + g + 8 * h, 5 * L - 1), l = q / 5, site = s.nbr[5 * i + opposite(q % 5)];
+              at[h] = l * n + site;
+#pragma unroll
+              for (int k = 0; k < 8; ++k) {
+                z[h][k] = 0.f;
+                if (kin.c[k] >= 0) {
+                  const int ll = wrap_slice(l + kin.dl[k], L), j = s.nbr[5 * site + kin.c[k]];
+                  z[h][k] = j == i ? xsh[ll] : xf[ll * n + j];
+                }
+              }
+            }
+            nn_tile_f(w, z, f0, f1);
             if (t == 0) {
               const int q0 = base + g, q1 = q0 + 8;
               if (q0 < 5 * L) {
                 fnew[q0] = f0;
-                pt += (double)f0 - (double)fc[centre(q0)];
+                pt += (double)f0 - (double)fc[at[0]];
               }
               if (q1 < 5 * L) {
                 fnew[q1] = f1;
-                pt += (double)f1 - (double)fc[centre(q1)];
+                pt += (double)f1 - (double)fc[at[1]];
               }
             }
           }
@@ -393,12 +497,8 @@ __global__ void __launch_bounds__(HQ_THREADS) nn_inner_kernel(Dev d, NNState nn,
             cn_block_commit(d, s.win, h1c, h2c, o3c, h1p, h2p, o3p);
             fc_stale = true;
           } else {
-            for (int q = threadIdx.x; q < 5 * L; q += HQ_THREADS) {
-              const int cidx = q % 5, sl = q / 5;
-              const int cx_ = (cidx == 1) - (cidx == 2), cy_ = (cidx == 3) - (cidx == 4);
-              const int j = (x - cx_ + d.nx) % d.nx + d.nx * ((y - cy_ + d.ny) % d.ny);
-              fc[(size_t)sl * n + j] = fnew[q];
-            }
+            for (int q = threadIdx.x; q < 5 * L; q += HQ_THREADS)
+              fc[(q / 5) * n + s.nbr[5 * i + opposite(q % 5)]] = fnew[q];
           }
         }
         __syncthreads();
@@ -464,7 +564,8 @@ __global__ void __launch_bounds__(HQ_THREADS) nn_batch_forward_kernel(Dev d, NNS
   extern __shared__ __align__(16) char nraw[];
   const int a = blockIdx.x, n = d.n, NL = d.n * d.L;
   const NNSmem s = nn_carve(n, nraw);
-  const NNFrags w = nn_build_frags(nn.wbf, s.frag, s.tcf);
+  build_cross(d, s.nbr);
+  const NNFrags w = nn_build_frags(nn.wbf, s.frag, s.tcf);  // (ends with a barrier)
   float* xa = nn.xb + (size_t)a * NL;  // read again by the backward pass
   to_inputs(Xs + (size_t)idx[a] * NL, nn.x0, xa, NL);
   const double F = fc_eval_all(d, s, w, xa, nullptr);
@@ -492,6 +593,9 @@ __global__ void __launch_bounds__(HQ_THREADS) nn_batch_backward_tc_kernel(Dev d,
   uint16_t* zl = zh + TC_K1 * TR_LD;
   uint16_t* d1h = zl + TC_K1 * TR_LD;
   uint16_t* d1l = d1h + TC_H * TR_LD;
+  int* nbr = (int*)(d1l + TC_H * TR_LD);
+  build_cross(d, nbr);
+  const NNLane kin = nn_lane_inputs();
   const NNFrags w = nn_build_frags(nn.wbf, frag, tcf);
   // W2^T fragments for d1 = d2 W2^T: B[k = u][n = v] = W2[v][u]
   uint2* w2t = frag + TC_FRAGS;
@@ -529,6 +633,13 @@ __global__ void __launch_bounds__(HQ_THREADS) nn_batch_backward_tc_kernel(Dev d,
     for (int j = 0; j < 8; ++j)
 #pragma unroll
       for (int e = 0; e < 4; ++e) acc1[j][e] = acc2[j][e] = 0.f;
+    float z[2][8];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      int a, pr;
+      rowpos(g + 8 * h, a, pr);  // the minibatch inputs of the forward kernel
+      patch_inputs(d, kin, nbr, nn.xb + (size_t)a * NL, pr / n, pr % n, z[h]);
+    }
 #pragma unroll
     for (int st = 0; st < 2; ++st) {
       uint32_t ahi[4], alo[4];
@@ -536,12 +647,7 @@ __global__ void __launch_bounds__(HQ_THREADS) nn_batch_backward_tc_kernel(Dev d,
       for (int q = 0; q < 4; ++q) {
         const int row = g + 8 * (q & 1);
         const int k = 16 * st + 2 * t + 8 * (q >> 1);
-        int a, pr;
-        rowpos(row, a, pr);
-        const float* xa = nn.xb + (size_t)a * NL;  // the minibatch inputs of the forward kernel
-        const float v0 = k < TC_IN ? xa[patch_pos(d, pr / n, pr % n, k)] : 0.f;
-        const float v1 = k + 1 < TC_IN ? xa[patch_pos(d, pr / n, pr % n, k + 1)] : 0.f;
-        split2(v0, v1, ahi[q], alo[q]);
+        split2(z[q & 1][4 * st + 2 * (q >> 1)], z[q & 1][4 * st + 2 * (q >> 1) + 1], ahi[q], alo[q]);
         // z^T staging (rows k >= 25 are zero)
         zh[k * TR_LD + 16 * warp + row] = (uint16_t)(ahi[q] & 0xffffu);
         zl[k * TR_LD + 16 * warp + row] = (uint16_t)(alo[q] & 0xffffu);

@@ -96,13 +96,28 @@ __device__ __forceinline__ void split2(float v0, float v1, uint32_t& hi, uint32_
   lo = pack_bf16(l0, l1);
 }
 
-// f of 16 patches by one warp.  zval(row, k) gives input k (0..24) of patch row (0..15) as a
-// float; it is called for k < 25 only.  Returns f of row g in f_g and of row g + 8 in f_g8
-// (g = lane / 4; every lane of the quad holds them).
-template <class ZF>
-__device__ __forceinline__ void nn_tile_f(const NNFrags& w, ZF zval, float& f_g, float& f_g8) {
-  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  float acc1[8][4];
+// The eight inputs k of a lane in layer 1's A fragments, q = 4 s + 2 half + p: k = 16 s + 2t + 8 half + p,
+// as slice offset dl = k / 5 - 2 and cross point c = k % 5 (k >= 25: padding, c = -1).  They are the same
+// for every tile, so index arithmetic on k is done once per kernel.
+struct NNLane {
+  int dl[8], c[8];
+};
+
+__device__ __forceinline__ NNLane nn_lane_inputs() {
+  const int t = threadIdx.x & 3;
+  NNLane n;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int k = 16 * (q >> 2) + 2 * t + 8 * ((q >> 1) & 1) + (q & 1);
+    n.dl[q] = k / 5 - 2;
+    n.c[q] = k < TC_IN ? k % 5 : -1;
+  }
+  return n;
+}
+
+// Layer 1 of a tile: acc1 = z W1.  z[h][q]: input q (NNLane order) of row g + 8h, zero for padding.
+__device__ __forceinline__ void nn_layer1(const NNFrags& w, const float (&z)[2][8], float (&acc1)[8][4]) {
+  const int lane = threadIdx.x & 31;
 #pragma unroll
   for (int j = 0; j < 8; ++j)
 #pragma unroll
@@ -111,13 +126,7 @@ __device__ __forceinline__ void nn_tile_f(const NNFrags& w, ZF zval, float& f_g,
   for (int s = 0; s < 2; ++s) {
     uint32_t ahi[4], alo[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int row = g + 8 * (q & 1);
-      const int k = 16 * s + 2 * t + 8 * (q >> 1);
-      const float v0 = k < TC_IN ? zval(row, k) : 0.f;
-      const float v1 = k + 1 < TC_IN ? zval(row, k + 1) : 0.f;
-      split2(v0, v1, ahi[q], alo[q]);
-    }
+    for (int q = 0; q < 4; ++q) split2(z[q & 1][4 * s + 2 * (q >> 1)], z[q & 1][4 * s + 2 * (q >> 1) + 1], ahi[q], alo[q]);
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const uint2 b = w.w1[(s * 8 + j) * 32 + lane];
@@ -125,9 +134,14 @@ __device__ __forceinline__ void nn_tile_f(const NNFrags& w, ZF zval, float& f_g,
       mma_bf16(acc1[j], alo, b);
     }
   }
-  float acc2[8][4];
+}
+
+// n-tiles J0 .. J0 + NJ - 1 of layer 2 from layer 1's accumulators.
+template <int J0, int NJ>
+__device__ __forceinline__ void nn_layer2(const NNFrags& w, const float (&acc1)[8][4], float (&acc2)[NJ][4]) {
+  const int lane = threadIdx.x & 31, t = lane & 3;
 #pragma unroll
-  for (int j = 0; j < 8; ++j)
+  for (int j = 0; j < NJ; ++j)
 #pragma unroll
     for (int e = 0; e < 4; ++e) acc2[j][e] = 0.f;
 #pragma unroll
@@ -142,28 +156,45 @@ __device__ __forceinline__ void nn_tile_f(const NNFrags& w, ZF zval, float& f_g,
       split2(fmaxf(acc1[j][2] + bb0, 0.f), fmaxf(acc1[j][3] + bb1, 0.f), ahi[2 * half + 1], alo[2 * half + 1]);
     }
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const uint2 b = w.w2[(s * 8 + j) * 32 + lane];
+    for (int j = 0; j < NJ; ++j) {
+      const uint2 b = w.w2[(s * 8 + J0 + j) * 32 + lane];
       mma_bf16(acc2[j], ahi, b);
       mma_bf16(acc2[j], alo, b);
     }
   }
-  float o0 = 0.f, o1 = 0.f;
+}
+
+// Layer 3's chain over n-tiles J0 .. J0 + NJ - 1, onto o0 (row g) and o1 (row g + 8): every evaluation
+// runs it in ascending order of the tiles, in one piece or handed from warp to warp.
+template <int J0, int NJ>
+__device__ __forceinline__ void nn_layer3(const NNFrags& w, const float (&acc2)[NJ][4], float& o0, float& o1) {
+  const int t = threadIdx.x & 3;
 #pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const int u = 8 * j + 2 * t;
+  for (int j = 0; j < NJ; ++j) {
+    const int u = 8 * (J0 + j) + 2 * t;
     const float bb0 = w.b2[u], bb1 = w.b2[u + 1], w0 = w.w3[u], w1 = w.w3[u + 1];
     o0 = fmaf(fmaxf(acc2[j][0] + bb0, 0.f), w0, o0);
     o0 = fmaf(fmaxf(acc2[j][1] + bb1, 0.f), w1, o0);
     o1 = fmaf(fmaxf(acc2[j][2] + bb0, 0.f), w0, o1);
     o1 = fmaf(fmaxf(acc2[j][3] + bb1, 0.f), w1, o1);
   }
-  o0 += __shfl_xor_sync(HQ_FULL, o0, 1);
-  o0 += __shfl_xor_sync(HQ_FULL, o0, 2);
-  o1 += __shfl_xor_sync(HQ_FULL, o1, 1);
-  o1 += __shfl_xor_sync(HQ_FULL, o1, 2);
-  f_g = o0 + w.b3;
-  f_g8 = o1 + w.b3;
+}
+
+__device__ __forceinline__ float nn_output(const NNFrags& w, float o) {
+  o += __shfl_xor_sync(HQ_FULL, o, 1);
+  o += __shfl_xor_sync(HQ_FULL, o, 2);
+  return o + w.b3;
+}
+
+// f of 16 patches by one warp from its inputs (nn_layer1's order): row g in f_g and row g + 8 in f_g8
+// (every lane of the quad holds them).
+__device__ __forceinline__ void nn_tile_f(const NNFrags& w, const float (&z)[2][8], float& f_g, float& f_g8) {
+  float acc1[8][4], acc2[8][4], o0 = 0.f, o1 = 0.f;
+  nn_layer1(w, z, acc1);
+  nn_layer2<0, 8>(w, acc1, acc2);
+  nn_layer3<0, 8>(w, acc2, o0, o1);
+  f_g = nn_output(w, o0);
+  f_g8 = nn_output(w, o1);
 }
 
 }  // namespace hq
@@ -188,7 +219,7 @@ constexpr int TR_FRAGS = TC_FRAGS + 4 * 8 * 32;  // + W2^T fragments
 
 __host__ __device__ inline size_t nn_train_tc_smem_bytes() {
   return sizeof(uint2) * TR_FRAGS + sizeof(float) * (TC_FLOATS + 3 * 8 * TC_H + 8) +
-         sizeof(uint16_t) * (size_t)TR_LD * (2 * TC_H + 2 * TC_H + 2 * TC_K1 + 2 * TC_H);
+         sizeof(uint16_t) * (size_t)TR_LD * (2 * TC_H + 2 * TC_H + 2 * TC_K1 + 2 * TC_H) + sizeof(int) * 5 * 256;
 }
 
 __device__ __forceinline__ void split1(float v, uint16_t& hi, uint16_t& lo) {

@@ -1,0 +1,379 @@
+// Dense linear algebra of a chain with its contractions on the tensor cores (hq_oz.cuh): blocked QR and Q formation, the triangular factor, LU and solves, products.
+// Column-major n x n matrices with stride ld = n (a multiple of 4, so that row pairs are 16-byte
+// aligned), one CTA per matrix.  What stays on the FP64 pipe is O(n^2) or narrow: panels of 16
+// columns, 16 x 16 triangles, scalings.
+#pragma once
+#include "hq_device.cuh"
+#include "hq_oz.cuh"
+#include "hq_lu.cuh"
+#include "hq_panel.cuh"
+
+namespace hq {
+
+// Rows of a staged block: 64, or 32 where 64 rows of n terms would not fit beside the rest.
+__host__ __device__ constexpr int oz_rows(int n) { return n <= 160 ? 64 : 32; }
+__host__ __device__ constexpr int oz_pad(int n) { return (n + 15) & ~15; }
+// bytes of the fragment scratch: a staged row block, or a QR panel in both fragment orders plus T
+__host__ __device__ constexpr size_t oz_frag_bytes(int n) {
+  return (size_t)oz_pad(n) * oz_rows(n) * 12 + 2 * 6 * 32 * 8;
+}
+
+struct OzScratch {
+  uint2* frag;   // oz_frag_bytes(n)
+  int* er;       // [oz_pad(n)] row bounds
+  int* ec;       // [oz_pad(n)] column bounds
+  double* tall;  // [oz_pad(n) / 16][16][16] triangular factors T of the QR panels
+  double* ws;    // [16][16]
+  int* ev;       // [oz_pad(n)] bounds of the reflector vectors
+  int n;
+};
+
+// Scratch of the QR: reflector scalars, 1 / D, pivot order.
+struct QrScratch {
+  double* tau;   // [16]
+  double* rinv;  // [n] 1 / D
+  int* perm;     // [n] perm[j] = original column placed at position j
+};
+
+struct RowPair {
+  double v0, v1;
+};
+__device__ __forceinline__ RowPair load_pair(const double* p) {
+  const double2 v = *reinterpret_cast<const double2*>(p);
+  return {v.x, v.y};
+}
+__device__ __forceinline__ void store_pair(double* p, double a, double b) {
+  *reinterpret_cast<double2*>(p) = make_double2(a, b);
+}
+
+// ---------------------------------------------------------------------- blocked QR
+// Column-pivoted QR in the form used for DQMC stabilisation by Bauer (SciPost Phys. Core 2,
+// 011 (2020)): the columns are ordered once by decreasing Euclidean norm, then factored by
+// unpivoted Householder QR.  The product being factored is column-graded (B..B U D), so the
+// one-time ordering gives the graded R that the UDV decomposition needs, without per-step
+// pivot searches and norm downdates.
+
+// Q <- columns of P ordered by decreasing norm (stable: ties keep index order); perm records the order.
+// Norms are compared through their IEEE bit patterns, which order non-negative doubles exactly like their
+// values.  norm2: n doubles of scratch.
+__device__ inline void prepivot(const double* P, double* Q, int ld, int n, const QrScratch& s, double* norm2) {
+  const int g = threadIdx.x >> 2, sub = threadIdx.x & 3;
+  for (int base = 0; base < n; base += HQ_THREADS / 4) {
+    const int c = base + g;
+    double a = 0.0;
+    if (c < n) {
+      const double* col = P + (size_t)c * ld;
+      for (int r = sub; r < n; r += 4) a = fma(col[r], col[r], a);
+    }
+    a = group_sum<4>(a);
+    if (c < n && sub == 0) norm2[c] = a;
+  }
+  __syncthreads();
+  for (int c = threadIdx.x; c < n; c += HQ_THREADS) {
+    const long long mine = __double_as_longlong(norm2[c]);
+    int rank = 0;
+    for (int o = 0; o < n; ++o) {
+      const long long other = __double_as_longlong(norm2[o]);
+      rank += (other > mine) || (other == mine && o < c);
+    }
+    s.perm[rank] = c;
+  }
+  __syncthreads();
+  for (int idx = threadIdx.x; idx < n * n; idx += HQ_THREADS) {
+    const int r = idx % n, j = idx / n;
+    Q[(size_t)j * ld + r] = P[(size_t)s.perm[j] * ld + r];
+  }
+  __syncthreads();
+}
+
+// Panel of kb <= 16 columns from j0 and its T factor; leaves the panel's row-term fragments in z.frag.
+template <int LM>
+__device__ __noinline__ void oz_panel(double* Q, double* V, int ld, int n, int j0, int kb, double* tau,
+                                      const OzScratch& z) {
+  PanelShared* ps = reinterpret_cast<PanelShared*>(z.frag);
+  const int m = n - j0;
+  if (LM <= 8 || m <= 64) panel_fixed<LM, 4>(Q, V, ld, n, j0, kb, ps, tau, z.ev);  // LM <= 8: n <= 64
+  else if (m <= 128) panel_fixed<LM, LM <= 8 ? 4 : 8>(Q, V, ld, n, j0, kb, ps, tau, z.ev);
+  else panel_fixed<LM, LM <= 8 ? 4 : 16>(Q, V, ld, n, j0, kb, ps, tau, z.ev);
+  stage_panel(z.frag, V, ld, n, j0, kb, z.ev);
+  // the sums go behind the fragments, where the block application stages T
+  const int nk = (m + 15) >> 4;
+  panel_t(z.frag, nk, kb, tau, z.ev + j0, reinterpret_cast<unsigned long long*>(z.frag + (size_t)nk * 2 * kOzDigits * 32),
+          z.ws, z.tall + (j0 >> 4) * 256);
+}
+
+// The reflectors in columns j0 .. j1 - 1 of V (zero above their first row) applied at once to columns c0 .. cend - 1, rows j0 .. n - 1, of A:
+//   kTrans:  A <- (I - V T V^T)^T A     (trailing update of the QR)
+//   !kTrans: A <- (I - V T V^T) A       (Q formation)
+// A warp takes 16 columns and runs W^T = A^T V, Z^T = W^T T (or W^T T^T) and A^T -= Z^T V^T back to back:
+// each result leaves the accumulators in the layout of the next left operand, so nothing but V's
+// and T's fragments is shared and A is read and written in place.  With fewer column groups than
+// warps, several warps form W of the same columns and share out the rows of the update.  kTrans follows
+// oz_panel, which has left V's row-term fragments in place.
+template <int LM, bool kTrans>
+__device__ __noinline__ void oz_wy_apply(const double* V, int ld, int n, int j0, int j1, const double* T, double* A,
+                                         int c0, int cend, const OzScratch& z) {
+  const int kb = j1 - j0, nr = n - j0, nk = (nr + 15) >> 4;
+  uint2* vk = z.frag;
+  uint2* vn = vk + (size_t)nk * 2 * kOzDigits * 32;
+  uint2* tf = vn + (size_t)nk * 2 * kOzDigits * 32;
+  int* et = z.ec;  // [16]
+  auto v = [&](int rr, int k) { return (k < kb && rr < nr) ? V[(size_t)(j0 + k) * ld + j0 + rr] : 0.0; };
+  auto evk = [&](int k) { return k < kb ? z.ev[j0 + k] : 128; };
+  if (!kTrans) stage_panel(vk, V, ld, n, j0, kb, z.ev);
+  oz_stage_rows(vn, z.er, nr, 16, [&](int r, int k) { return v(r, k); });
+  oz_stage_rows(tf, et, 16, 16, [&](int r, int k) { return kTrans ? T[k * 16 + r] : T[r * 16 + k]; });
+  __syncthreads();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const int ncg = (cend - c0 + 15) >> 4;
+  const int parts = ncg >= HQ_WARPS ? 1 : HQ_WARPS / ncg;
+  const int rp = ((nr + parts - 1) / parts + 7) & ~7;
+  for (int unit = warp; unit < ((ncg * parts + HQ_WARPS - 1) / HQ_WARPS) * HQ_WARPS; unit += HQ_WARPS) {
+    const bool work = unit < ncg * parts;
+    const int ca = c0 + (unit % ncg) * 16 + g, cb = ca + 8, rb = work ? (unit / ncg) * rp : nr;
+    const double* pa = A + (size_t)(ca < cend ? ca : c0) * ld + j0;
+    const double* pb = A + (size_t)(cb < cend ? cb : c0) * ld + j0;
+    uint32_t a[4][kOzDigits];
+    int E[2] = {128, 128};
+    if (work && rb < nr) {
+      uint32_t ma = 0, mb = 0;
+      for (int r = 2 * t; r < nr; r += 8) {
+        const RowPair x = load_pair(pa + r), y = load_pair(pb + r);
+        ma = max(ma, max(oz_abs_hi(x.v0), oz_abs_hi(x.v1)));
+        mb = max(mb, max(oz_abs_hi(y.v0), oz_abs_hi(y.v1)));
+      }
+      ma = max(ma, __shfl_xor_sync(HQ_FULL, ma, 1));
+      mb = max(mb, __shfl_xor_sync(HQ_FULL, mb, 1));
+      ma = max(ma, __shfl_xor_sync(HQ_FULL, ma, 2));
+      mb = max(mb, __shfl_xor_sync(HQ_FULL, mb, 2));
+      E[0] = oz_bound(ma);
+      E[1] = oz_bound(mb);
+      // W^T: sums over up to 256 rows fit one accumulator, because |v|^2 < 16 bounds the sum by
+      // 4 sqrt(n) times the column's largest entry
+      long long Tw[2][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}};
+      for (int ks = 0; ks < nk; ++ks) {
+        const int r = 16 * ks + 2 * t;
+        const RowPair z0{0.0, 0.0};
+        const RowPair x0 = r < nr ? load_pair(pa + r) : z0, x1 = r < nr ? load_pair(pb + r) : z0;
+        const RowPair x2 = r + 8 < nr ? load_pair(pa + r + 8) : z0, x3 = r + 8 < nr ? load_pair(pb + r + 8) : z0;
+        oz_split<kOzP>(x0.v0, x0.v1, E[0], E[0], a[0]);
+        oz_split<kOzP>(x1.v0, x1.v1, E[1], E[1], a[1]);
+        oz_split<kOzP>(x2.v0, x2.v1, E[0], E[0], a[2]);
+        oz_split<kOzP>(x3.v0, x3.v1, E[1], E[1], a[3]);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const uint2* fr = vk + (size_t)(ks * 2 + j) * kOzDigits * 32 + lane;
+          oz_mma(a, [&](int d) { return fr[d * 32]; }, Tw[j]);
+        }
+      }
+      double w[2][4];
+#pragma unroll
+      for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) w[j][e] = oz_scale((double)Tw[j][e], oz_expo<kOzP>(evk(8 * j + 2 * t + (e & 1)), E[e >> 1]));
+      oz_left_from_acc(w, a, E);
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        long long Tz[4] = {0, 0, 0, 0};
+        const uint2* fr = tf + (size_t)j * kOzDigits * 32 + lane;
+        oz_mma(a, [&](int d) { return fr[d * 32]; }, Tz);
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          w[j][e] = oz_scale((double)Tz[e], oz_expo<kOzP>(et[8 * j + 2 * t + (e & 1)], E[e >> 1]));
+      }
+      oz_left_from_acc(w, a, E);
+    }
+    if (parts > 1) __syncthreads();  // W of every warp is formed before rows change
+    if (work && rb < nr)
+      oz_apply_rows(vn + (size_t)(rb >> 3) * kOzDigits * 32, z.er + rb, min(rp, nr - rb), a, E, ca, cb, cend,
+                    [&](int r, int c, double s0, double s1) {
+                      double* p = A + (size_t)c * ld + j0 + rb + r;
+                      const RowPair x = load_pair(p);
+                      store_pair(p, x.v0 - s0, x.v1 - s1);
+                    });
+  }
+  __syncthreads();
+}
+
+// Householder QR in panels of 16 columns; the trailing columns take each panel's reflectors as one
+// block.  R goes to the upper triangle of Q (below it Q is left undefined), the reflector vectors to V,
+// and the panels' T factors are kept for the Q formation.
+template <int LM>
+__device__ inline void oz_qr(double* Q, double* V, int ld, int n, const QrScratch& s, const OzScratch& z) {
+  for (int j0 = 0; j0 < n; j0 += 16) {
+    const int j1 = min(j0 + 16, n);
+    oz_panel<LM>(Q, V, ld, n, j0, j1 - j0, s.tau, z);
+    if (j1 < n) oz_wy_apply<LM, true>(V, ld, n, j0, j1, z.tall + (j0 >> 4) * 256, Q, j1, n, z);
+  }
+}
+
+// U <- H_0 ... H_{n-1}: the panels' blocks applied to the identity, last panel first (columns left
+// of a panel are still unit vectors there).
+template <int LM>
+__device__ inline void oz_form_q(const double* V, int ld, int n, double* U, const OzScratch& z) {
+  set_identity(U, ld, n);
+  __syncthreads();
+  for (int j0 = ((n - 1) >> 4) << 4; j0 >= 0; j0 -= 16)
+    oz_wy_apply<LM, false>(V, ld, n, j0, min(j0 + 16, n), z.tall + (j0 >> 4) * 256, U, j0, n, z);
+}
+
+// Tout = D^-1 R (rows of Tprev in pivot order): T' Tprev with T' = D^-1 R Pi^T.
+template <int LM, bool kWide>
+__device__ __noinline__ void oz_t_product(const double* P, int n, const int* perm, const double* rinv,
+                                          const double* Tprev, double* Tout, const OzScratch& z) {
+  auto fr = [&](int r, int k) { return k >= r ? P[(size_t)k * n + r] * rinv[r] : 0.0; };
+  oz_row_bounds(n, n, z.er, fr);
+  oz_col_bounds(Tprev, n, n, n, z.ec);
+  __syncthreads();
+  oz_gemm<kWide, true>(
+      n, n, n, oz_rows(n), z.frag, fr, [&](int r) { return z.er[r]; },
+      [&](int k, int c) { return Tprev[(size_t)c * n + perm[k]]; }, [&](int c) { return z.ec[c]; },
+      [&](int r, int c, double v0, double v1) { store_pair(Tout + (size_t)c * n + r, v0, v1); });
+}
+
+template <int LM>
+__device__ inline void oz_t_update(const double* P, int n, const QrScratch& s, double* D, const double* Tprev,
+                                   double* Tout, const OzScratch& z) {
+  for (int j = threadIdx.x; j < n; j += HQ_THREADS) {
+    const double dj = fabs(P[(size_t)j * n + j]);
+    D[j] = dj;
+    s.rinv[j] = 1.0 / dj;
+  }
+  __syncthreads();
+  if (Tprev == nullptr) {
+    for (int idx = threadIdx.x; idx < n * n; idx += HQ_THREADS) {
+      const int j = idx % n, c = idx / n;
+      Tout[(size_t)s.perm[c] * n + j] = (c >= j) ? P[(size_t)c * n + j] * s.rinv[j] : 0.0;
+    }
+    __syncthreads();
+  } else if (LM > 8 && n > 64) {
+    oz_t_product<LM, true>(P, n, s.perm, s.rinv, Tprev, Tout, z);
+  } else {
+    oz_t_product<LM, false>(P, n, s.perm, s.rinv, Tprev, Tout, z);
+  }
+}
+
+// C = op(A) op(B) diag(cd) (cd may be null), optionally with B's rows scaled by kd first.
+template <int LM, bool kWide, bool TA, bool TB>
+__device__ __noinline__ void oz_product_mm(int n, const double* A, const double* B, const double* kd, const double* cd,
+                                           double* C, const OzScratch& z) {
+  auto fa = [&](int r, int k) { return TA ? A[(size_t)r * n + k] : A[(size_t)k * n + r]; };
+  auto fb = [&](int k, int c) {
+    const double v = TB ? B[(size_t)k * n + c] : B[(size_t)c * n + k];
+    return kd ? v * kd[k] : v;
+  };
+  if (TA) oz_col_bounds(A, n, n, n, z.er);
+  else oz_row_bounds(n, n, z.er, fa);
+  if (TB) oz_row_bounds(n, n, z.ec, [&](int c, int k) { return fb(k, c); });
+  else if (kd) oz_row_bounds(n, n, z.ec, [&](int c, int k) { return fb(k, c); });
+  else oz_col_bounds(B, n, n, n, z.ec);
+  __syncthreads();
+  oz_gemm<kWide, false>(
+      n, n, n, oz_rows(n), z.frag, fa, [&](int r) { return z.er[r]; }, fb, [&](int c) { return z.ec[c]; },
+      [&](int r, int c, double v0, double v1) {
+        if (cd) {
+          v0 *= cd[c];
+          v1 *= cd[c];
+        }
+        store_pair(C + (size_t)c * n + r, v0, v1);
+      });
+}
+
+template <int LM, bool TA, bool TB>
+__device__ inline void oz_mm(int n, const double* A, const double* B, const double* kd, const double* cd, double* C,
+                             const OzScratch& z) {
+  if (LM > 8 && n > 64) oz_product_mm<LM, true, TA, TB>(n, A, B, kd, cd, C, z);
+  else oz_product_mm<LM, false, TA, TB>(n, A, B, kd, cd, C, z);
+}
+
+// Flush of delayed updates: G(r, c) += sum_m A[m][r] B[m][c], m < kk (A, B [kk][n]).
+template <int LM>
+__device__ __noinline__ void oz_flush(double* G, const double* A, const double* B, int n, int kk, const OzScratch& z) {
+  for (int m0 = 0; m0 < kk; m0 += 16)
+    oz_rank16<false>(0, n, 0, n, min(16, kk - m0), z.frag, z.er, [&](int r, int k) { return A[(size_t)(m0 + k) * n + r]; },
+              [&](int k, int c) { return B[(size_t)(m0 + k) * n + c]; },
+              [&](int r, int c, double s0, double s1) {
+                double* p = G + (size_t)c * n + r;
+                const RowPair x = load_pair(p);
+                store_pair(p, x.v0 + s0, x.v1 + s1);
+              });
+}
+
+// ------------------------------------------------------------ separable propagator
+// P <- the product of `count` slice matrices times the start: identity, or with U its columns times D.
+//   kAfter:  P <- diag(d_k) E P per slice (B^T = exp(-dtau V) exp(-dtau K), top-down products)
+//   !kAfter: P <- E diag(d_k) P           (B = exp(-dtau K) exp(-dtau V))
+// dv(k, r): diagonal entry r of the k-th slice applied.  A warp keeps its columns in registers through
+// all slices; dbuf holds the diagonals of `cap` slices at a time.
+template <bool kAfter, class DV>
+__device__ __forceinline__ void oz_slices(int nx, int ny, int n, const OzKin& K, double* P, const double* U,
+                                          const double* D, int count, DV dv, double* dbuf, int cap) {
+  for (int k0 = 0; k0 < count; k0 += cap) {
+    const int m = min(cap, count - k0);
+    __syncthreads();
+    for (int idx = threadIdx.x; idx < m * n; idx += HQ_THREADS) dbuf[idx] = dv(k0 + idx / n, idx % n);
+    __syncthreads();
+    oz_kin_lines(
+        nx, ny, n,
+        [&](int c, int i, double& v0, double& v1) {
+          if (k0 > 0) {
+            const RowPair p = load_pair(P + (size_t)c * n + i);
+            v0 = p.v0;
+            v1 = p.v1;
+          } else if (U) {
+            const RowPair p = load_pair(U + (size_t)c * n + i);
+            v0 = p.v0 * D[c];
+            v1 = p.v1 * D[c];
+          } else {
+            v0 = i == c ? 1.0 : 0.0;
+            v1 = i + 1 == c ? 1.0 : 0.0;
+          }
+        },
+        [&](double (&z)[2][4], bool two_x, bool two_y, auto visit) {
+          for (int k = 0; k < m; ++k) {
+            const double* dk = dbuf + k * n;
+            auto scale = [&](bool on, int, int i, double& v0, double& v1) {
+              if (on) {
+                v0 *= dk[i];
+                v1 *= dk[i + 1];
+              }
+            };
+            if (!kAfter) visit(scale);
+            oz_kin_tile(K, z, two_x, two_y);
+            if (kAfter) visit(scale);
+          }
+        },
+        [&](int c, int i, double v0, double v1) { store_pair(P + (size_t)c * n + i, v0, v1); });
+  }
+  __syncthreads();
+}
+
+// G <- E diag(d) G diag(rd) E^-1 (the wrap; F the fragments of E, Fi those of E^-1).
+template <int LM>
+__device__ __noinline__ void oz_wrap(int nx, int ny, int n, const OzKin& F, const OzKin& Fi, double* G, const double* d,
+                                     const double* rd) {
+  oz_kin_lines(
+      nx, ny, n,
+      [&](int c, int i, double& v0, double& v1) {
+        const RowPair p = load_pair(G + (size_t)c * n + i);
+        v0 = (d[i] * p.v0) * rd[c];
+        v1 = (d[i + 1] * p.v1) * rd[c];
+      },
+      [&](double (&z)[2][4], bool two_x, bool two_y, auto) { oz_kin_tile(F, z, two_x, two_y); },
+      [&](int c, int i, double v0, double v1) { store_pair(G + (size_t)c * n + i, v0, v1); });
+  __syncthreads();
+  oz_kin_lines(
+      nx, ny, n,
+      [&](int r, int i, double& v0, double& v1) {
+        v0 = G[(size_t)i * n + r];
+        v1 = G[(size_t)(i + 1) * n + r];
+      },
+      [&](double (&z)[2][4], bool two_x, bool two_y, auto) { oz_kin_tile(Fi, z, two_x, two_y); },
+      [&](int r, int i, double v0, double v1) {
+        G[(size_t)i * n + r] = v0;
+        G[(size_t)(i + 1) * n + r] = v1;
+      });
+  __syncthreads();
+}
+
+}  // namespace hq
