@@ -163,6 +163,12 @@ __device__ __noinline__ void slice_product(const Dev& d, const Smem& sm, double*
                                            int count, SliceDiag src) {
   const int n = d.n;
   HQ_TIC(kin);
+  if (n <= kTiny) {
+    tiny_slices<kAfter>(d.nx, d.ny, n, sm.ex, sm.ey, P, U, D, count, [&](int k, int r) { return src(d, k, r); },
+                        reinterpret_cast<double*>(sm.oz.frag));
+    HQ_TOC(kin, SEC_KIN);
+    return;
+  }
   const int cap = (int)(oz_frag_bytes(n) / (sizeof(double) * n));
   oz_slices<kAfter>(d.nx, d.ny, n, sm.kf, P, U, D, count, [&](int k, int r) { return src(d, k, r); },
                     reinterpret_cast<double*>(sm.oz.frag), cap);

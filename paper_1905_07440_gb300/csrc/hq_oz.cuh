@@ -162,33 +162,37 @@ __device__ __forceinline__ uint32_t oz_trans8x8(uint32_t v) {
 }
 
 // --------------------------------------------------------------- line exponents
-// e[c] = bound of column c of a rows x cols matrix (one warp per column).  No barrier.
-__device__ inline void oz_col_bounds(const double* A, int ld, int rows, int cols, int* e) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int c = warp; c < cols; c += HQ_WARPS) {
-    uint32_t m = 0;
-    for (int r = lane; r < rows; r += 32) m = max(m, oz_abs_hi(A[(size_t)c * ld + r]));
-    m = __reduce_max_sync(HQ_FULL, m);
-    if (lane == 0) e[c] = oz_bound(m);
-  }
-}
-
-// e[r] = bound of row r, f(r, k) for k0(r) <= k < K; e must not be read before the closing barrier.
+// e[r] = bound of line r (0 <= r < lines) over its K entries f(r, k).  along_k: consecutive k are consecutive
+// in memory (a warp per line), else consecutive lines are (a thread per line, K shared out).  Ends with a
+// barrier.
 template <class F>
-__device__ inline void oz_row_bounds(int rows, int K, int* e, F f) {
+__device__ inline void oz_line_bounds(bool along_k, int lines, int K, int* e, F f) {
+  if (along_k) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll 1
+    for (int r = warp; r < lines; r += HQ_WARPS) {
+      uint32_t m = 0;
+#pragma unroll 2
+      for (int k = lane; k < K; k += 32) m = max(m, oz_abs_hi(f(r, k)));
+      m = __reduce_max_sync(HQ_FULL, m);
+      if (lane == 0) e[r] = oz_bound(m);
+    }
+    __syncthreads();
+    return;
+  }
   uint32_t* m = reinterpret_cast<uint32_t*>(e);
-  for (int r = threadIdx.x; r < rows; r += HQ_THREADS) m[r] = 0;
+  for (int r = threadIdx.x; r < lines; r += HQ_THREADS) m[r] = 0;
   __syncthreads();
-  const int parts = rows >= HQ_THREADS ? 1 : HQ_THREADS / rows;
-  for (int w = threadIdx.x; w < rows * parts; w += HQ_THREADS) {
-    const int r = w % rows;
+  const int parts = lines >= HQ_THREADS ? 1 : HQ_THREADS / lines;
+  const int r = threadIdx.x % lines, p = threadIdx.x / lines;
+  if (p < parts) {
     uint32_t b = 0;
-    for (int k = w / rows; k < K; k += parts) b = max(b, oz_abs_hi(f(r, k)));
-    if (parts == 1) m[r] = b;
-    else atomicMax(&m[r], b);
+#pragma unroll 4
+    for (int k = p; k < K; k += parts) b = max(b, oz_abs_hi(f(r, k)));
+    atomicMax(&m[r], b);
   }
   __syncthreads();
-  for (int r = threadIdx.x; r < rows; r += HQ_THREADS) e[r] = oz_bound(m[r]);
+  for (int q = threadIdx.x; q < lines; q += HQ_THREADS) e[q] = oz_bound(m[q]);
   __syncthreads();
 }
 
@@ -214,9 +218,9 @@ __device__ __forceinline__ void oz_stage(uint2* frag, int k0, int nk, int nt, F 
 // out(r, c, v0, v1) receives entries (r, c), (r + 1, c) of the M x N product sum_k A(r, k) B(k, c):
 // fa(r, k), fb(k, c) values (asked only inside the ranges), ea(r), eb(c) bounds.  Row blocks of RB
 // rows of A are split once into shared-memory fragments (all K terms); a warp then takes 16
-// columns x 32 rows, splitting its columns of B in registers, so no other barrier is needed.
+// columns x 8 NT rows, splitting its columns of B in registers, so no other barrier is needed.
 // kTri: A(r, k) = 0 for k < r (the sum starts at the row block's first row).
-template <bool kWide, bool kTri, class FA, class EA, class FB, class EB, class OUT>
+template <int NT, bool kWide, bool kTri, class FA, class EA, class FB, class EB, class OUT>
 __device__ __forceinline__ void oz_gemm(int M, int N, int K, int RB, uint2* frag, FA fa, EA ea, FB fb, EB eb,
                                         OUT out) {
   constexpr int P = kOzP;
@@ -229,16 +233,17 @@ __device__ __forceinline__ void oz_gemm(int M, int N, int K, int RB, uint2* frag
                 [&](int line, int k) { return (r0 + line < M && k < K) ? fa(r0 + line, k) : 0.0; },
                 [&](int line) { return r0 + line < M ? ea(r0 + line) : 128; });
     __syncthreads();
-    const int nh = (min(RB, M - r0) + 31) >> 5;
+    const int nh = (min(RB, M - r0) + 8 * NT - 1) / (8 * NT);
     for (int unit = warp; unit < ncg * nh; unit += HQ_WARPS) {
-      const int c0 = (unit % ncg) * 16, half = unit / ncg;
+      const int c0 = (unit % ncg) * 16, part = unit / ncg;
       const int ca = c0 + g, cb = c0 + g + 8;
       const int Ea = ca < N ? eb(ca) : 128, Eb = cb < N ? eb(cb) : 128;
-      long long T[4][4], H[4][4];
+      long long T[NT][4], H[NT][4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
+      for (int j = 0; j < NT; ++j)
 #pragma unroll
         for (int e = 0; e < 4; ++e) T[j][e] = H[j][e] = 0;
+#pragma unroll 1
       for (int ks = k0; ks < nk; ++ks) {
         const int k = 16 * ks + 2 * t;
         auto get = [&](int kk, int c) { return (kk < K && c < N) ? fb(kk, c) : 0.0; };
@@ -248,15 +253,15 @@ __device__ __forceinline__ void oz_gemm(int M, int N, int K, int RB, uint2* frag
         oz_split<P>(get(k + 8, ca), get(k + 9, ca), Ea, Ea, a[2]);
         oz_split<P>(get(k + 8, cb), get(k + 9, cb), Eb, Eb, a[3]);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const uint2* fr = frag + (size_t)(ks * nt + half * 4 + j) * kOzDigits * 32 + lane;
+        for (int j = 0; j < NT; ++j) {
+          const uint2* fr = frag + (size_t)(ks * nt + part * NT + j) * kOzDigits * 32 + lane;
           if (kWide) oz_mma_wide(a, [&](int d) { return fr[d * 32]; }, H[j], T[j]);
           else oz_mma(a, [&](int d) { return fr[d * 32]; }, T[j]);
         }
       }
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int r = r0 + half * 32 + 8 * j + 2 * t;
+      for (int j = 0; j < NT; ++j) {
+        const int r = r0 + part * 8 * NT + 8 * j + 2 * t;
         if (r >= M) continue;
         double v[4];
 #pragma unroll
@@ -332,19 +337,21 @@ __device__ __forceinline__ void oz_apply_rows(const uint2* frag, const int* er, 
   }
 }
 
+// (The callers keep to few instances with runtime strides: a chunk of the chain runs through all of this
+// code once per factorisation step, and what is instantiated twice is fetched twice.)
 // out(r, c, s0, s1): s = sum_k A(r, k) B(k, c) for r0 <= r < r1, c0 <= c < c1 and kb <= 16 terms; fa, fb
-// values.  Reads of fa and fb must not overlap what `out` writes, except that with kOnePart (a warp
+// values.  Reads of fa and fb must not overlap what `out` writes, except that with one_part (a warp
 // owns its columns whole) `out` may overwrite the column entries that fb reads.  Ends with a barrier.
-template <bool kOnePart, class FA, class FB, class OUT>
-__device__ __forceinline__ void oz_rank16(int r0, int r1, int c0, int c1, int kb, uint2* frag, int* er, FA fa, FB fb,
-                                          OUT out) {
+template <class FA, class FB, class OUT>
+__device__ __forceinline__ void oz_rank16(bool one_part, int r0, int r1, int c0, int c1, int kb, uint2* frag, int* er,
+                                          FA fa, FB fb, OUT out) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int nr = r1 - r0;
   oz_stage_rows(frag, er, nr, kb, [&](int r, int k) { return fa(r0 + r, k); });
   __syncthreads();
   // few columns: the row range is shared out too, so that every warp has work
   const int ncg = (c1 - c0 + 15) >> 4;
-  const int parts = kOnePart || ncg >= HQ_WARPS ? 1 : HQ_WARPS / ncg;
+  const int parts = one_part || ncg >= HQ_WARPS ? 1 : HQ_WARPS / ncg;
   const int rp = (((nr + parts - 1) / parts) + 7) & ~7;
   for (int unit = warp; unit < ncg * parts; unit += HQ_WARPS) {
     const int ca = c0 + (unit % ncg) * 16 + g, cb = ca + 8, rb = (unit / ncg) * rp;

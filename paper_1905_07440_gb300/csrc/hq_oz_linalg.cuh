@@ -46,6 +46,11 @@ __device__ __forceinline__ void store_pair(double* p, double a, double b) {
   *reinterpret_cast<double2*>(p) = make_double2(a, b);
 }
 
+// Matrices of up to kTiny rows (lattices of up to 16 sites): one MMA step holds a whole product, and its
+// splits and conversions take 12 thousand cycles where the FP64 pipe needs 2 thousand for the 16 DFMAs per
+// thread.  So products, the triangular factor and Q stay in FP64 there.
+constexpr int kTiny = 16;
+
 // ---------------------------------------------------------------------- blocked QR
 // Column-pivoted QR in the form used for DQMC stabilisation by Bauer (SciPost Phys. Core 2,
 // 011 (2020)): the columns are ordered once by decreasing Euclidean norm, then factored by
@@ -103,15 +108,15 @@ __device__ __noinline__ void oz_panel(double* Q, double* V, int ld, int n, int j
 }
 
 // The reflectors in columns j0 .. j1 - 1 of V (zero above their first row) applied at once to columns c0 .. cend - 1, rows j0 .. n - 1, of A:
-//   kTrans:  A <- (I - V T V^T)^T A     (trailing update of the QR)
-//   !kTrans: A <- (I - V T V^T) A       (Q formation)
+//   trans:  A <- (I - V T V^T)^T A     (trailing update of the QR)
+//   !trans: A <- (I - V T V^T) A       (Q formation)
 // A warp takes 16 columns and runs W^T = A^T V, Z^T = W^T T (or W^T T^T) and A^T -= Z^T V^T back to back:
 // each result leaves the accumulators in the layout of the next left operand, so nothing but V's
 // and T's fragments is shared and A is read and written in place.  With fewer column groups than
-// warps, several warps form W of the same columns and share out the rows of the update.  kTrans follows
+// warps, several warps form W of the same columns and share out the rows of the update.  trans follows
 // oz_panel, which has left V's row-term fragments in place.
-template <int LM, bool kTrans>
-__device__ __noinline__ void oz_wy_apply(const double* V, int ld, int n, int j0, int j1, const double* T, double* A,
+template <int LM>
+__device__ __noinline__ void oz_wy_apply(bool trans, const double* V, int ld, int n, int j0, int j1, const double* T, double* A,
                                          int c0, int cend, const OzScratch& z) {
   const int kb = j1 - j0, nr = n - j0, nk = (nr + 15) >> 4;
   uint2* vk = z.frag;
@@ -120,9 +125,9 @@ __device__ __noinline__ void oz_wy_apply(const double* V, int ld, int n, int j0,
   int* et = z.ec;  // [16]
   auto v = [&](int rr, int k) { return (k < kb && rr < nr) ? V[(size_t)(j0 + k) * ld + j0 + rr] : 0.0; };
   auto evk = [&](int k) { return k < kb ? z.ev[j0 + k] : 128; };
-  if (!kTrans) stage_panel(vk, V, ld, n, j0, kb, z.ev);
+  if (!trans) stage_panel(vk, V, ld, n, j0, kb, z.ev);
   oz_stage_rows(vn, z.er, nr, 16, [&](int r, int k) { return v(r, k); });
-  oz_stage_rows(tf, et, 16, 16, [&](int r, int k) { return kTrans ? T[k * 16 + r] : T[r * 16 + k]; });
+  oz_stage_rows(tf, et, 16, 16, [&](int r, int k) { return trans ? T[k * 16 + r] : T[r * 16 + k]; });
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int ncg = (cend - c0 + 15) >> 4;
@@ -137,6 +142,7 @@ __device__ __noinline__ void oz_wy_apply(const double* V, int ld, int n, int j0,
     int E[2] = {128, 128};
     if (work && rb < nr) {
       uint32_t ma = 0, mb = 0;
+#pragma unroll 2
       for (int r = 2 * t; r < nr; r += 8) {
         const RowPair x = load_pair(pa + r), y = load_pair(pb + r);
         ma = max(ma, max(oz_abs_hi(x.v0), oz_abs_hi(x.v1)));
@@ -151,6 +157,7 @@ __device__ __noinline__ void oz_wy_apply(const double* V, int ld, int n, int j0,
       // W^T: sums over up to 256 rows fit one accumulator, because |v|^2 < 16 bounds the sum by
       // 4 sqrt(n) times the column's largest entry
       long long Tw[2][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}};
+#pragma unroll 1
       for (int ks = 0; ks < nk; ++ks) {
         const int r = 16 * ks + 2 * t;
         const RowPair z0{0.0, 0.0};
@@ -203,7 +210,7 @@ __device__ inline void oz_qr(double* Q, double* V, int ld, int n, const QrScratc
   for (int j0 = 0; j0 < n; j0 += 16) {
     const int j1 = min(j0 + 16, n);
     oz_panel<LM>(Q, V, ld, n, j0, j1 - j0, s.tau, z);
-    if (j1 < n) oz_wy_apply<LM, true>(V, ld, n, j0, j1, z.tall + (j0 >> 4) * 256, Q, j1, n, z);
+    if (j1 < n) oz_wy_apply<LM>(true, V, ld, n, j0, j1, z.tall + (j0 >> 4) * 256, Q, j1, n, z);
   }
 }
 
@@ -211,10 +218,26 @@ __device__ inline void oz_qr(double* Q, double* V, int ld, int n, const QrScratc
 // of a panel are still unit vectors there).
 template <int LM>
 __device__ inline void oz_form_q(const double* V, int ld, int n, double* U, const OzScratch& z) {
+  if (n <= kTiny) {  // one panel: U = I - V (T V^T), an entry per thread
+    double* W = z.ws;
+    const int r = threadIdx.x >> 4, c = threadIdx.x & 15;
+    double a = 0.0;
+    if (c < n)
+      for (int k = r; k < n; ++k) a = fma(z.tall[r * 16 + k], V[(size_t)k * ld + c], a);
+    W[r * 16 + c] = a;
+    __syncthreads();
+    if (r < n && c < n) {
+      a = r == c ? 1.0 : 0.0;
+      for (int k = 0; k <= r; ++k) a = fma(-V[(size_t)k * ld + r], W[k * 16 + c], a);
+      U[(size_t)c * ld + r] = a;
+    }
+    __syncthreads();
+    return;
+  }
   set_identity(U, ld, n);
   __syncthreads();
   for (int j0 = ((n - 1) >> 4) << 4; j0 >= 0; j0 -= 16)
-    oz_wy_apply<LM, false>(V, ld, n, j0, min(j0 + 16, n), z.tall + (j0 >> 4) * 256, U, j0, n, z);
+    oz_wy_apply<LM>(false, V, ld, n, j0, min(j0 + 16, n), z.tall + (j0 >> 4) * 256, U, j0, n, z);
 }
 
 // Tout = D^-1 R (rows of Tprev in pivot order): T' Tprev with T' = D^-1 R Pi^T.
@@ -222,10 +245,9 @@ template <int LM, bool kWide>
 __device__ __noinline__ void oz_t_product(const double* P, int n, const int* perm, const double* rinv,
                                           const double* Tprev, double* Tout, const OzScratch& z) {
   auto fr = [&](int r, int k) { return k >= r ? P[(size_t)k * n + r] * rinv[r] : 0.0; };
-  oz_row_bounds(n, n, z.er, fr);
-  oz_col_bounds(Tprev, n, n, n, z.ec);
-  __syncthreads();
-  oz_gemm<kWide, true>(
+  oz_line_bounds(false, n, n, z.er, fr);
+  oz_line_bounds(true, n, n, z.ec, [&](int c, int k) { return Tprev[(size_t)c * n + k]; });
+  oz_gemm<LM <= 8 ? 2 : 4, kWide, true>(
       n, n, n, oz_rows(n), z.frag, fr, [&](int r) { return z.er[r]; },
       [&](int k, int c) { return Tprev[(size_t)c * n + perm[k]]; }, [&](int c) { return z.ec[c]; },
       [&](int r, int c, double v0, double v1) { store_pair(Tout + (size_t)c * n + r, v0, v1); });
@@ -246,6 +268,14 @@ __device__ inline void oz_t_update(const double* P, int n, const QrScratch& s, d
       Tout[(size_t)s.perm[c] * n + j] = (c >= j) ? P[(size_t)c * n + j] * s.rinv[j] : 0.0;
     }
     __syncthreads();
+  } else if (n <= kTiny) {
+    const int r = threadIdx.x & 15, c = threadIdx.x >> 4;
+    if (r < n && c < n) {
+      double a = 0.0;
+      for (int k = r; k < n; ++k) a = fma(P[(size_t)k * n + r], Tprev[(size_t)c * n + s.perm[k]], a);
+      Tout[(size_t)c * n + r] = a * s.rinv[r];
+    }
+    __syncthreads();
   } else if (LM > 8 && n > 64) {
     oz_t_product<LM, true>(P, n, s.perm, s.rinv, Tprev, Tout, z);
   } else {
@@ -253,22 +283,19 @@ __device__ inline void oz_t_update(const double* P, int n, const QrScratch& s, d
   }
 }
 
-// C = op(A) op(B) diag(cd) (cd may be null), optionally with B's rows scaled by kd first.
-template <int LM, bool kWide, bool TA, bool TB>
-__device__ __noinline__ void oz_product_mm(int n, const double* A, const double* B, const double* kd, const double* cd,
-                                           double* C, const OzScratch& z) {
-  auto fa = [&](int r, int k) { return TA ? A[(size_t)r * n + k] : A[(size_t)k * n + r]; };
+// C = A diag(kd) B diag(cd) (kd, cd may be null) with A(r, k) = A[r ar + k ak], B(k, c) = B[k bk + c bc] (each with a
+// unit stride), C column-major.
+template <int LM, bool kWide>
+__device__ __noinline__ void oz_product_mm(int n, const double* A, int ar, int ak, const double* B, int bk, int bc,
+                                           const double* kd, const double* cd, double* C, const OzScratch& z) {
+  auto fa = [&](int r, int k) { return A[(size_t)r * ar + (size_t)k * ak]; };
   auto fb = [&](int k, int c) {
-    const double v = TB ? B[(size_t)k * n + c] : B[(size_t)c * n + k];
+    const double v = B[(size_t)k * bk + (size_t)c * bc];
     return kd ? v * kd[k] : v;
   };
-  if (TA) oz_col_bounds(A, n, n, n, z.er);
-  else oz_row_bounds(n, n, z.er, fa);
-  if (TB) oz_row_bounds(n, n, z.ec, [&](int c, int k) { return fb(k, c); });
-  else if (kd) oz_row_bounds(n, n, z.ec, [&](int c, int k) { return fb(k, c); });
-  else oz_col_bounds(B, n, n, n, z.ec);
-  __syncthreads();
-  oz_gemm<kWide, false>(
+  oz_line_bounds(ak == 1, n, n, z.er, fa);
+  oz_line_bounds(bk == 1, n, n, z.ec, [&](int c, int k) { return fb(k, c); });
+  oz_gemm<LM <= 8 ? 2 : 4, kWide, false>(
       n, n, n, oz_rows(n), z.frag, fa, [&](int r) { return z.er[r]; }, fb, [&](int c) { return z.ec[c]; },
       [&](int r, int c, double v0, double v1) {
         if (cd) {
@@ -282,21 +309,31 @@ __device__ __noinline__ void oz_product_mm(int n, const double* A, const double*
 template <int LM, bool TA, bool TB>
 __device__ inline void oz_mm(int n, const double* A, const double* B, const double* kd, const double* cd, double* C,
                              const OzScratch& z) {
-  if (LM > 8 && n > 64) oz_product_mm<LM, true, TA, TB>(n, A, B, kd, cd, C, z);
-  else oz_product_mm<LM, false, TA, TB>(n, A, B, kd, cd, C, z);
+  if (n <= kTiny) {
+    const int r = threadIdx.x & 15, c = threadIdx.x >> 4;
+    __syncthreads();
+    if (r < n && c < n) {
+      double a = 0.0;
+      for (int k = 0; k < n; ++k) {
+        const double b = TB ? B[k * n + c] : B[c * n + k];
+        a = fma(TA ? A[r * n + k] : A[k * n + r], kd ? b * kd[k] : b, a);
+      }
+      C[c * n + r] = cd ? a * cd[c] : a;
+    }
+    __syncthreads();
+    return;
+  }
+  const int ar = TA ? n : 1, ak = TA ? 1 : n, bk = TB ? n : 1, bc = TB ? 1 : n;
+  if (LM > 8 && n > 64) oz_product_mm<LM, true>(n, A, ar, ak, B, bk, bc, kd, cd, C, z);
+  else oz_product_mm<LM, false>(n, A, ar, ak, B, bk, bc, kd, cd, C, z);
 }
 
 // Flush of delayed updates: G(r, c) += sum_m A[m][r] B[m][c], m < kk (A, B [kk][n]).
 template <int LM>
-__device__ __noinline__ void oz_flush(double* G, const double* A, const double* B, int n, int kk, const OzScratch& z) {
+__device__ inline void oz_flush(double* G, const double* A, const double* B, int n, int kk, const OzScratch& z) {
   for (int m0 = 0; m0 < kk; m0 += 16)
-    oz_rank16<false>(0, n, 0, n, min(16, kk - m0), z.frag, z.er, [&](int r, int k) { return A[(size_t)(m0 + k) * n + r]; },
-              [&](int k, int c) { return B[(size_t)(m0 + k) * n + c]; },
-              [&](int r, int c, double s0, double s1) {
-                double* p = G + (size_t)c * n + r;
-                const RowPair x = load_pair(p);
-                store_pair(p, x.v0 + s0, x.v1 + s1);
-              });
+    oz_rank<LM>(Rank16{A + (size_t)m0 * n, 1, n, B + (size_t)m0 * n, n, 1, G, n, 1.0, 1.0}, 0, n, 0, n, min(16, kk - m0),
+                z.frag, z.er);
 }
 
 // ------------------------------------------------------------ separable propagator
@@ -345,6 +382,35 @@ __device__ __forceinline__ void oz_slices(int nx, int ny, int n, const OzKin& K,
         },
         [&](int c, int i, double v0, double v1) { store_pair(P + (size_t)c * n + i, v0, v1); });
   }
+  __syncthreads();
+}
+
+// The same for n <= kTiny in FP64: a matrix entry per thread, the columns in shared memory (buf: 512
+// doubles) between the two passes of a slice.
+template <bool kAfter, class DV>
+__device__ __forceinline__ void tiny_slices(int nx, int ny, int n, const double* ex, const double* ey, double* P,
+                                            const double* U, const double* D, int count, DV dv, double* buf) {
+  const int i = threadIdx.x & 15, c = threadIdx.x >> 4, x = i % nx, y = i / nx;
+  const bool on = i < n && c < n;
+  double *A = buf + 16 * c, *T = buf + 256 + 16 * c;
+  double v = 0.0;
+  if (on) v = U ? U[(size_t)c * n + i] * D[c] : (i == c ? 1.0 : 0.0);
+  for (int k = 0; k < count; ++k) {
+    const double d = on ? dv(k, i) : 0.0;
+    __syncthreads();
+    A[i] = kAfter ? v : v * d;
+    __syncthreads();
+    double a = 0.0;
+    if (on)
+      for (int b = 0; b < nx; ++b) a = fma(ex[x * nx + b], A[b + nx * y], a);
+    T[i] = a;
+    __syncthreads();
+    v = 0.0;
+    if (on)
+      for (int b = 0; b < ny; ++b) v = fma(ey[y * ny + b], T[x + nx * b], v);
+    if (kAfter) v *= d;
+  }
+  if (on) P[(size_t)c * n + i] = v;
   __syncthreads();
 }
 

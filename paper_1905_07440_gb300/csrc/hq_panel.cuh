@@ -42,7 +42,7 @@ constexpr int kPanelWarps = 4;  // warps of a panel held in FP64 (hq_lu.cuh): on
 // shared scratch of a panel (inside the fragment scratch)
 struct PanelShared {
   __int128 part[HQ_WARPS][16];
-  long long arow[16];
+  double arow[16];
   long long m[16];
   long long b;
   uint32_t cmax[16];
@@ -151,21 +151,36 @@ __device__ __noinline__ void panel_fixed(double* Q, double* V, int ld, int n, in
       if (!(lane & o)) ps->part[warp][((idx + jb) & (CPT - 1)) * G + cq] = idx < left ? p[0] : (__int128)0;
       if (row == j) {
 #pragma unroll
-        for (int i = 0; i < CPT; ++i) ps->arow[((i + jb) & (CPT - 1)) * G + cq] = x[i];
+        for (int i = 0; i < CPT; ++i)
+          if (i < left) ps->arow[(i + jb) * G + cq] = (double)x[i];
       }
       bar_warps(nthr);
+      // warp 0: the step's scalars.  Every FP64 instruction holds the pipe for 64 cycles, so their number
+      // counts, not the depth of the chain: 13 up to the coefficients; records come after the barrier.
+      double nrm = 0.0, gam = 0.0, aa = 0.0;
+      int h = 0;
+      bool zero = false, neg = false;
       if (warp == 0) {
         const int c = lane & 15;
-        const double a = (double)ps->arow[c];
         __int128 t = 0;
         for (int w = lane >> 4; w < nw; w += 2) t += ps->part[w][c];
-        t = add_from(t, t, 16);
-        // S_j > 0; for the others a rounding of 2^11 against norms of 2^60 does not matter
-        const double d = fma((double)(long long)(t >> 64), 18446744073709551616.0, (double)(unsigned long long)t);
+        if (nw > 1) t = add_from(t, t, 16);
+        else t = lane < 16 ? t : (__int128)0;
+        // leading 62 bits of the sum: one conversion
+        const bool minus = t < 0;
+        const unsigned __int128 u = minus ? (unsigned __int128)(-t) : (unsigned __int128)t;
+        const unsigned long long uh = (unsigned long long)(u >> 64), ul = (unsigned long long)u;
+        const int up = uh ? 66 - __clzll((long long)uh) : 0;  // bits above 62
+        const long long lead = uh ? (long long)((uh << (64 - up)) | (ul >> up)) : (long long)(ul >> 2);
+        const double d0 = (double)lead;
+        const double a = ps->arow[c];
+        const int ud = uh ? up : 2;
+        double d = shift_exponent(minus ? -d0 : d0, ud);
         const double Sj = __shfl_sync(HQ_FULL, d, j);
-        const double al0 = __shfl_sync(HQ_FULL, a, j);
-        const int hs = __double2hiint(Sj), es = (hs >> 20) - 1023, h = es >> 1;
-        const bool zero = (hs & 0x7fffffff) == 0;
+        const double al0 = ps->arow[j];
+        const int hs = __double2hiint(Sj), es = (hs >> 20) - 1023;
+        h = es >> 1;
+        zero = (hs & 0x7fffffff) == 0;
         // s = S / 4^h in [1, 4): everything below is in units of 2^h of column j
         const double s = zero ? 1.0 : __hiloint2double((hs & 0xfffff) | ((1023 + (es & 1)) << 20), __double2loint(Sj));
         const float sf = __uint_as_float((uint32_t)__double2hiint(s) * 8u - ((1023u - 127u) << 23) +
@@ -174,30 +189,36 @@ __device__ __noinline__ void panel_fixed(double* Q, double* V, int ld, int n, in
         const double y0 = float_bits_to_double(yf);
         const double q = s * y0;
         const double al = shift_exponent(al0, -h);
-        const bool neg = __double2hiint(al) < 0;
-        const double aa = fabs(al);
+        neg = __double2hiint(al) < 0;
+        aa = fabs(al);
+        // |al| <= 2 as a float, from its bits (0 when it does not matter for the seed)
+        const int ah = __double2hiint(aa);
+        const float af = ah > (900 << 20) ? __uint_as_float(((uint32_t)(ah - (896 << 20)) << 3) | ((uint32_t)__double2loint(aa) >> 29))
+                                          : 0.f;
+        const double g0 = float_bits_to_double(__fdividef(1.f, fmaf(af, sf * yf, sf)));
         const double e1 = fma(-q, y0, 1.0);
-        const double g0 = float_bits_to_double(__fdividef(1.f, fmaf((float)aa, sf * yf, sf)));
-        const double y = fma(y0 * e1, fma(0.375, e1, 0.5), y0);  // 1 / sqrt(s), third order
-        const double nrm = s * y;
+        nrm = fma(q * e1, fma(0.375, e1, 0.5), q);  // sqrt(s): s / sqrt(s), third order
         const double td = fma(aa, nrm, s);
         const double wc = fma(neg ? -nrm : nrm, a, shift_exponent(d, -h));  // v^T x_c
         const double e2 = fma(-td, g0, 1.0);
-        const double gam = fma(g0, fma(e2, e2, e2), g0);  // 2 / v^T v
-        if (lane < 16) ps->m[c] = (c > j && c < kb && !zero) ? __double2ll_rn(gam * wc) : 0ll;
+        gam = fma(g0, fma(e2, e2, e2), g0);  // 2 / v^T v
+        const double phi = gam * wc;
+        if (lane < 16) ps->m[c] = (c > j && c < kb && !zero) ? __double2ll_rn(phi) : 0ll;
         if (lane == 0) {
           // b 2^59 as an integer, from the bits of |b| in [1, 2]
           const unsigned long long bits = (unsigned long long)__double_as_longlong(nrm);
           const unsigned long long bi = ((bits & 0xfffffffffffffull) | 0x10000000000000ull) << ((int)(bits >> 52) - 1023 + 7);
           ps->b = zero ? 0ll : (neg ? (long long)bi : -(long long)bi);
           ps->shift = zero ? 0 : max(59 - h, 0);
-          tau[j] = bad ? nanv : (zero ? 0.0 : gam);
-          ev[j0 + j] = zero ? kOzUnit : oz_bound(oz_abs_hi(aa + nrm));
-          const int k = h + oz_bound(ps->cmax[j]) - 1023 - B;
-          Q[(size_t)(j0 + j) * ld + j0 + j] = bad ? nanv : (zero ? 0.0 : oz_scale(neg ? nrm : -nrm, k));
         }
       }
       bar_warps(nthr);
+      if (tid == 0) {
+        tau[j] = bad ? nanv : (zero ? 0.0 : gam);
+        ev[j0 + j] = zero ? kOzUnit : oz_bound(oz_abs_hi(aa + nrm));
+        const int k = h + oz_bound(ps->cmax[j]) - 1023 - B;
+        Q[(size_t)(j0 + j) * ld + j0 + j] = bad ? nanv : (zero ? 0.0 : oz_scale(neg ? nrm : -nrm, k));
+      }
       const long long v = row < j ? 0ll : (long long)((unsigned long long)xj << ps->shift) - (row == j ? ps->b : 0ll);
       const int v1 = (int)(v >> 30), v0 = (int)(v & 0x3fffffff);
 #pragma unroll
@@ -243,9 +264,7 @@ __device__ __forceinline__ void stage_panel(uint2* vk, const double* V, int ld, 
 // T of H_j0 ... = I - V T V^T (upper triangular, compact WY: Schreiber and Van Loan, SIAM J. Sci. Stat.
 // Comput. 10 (1989)).  V^T V comes from the staged fragments (a right fragment holds the same values
 // as the left fragment of its transpose), the k-steps shared out over the warps and their integer sums
-// added in shared memory; then warp 0 forms T: the two 8 x 8 diagonal blocks (a row per lane) and
-// the off-diagonal one as -T11 S12 T22, which halves the chain of dependent FP64 instructions of a
-// 16-column recurrence.  S, T: [16][16]; ends with a barrier.
+// added in shared memory.  S, T: [16][16]; ends with a barrier.
 __device__ inline void panel_t(const uint2* vk, int nk, int kb, const double* tau, const int* ev, unsigned long long* sum,
                                double* S, double* T) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
@@ -283,12 +302,14 @@ __device__ inline void panel_t(const uint2* vk, int nk, int kb, const double* ta
     S[tid] = (a < b && b < kb) ? oz_scale((double)(long long)sum[tid], oz_expo<kOzP>(ev[a], ev[b])) : 0.0;
   }
   __syncthreads();
+  // T by doubling: 4 x 4 diagonal blocks (a row per lane), then off-diagonal blocks -T11 S12 T22 of 4 and
+  // of 8; S12 T22 is kept in S's place.  34 dependent FP64 instructions instead of 136 of the recurrence.
   if (warp == 0) {
     if (lane < 16) {
-      const int i = lane & 7, o = lane & 8;
-      double x[8];
+      const int i = lane & 3, o = lane & 12;
+      double x[4];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
+      for (int j = 0; j < 4; ++j) {
         const double tj = o + j < kb ? tau[o + j] : 0.0;
         double a = 0.0;
 #pragma unroll
@@ -298,27 +319,31 @@ __device__ inline void panel_t(const uint2* vk, int nk, int kb, const double* ta
       }
     }
     __syncwarp();
-    double y[2];
+    const int o = lane < 16 ? 0 : 8, r = (lane >> 2) & 3, c = lane & 3;
+    double a = 0.0;
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const int r = (lane >> 3) + 4 * u, c = lane & 7;
-      double a = 0.0;
-#pragma unroll
-      for (int k = 0; k < 8; ++k) a = fma(S[r * 16 + 8 + k], T[(8 + k) * 16 + 8 + c], a);
-      y[u] = a;
-    }
+    for (int k = 0; k < 4; ++k) a = fma(S[(o + r) * 16 + o + 4 + k], T[(o + 4 + k) * 16 + o + 4 + c], a);
     __syncwarp();
-#pragma unroll
-    for (int u = 0; u < 2; ++u) S[((lane >> 3) + 4 * u) * 16 + 8 + (lane & 7)] = y[u];
+    S[(o + r) * 16 + o + 4 + c] = a;
     __syncwarp();
+    a = 0.0;
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const int r = (lane >> 3) + 4 * u, c = lane & 7;
-      double a = 0.0;
+    for (int k = 0; k < 4; ++k) a = fma(T[(o + r) * 16 + o + k], S[(o + k) * 16 + o + 4 + c], a);
+    T[(o + r) * 16 + o + 4 + c] = -a;
+  }
+  __syncthreads();
+  if (tid < 64) {
+    const int r = tid >> 3, c = tid & 7;
+    double a = 0.0;
 #pragma unroll
-      for (int k = 0; k < 8; ++k) a = fma(T[r * 16 + k], S[k * 16 + 8 + c], a);
-      T[r * 16 + 8 + c] = -a;
-    }
+    for (int k = 0; k < 8; ++k) a = fma(S[r * 16 + 8 + k], T[(8 + k) * 16 + 8 + c], a);
+    bar_warps(64);
+    S[r * 16 + 8 + c] = a;
+    bar_warps(64);
+    a = 0.0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) a = fma(T[r * 16 + k], S[k * 16 + 8 + c], a);
+    T[r * 16 + 8 + c] = -a;
   }
   __syncthreads();
 }
