@@ -17,16 +17,17 @@ static_assert(CN_NP == HQ_CNN_PARAMS, "parameter count");
 constexpr int CN_TILE = 32;  // points per staged tile in the weight-gradient passes
 
 // ------------------------------------------------------------------------ evaluation
-// F_cnn of every chain (grid = chains); refreshes the chain's cached activations.
-__global__ void __launch_bounds__(HQ_THREADS) cnn_eval_kernel(Dev d, CnnState cn, const double* Xall, double* Fout,
-                                                              double x0) {
+// F_cnn of every chain (grid = chains); refreshes the chain's caches and network inputs.
+__global__ void __launch_bounds__(HQ_THREADS, 2) cnn_eval_kernel(Dev d, CnnState cn, const double* Xall, double* Fout,
+                                                                 double x0) {
   extern __shared__ __align__(16) char craw[];
-  float* w = (float*)craw;
-  double* red = (double*)(w + CN_WPAD);
+  __shared__ double red[HQ_WARPS];
   const int c = blockIdx.x, NL = d.n * d.L;
-  cn_load_weights(cn.wbf, w);
-  const double F = cn_forward_all(d, w, Xall + (size_t)c * NL, x0, cn.h1c + (size_t)c * NL * CN_C,
-                                  cn.h2c + (size_t)c * NL * CN_C, cn.o3c + (size_t)c * NL, red);
+  const double* X = Xall + (size_t)c * NL;
+  float* xf = cn.xf + (size_t)c * NL;
+  for (int k = threadIdx.x; k < NL; k += HQ_THREADS) xf[k] = (float)(X[k] - x0);
+  const CnSm w = cn_setup(cn.wbf, craw);  // (ends with a barrier)
+  const double F = cn_refresh(d, w, xf, cn.h1c + (size_t)c * NL * 8, cn.s2c + (size_t)c * NL, red);
   if (threadIdx.x == 0) Fout[c] = F;
 }
 
@@ -83,7 +84,7 @@ __global__ void __launch_bounds__(HQ_THREADS) cnn_train_kernel(Dev d, CnnState c
   for (int a = blockIdx.x; a < B; a += gridDim.x) {
     const double* X = Xs + (size_t)idx[a] * NL;
     // forward
-    const double F = cn_forward_all(d, s.w, X, x0, A1, A2, nullptr, s.red);
+    const double F = cn_forward_all(d, s.w, X, x0, A1, A2, s.red);
     if (tid == 0) Fb[a] = F;
     const float sg = (float)(2.0 * (F - ys[idx[a]]) / B);
     // layer 3: dF/dW3[t][ci] = sum_q h2(q)[ci] for every t; dF/db3 = L N
@@ -264,7 +265,7 @@ static double mean_field_shift(const Dev& d) { return -d.g / (d.mass * d.omega *
 
 cudaError_t cnn_launch_eval(const Dev& d, const CnnState& cn, const double* X, double* F, int /*write_cache*/,
                             cudaStream_t s) {
-  const size_t sb = sizeof(float) * CN_WPAD + sizeof(double) * HQ_WARPS;
+  const size_t sb = cn_smem_bytes();
   opt_in_smem((const void*)cnn_eval_kernel, sb);
   cnn_eval_kernel<<<d.n_chains, HQ_THREADS, sb, s>>>(d, cn, X, F, mean_field_shift(d));
   return cudaGetLastError();

@@ -7,11 +7,11 @@
 // 1 -> 16 -> 16 -> 1 channels, ReLU after the first two, and F_cnn(X) = sum of the last
 // layer over every point; the input is z = X - x0 with x0 = -g/(M Omega^2).  Tap
 // t = 9 (dl + 1) + 3 (dy + 1) + (dx + 1) reads (l + dl, y + dy, x + dx).  Weights are
-// bfloat16, arithmetic FP32; every path computes a point through the same functions in the
-// same order, so a value recomputed in a block-move window equals the cached one bit for bit.
+// bfloat16, arithmetic FP32.
 #pragma once
 #include "hq_device.cuh"
 #include "hq_internal.h"
+#include "hq_nn_tc.cuh"
 
 namespace hq {
 
@@ -19,7 +19,6 @@ constexpr int CN_T = 27, CN_C = kCnnC;
 constexpr int CN_W1 = 0, CN_B1 = CN_T * CN_C, CN_W2 = CN_B1 + CN_C, CN_B2 = CN_W2 + CN_T * CN_C * CN_C,
               CN_W3 = CN_B2 + CN_C, CN_B3 = CN_W3 + CN_T * CN_C, CN_NP = CN_B3 + 1;
 constexpr int CN_WPAD = (CN_NP + 3) & ~3;
-constexpr int CN_WIN = 49;  // sites within torus distance 3
 
 __device__ inline void cn_load_weights(const uint16_t* wb, float* w) {
   for (int k = threadIdx.x; k < CN_WPAD; k += blockDim.x) w[k] = (k < CN_NP) ? bf16_to_float(wb[k]) : 0.f;
@@ -32,17 +31,15 @@ __device__ __forceinline__ int cn_site(const Dev& d, int i, int dy, int dx) {
   return (x + dx + d.nx) % d.nx + d.nx * ((y + dy + d.ny) % d.ny);
 }
 
-// Layer-1 activations (after ReLU) at (l, i); site cs of every slice is shifted by cdx.
-__device__ __forceinline__ void cn_layer1(const Dev& d, const float* w, const double* X, double x0, int l, int i,
-                                          int cs, double cdx, float* out) {
+// ------------------------------------------------------------------ training path (FP32, a thread per point)
+// Layer-1 activations (after ReLU) at (l, i).
+__device__ __forceinline__ void cn_layer1(const Dev& d, const float* w, const double* X, double x0, int l, int i, float* out) {
   float a[CN_C];
 #pragma unroll
   for (int c = 0; c < CN_C; ++c) a[c] = w[CN_B1 + c];
   for (int t = 0; t < CN_T; ++t) {
     const int ll = (l + t / 9 - 1 + d.L) % d.L, j = cn_site(d, i, (t / 3) % 3 - 1, t % 3 - 1);
-    double v = X[(size_t)ll * d.n + j];
-    if (j == cs) v = v + cdx;
-    const float z = (float)(v - x0);
+    const float z = (float)(X[(size_t)ll * d.n + j] - x0);
 #pragma unroll
     for (int c = 0; c < CN_C; ++c) a[c] = fmaf(z, w[CN_W1 + t * CN_C + c], a[c]);
   }
@@ -101,11 +98,11 @@ __device__ __forceinline__ float cn_layer3(const Dev& d, const float* w, int l, 
 }
 
 // F_cnn of one field configuration by the whole CTA; layer outputs go to h1 [L N][16],
-// h2 [L N][16] and (if o3 != nullptr) o3 [L N].  Returns F in every thread.
+// h2 [L N][16].  Returns F in every thread.
 __device__ inline double cn_forward_all(const Dev& d, const float* w, const double* X, double x0, float* h1, float* h2,
-                                        float* o3, double* red) {
+                                        double* red) {
   const int n = d.n, NL = d.n * d.L;
-  for (int p = threadIdx.x; p < NL; p += blockDim.x) cn_layer1(d, w, X, x0, p / n, p % n, -1, 0.0, h1 + (size_t)p * CN_C);
+  for (int p = threadIdx.x; p < NL; p += blockDim.x) cn_layer1(d, w, X, x0, p / n, p % n, h1 + (size_t)p * CN_C);
   __syncthreads();
   auto h1at = [&](int ll, int j) { return h1 + ((size_t)ll * n + j) * CN_C; };
   for (int p = threadIdx.x; p < NL; p += blockDim.x) cn_layer2(d, w, p / n, p % n, h1at, h2 + (size_t)p * CN_C);
@@ -114,101 +111,264 @@ __device__ inline double cn_forward_all(const Dev& d, const float* w, const doub
   double part = 0.0;
   for (int p = threadIdx.x; p < NL; p += blockDim.x) {
     const float o = cn_layer3(d, w, p / n, p % n, h2at);
-    if (o3) o3[p] = o;
     part += (double)o;
   }
   return block_sum(part, red);
 }
 
-// Sites within torus distance 1, 2, 3 of site i (each listed once, ascending) and the
-// position of every site in the radius-1 and radius-2 lists (-1 outside).  Shared memory:
-// cnt[4], lst [3][CN_WIN], pos [2][n].  Thread 0 builds; ends with a barrier.
-struct CnWindow {
-  int* cnt;
-  int* lst;
-  int* pos;
+// ------------------------------------------------------------------ sampling path
+// Evaluation and block-move windows on the tensor cores.  Two facts keep the work small:
+//
+//   * F_cnn sums the last layer over the whole torus, so F_cnn = L N b3 + sum_q wbar . h2(q) with
+//     wbar = sum_t W3[t]: the third convolution is a dot product per point.  wbar is kept as two floats.
+//     A point's cache is that one number, and a block move recomputes layer 1 within lattice distance 1
+//     and layer 2 within 2 of its site (every slice), no outputs beyond.
+//   * Layer 2 (27 taps x 16 x 16) runs as m16n8k16 MMAs, 16 points per warp.  Weights are bfloat16
+//     already; a layer-1 value is split into three bfloat16 terms (24 bits: exact), once when it is
+//     written, and stored as fragments' register pairs: uint4 (hi, mid, lo, 0) per two channels.  Each
+//     tap's three products are added to the FP32 sums with FADDs, so no rounding of the tensor core's
+//     own accumulation carries over from tap to tap.
+//
+// Every path computes a point through cn_tile in the same order, so a value recomputed in a window
+// equals the cached one bit for bit.  (The scalar form took 600 thousand cycles per block move at 8x8,
+// L = 40: FP64 input conversions, a window list built by one thread, weights re-read per point.)
+struct CnSm {
+  const uint2* w2;                       // [27][2][32] fragments of W2
+  const float *w1, *b1, *b2, *wh, *wl;   // W1 [27][16], biases, wbar = wh + wl
+  float b3;
 };
 
-__device__ inline void cn_build_window(const Dev& d, int i, const CnWindow& wd) {
-  if (threadIdx.x == 0) {
-    const int xi = i % d.nx, yi = i / d.nx;
-    int c1 = 0, c2 = 0, c3 = 0;
-    for (int j = 0; j < d.n; ++j) {
-      int ax = abs(j % d.nx - xi), ay = abs(j / d.nx - yi);
-      ax = min(ax, d.nx - ax);
-      ay = min(ay, d.ny - ay);
-      const int r = max(ax, ay);
-      wd.pos[j] = -1;
-      wd.pos[d.n + j] = -1;
-      if (r <= 1) { wd.pos[j] = c1; wd.lst[c1++] = j; }
-      if (r <= 2) { wd.pos[d.n + j] = c2; wd.lst[CN_WIN + c2++] = j; }
-      if (r <= 3) wd.lst[2 * CN_WIN + c3++] = j;
-    }
-    wd.cnt[0] = c1;
-    wd.cnt[1] = c2;
-    wd.cnt[2] = c3;
+constexpr int CN_FRAGS = CN_T * 2 * 32, CN_FLOATS = CN_T * CN_C + 4 * CN_C + 4;
+__host__ __device__ inline size_t cn_smem_bytes() { return sizeof(uint2) * CN_FRAGS + sizeof(float) * CN_FLOATS; }
+
+// all threads; ends with a barrier
+__device__ inline CnSm cn_setup(const uint16_t* wb, char* mem) {
+  uint2* fr = reinterpret_cast<uint2*>(mem);
+  float* f = reinterpret_cast<float*>(fr + CN_FRAGS);
+  for (int e = threadIdx.x; e < CN_FRAGS; e += blockDim.x) {
+    const int lane = e & 31, nt = (e >> 5) & 1, tap = e >> 6, g = lane >> 2, t = lane & 3;
+    const uint16_t* W = wb + CN_W2 + tap * CN_C * CN_C + 8 * nt + g;
+    auto w = [&](int ci) { return (uint32_t)W[ci * CN_C]; };
+    fr[e] = make_uint2(w(2 * t) | (w(2 * t + 1) << 16), w(2 * t + 8) | (w(2 * t + 9) << 16));
+  }
+  float *w1 = f, *b1 = w1 + CN_T * CN_C, *b2 = b1 + CN_C, *wh = b2 + CN_C, *wl = wh + CN_C;
+  for (int e = threadIdx.x; e < CN_T * CN_C; e += blockDim.x) w1[e] = bf16_to_float(wb[CN_W1 + e]);
+  for (int c = threadIdx.x; c < CN_C; c += blockDim.x) {
+    b1[c] = bf16_to_float(wb[CN_B1 + c]);
+    b2[c] = bf16_to_float(wb[CN_B2 + c]);
+    double s = 0.0;
+    for (int t = 0; t < CN_T; ++t) s += (double)bf16_to_float(wb[CN_W3 + t * CN_C + c]);
+    wh[c] = (float)s;
+    wl[c] = (float)(s - (double)(float)s);
   }
   __syncthreads();
+  return CnSm{fr, w1, b1, b2, wh, wl, bf16_to_float(wb[CN_B3])};
 }
 
-// F_cnn(X') - F_cnn(X) for X'(i, .) = X(i, .) + dx, from the cached activations of X: the
-// proposal's layer-1 values in the radius-1 window, layer-2 in radius 2, outputs in radius 3
-// (every slice) go to h1p / h2p / o3p.  Called by the whole CTA after cn_build_window;
-// returns the difference in every thread.
-__device__ inline double cn_block_delta(const Dev& d, const float* w, const CnWindow& wd, const double* X, double x0,
-                                        int i, double dx, const float* h1c, const float* h2c, const float* o3c,
-                                        float* h1p, float* h2p, float* o3p, double* red) {
-  const int n = d.n, L = d.L;
-  const int n1 = wd.cnt[0], n2 = wd.cnt[1], n3 = wd.cnt[2];
-  const int* l1 = wd.lst;
-  const int* l2 = wd.lst + CN_WIN;
-  const int* l3 = wd.lst + 2 * CN_WIN;
-  const int* pos1 = wd.pos;
-  const int* pos2 = wd.pos + n;
-  for (int q = threadIdx.x; q < n1 * L; q += blockDim.x) {
-    const int l = q / n1, k = q % n1;
-    cn_layer1(d, w, X, x0, l, l1[k], i, dx, h1p + (size_t)q * CN_C);
+// Two non-negative activations as packed bfloat16 pairs hi + mid + lo.
+__device__ __forceinline__ uint4 cn_split(float a, float b) {
+  auto three = [](float v, uint32_t& h, uint32_t& m, uint32_t& l) {
+    h = float_to_bf16(v);
+    const float r = v - bf16_to_float((uint16_t)h);
+    m = float_to_bf16(r);
+    l = float_to_bf16(r - bf16_to_float((uint16_t)m));
+  };
+  uint32_t ah, am, al, bh, bm, bl;
+  three(a, ah, am, al);
+  three(b, bh, bm, bl);
+  return make_uint4(ah | (bh << 16), am | (bm << 16), al | (bl << 16), 0u);
+}
+
+__device__ __forceinline__ int cn_wrap(int a, int n) { return a < 0 ? a + n : (a >= n ? a - n : a); }
+
+// Channels 8 half .. 8 half + 7 of layer 1 (after ReLU) at (l, x, y) to out[4 half ..]; z(ll, j): input.
+template <class Z>
+__device__ __forceinline__ void cn_point1(const Dev& d, const CnSm& w, int l, int x, int y, int half, Z z, uint4* out) {
+  float a[8];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) a[c] = w.b1[8 * half + c];
+#pragma unroll 1
+  for (int dl = -1; dl <= 1; ++dl) {
+    const int ll = cn_wrap(l + dl, d.L);
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+      const float v = z(ll, cn_wrap(x + q % 3 - 1, d.nx) + d.nx * cn_wrap(y + q / 3 - 1, d.ny));
+      const float* W = w.w1 + (9 * (dl + 1) + q) * CN_C + 8 * half;
+#pragma unroll
+      for (int c = 0; c < 8; ++c) a[c] = fmaf(v, W[c], a[c]);
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < 4; ++c) out[4 * half + c] = cn_split(fmaxf(a[2 * c], 0.f), fmaxf(a[2 * c + 1], 0.f));
+}
+
+// Lattice window around a site: columns x0 .. x0 + wx - 1 (periodic), rows likewise; all of the lattice in a
+// direction shorter than the window.
+struct CnBox {
+  int x0, y0, wx, wy;
+  __device__ __forceinline__ int count() const { return wx * wy; }
+  __device__ __forceinline__ int x(const Dev& d, int k) const { return cn_wrap(x0 + k % wx, d.nx); }
+  __device__ __forceinline__ int y(const Dev& d, int k) const { return cn_wrap(y0 + k / wx, d.ny); }
+};
+__device__ __forceinline__ CnBox cn_box(const Dev& d, int i, int radius) {
+  const int w = 2 * radius + 1, x = i % d.nx, y = i / d.nx;
+  return CnBox{w < d.nx ? cn_wrap(x - radius, d.nx) : 0, w < d.ny ? cn_wrap(y - radius, d.ny) : 0, min(w, d.nx), min(w, d.ny)};
+}
+
+// wbar . h2 of 16 points by one warp: rows g, g + 8 are the points (l, x, y)[2].  Layer-1 values of sites in
+// `box` come from `win` ([L][box][8]), of the others from `cur` ([L][n][8]).  Every lane of a quad gets both.
+__device__ __forceinline__ void cn_tile(const Dev& d, const CnSm& w, const int (&l)[2], const int (&x)[2], const int (&y)[2],
+                                        const uint4* cur, const uint4* win, const CnBox& box, float (&s)[2]) {
+  const int lane = threadIdx.x & 31, t = lane & 3;
+  float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+  // per row: site columns and rows of the three offsets, and their places in the window (-1 outside)
+  int xs[2][3], ys[2][3], px[2][3], py[2][3];
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int o = 0; o < 3; ++o) {
+      xs[h][o] = cn_wrap(x[h] + o - 1, d.nx);
+      ys[h][o] = cn_wrap(y[h] + o - 1, d.ny);
+      const int a = cn_wrap(xs[h][o] - box.x0, d.nx), b = cn_wrap(ys[h][o] - box.y0, d.ny);
+      px[h][o] = a < box.wx ? a : -1;
+      py[h][o] = b < box.wy ? b : -1;
+      ys[h][o] *= d.nx;
+    }
+  const int n1 = box.count();
+#pragma unroll 1
+  for (int dl = 0; dl < 3; ++dl) {
+    const uint4 *c[2], *v[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int ll = cn_wrap(l[h] + dl - 1, d.L);
+      c[h] = cur + (size_t)ll * d.n * 8;
+      v[h] = win + (size_t)ll * n1 * 8;
+    }
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+      const uint4* p[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int a = px[h][q % 3], b = py[h][q / 3];
+        p[h] = (a >= 0 && b >= 0) ? v[h] + (b * box.wx + a) * 8 : c[h] + (ys[h][q / 3] + xs[h][q % 3]) * 8;
+      }
+      const uint4 a0 = p[0][t], a1 = p[1][t], a2 = p[0][t + 4], a3 = p[1][t + 4];
+      const uint32_t hi[4] = {a0.x, a1.x, a2.x, a3.x}, mid[4] = {a0.y, a1.y, a2.y, a3.y}, lo[4] = {a0.z, a1.z, a2.z, a3.z};
+#pragma unroll
+      for (int nt = 0; nt < 2; ++nt) {
+        const uint2 b = w.w2[((9 * dl + q) * 2 + nt) * 32 + lane];
+        float e[4] = {0.f, 0.f, 0.f, 0.f};
+        mma_bf16(e, lo, b);
+        mma_bf16(e, mid, b);
+        mma_bf16(e, hi, b);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) acc[nt][k] += e[k];
+      }
+    }
+  }
+  s[0] = s[1] = 0.f;
+#pragma unroll
+  for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int ch = 8 * nt + 2 * t + (k & 1);
+      const float h2 = fmaxf(acc[nt][k] + w.b2[ch], 0.f);
+      s[k >> 1] = fmaf(h2, w.wh[ch], fmaf(h2, w.wl[ch], s[k >> 1]));
+    }
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    s[h] += __shfl_xor_sync(HQ_FULL, s[h], 1);
+    s[h] += __shfl_xor_sync(HQ_FULL, s[h], 2);
+  }
+}
+
+// F_cnn of one configuration by the whole CTA from the network inputs xf [L][n]; layer 1 goes to h1
+// [L][n][8] and every point's wbar . h2 to s2 [L][n].  Returns F in every thread.
+__device__ inline double cn_refresh(const Dev& d, const CnSm& w, const float* xf, uint4* h1, float* s2, double* red) {
+  const int n = d.n, NL = d.n * d.L, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2;
+  for (int e = threadIdx.x; e < 2 * NL; e += HQ_THREADS) {
+    const int p = e >> 1, l = p / n, i = p % n;
+    cn_point1(d, w, l, i % d.nx, i / d.nx, e & 1, [&](int ll, int j) { return xf[ll * n + j]; }, h1 + (size_t)p * 8);
   }
   __syncthreads();
-  auto h1at = [&](int ll, int j) {
-    const int k = pos1[j];
-    return k >= 0 ? h1p + ((size_t)ll * n1 + k) * CN_C : h1c + ((size_t)ll * n + j) * CN_C;
-  };
-  for (int q = threadIdx.x; q < n2 * L; q += blockDim.x) {
-    const int l = q / n2, k = q % n2;
-    cn_layer2(d, w, l, l2[k], h1at, h2p + (size_t)q * CN_C);
-  }
-  __syncthreads();
-  auto h2at = [&](int ll, int j) {
-    const int k = pos2[j];
-    return k >= 0 ? h2p + ((size_t)ll * n2 + k) * CN_C : h2c + ((size_t)ll * n + j) * CN_C;
-  };
+  const CnBox none{0, 0, 0, 0};
   double part = 0.0;
-  for (int q = threadIdx.x; q < n3 * L; q += blockDim.x) {
-    const int l = q / n3, k = q % n3, j = l3[k];
-    const float o = cn_layer3(d, w, l, j, h2at);
-    o3p[q] = o;
-    part += (double)o - (double)o3c[(size_t)l * n + j];
+  for (int base = warp * 16; base < NL; base += HQ_WARPS * 16) {
+    int l[2], x[2], y[2];
+    float s[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int p = min(base + g + 8 * h, NL - 1), i = p % n;
+      l[h] = p / n;
+      x[h] = i % d.nx;
+      y[h] = i / d.nx;
+    }
+    cn_tile(d, w, l, x, y, h1, h1, none, s);
+    if ((lane & 3) == 0) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int p = base + g + 8 * h;
+        if (p < NL) {
+          s2[p] = s[h];
+          part += (double)s[h];
+        }
+      }
+    }
+  }
+  return block_sum(part, red) + (double)NL * (double)w.b3;
+}
+
+// F_cnn(X') - F_cnn(X) for X'(i, .) = X(i, .) + dx: z'(l, i) = xsh[l], the other inputs from xf; h1, s2 the caches
+// of X; the proposal's layer 1 (radius 1) goes to h1p, its points (radius 2) to s2p.  Called by the
+// whole CTA; returns the difference in every thread.
+__device__ inline double cn_block_delta(const Dev& d, const CnSm& w, const float* xf, const float* xsh, int i,
+                                        const uint4* h1, const float* s2, uint4* h1p, float* s2p, double* red) {
+  const int n = d.n, L = d.L, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2;
+  const CnBox b1 = cn_box(d, i, 1), b2 = cn_box(d, i, 2);
+  const int n1 = b1.count(), n2 = b2.count();
+  for (int e = threadIdx.x; e < 2 * n1 * L; e += HQ_THREADS) {
+    const int q = e >> 1, l = q / n1, k = q % n1;
+    cn_point1(d, w, l, b1.x(d, k), b1.y(d, k), e & 1, [&](int ll, int j) { return j == i ? xsh[ll] : xf[ll * n + j]; },
+              h1p + (size_t)q * 8);
+  }
+  __syncthreads();
+  double part = 0.0;
+  for (int base = warp * 16; base < n2 * L; base += HQ_WARPS * 16) {
+    int l[2], x[2], y[2];
+    float s[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int q = min(base + g + 8 * h, n2 * L - 1), k = q % n2;
+      l[h] = q / n2;
+      x[h] = b2.x(d, k);
+      y[h] = b2.y(d, k);
+    }
+    cn_tile(d, w, l, x, y, h1, h1p, b1, s);
+    if ((lane & 3) == 0) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int q = base + g + 8 * h;
+        if (q < n2 * L) {
+          s2p[q] = s[h];
+          part += (double)s[h] - (double)s2[l[h] * n + x[h] + d.nx * y[h]];
+        }
+      }
+    }
   }
   return block_sum(part, red);
 }
 
-// Accepted block move: the window values become the cached activations.
-__device__ inline void cn_block_commit(const Dev& d, const CnWindow& wd, float* h1c, float* h2c, float* o3c,
-                                       const float* h1p, const float* h2p, const float* o3p) {
-  const int n = d.n, L = d.L;
-  const int n1 = wd.cnt[0], n2 = wd.cnt[1], n3 = wd.cnt[2];
-  for (int q = threadIdx.x; q < n1 * L * 4; q += blockDim.x) {
-    const int pt = q / 4, v = q % 4, l = pt / n1, j = wd.lst[pt % n1];
-    reinterpret_cast<float4*>(h1c + ((size_t)l * n + j) * CN_C)[v] = reinterpret_cast<const float4*>(h1p + (size_t)pt * CN_C)[v];
+// Accepted block move: the window values become the caches.  Ends with a barrier.
+__device__ inline void cn_block_commit(const Dev& d, int i, uint4* h1, float* s2, const uint4* h1p, const float* s2p) {
+  const CnBox b1 = cn_box(d, i, 1), b2 = cn_box(d, i, 2);
+  const int n = d.n, L = d.L, n1 = b1.count(), n2 = b2.count();
+  for (int e = threadIdx.x; e < n1 * L * 8; e += HQ_THREADS) {
+    const int q = e >> 3, l = q / n1, k = q % n1;
+    h1[((size_t)l * n + b1.x(d, k) + d.nx * b1.y(d, k)) * 8 + (e & 7)] = h1p[e];
   }
-  for (int q = threadIdx.x; q < n2 * L * 4; q += blockDim.x) {
-    const int pt = q / 4, v = q % 4, l = pt / n2, j = wd.lst[CN_WIN + pt % n2];
-    reinterpret_cast<float4*>(h2c + ((size_t)l * n + j) * CN_C)[v] = reinterpret_cast<const float4*>(h2p + (size_t)pt * CN_C)[v];
-  }
-  for (int q = threadIdx.x; q < n3 * L; q += blockDim.x) {
-    const int l = q / n3, j = wd.lst[2 * CN_WIN + q % n3];
-    o3c[(size_t)l * n + j] = o3p[q];
+  for (int q = threadIdx.x; q < n2 * L; q += HQ_THREADS) {
+    const int l = q / n2, k = q % n2;
+    s2[l * n + b2.x(d, k) + d.nx * b2.y(d, k)] = s2p[q];
   }
   __syncthreads();
 }

@@ -925,7 +925,7 @@ constexpr int kCnnParamsPad = (HQ_CNN_PARAMS + 3) & ~3;
 
 struct NNLayout {
   size_t wbf, master, grad, am, av, partials, fcache, fnew, X0, ld0, F0, F1, pc, Fb, loss, idx, counters, dFpath, G0, xf, xb;
-  size_t cwbf, cmaster, cgrad, cam, cav, cpartials, h1c, h2c, o3c, h1p, h2p, o3p, tr, cFb, cF;
+  size_t cwbf, cmaster, cgrad, cam, cav, cpartials, h1c, s2c, h1p, s2p, tr, cFb, cF;
   int train_ctas;
   size_t total;
 };
@@ -965,12 +965,10 @@ NNLayout nn_layout(const hq::Dev& d, int max_batch, int max_samples) {
   l.cam = take(4 * PC);
   l.cav = take(4 * PC);
   l.cpartials = take(4 * PC * l.train_ctas);
-  l.h1c = take(4 * C * NL * CH);
-  l.h2c = take(4 * C * NL * CH);
-  l.o3c = take(4 * C * NL);
-  l.h1p = take(4 * C * 9 * d.L * CH);
-  l.h2p = take(4 * C * 25 * d.L * CH);
-  l.o3p = take(4 * C * 49 * d.L);
+  l.h1c = take(16 * C * NL * (CH / 2));
+  l.s2c = take(4 * C * NL);
+  l.h1p = take(16 * C * 9 * d.L * (CH / 2));
+  l.s2p = take(4 * C * 25 * d.L);
   l.tr = take(4 * (size_t)l.train_ctas * 3 * NL * CH);
   l.cFb = take(8 * (size_t)max_batch);
   l.cF = take(8 * C);
@@ -1038,12 +1036,11 @@ int hq_nn_attach(hq_engine* e, void* arena, size_t bytes, int max_batch, int max
   cn.adam_v = (float*)(a + l.cav);
   cn.partials = (float*)(a + l.cpartials);
   cn.train_ctas = l.train_ctas;
-  cn.h1c = (float*)(a + l.h1c);
-  cn.h2c = (float*)(a + l.h2c);
-  cn.o3c = (float*)(a + l.o3c);
-  cn.h1p = (float*)(a + l.h1p);
-  cn.h2p = (float*)(a + l.h2p);
-  cn.o3p = (float*)(a + l.o3p);
+  cn.h1c = (uint4*)(a + l.h1c);
+  cn.s2c = (float*)(a + l.s2c);
+  cn.h1p = (uint4*)(a + l.h1p);
+  cn.s2p = (float*)(a + l.s2p);
+  cn.xf = nn.xf;
   cn.tr = (float*)(a + l.tr);
   cn.Fb = (double*)(a + l.cFb);
   cn.F = (double*)(a + l.cF);

@@ -120,9 +120,8 @@ struct NNState {
 };
 
 // Periodic 3D convolutional action for block moves: three 3x3x3 layers 1 -> 16 -> 16 -> 1
-// on the (x, y, tau) torus, summed over every point.  Activations are stored after the ReLU,
-// 16 floats per point (point-major).  Window buffers hold the block-move proposal around the
-// moved site: radius 1 (layer 1), 2 (layer 2), 3 (layer 3) in the lattice, every slice.
+// on the (x, y, tau) torus, summed over every point.  Window buffers hold the block-move proposal
+// around the moved site: radius 1 (layer 1) and 2 (layer 2) in the lattice, every slice.
 constexpr int kCnnC = 16;
 constexpr int kCnnTrainCtas = 152;
 struct CnnState {
@@ -134,12 +133,11 @@ struct CnnState {
   float* adam_v;
   float* partials;      // [train_ctas][padded params]
   int train_ctas;
-  float* h1c;           // [C][L N][16] layer-1 activations of the current fields
-  float* h2c;           // [C][L N][16]
-  float* o3c;           // [C][L N] layer-3 outputs
-  float* h1p;           // [C][9 L][16] proposal, window radius 1
-  float* h2p;           // [C][25 L][16] radius 2
-  float* o3p;           // [C][49 L] radius 3
+  uint4* h1c;           // [C][L N][8] layer-1 activations of the current fields (split, by channel pairs)
+  float* s2c;           // [C][L N] every point's share of F
+  uint4* h1p;           // [C][9 L][8] proposal, window radius 1
+  float* s2p;           // [C][25 L] radius 2
+  float* xf;            // [C][L N] network inputs (float)(X - x0), the patch network's table
   float* tr;            // [train_ctas][3][L N][16] training activations and gradients
   double* Fb;           // [max batch] minibatch F
   double* F;            // [C]

@@ -47,14 +47,14 @@ struct NNSmem {
   double* pds;   // [n] dtau dS_ph
   double* gacc;  // [NN_GROUPS] per-group sums
   double* scal;  // [8]
-  float* cw;     // [CN_WPAD] convolutional weights (with_cnn)
-  CnWindow win;  // block-move window (with_cnn)
+  char* cw;      // convolutional weights (with_cnn)
 };
 
 __host__ __device__ inline size_t nn_smem_bytes(int n, bool with_cnn = false) {
   size_t b = sizeof(uint2) * TC_FRAGS + sizeof(double) * (HQ_WARPS + 3 * (size_t)n + NN_GROUPS + 8) +
              sizeof(float) * (TC_FLOATS + 32 + 128 + (size_t)n) + sizeof(int) * (4 + 5 * (size_t)n);
-  if (with_cnn) b += sizeof(float) * CN_WPAD + sizeof(int) * (4 + 3 * CN_WIN + 2 * (size_t)n);
+  b = (b + 15) & ~(size_t)15;
+  if (with_cnn) b += cn_smem_bytes();
   return b;
 }
 
@@ -75,14 +75,7 @@ __device__ inline NNSmem nn_carve(int n, char* base, bool with_cnn = false) {
   s.flag = (volatile int*)f; f += 4;
   s.pxf = f; f += n;
   s.nbr = (int*)f; f += 5 * n;
-  s.cw = nullptr;
-  if (with_cnn) {
-    s.cw = f; f += CN_WPAD;
-    int* q = (int*)f;
-    s.win.cnt = q; q += 4;
-    s.win.lst = q; q += 3 * CN_WIN;
-    s.win.pos = q;
-  }
+  s.cw = with_cnn ? base + nn_smem_bytes(n) : nullptr;
   return s;
 }
 
@@ -233,22 +226,18 @@ __global__ void __launch_bounds__(HQ_THREADS, 2) nn_inner_kernel(Dev d, NNState 
   const NNSmem s = nn_carve(n, nraw, use_cnn != 0);
   build_cross(d, s.nbr);
   const NNFrags w = nn_build_frags(nn.wbf, s.frag, s.tcf);  // (ends with a barrier)
-  if (use_cnn) cn_load_weights(cn.wbf, s.cw);
+  CnSm cw{};
+  if (use_cnn) cw = cn_setup(cn.wbf, s.cw);
   double* X = d.X + (size_t)c * NL;
   float* xf = nn.xf + (size_t)c * NL;  // inputs of the current fields, kept with X below
   to_inputs(X, nn.x0, xf, NL);
   float* fc = nn.fcache + (size_t)c * NL;
   float* fnew = nn.fnew + (size_t)c * 6 * L;
   float* xsh = fnew + 5 * L;  // inputs of the moved site's proposed values (block moves)
-  float *h1c = nullptr, *h2c = nullptr, *o3c = nullptr, *h1p = nullptr, *h2p = nullptr, *o3p = nullptr;
-  if (use_cnn) {
-    h1c = cn.h1c + (size_t)c * NL * CN_C;
-    h2c = cn.h2c + (size_t)c * NL * CN_C;
-    o3c = cn.o3c + (size_t)c * NL;
-    h1p = cn.h1p + (size_t)c * 9 * L * CN_C;
-    h2p = cn.h2p + (size_t)c * 25 * L * CN_C;
-    o3p = cn.o3p + (size_t)c * CN_WIN * L;
-  }
+  uint4* h1c = cn.h1c + (size_t)c * NL * 8;
+  float* s2c = cn.s2c + (size_t)c * NL;
+  uint4* h1p = cn.h1p + (size_t)c * 9 * L * 8;
+  float* s2p = cn.s2p + (size_t)c * 25 * L;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, g = lane >> 2, t = lane & 3;
   const uint32_t* id = d.cid + 4 * (size_t)c;
   const uint32_t key0 = id[0], key1 = id[1], chain = id[2], step = id[3];
@@ -415,7 +404,7 @@ __global__ void __launch_bounds__(HQ_THREADS, 2) nn_inner_kernel(Dev d, NNState 
     }
     if (!local_part && do_block) {
       if (use_cnn && cn_stale) {
-        cn_forward_all(d, s.cw, X, nn.x0, h1c, h2c, o3c, s.red);
+        cn_refresh(d, cw, xf, h1c, s2c, s.red);
         cn_stale = false;
       }
       for (int i0 = 0; i0 < Wb; ++i0) {
@@ -438,8 +427,7 @@ __global__ void __launch_bounds__(HQ_THREADS, 2) nn_inner_kernel(Dev d, NNState 
         const double dS = pfac * a;
         double dF;
         if (use_cnn) {
-          cn_build_window(d, i, s.win);
-          dF = cn_block_delta(d, s.cw, s.win, X, nn.x0, i, dx, h1c, h2c, o3c, h1p, h2p, o3p, s.red);
+          dF = cn_block_delta(d, cw, xf, xsh, i, h1c, s2c, h1p, s2p, s.red);
         } else {
           // the 5 L patches containing site i: patch q has centre (q / 5, i - c), c = q % 5; warp
           // w takes the tiles w, w + 8, ... of 16 patches
@@ -494,7 +482,7 @@ __global__ void __launch_bounds__(HQ_THREADS, 2) nn_inner_kernel(Dev d, NNState 
             xf[(size_t)sl * n + i] = net_input(v, nn.x0);
           }
           if (use_cnn) {
-            cn_block_commit(d, s.win, h1c, h2c, o3c, h1p, h2p, o3p);
+            cn_block_commit(d, i, h1c, s2c, h1p, s2p);
             fc_stale = true;
           } else {
             for (int q = threadIdx.x; q < 5 * L; q += HQ_THREADS)
