@@ -165,7 +165,7 @@ __device__ __noinline__ void slice_product(const Dev& d, const Smem& sm, double*
   HQ_TIC(kin);
   if (n <= kTiny) {
     tiny_slices<kAfter>(d.nx, d.ny, n, sm.ex, sm.ey, P, U, D, count, [&](int k, int r) { return src(d, k, r); },
-                        reinterpret_cast<double*>(sm.oz.frag));
+                        reinterpret_cast<double*>(sm.oz.frag), (int)(oz_frag_bytes(n) / sizeof(double) - 512) / n);
     HQ_TOC(kin, SEC_KIN);
     return;
   }

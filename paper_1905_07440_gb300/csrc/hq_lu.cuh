@@ -1,11 +1,10 @@
 // LU with partial pivoting and its solves: panels of 16 columns in registers, everything else as 16-term products on the tensor cores (hq_oz.cuh).
 //
-// A panel is held by four warps, one per scheduler (see hq_panel.cuh: FP64 instructions are what counts),
-// with one row per thread (two for m > 128) or G = 2, 4 threads per row for m <= 64, 32.  A column step
-// needs one barrier: every warp offers its best remaining row (largest high word, by one REDUX) with that
-// row's entries, and after the barrier all threads take the best offer and update their own rows.  Rows
-// are not moved; each thread tracks the position its rows end at.  The column-by-column form in memory took
-// four barriers and about 5800 cycles per column at n = 64.
+// A panel is held by four warps as in hq_panel.cuh (column c in warp c % 4, its rows over the lanes).  Per step
+// the pivot column goes to all warps through shared memory (one barrier); every warp then finds the pivot
+// (largest high word, one REDUX) and updates its own columns, so no row crosses warps.  Rows are not moved;
+// every lane tracks the position its rows end at.  The column-by-column form in memory took four barriers
+// and about 5800 cycles per column at n = 64.
 // Triangles: the 16 x 16 diagonal blocks are inverted once (one warp each, 60 dependent FP64
 // instructions), so the triangular solves become products too.
 #pragma once
@@ -28,41 +27,44 @@ __device__ __forceinline__ double recip_fp64(double u) {
 }
 
 struct LuShared {
-  double row[2][kPanelWarps][16];
-  int key[2][kPanelWarps], pos[2][kPanelWarps];
+  double col[2][256];
 };
 
 // Columns p0 .. p0 + kb - 1, rows p0 .. n - 1 of A, in place (L below, U on and above the diagonal, rows
 // in pivot order); piv[p0 + j] = the row swapped with p0 + j at step j.  Ends with a barrier.
-template <int LM, int CPT, int RPT>
+template <int LM, int RPL>
 __device__ __noinline__ void lu_panel_rows(double* A, int ld, int n, int p0, int kb, int* piv, LuShared* ls) {
-  constexpr int G = 16 / CPT, LG = G == 4 ? 2 : G == 2 ? 1 : 0, kThreads = 32 * kPanelWarps, kRows = kThreads / G;
+  constexpr int kThreads = 32 * kPanelWarps;
   const int m = n - p0, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (warp < kPanelWarps) {
-    const int row0 = tid >> LG, cq = tid & (G - 1);
-    double x[RPT][CPT];
-    int pos[RPT];
-    bool active[RPT];
+    double x[RPL][4];
+    int pos[RPL];
+    bool active[RPL];
 #pragma unroll
-    for (int r = 0; r < RPT; ++r) {
-      pos[r] = row0 + r * kRows;
+    for (int r = 0; r < RPL; ++r) {
+      pos[r] = lane + 32 * r;
       active[r] = pos[r] < m;
 #pragma unroll
-      for (int i = 0; i < CPT; ++i) {
-        const int c = i * G + cq;
+      for (int i = 0; i < 4; ++i) {
+        const int c = 4 * i + warp;
         x[r][i] = (active[r] && c < kb) ? A[(size_t)(p0 + c) * ld + p0 + pos[r]] : 0.0;
       }
     }
+    if (warp == 0) {
+#pragma unroll
+      for (int r = 0; r < RPL; ++r) ls->col[0][lane + 32 * r] = x[r][0];
+    }
+    bar_warps(kThreads);
 #pragma unroll 1
     for (int j = 0; j < kb; ++j) {
-      // x[.][i] holds column ((i + jb) % CPT) G + cq; entries i < CPT - jb are the columns not yet done
-      const int jo = j & (G - 1), jb = j >> LG, left = CPT - jb, b = j & 1;
-      double xj[RPT];
+      // x[.][i] is column 4 ((i + done) % 4) + warp; the warp's columns after j are entries first .. left - 1
+      const int jw = j & 3, done = j >> 2, left = 4 - done, first = warp <= jw ? 1 : 0;
+      double xj[RPL];
       uint32_t key = 0;
       int kr = 0;
 #pragma unroll
-      for (int r = 0; r < RPT; ++r) {
-        xj[r] = G == 1 ? x[r][0] : __shfl_sync(HQ_FULL, x[r][0], (lane & ~(G - 1)) | jo);
+      for (int r = 0; r < RPL; ++r) {
+        xj[r] = ls->col[j & 1][lane + 32 * r];
         const uint32_t k = active[r] ? oz_abs_hi(xj[r]) + 1u : 0u;
         if (k > key) {
           key = k;
@@ -70,69 +72,71 @@ __device__ __noinline__ void lu_panel_rows(double* A, int ld, int n, int p0, int
         }
       }
       const uint32_t best = __reduce_max_sync(HQ_FULL, key);
-      const int cand = (__ffs(__ballot_sync(HQ_FULL, key == best)) - 1) & ~(G - 1);
-      const bool mine = (lane & ~(G - 1)) == cand;
-      if (mine) {
+      const int win = __ffs(__ballot_sync(HQ_FULL, key == best)) - 1;
+      auto pick = [&](const double (&v)[RPL]) {
+        double w = v[0];
 #pragma unroll
-        for (int r = 0; r < RPT; ++r)
-          if (r == kr) {
+        for (int r = 1; r < RPL; ++r)
+          if (kr == r) w = v[r];
+        return __shfl_sync(HQ_FULL, w, win);
+      };
+      int pk = pos[0];
 #pragma unroll
-            for (int i = 0; i < CPT; ++i) ls->row[b][warp][((i + jb) & (CPT - 1)) * G + cq] = x[r][i];
-            if (cq == 0) {
-              ls->key[b][warp] = (int)best;
-              ls->pos[b][warp] = pos[r];
-            }
-          }
-      }
-      bar_warps(kThreads);
-      int win = 0;
-      uint32_t top = (uint32_t)ls->key[b][0];
-#pragma unroll
-      for (int w = 1; w < kPanelWarps; ++w) {
-        const uint32_t k = (uint32_t)ls->key[b][w];
-        if (k > top) {
-          top = k;
-          win = w;
-        }
-      }
-      const double* u = ls->row[b][win];
-      const int from = ls->pos[b][win];
+      for (int r = 1; r < RPL; ++r)
+        if (kr == r) pk = pos[r];
+      const int from = __shfl_sync(HQ_FULL, pk, win);
+      const double rp = recip_fp64(pick(xj));
       if (tid == 0) piv[p0 + j] = p0 + from;
-      const double rp = recip_fp64(u[j]);
 #pragma unroll
-      for (int r = 0; r < RPT; ++r) {
-        if (warp == win && mine && r == kr) {
+      for (int r = 0; r < RPL; ++r) {
+        if (lane == win && kr == r) {
           pos[r] = j;
           active[r] = false;
         } else if (pos[r] == j) {
           pos[r] = from;
         }
-        const double l = xj[r] * rp;
+      }
+      double l[RPL];
 #pragma unroll
-        for (int i = 0; i < CPT; ++i)
-          if (i < left) {
-            const int c = i * G + jb * G + cq;
-            const double upd = fma(-l, u[c], x[r][i]);
-            if (active[r]) {
-              if (c > j) x[r][i] = upd;
-              else if (c == j) x[r][i] = l;
-            }
-          }
-        if (jo == G - 1) {
-          const double first = x[r][0];
+      for (int r = 0; r < RPL; ++r) l[r] = active[r] ? xj[r] * rp : 0.0;
 #pragma unroll
-          for (int i = 0; i + 1 < CPT; ++i) x[r][i] = x[r][i + 1];
-          x[r][CPT - 1] = first;
+      for (int i = 0; i < 4; ++i)
+        if (i < left && i >= first) {
+          double col[RPL];
+#pragma unroll
+          for (int r = 0; r < RPL; ++r) col[r] = x[r][i];
+          const double u = pick(col);
+#pragma unroll
+          for (int r = 0; r < RPL; ++r) x[r][i] = fma(-l[r], u, x[r][i]);
+        }
+      if (j + 1 < kb && warp == ((j + 1) & 3)) {
+        const bool turned = jw == 3;  // warp 0 takes its next column
+#pragma unroll
+        for (int r = 0; r < RPL; ++r) ls->col[(j + 1) & 1][lane + 32 * r] = turned ? x[r][1] : x[r][0];
+      }
+      if (warp == jw) {
+#pragma unroll
+        for (int r = 0; r < RPL; ++r)
+          if (active[r]) x[r][0] = l[r];
+      }
+      if (jw == 3) {
+#pragma unroll
+        for (int r = 0; r < RPL; ++r) {
+          const double f = x[r][0];
+#pragma unroll
+          for (int i = 0; i < 3; ++i) x[r][i] = x[r][i + 1];
+          x[r][3] = f;
         }
       }
+      bar_warps(kThreads);
     }
-    const int jb = kb >> LG;
+    const int done = kb >> 2;
 #pragma unroll
-    for (int r = 0; r < RPT; ++r)
-      if (row0 + r * kRows < m) {
+    for (int r = 0; r < RPL; ++r)
+      if (lane + 32 * r < m) {
 #pragma unroll
-        for (int i = 0; i < CPT; ++i) {
-          const int c = ((i + jb) & (CPT - 1)) * G + cq;
+        for (int i = 0; i < 4; ++i) {
+          const int c = 4 * ((i + done) & 3) + warp;
           if (c < kb) A[(size_t)(p0 + c) * ld + p0 + pos[r]] = x[r][i];
         }
       }
@@ -248,10 +252,10 @@ __device__ inline double oz_lu(double* A, int n, int* piv, double* red, double* 
   LuShared* ls = reinterpret_cast<LuShared*>(frag);
   for (int p0 = 0; p0 < n; p0 += 16) {
     const int kb = min(16, n - p0), p1 = p0 + kb, m = n - p0;
-    if (m <= 32) lu_panel_rows<LM, 4, 1>(A, n, n, p0, kb, piv, ls);
-    else if (LM <= 8 || m <= 64) lu_panel_rows<LM, 8, 1>(A, n, n, p0, kb, piv, ls);  // LM <= 8: n <= 64
-    else if (m <= 128) lu_panel_rows<LM, LM <= 8 ? 8 : 16, 1>(A, n, n, p0, kb, piv, ls);
-    else lu_panel_rows<LM, LM <= 8 ? 8 : 16, LM <= 8 ? 1 : 2>(A, n, n, p0, kb, piv, ls);
+    if (m <= 32) lu_panel_rows<LM, 1>(A, n, n, p0, kb, piv, ls);
+    else if (LM <= 8 || m <= 64) lu_panel_rows<LM, 2>(A, n, n, p0, kb, piv, ls);  // LM <= 8: n <= 64
+    else if (m <= 128) lu_panel_rows<LM, LM <= 8 ? 2 : 4>(A, n, n, p0, kb, piv, ls);
+    else lu_panel_rows<LM, LM <= 8 ? 2 : 8>(A, n, n, p0, kb, piv, ls);
     double* M = tri + (p0 >> 4) * 256;
     if (tid < 32) invert_triangle<true>(A, n, p0, kb, M);
     else
@@ -279,12 +283,27 @@ template <int LM>
 __device__ inline void oz_lu_solve(const double* A, int n, const int* piv, double* Y, double* tri, uint2* frag,
                                    int* er) {
   const int tid = threadIdx.x, warp = tid >> 5;
-  for (int c = tid; c < n; c += HQ_THREADS) {
-    double* y = Y + (size_t)c * n;
+  // all row swaps at once: thread 0 turns them into a permutation, then a warp moves a column
+  int* perm = er;
+  if (tid == 0) {
+    for (int r = 0; r < n; ++r) perm[r] = r;
     for (int j = 0; j < n; ++j) {
-      const int p = piv[j];
-      if (p != j) { const double v = y[j]; y[j] = y[p]; y[p] = v; }
+      const int p = piv[j], v = perm[j];
+      perm[j] = perm[p];
+      perm[p] = v;
     }
+  }
+  __syncthreads();
+  for (int c = warp; c < n; c += HQ_WARPS) {
+    double* y = Y + (size_t)c * n;
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if ((tid & 31) + 32 * u < n) v[u] = y[perm[(tid & 31) + 32 * u]];
+    __syncwarp();
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if ((tid & 31) + 32 * u < n) y[(tid & 31) + 32 * u] = v[u];
   }
   __syncthreads();
   for (int p0 = 0; p0 < n; p0 += 16) {

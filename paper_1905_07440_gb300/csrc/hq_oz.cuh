@@ -453,6 +453,49 @@ __device__ __forceinline__ void oz_kin_split(const double (&z)[2][4], bool two_x
       oz_split<kOzP>(z[w][2 * h], z[w][2 * h + 1], E[h][w], E[h][w], q[2 * w + h]);
 }
 
+// Digits of the tile sums T (units as oz_mma's) straight from the integers: the sums of a block share one
+// scale (E, with the factor's bound kex), so all they need is a common shift that brings the largest
+// below 2^58.  Without the way through doubles (conversion, exponent, mantissa) this is about half of the
+// instructions of a split.  E becomes the bounds of the shifted blocks.
+__device__ __forceinline__ void oz_kin_resplit(const long long (&T)[2][4], int kex, bool two_x, bool two_y,
+                                               uint32_t (&q)[4][kOzDigits], int (&E)[2][2]) {
+  constexpr unsigned long long kBias = 512ull * (1ull + (1ull << 10) + (1ull << 20) + (1ull << 30) + (1ull << 40) +
+                                                 (1ull << 50));
+  auto mag = [](long long v) { return (uint32_t)((v ^ (v >> 63)) >> 32); };
+  uint32_t m[2][2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int w = 0; w < 2; ++w) m[h][w] = max(mag(T[w][2 * h]), mag(T[w][2 * h + 1]));
+  if (!two_x) {
+    m[0][0] = m[0][1] = max(m[0][0], m[0][1]);
+    m[1][0] = m[1][1] = max(m[1][0], m[1][1]);
+  }
+  if (!two_y) {
+    m[0][0] = m[1][0] = max(m[0][0], m[1][0]);
+    m[0][1] = m[1][1] = max(m[0][1], m[1][1]);
+  }
+  if (!two_x && !two_y) {
+    m[0][0] = m[0][1] = m[1][0] = m[1][1] = __reduce_max_sync(HQ_FULL, m[0][0]);
+  } else {
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int w = 0; w < 2; ++w) m[h][w] = __reduce_max_sync(HQ_FULL, m[h][w]);
+  }
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int w = 0; w < 2; ++w) {
+      const int up = 58 - (64 - __clz((int)m[h][w]));  // |T| < 2^(64 - clz)
+      const unsigned long long u = up >= 0 ? (unsigned long long)T[w][2 * h] << up : (unsigned long long)(T[w][2 * h] >> -up);
+      const unsigned long long v =
+          up >= 0 ? (unsigned long long)T[w][2 * h + 1] << up : (unsigned long long)(T[w][2 * h + 1] >> -up);
+      oz_pack(kBias + u, kBias + v, q[2 * w + h]);
+      E[h][w] += kex - 1021 - up;
+    }
+}
+
 // Z <- F_y Z F_x^T for a tile.
 __device__ __forceinline__ void oz_kin_tile(const OzKin& K, double (&z)[2][4], bool two_x, bool two_y) {
   const int lane = threadIdx.x & 31;
@@ -460,16 +503,14 @@ __device__ __forceinline__ void oz_kin_tile(const OzKin& K, double (&z)[2][4], b
   int E[2][2];
   // over x: the tile is the left operand
   oz_kin_split(z, two_x, two_y, q, E);
+  long long T[2][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}};
 #pragma unroll
   for (int w = 0; w < 2; ++w) {
-    long long T[4] = {0, 0, 0, 0};
     const uint2* fr = K.fx + w * 6 * 32 + lane;
-    oz_mma(q, [&](int d) { return fr[d * 32]; }, T);
-#pragma unroll
-    for (int e = 0; e < 4; ++e) z[w][e] = oz_scale((double)T[e], oz_expo<kOzP>(E[e >> 1][w], K.ex));
+    oz_mma(q, [&](int d) { return fr[d * 32]; }, T[w]);
   }
   // over y: the tile is the right operand (8 x 8 blocks transposed in registers)
-  oz_kin_split(z, two_x, two_y, q, E);
+  oz_kin_resplit(T, K.ex, two_x, two_y, q, E);
 #pragma unroll
   for (int b = 0; b < 4; ++b)
 #pragma unroll
@@ -485,10 +526,10 @@ __device__ __forceinline__ void oz_kin_tile(const OzKin& K, double (&z)[2][4], b
   }
 #pragma unroll
   for (int w = 0; w < 2; ++w) {
-    long long T[4] = {0, 0, 0, 0};
-    oz_mma(a, [&](int d) { return make_uint2(q[2 * w][d], q[2 * w + 1][d]); }, T);
+    long long S[4] = {0, 0, 0, 0};
+    oz_mma(a, [&](int d) { return make_uint2(q[2 * w][d], q[2 * w + 1][d]); }, S);
 #pragma unroll
-    for (int e = 0; e < 4; ++e) z[w][e] = oz_scale((double)T[e], oz_expo<kOzP>(E[e >> 1][w], K.ey));
+    for (int e = 0; e < 4; ++e) z[w][e] = oz_scale((double)S[e], oz_expo<kOzP>(E[e >> 1][w], K.ey));
   }
 }
 

@@ -97,9 +97,10 @@ __device__ __noinline__ void oz_panel(double* Q, double* V, int ld, int n, int j
                                       const OzScratch& z) {
   PanelShared* ps = reinterpret_cast<PanelShared*>(z.frag);
   const int m = n - j0;
-  if (LM <= 8 || m <= 64) panel_fixed<LM, 4>(Q, V, ld, n, j0, kb, ps, tau, z.ev);  // LM <= 8: n <= 64
-  else if (m <= 128) panel_fixed<LM, LM <= 8 ? 4 : 8>(Q, V, ld, n, j0, kb, ps, tau, z.ev);
-  else panel_fixed<LM, LM <= 8 ? 4 : 16>(Q, V, ld, n, j0, kb, ps, tau, z.ev);
+  if (m <= 32) panel_house<LM, 1>(Q, V, ld, n, j0, kb, ps, tau, z.ev);
+  else if (LM <= 8 || m <= 64) panel_house<LM, 2>(Q, V, ld, n, j0, kb, ps, tau, z.ev);  // LM <= 8: n <= 64
+  else if (m <= 128) panel_house<LM, LM <= 8 ? 2 : 4>(Q, V, ld, n, j0, kb, ps, tau, z.ev);
+  else panel_house<LM, LM <= 8 ? 2 : 8>(Q, V, ld, n, j0, kb, ps, tau, z.ev);
   stage_panel(z.frag, V, ld, n, j0, kb, z.ev);
   // the sums go behind the fragments, where the block application stages T
   const int nk = (m + 15) >> 4;
@@ -328,12 +329,23 @@ __device__ inline void oz_mm(int n, const double* A, const double* B, const doub
   else oz_product_mm<LM, false>(n, A, ar, ak, B, bk, bc, kd, cd, C, z);
 }
 
-// Flush of delayed updates: G(r, c) += sum_m A[m][r] B[m][c], m < kk (A, B [kk][n]).
+// Flush of delayed updates: G(r, c) += sum_m A[m][r] B[m][c], m < kk (A, B [kk][n]).  The wide class has an
+// instance of its own (its 65 thousand entries outweigh the code; 16x16 local sweeps 430 -> 390 ms).
 template <int LM>
-__device__ inline void oz_flush(double* G, const double* A, const double* B, int n, int kk, const OzScratch& z) {
-  for (int m0 = 0; m0 < kk; m0 += 16)
-    oz_rank<LM>(Rank16{A + (size_t)m0 * n, 1, n, B + (size_t)m0 * n, n, 1, G, n, 1.0, 1.0}, 0, n, 0, n, min(16, kk - m0),
-                z.frag, z.er);
+__device__ __noinline__ void oz_flush(double* G, const double* A, const double* B, int n, int kk, const OzScratch& z) {
+  for (int m0 = 0; m0 < kk; m0 += 16) {
+    const int kb = min(16, kk - m0);
+    if (LM <= 8)
+      oz_rank<LM>(Rank16{A + (size_t)m0 * n, 1, n, B + (size_t)m0 * n, n, 1, G, n, 1.0, 1.0}, 0, n, 0, n, kb, z.frag, z.er);
+    else
+      oz_rank16(false, 0, n, 0, n, kb, z.frag, z.er, [&](int r, int k) { return A[(m0 + k) * n + r]; },
+                [&](int k, int c) { return B[(m0 + k) * n + c]; },
+                [&](int r, int c, double s0, double s1) {
+                  double* p = G + c * n + r;
+                  const RowPair x = load_pair(p);
+                  store_pair(p, x.v0 + s0, x.v1 + s1);
+                });
+  }
 }
 
 // ------------------------------------------------------------ separable propagator
@@ -386,18 +398,23 @@ __device__ __forceinline__ void oz_slices(int nx, int ny, int n, const OzKin& K,
 }
 
 // The same for n <= kTiny in FP64: a matrix entry per thread, the columns in shared memory (buf: 512
-// doubles) between the two passes of a slice.
+// doubles and `cap` slices' diagonals) between the two passes of a slice.
 template <bool kAfter, class DV>
 __device__ __forceinline__ void tiny_slices(int nx, int ny, int n, const double* ex, const double* ey, double* P,
-                                            const double* U, const double* D, int count, DV dv, double* buf) {
+                                            const double* U, const double* D, int count, DV dv, double* buf, int cap) {
+  double* dbuf = buf + 512;  // [cap][n] diagonals of a run of slices
   const int i = threadIdx.x & 15, c = threadIdx.x >> 4, x = i % nx, y = i / nx;
   const bool on = i < n && c < n;
   double *A = buf + 16 * c, *T = buf + 256 + 16 * c;
   double v = 0.0;
   if (on) v = U ? U[(size_t)c * n + i] * D[c] : (i == c ? 1.0 : 0.0);
   for (int k = 0; k < count; ++k) {
-    const double d = on ? dv(k, i) : 0.0;
-    __syncthreads();
+    if (k % cap == 0) {
+      __syncthreads();
+      for (int w = threadIdx.x; w < min(cap, count - k) * n; w += HQ_THREADS) dbuf[w] = dv(k + w / n, w % n);
+      __syncthreads();
+    }
+    const double d = on ? dbuf[(k % cap) * n + i] : 0.0;
     A[i] = kAfter ? v : v * d;
     __syncthreads();
     double a = 0.0;
