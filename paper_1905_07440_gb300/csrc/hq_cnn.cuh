@@ -167,16 +167,10 @@ __device__ inline CnSm cn_setup(const uint16_t* wb, char* mem) {
 
 // Two non-negative activations as packed bfloat16 pairs hi + mid + lo.
 __device__ __forceinline__ uint4 cn_split(float a, float b) {
-  auto three = [](float v, uint32_t& h, uint32_t& m, uint32_t& l) {
-    h = float_to_bf16(v);
-    const float r = v - bf16_to_float((uint16_t)h);
-    m = float_to_bf16(r);
-    l = float_to_bf16(r - bf16_to_float((uint16_t)m));
-  };
-  uint32_t ah, am, al, bh, bm, bl;
-  three(a, ah, am, al);
-  three(b, bh, bm, bl);
-  return make_uint4(ah | (bh << 16), am | (bm << 16), al | (bl << 16), 0u);
+  const uint32_t h = cvt_bf16x2(a, b);
+  const float ra = a - __uint_as_float(h << 16), rb = b - __uint_as_float(h & 0xffff0000u);
+  const uint32_t m = cvt_bf16x2(ra, rb);
+  return make_uint4(h, m, cvt_bf16x2(ra - __uint_as_float(m << 16), rb - __uint_as_float(m & 0xffff0000u)), 0u);
 }
 
 __device__ __forceinline__ int cn_wrap(int a, int n) { return a < 0 ? a + n : (a >= n ? a - n : a); }

@@ -50,13 +50,28 @@ static constexpr int kSmemVecs = 9;
 // Kernel template class of a lattice: both sides up to 8 (N <= 64, two CTAs per SM), or up to 16.
 static inline int lmax_of(int nx, int ny) { return (nx > ny ? nx : ny) <= 8 ? 8 : 16; }
 
-// Shared memory of one chain's CTA: the layout of carve().
-size_t smem_bytes(const Dev& d) {
-  const int n = d.n;
-  return (size_t)(2 * d.nx * d.nx + 2 * d.ny * d.ny + kSmemVecs * n + 16 + 32 + 16 + 16 * oz_pad(n) + 256) *
-             sizeof(double) +
-         oz_frag_bytes(n) + 2 * kOzKinBytes + (size_t)(4 * oz_pad(n) + 2 * n + 8) * sizeof(int);
+// Shared memory of one chain's CTA without the fragment scratch.
+__host__ __device__ inline size_t smem_base_bytes(int nx, int ny, int n) {
+  return (size_t)(2 * nx * nx + 2 * ny * ny + kSmemVecs * n + 16 + 32 + 16 + 16 * oz_pad(n) + 256) * sizeof(double) +
+         2 * kOzKinBytes + (size_t)(4 * oz_pad(n) + 2 * n + 8) * sizeof(int);
 }
+
+// The delayed-update vectors A, B [k][n] sit behind a flush's fragments (oz_pad(n) 192 bytes) in that scratch
+// while a slice's moves run: every accepted move reads all pending ones, and through L2 those reads took
+// longer than the sums.  They stay in global memory where the scratch would pass the CTA's share of an SM
+// (two CTAs with both sides up to 8, else one).
+__host__ __device__ inline size_t delayed_bytes(int n, int k) { return (size_t)2 * k * n * sizeof(double); }
+__host__ __device__ inline bool delayed_in_smem(int nx, int ny, int n, int k) {
+  const size_t cap = nx <= 8 && ny <= 8 ? 112 * 1024 : 224 * 1024;
+  return smem_base_bytes(nx, ny, n) + (size_t)oz_pad(n) * 192 + delayed_bytes(n, k) <= cap;
+}
+__host__ __device__ inline size_t scratch_bytes(int nx, int ny, int n, int k) {
+  const size_t f = oz_frag_bytes(n), v = (size_t)oz_pad(n) * 192 + delayed_bytes(n, k);
+  return delayed_in_smem(nx, ny, n, k) && v > f ? v : f;
+}
+
+// Shared memory of one chain's CTA: the layout of carve().
+size_t smem_bytes(const Dev& d) { return smem_base_bytes(d.nx, d.ny, d.n) + scratch_bytes(d.nx, d.ny, d.n, d.k); }
 
 __device__ inline Smem carve(const Dev& d, double* base) {
   Smem s;
@@ -79,7 +94,7 @@ __device__ inline Smem carve(const Dev& d, double* base) {
   s.red = p; p += 32;
   s.scal = p; p += 16;
   // 16-byte aligned: every count above is even (nx, ny and n are even)
-  s.oz.frag = reinterpret_cast<uint2*>(p); p += oz_frag_bytes(n) / sizeof(double);
+  s.oz.frag = reinterpret_cast<uint2*>(p); p += scratch_bytes(d.nx, d.ny, n, d.k) / sizeof(double);
   s.kin_mem = reinterpret_cast<char*>(p); p += 2 * kOzKinBytes / sizeof(double);
   s.oz.tall = p; p += oz_pad(n) * 16;
   s.oz.ws = p; p += 256;
@@ -441,8 +456,10 @@ __device__ __noinline__ void local_chunk_body(const Dev& d, int c, int s0, int s
   load_kinetic(d, sm);
   double* X = d.X + (size_t)c * L * n;
   double* G = d.G + (size_t)c * n * n;
-  double* A = d.Adl + (size_t)c * k * n;
-  double* B = d.Bdl + (size_t)c * k * n;
+  const bool in_smem = delayed_in_smem(d.nx, d.ny, n, k);
+  double* A = in_smem ? reinterpret_cast<double*>(reinterpret_cast<char*>(sm.oz.frag) + (size_t)oz_pad(n) * 192)
+                      : d.Adl + (size_t)c * k * n;
+  double* B = in_smem ? A + k * n : d.Bdl + (size_t)c * k * n;
   const uint32_t* id = d.cid + 4 * (size_t)c;
   const uint32_t key0 = id[0], key1 = id[1], chain = id[2], sweep = id[3];
   long long n_acc = 0;

@@ -88,12 +88,17 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], 
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b.x), "r"(b.y));
 }
 
+// two floats to packed bfloat16, round to nearest even (a in the low half): one instruction
+__device__ __forceinline__ uint32_t cvt_bf16x2(float a, float b) {
+  uint32_t r;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;\n" : "=r"(r) : "f"(b), "f"(a));
+  return r;
+}
+
 // v = hi + lo in bfloat16 (hi, lo packed by pairs: first element in the low half)
 __device__ __forceinline__ void split2(float v0, float v1, uint32_t& hi, uint32_t& lo) {
-  const uint16_t h0 = float_to_bf16(v0), h1 = float_to_bf16(v1);
-  const uint16_t l0 = float_to_bf16(v0 - bf16_to_float(h0)), l1 = float_to_bf16(v1 - bf16_to_float(h1));
-  hi = pack_bf16(h0, h1);
-  lo = pack_bf16(l0, l1);
+  hi = cvt_bf16x2(v0, v1);
+  lo = cvt_bf16x2(v0 - __uint_as_float(hi << 16), v1 - __uint_as_float(hi & 0xffff0000u));
 }
 
 // The eight inputs k of a lane in layer 1's A fragments, q = 4 s + 2 half + p: k = 16 s + 2t + 8 half + p,
@@ -223,8 +228,10 @@ __host__ __device__ inline size_t nn_train_tc_smem_bytes() {
 }
 
 __device__ __forceinline__ void split1(float v, uint16_t& hi, uint16_t& lo) {
-  hi = float_to_bf16(v);
-  lo = float_to_bf16(v - bf16_to_float(hi));
+  uint32_t h, l;
+  split2(v, 0.f, h, l);
+  hi = (uint16_t)h;
+  lo = (uint16_t)l;
 }
 
 __device__ __forceinline__ uint32_t ld32(const uint16_t* p) { return *reinterpret_cast<const uint32_t*>(p); }
