@@ -139,11 +139,12 @@ __device__ __forceinline__ void set_identity(double* A, int ld, int n) {
   }
 }
 
-__device__ __forceinline__ void copy_mat(double* B, const double* A, int ld, int n) {
-  for (int idx = threadIdx.x; idx < n * n; idx += HQ_THREADS) {
-    const int r = idx % n, c = idx / n;
-    B[(size_t)c * ld + r] = A[(size_t)c * ld + r];
-  }
+// B <- A (n x n, contiguous, n^2 a multiple of 16)
+__device__ __forceinline__ void copy_mat(double* B, const double* A, int n) {
+  const double2* a = reinterpret_cast<const double2*>(A);
+  double2* b = reinterpret_cast<double2*>(B);
+#pragma unroll 4
+  for (int idx = threadIdx.x; idx < n * n / 2; idx += HQ_THREADS) b[idx] = a[idx];
 }
 
 // Sum over groups of G lanes (the warp's 32 lanes all take part).

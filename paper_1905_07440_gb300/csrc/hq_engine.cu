@@ -149,7 +149,7 @@ Layout layout(const hq_params& p, int C, int max_series) {
     l.expV = take(sizeof(double) * C * L * n);
     l.cmat = take(sizeof(double) * C * 2 * nch * nn);
     l.cbuf = take(sizeof(int) * C);
-    l.corr = take(sizeof(double) * C * (2 * n * L + L));
+    l.corr = take(sizeof(double) * C * (2 * n * L + ((L + 1) & ~(size_t)1)));
   }
   l.total = off;
   return l;

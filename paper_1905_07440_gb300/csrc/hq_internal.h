@@ -65,7 +65,7 @@ struct Dev {
   double* expV;       // [C][L][N] exp(-dtau V) of the current fields
   double* cmat;       // [C][2][n_chunks][N*N] chunk products, current and proposed
   int* cbuf;          // [C] index of the current buffer
-  double* corr;       // [C][2 N L + L] correction vectors of every chunk, shifted diagonal
+  double* corr;       // [C][2 N L + L (even)] correction vectors of every chunk, shifted diagonal
 };
 
 // A heterogeneous group of engines swept together (device copy of each engine's

@@ -258,8 +258,8 @@ __device__ __noinline__ double udv_top_down(const Dev& d, int c, const Smem& sm,
     double* t = Tc; Tc = Tn; Tn = t;
     if (store && lo > 0) {
       const size_t b = (size_t)c * d.n_bound + (lo / nw - 1);
-      copy_mat(d.stU + b * n * n, U, n, n);
-      copy_mat(d.stT + b * n * n, Tc, n, n);
+      copy_mat(d.stU + b * n * n, U, n);
+      copy_mat(d.stT + b * n * n, Tc, n);
       for (int r = threadIdx.x; r < n; r += HQ_THREADS) d.stD[b * n + r] = sm.dv[r];
       __syncthreads();
     }
@@ -317,7 +317,7 @@ __device__ __noinline__ void udv_bottom_half(const Dev& d, int c, const Smem& sm
     slice_product<LMAX, false>(d, sm, P, first ? nullptr : UR, DR, s1 - s0,
                                SliceDiag{X, nullptr, s0, 1, -1, 0.0});
     udv_step<LMAX>(sm, P, Q, n, UR, DR, first ? nullptr : TR, T2);
-    copy_mat(TR, T2, n, n);
+    copy_mat(TR, T2, n);
     __syncthreads();
   }
 }
@@ -607,7 +607,7 @@ __device__ __noinline__ void local_chunk_body(const Dev& d, int c, int s0, int s
   HQ_TIC(rq);
   double* Q = chain_work(d, c, WK_M1);
   udv_step<LMAX>(sm, P, Q, n, UR, DR, first ? nullptr : TR, T2);
-  copy_mat(TR, T2, n, n);
+  copy_mat(TR, T2, n);
   __syncthreads();
   HQ_TOC(rq, SEC_RESTAB_QR);
   HQ_TIC(rg);
@@ -620,7 +620,7 @@ __device__ __noinline__ void local_chunk_body(const Dev& d, int c, int s0, int s
   }
   err = block_max(err, sm.red);
   bad = block_max(bad, sm.red);
-  copy_mat(G, Gf, n, n);
+  copy_mat(G, Gf, n);
   if (threadIdx.x == 0) {
     double* acc = d.acc + (size_t)c * kAccSlots;
     acc[ACC_WRAP] = fmax(acc[ACC_WRAP], err);
@@ -691,9 +691,10 @@ __device__ inline double* chunk_mat(const Dev& d, int c, int buf, int q) {
   return d.cmat + (((size_t)c * 2 + buf) * d.n_chunks + q) * (size_t)d.n * d.n;
 }
 
-// per chain: V (n x L), R (n x L), shifted diagonal entry per slice (L)
+// per chain: V (n x L), R (n x L), shifted diagonal entry per slice (L, an even stride keeps every chain's
+// vectors 16-byte aligned)
 __device__ inline double* chain_corr(const Dev& d, int c) {
-  return d.corr + (size_t)c * (2 * (size_t)d.n * d.L + d.L);
+  return d.corr + (size_t)c * (2 * (size_t)d.n * d.L + ((d.L + 1) & ~1));
 }
 
 // exp(-dtau V) of every slice and the chunk products M_q of chain c (current buffer).
@@ -713,68 +714,6 @@ __device__ __noinline__ void build_chunks(const Dev& d, const Smem& sm, int c) {
 }
 
 // log|det M(X')| for X' = X + dx e_site (all slices) from the chunk propagators.
-// One step of the correction-vector chains of every chunk at once.  Column s of V (or R)
-// belongs to chunk q = s / n_wrap, position k = s - q n_wrap in a chunk of length m_q.
-//   V step (1 <= step < n_wrap): columns with k >= m_q - step get A'_t = D'_t E, t = hi_q - 1 - step
-//   R step (0 <= step < n_wrap): columns with k <= step get A_t^T = E D_t,      t = lo_q + step
-// D_t = exp(-dtau V_t) from the cache ev, D'_t the same with entry `site` replaced by xs[t].
-template <int LMAX, bool RCHAIN>
-__device__ void corr_step(const Dev& d, const Smem& sm, double* W, int step, int site, const double* ev,
-                          const double* xs) {
-  const int n = d.n, L = d.L, nw = d.n_wrap, nx = d.nx, ny = d.ny;
-  for (int line = threadIdx.x; line < ny * L; line += HQ_THREADS) {
-    const int y = line % ny, col = line / ny;
-    const int q = col / nw, k = col - q * nw, lo = q * nw, m = min(nw, L - lo);
-    const bool on = (step < m) && (RCHAIN ? (k <= step) : (k >= m - step));
-    if (!on) continue;
-    const int t = RCHAIN ? lo + step : lo + m - 1 - step;
-    double* base = W + (size_t)col * n + nx * y;
-    double v[LMAX];
-#pragma unroll
-    for (int b = 0; b < LMAX; ++b) {
-      v[b] = (b < nx) ? base[b] : 0.0;
-      if (RCHAIN && b < nx) v[b] *= ev[(size_t)t * n + nx * y + b];
-    }
-#pragma unroll
-    for (int a = 0; a < LMAX; ++a) {
-      if (a < nx) {
-        double acc = 0.0;
-#pragma unroll
-        for (int b = 0; b < LMAX; ++b)
-          if (b < nx) acc = fma(sm.ex[a * nx + b], v[b], acc);
-        base[a] = acc;
-      }
-    }
-  }
-  __syncthreads();
-  for (int line = threadIdx.x; line < nx * L; line += HQ_THREADS) {
-    const int x = line % nx, col = line / nx;
-    const int q = col / nw, k = col - q * nw, lo = q * nw, m = min(nw, L - lo);
-    const bool on = (step < m) && (RCHAIN ? (k <= step) : (k >= m - step));
-    if (!on) continue;
-    const int t = RCHAIN ? lo + step : lo + m - 1 - step;
-    double* base = W + (size_t)col * n + x;
-    double v[LMAX];
-#pragma unroll
-    for (int b = 0; b < LMAX; ++b) v[b] = (b < ny) ? base[b * nx] : 0.0;
-#pragma unroll
-    for (int a = 0; a < LMAX; ++a) {
-      if (a < ny) {
-        double acc = 0.0;
-#pragma unroll
-        for (int b = 0; b < LMAX; ++b)
-          if (b < ny) acc = fma(sm.ey[a * ny + b], v[b], acc);
-        if (!RCHAIN) {
-          const int r = x + nx * a;
-          acc *= (r == site) ? xs[t] : ev[(size_t)t * n + r];
-        }
-        base[a * nx] = acc;
-      }
-    }
-  }
-  __syncthreads();
-}
-
 template <int LMAX>
 __device__ __noinline__ double udv_top_down_cm(const Dev& d, int c, const Smem& sm, int site, double dx) {
   const int n = d.n, L = d.L, nw = d.n_wrap;
@@ -792,36 +731,16 @@ __device__ __noinline__ double udv_top_down_cm(const Dev& d, int c, const Smem& 
   const double delta = expm1(-d.dtau * d.g * dx);
   HQ_TIC(cv);
   for (int s = threadIdx.x; s < L; s += HQ_THREADS) xs[s] = exp(-d.dtau * (d.g * (X[(size_t)s * n + site] + dx) - d.mu));
-  for (int idx = threadIdx.x; idx < n * L; idx += HQ_THREADS) {
-    const double e = (idx % n == site) ? 1.0 : 0.0;
-    Vc[idx] = e;
-    Rc[idx] = e;
-  }
   __syncthreads();
-  // column s of V: A'_lo .. A'_{s-1} e_site; of R: A_{hi-1}^T .. A_s^T e_site (chunk [lo, hi))
-  for (int step = 1; step < nw; ++step) corr_step<LMAX, false>(d, sm, Vc, step, site, ev, xs);
-  for (int step = 0; step < nw; ++step) corr_step<LMAX, true>(d, sm, Rc, step, site, ev, xs);
-  // M'_q = M_q + delta sum_{s in q} V_s R_s^T for every chunk (four outputs per thread)
-  const int nn4 = (n * n) >> 2;
-  for (int idx = threadIdx.x; idx < d.n_chunks * nn4; idx += HQ_THREADS) {
-    const int q = idx / nn4, e0 = (idx - q * nn4) * 4;
+  oz_corr<LMAX>(d.nx, d.ny, n, L, nw, d.n_chunks, sm.kf, site, ev, xs, Vc, Rc);
+  // M'_q = M_q + delta sum_{s in q} V_s R_s^T for every chunk
+  for (int q = 0; q < d.n_chunks; ++q) {
     const int lo = q * nw, m = min(nw, L - lo);
     const double* M = chunk_mat(d, c, cur, q);
     double* Mn = chunk_mat(d, c, 1 - cur, q);
-    const int col = e0 / n, r0 = e0 - col * n;  // four consecutive rows of one column (n % 4 == 0)
-    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-    for (int k = 0; k < m; ++k) {
-      const double* vk = Vc + (size_t)(lo + k) * n + r0;
-      const double rk = Rc[(size_t)(lo + k) * n + col];
-      a0 = fma(vk[0], rk, a0);
-      a1 = fma(vk[1], rk, a1);
-      a2 = fma(vk[2], rk, a2);
-      a3 = fma(vk[3], rk, a3);
-    }
-    Mn[e0] = fma(delta, a0, M[e0]);
-    Mn[e0 + 1] = fma(delta, a1, M[e0 + 1]);
-    Mn[e0 + 2] = fma(delta, a2, M[e0 + 2]);
-    Mn[e0 + 3] = fma(delta, a3, M[e0 + 3]);
+    for (int k0 = 0; k0 < m; k0 += 16)
+      oz_rank<LMAX>(Rank16{Vc + (size_t)(lo + k0) * n, 1, n, Rc + (size_t)(lo + k0) * n, n, 1, k0 == 0 ? M : Mn, Mn, n, delta, 1.0},
+                    0, n, 0, n, min(16, m - k0), sm.oz.frag, sm.oz.er);
   }
   __syncthreads();
   HQ_TOC(cv, SEC_DL);
@@ -830,7 +749,7 @@ __device__ __noinline__ double udv_top_down_cm(const Dev& d, int c, const Smem& 
     double* Mn = chunk_mat(d, c, 1 - cur, q);
     HQ_TIC(gm);
     if (first) {
-      copy_mat(P, Mn, n, n);
+      copy_mat(P, Mn, n);
     } else {
       oz_mm<LMAX, false, false>(n, Mn, U, nullptr, sm.dv, P, sm.oz);
     }

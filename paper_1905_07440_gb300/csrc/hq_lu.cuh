@@ -206,7 +206,7 @@ __device__ inline void invert_triangle(const double* A, int ld, int p0, int kb, 
   __syncwarp();
 }
 
-// C(r, c) <- base C(r, c) + sign sum_k A(r, k) B(k, c) for r0 <= r < r1, c0 <= c < c1, k < kb <= 16, with A(r, k) =
+// C(r, c) <- base Cin(r, c) + sign sum_k A(r, k) B(k, c) for r0 <= r < r1, c0 <= c < c1, k < kb <= 16, with A(r, k) =
 // A[r ar + k ak], B(k, c) = B[k bk + c bc] and C column-major (ldc).  With base = 0 B may be rows of C's
 // own columns (each warp reads a column's terms before it writes).  Ends with a barrier.
 struct Rank16 {
@@ -214,6 +214,7 @@ struct Rank16 {
   int ar, ak;
   const double* B;
   int bk, bc;
+  const double* Cin;
   double* C;
   int ldc;
   double sign, base;
@@ -221,27 +222,27 @@ struct Rank16 {
 
 template <int LM>
 __device__ __noinline__ void oz_rank(const Rank16 q, int r0, int r1, int c0, int c1, int kb, uint2* frag, int* er) {
-  oz_rank16(q.base == 0.0, r0, r1, c0, c1, kb, frag, er, [&](int r, int k) { return q.A[(size_t)r * q.ar + (size_t)k * q.ak]; },
+  oz_rank16<LM <= 8 ? 1 : 2>(q.base == 0.0, r0, r1, c0, c1, kb, frag, er, [&](int r, int k) { return q.A[(size_t)r * q.ar + (size_t)k * q.ak]; },
             [&](int k, int c) { return q.B[(size_t)k * q.bk + (size_t)c * q.bc]; },
             [&](int r, int c, double s0, double s1) {
-              double2* p = reinterpret_cast<double2*>(q.C + (size_t)c * q.ldc + r);
+              const size_t at = (size_t)c * q.ldc + r;
               double2 v = make_double2(0.0, 0.0);
-              if (q.base != 0.0) v = *p;
-              *p = make_double2(fma(q.sign, s0, v.x), fma(q.sign, s1, v.y));
+              if (q.base != 0.0) v = *reinterpret_cast<const double2*>(q.Cin + at);
+              *reinterpret_cast<double2*>(q.C + at) = make_double2(fma(q.sign, s0, v.x), fma(q.sign, s1, v.y));
             });
 }
 
 // Y(p0 : p0 + kb, c0 : c1) <- M Y(p0 : p0 + kb, c0 : c1) for a 16 x 16 row-major M.
 template <int LM>
 __device__ inline void oz_left16(const double* M, double* Y, int ld, int p0, int kb, int c0, int c1, uint2* frag, int* er) {
-  oz_rank<LM>(Rank16{M, 16, 1, Y + p0, 1, ld, Y + p0, ld, 1.0, 0.0}, 0, kb, c0, c1, kb, frag, er);
+  oz_rank<LM>(Rank16{M, 16, 1, Y + p0, 1, ld, nullptr, Y + p0, ld, 1.0, 0.0}, 0, kb, c0, c1, kb, frag, er);
 }
 
 // C(r0:r1, c0:c1) -= A(r0:r1, k0:k0+kb) B(k0:k0+kb, c0:c1), kb <= 16.
 template <int LM>
 __device__ inline void oz_rank_update(double* C, const double* A, const double* B, int ld, int r0, int r1, int c0, int c1,
                                       int k0, int kb, uint2* frag, int* er) {
-  oz_rank<LM>(Rank16{A + (size_t)k0 * ld, 1, ld, B + k0, 1, ld, C, ld, -1.0, 1.0}, r0, r1, c0, c1, kb, frag, er);
+  oz_rank<LM>(Rank16{A + (size_t)k0 * ld, 1, ld, B + k0, 1, ld, C, C, ld, -1.0, 1.0}, r0, r1, c0, c1, kb, frag, er);
 }
 
 // In place LU of A; tri: oz_pad(n) / 16 blocks of 16 x 16, left holding the inverses of L's diagonal

@@ -317,22 +317,32 @@ __device__ __forceinline__ void oz_left_from_acc(const double (&w)[2][4], uint32
 
 // For the warp's 16 columns ca = c0 + g, cb = c0 + g + 8 and rows 0 .. nr - 1:
 // io(r, c, v0, v1) gets the products of rows r, r + 1 (from the staged coefficients) with the
-// column's left fragment.
-template <class IO>
+// column's left fragment.  NT tiles of 8 rows at a time: with two, one tile's conversions fill the gaps of the
+// other's MMA chains.
+template <int NT, class IO>
 __device__ __forceinline__ void oz_apply_rows(const uint2* frag, const int* er, int nr, const uint32_t (&a)[4][kOzDigits],
                                               const int (&E)[2], int ca, int cb, int cend, IO io) {
   const int lane = threadIdx.x & 31, t = lane & 3;
-  for (int tile = 0; 8 * tile < nr; ++tile) {
-    const uint2* fr = frag + (size_t)tile * kOzDigits * 32 + lane;
-    long long T[4] = {0, 0, 0, 0};
-    oz_mma(a, [&](int d) { return fr[d * 32]; }, T);
-    const int r = 8 * tile + 2 * t;
-    if (r < nr) {
-      const int E0 = er[r], E1 = er[r + 1];
-      if (ca < cend)
-        io(r, ca, oz_scale((double)T[0], oz_expo<kOzP>(E0, E[0])), oz_scale((double)T[1], oz_expo<kOzP>(E1, E[0])));
-      if (cb < cend)
-        io(r, cb, oz_scale((double)T[2], oz_expo<kOzP>(E0, E[1])), oz_scale((double)T[3], oz_expo<kOzP>(E1, E[1])));
+#pragma unroll 1
+  for (int tile = 0; 8 * tile < nr; tile += NT) {
+    long long T[NT][4];
+#pragma unroll
+    for (int j = 0; j < NT; ++j) {
+      const uint2* fr = frag + (size_t)(tile + j) * kOzDigits * 32 + lane;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) T[j][e] = 0;
+      oz_mma(a, [&](int d) { return fr[d * 32]; }, T[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < NT; ++j) {
+      const int r = 8 * (tile + j) + 2 * t;
+      if (r < nr) {
+        const int E0 = er[r], E1 = er[r + 1];
+        if (ca < cend)
+          io(r, ca, oz_scale((double)T[j][0], oz_expo<kOzP>(E0, E[0])), oz_scale((double)T[j][1], oz_expo<kOzP>(E1, E[0])));
+        if (cb < cend)
+          io(r, cb, oz_scale((double)T[j][2], oz_expo<kOzP>(E0, E[1])), oz_scale((double)T[j][3], oz_expo<kOzP>(E1, E[1])));
+      }
     }
   }
 }
@@ -342,7 +352,7 @@ __device__ __forceinline__ void oz_apply_rows(const uint2* frag, const int* er, 
 // out(r, c, s0, s1): s = sum_k A(r, k) B(k, c) for r0 <= r < r1, c0 <= c < c1 and kb <= 16 terms; fa, fb
 // values.  Reads of fa and fb must not overlap what `out` writes, except that with one_part (a warp
 // owns its columns whole) `out` may overwrite the column entries that fb reads.  Ends with a barrier.
-template <class FA, class FB, class OUT>
+template <int NT, class FA, class FB, class OUT>
 __device__ __forceinline__ void oz_rank16(bool one_part, int r0, int r1, int c0, int c1, int kb, uint2* frag, int* er,
                                           FA fa, FB fb, OUT out) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
@@ -352,7 +362,7 @@ __device__ __forceinline__ void oz_rank16(bool one_part, int r0, int r1, int c0,
   // few columns: the row range is shared out too, so that every warp has work
   const int ncg = (c1 - c0 + 15) >> 4;
   const int parts = one_part || ncg >= HQ_WARPS ? 1 : HQ_WARPS / ncg;
-  const int rp = (((nr + parts - 1) / parts) + 7) & ~7;
+  const int rp = (((nr + parts - 1) / parts) + 8 * NT - 1) / (8 * NT) * (8 * NT);
   for (int unit = warp; unit < ncg * parts; unit += HQ_WARPS) {
     const int ca = c0 + (unit % ncg) * 16 + g, cb = ca + 8, rb = (unit / ncg) * rp;
     if (rb >= nr) continue;
@@ -367,7 +377,7 @@ __device__ __forceinline__ void oz_rank16(bool one_part, int r0, int r1, int c0,
     uint32_t a[4][kOzDigits];
     int E[2];
     oz_left_from_acc(w, a, E);
-    oz_apply_rows(frag + (size_t)(rb >> 3) * kOzDigits * 32, er + rb, min(rp, nr - rb), a, E, ca, cb, c1,
+    oz_apply_rows<NT>(frag + (size_t)(rb >> 3) * kOzDigits * 32, er + rb, min(rp, nr - rb), a, E, ca, cb, c1,
                   [&](int r, int c, double s0, double s1) { out(r0 + rb + r, c, s0, s1); });
   }
   __syncthreads();

@@ -133,7 +133,8 @@ __device__ __noinline__ void oz_wy_apply(bool trans, const double* V, int ld, in
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int ncg = (cend - c0 + 15) >> 4;
   const int parts = ncg >= HQ_WARPS ? 1 : HQ_WARPS / ncg;
-  const int rp = ((nr + parts - 1) / parts + 7) & ~7;
+  constexpr int kTiles = LM <= 8 ? 1 : 2;
+  const int rp = ((nr + parts - 1) / parts + 8 * kTiles - 1) / (8 * kTiles) * (8 * kTiles);
   for (int unit = warp; unit < ((ncg * parts + HQ_WARPS - 1) / HQ_WARPS) * HQ_WARPS; unit += HQ_WARPS) {
     const bool work = unit < ncg * parts;
     const int ca = c0 + (unit % ncg) * 16 + g, cb = ca + 8, rb = work ? (unit / ncg) * rp : nr;
@@ -193,7 +194,7 @@ __device__ __noinline__ void oz_wy_apply(bool trans, const double* V, int ld, in
     }
     if (parts > 1) __syncthreads();  // W of every warp is formed before rows change
     if (work && rb < nr)
-      oz_apply_rows(vn + (size_t)(rb >> 3) * kOzDigits * 32, z.er + rb, min(rp, nr - rb), a, E, ca, cb, cend,
+      oz_apply_rows<kTiles>(vn + (size_t)(rb >> 3) * kOzDigits * 32, z.er + rb, min(rp, nr - rb), a, E, ca, cb, cend,
                     [&](int r, int c, double s0, double s1) {
                       double* p = A + (size_t)c * ld + j0 + rb + r;
                       const RowPair x = load_pair(p);
@@ -336,9 +337,9 @@ __device__ __noinline__ void oz_flush(double* G, const double* A, const double* 
   for (int m0 = 0; m0 < kk; m0 += 16) {
     const int kb = min(16, kk - m0);
     if (LM <= 8)
-      oz_rank<LM>(Rank16{A + (size_t)m0 * n, 1, n, B + (size_t)m0 * n, n, 1, G, n, 1.0, 1.0}, 0, n, 0, n, kb, z.frag, z.er);
+      oz_rank<LM>(Rank16{A + (size_t)m0 * n, 1, n, B + (size_t)m0 * n, n, 1, G, G, n, 1.0, 1.0}, 0, n, 0, n, kb, z.frag, z.er);
     else
-      oz_rank16(false, 0, n, 0, n, kb, z.frag, z.er, [&](int r, int k) { return A[(m0 + k) * n + r]; },
+      oz_rank16<2>(false, 0, n, 0, n, kb, z.frag, z.er, [&](int r, int k) { return A[(m0 + k) * n + r]; },
                 [&](int k, int c) { return B[(m0 + k) * n + c]; },
                 [&](int r, int c, double s0, double s1) {
                   double* p = G + c * n + r;
@@ -428,6 +429,64 @@ __device__ __forceinline__ void tiny_slices(int nx, int ny, int n, const double*
     if (kAfter) v *= d;
   }
   if (on) P[(size_t)c * n + i] = v;
+  __syncthreads();
+}
+
+// Correction vectors of a block move at `site` (chunk q: slices lo .. lo + m - 1, lo = q nw, D_t = exp(-dtau V_t)
+// from ev [L][n], D'_t the same with the shifted entry xs[t] at the site):
+//   V column lo + s: D'_lo E ... D'_(lo+s-1) E e_site             (s = 0 .. m - 1 slices)
+//   R column lo + m - s: E D_(lo+m-1) ... E D_(lo+m-s) e_site     (s = 1 .. m)
+// A vector is a matrix column to the kinetic tiles; columns of different chunks with the same s share a
+// tile, and a warp runs a tile's s slices in registers.  Longest first over the warps.  (As FP64 line
+// passes over all vectors, one slice per barrier pair, this took 1.1 million cycles per move at 8x8, L = 80.)
+template <int LM>
+__device__ __noinline__ void oz_corr(int nx, int ny, int n, int L, int nw, int nq, const OzKin& K, int site,
+                                     const double* ev, const double* xs, double* V, double* R) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const bool two_x = nx <= 8, two_y = ny <= 8;
+  const int per = (two_x ? 2 : 1) * (two_y ? 2 : 1), tg = (nq + per - 1) / per;
+  for (int idx = threadIdx.x; idx < nq * n; idx += HQ_THREADS)
+    V[(size_t)(idx / n) * nw * n + idx % n] = idx % n == site ? 1.0 : 0.0;
+#pragma unroll 1
+  for (int task = warp; task < (2 * nw - 1) * tg; task += HQ_WARPS) {
+    const int rest = task - tg;
+    const bool right = task < tg || rest % (2 * tg) < tg;
+    const int s = task < tg ? nw : nw - 1 - rest / (2 * tg), gq = task < tg ? task : rest % tg;
+    double z[2][4];
+    auto visit = [&](auto f) {
+#pragma unroll
+      for (int w = 0; w < 2; ++w)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int x = two_x ? 2 * t : 8 * w + 2 * t, y = two_y ? g : 8 * h + g;
+          const int q = gq * per + (two_y ? h : 0) * (two_x ? 2 : 1) + (two_x ? w : 0);
+          const int lo = q * nw, m = min(nw, L - lo);
+          f(x < nx && y < ny && q < nq && (right ? s <= m : s < m), right ? lo + m - s : lo + s, x + nx * y, z[w][2 * h],
+            z[w][2 * h + 1]);
+        }
+    };
+    visit([&](bool on, int, int i, double& v0, double& v1) {
+      v0 = on && i == site ? 1.0 : 0.0;
+      v1 = on && i + 1 == site ? 1.0 : 0.0;
+    });
+#pragma unroll 1
+    for (int u = 0; u < s; ++u) {
+      auto scale = [&](bool on, int col, int i, double& v0, double& v1) {
+        if (!on) return;
+        const int at = right ? col + u : col - 1 - u;
+        const RowPair e = load_pair(ev + (size_t)at * n + i);
+        v0 *= !right && i == site ? xs[at] : e.v0;
+        v1 *= !right && i + 1 == site ? xs[at] : e.v1;
+      };
+      if (right) visit(scale);
+      oz_kin_tile(K, z, two_x, two_y);
+      if (!right) visit(scale);
+    }
+    double* W = right ? R : V;
+    visit([&](bool on, int col, int i, double& v0, double& v1) {
+      if (on) store_pair(W + (size_t)col * n + i, v0, v1);
+    });
+  }
   __syncthreads();
 }
 
