@@ -3,18 +3,19 @@
 // F_cnn(X) = sum over the (x, y, tau) torus of a three-layer periodic 3x3x3 network (see
 // hq_cnn.cuh).  Training fits F_cnn(X_a) to log|det M(X_a)| minus the sample mean by mean
 // squared error, as for the patch network.  Because F_cnn is a plain sum of the last layer,
-// dF/d(layer-2 output at any point) is the same vector sum_t W3[t][.], which makes the first
-// backward step a masked constant.  Every gradient entry is owned by one thread and summed
-// over the CTA's samples in a fixed order; the per-CTA partials are summed in a fixed order by
-// the Adam kernel, so training is deterministic.
+// dF/d(layer-2 output at any point) is the same vector sum_t W3[t][.], so the error behind layer 2
+// is a mask times a constant: both contractions with it (the gradient of W2 over points, the error of
+// layer 1 over channels) are MMAs with an exact 0/1 operand.  Every sample is shared out over
+// several CTAs; sums run in a fixed order and the per-CTA partials are added in a fixed order by the
+// Adam kernel, so training is deterministic.
+#include <algorithm>
+
 #include "hq_cnn.cuh"
 #include "../../include/holstein_dqmc.h"
 
 namespace hq {
 
 static_assert(CN_NP == HQ_CNN_PARAMS, "parameter count");
-
-constexpr int CN_TILE = 32;  // points per staged tile in the weight-gradient passes
 
 // ------------------------------------------------------------------------ evaluation
 // F_cnn of every chain (grid = chains); refreshes the chain's caches and network inputs.
@@ -32,199 +33,348 @@ __global__ void __launch_bounds__(HQ_THREADS, 2) cnn_eval_kernel(Dev d, CnnState
 }
 
 // ------------------------------------------------------------------------ training
-struct CnTrainSmem {
-  float* w;      // [CN_WPAD]
-  float* nbh;    // [CN_TILE][27][16] staged neighbourhoods (layer-1 values or inputs)
-  float* dt;     // [CN_TILE][16] staged gradients at the tile's points
-  float* hs;     // [HQ_THREADS][16] per-thread channel sums
-  float* w3s;    // [16] sum over taps of W3
-  double* red;   // [HQ_WARPS]
-  double* scal;  // [2]
+// Scratch of one sample of a round (samples trained at a time), in cn.tr: layer-1 activations (split), network
+// inputs, layer-2 masks (a bit per channel), per-part channel sums of layer 2 and shares of F.
+struct CnSample {
+  uint4* h1;       // [L N][8]
+  float* z;        // [L N]
+  uint16_t* mask;  // [L N]
+  float* hs;       // [kCnnParts][16]
+  double* f;       // [kCnnParts]
 };
+__host__ __device__ inline size_t cn_sample_bytes(size_t NL) {
+  return NL * 128 + ((NL * 4 + 15) & ~(size_t)15) + ((NL * 2 + 15) & ~(size_t)15) + kCnnParts * (16 * 4 + 8);
+}
+size_t cnn_sample_bytes(size_t NL) { return (cn_sample_bytes(NL) + 255) & ~(size_t)255; }
 
-__host__ __device__ inline size_t cn_train_smem_bytes() {
-  return sizeof(float) * (CN_WPAD + CN_TILE * CN_T * CN_C + CN_TILE * CN_C + HQ_THREADS * CN_C + CN_C) +
-         sizeof(double) * (HQ_WARPS + 2);
+__device__ __forceinline__ CnSample cn_sample(const CnnState& cn, size_t NL, int a) {
+  char* p = cn.tr + (size_t)a * ((cn_sample_bytes(NL) + 255) & ~(size_t)255);
+  CnSample s;
+  s.h1 = (uint4*)p; p += NL * 128;
+  s.z = (float*)p; p += (NL * 4 + 15) & ~(size_t)15;
+  s.mask = (uint16_t*)p; p += (NL * 2 + 15) & ~(size_t)15;
+  s.f = (double*)p; p += kCnnParts * 8;
+  s.hs = (float*)p;
+  return s;
 }
 
-// One minibatch: each CTA takes samples a = blockIdx.x, + gridDim.x, ...; forward with the
-// activations kept in the CTA's slice of cn.tr, then the backward passes.  Writes F_a to Fb
-// and the CTA's summed gradient to partials[blockIdx.x].
-__global__ void __launch_bounds__(HQ_THREADS) cnn_train_kernel(Dev d, CnnState cn, const double* Xs,
-                                                               const double* ys, const int* idx, int B, double x0,
-                                                               double* Fb, float* partials) {
+// Network inputs of the round's samples.
+__global__ void cnn_inputs_kernel(Dev d, CnnState cn, const double* Xs, const int* idx, double x0) {
+  const int NL = d.n * d.L, a = blockIdx.y;
+  const CnSample s = cn_sample(cn, NL, a);
+  const double* X = Xs + (size_t)idx[a] * NL;
+  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < NL; k += gridDim.x * blockDim.x) s.z[k] = (float)(X[k] - x0);
+}
+
+__global__ void __launch_bounds__(HQ_THREADS) cnn_layer1_kernel(Dev d, CnnState cn) {
   extern __shared__ __align__(16) char craw[];
-  CnTrainSmem s;
-  float* f = (float*)craw;
-  s.w = f; f += CN_WPAD;
-  s.nbh = f; f += CN_TILE * CN_T * CN_C;
-  s.dt = f; f += CN_TILE * CN_C;
-  s.hs = f; f += HQ_THREADS * CN_C;
-  s.w3s = f; f += CN_C;
-  s.red = (double*)f;
-  s.scal = s.red + HQ_WARPS;
-  cn_load_weights(cn.wbf, s.w);
-  const int n = d.n, NL = d.n * d.L, tid = threadIdx.x;
-  if (tid < CN_C) {
+  const CnSm w = cn_setup<false>(cn.wbf, craw);
+  const int n = d.n, NL = d.n * d.L;
+  const CnSample s = cn_sample(cn, NL, blockIdx.y);
+  for (int e = blockIdx.x * HQ_THREADS + threadIdx.x; e < 2 * NL; e += gridDim.x * HQ_THREADS) {
+    const int p = e >> 1, l = p / n, i = p % n;
+    cn_point1(d, w, l, i % d.nx, i / d.nx, e & 1, [&](int ll, int j) { return s.z[ll * n + j]; }, s.h1 + (size_t)p * 8);
+  }
+}
+
+// the points of part `part` of `parts`: whole tiles of 16
+__device__ __forceinline__ void cn_part(int NL, int part, int parts, int& p0, int& p1) {
+  const int tiles = (NL + 15) >> 4;
+  p0 = (int)((long long)tiles * part / parts) * 16;
+  p1 = min((int)((long long)tiles * (part + 1) / parts) * 16, NL);
+}
+
+// Layer 2 of the round's samples: masks, channel sums and shares of F (grid: parts x samples).
+__global__ void __launch_bounds__(HQ_THREADS, 2) cnn_layer2_kernel(Dev d, CnnState cn) {
+  extern __shared__ __align__(16) char craw[];
+  __shared__ double red[HQ_WARPS];
+  __shared__ float ch[HQ_WARPS][CN_C];
+  const CnSm w = cn_setup(cn.wbf, craw);
+  const int n = d.n, NL = d.n * d.L, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const CnSample s = cn_sample(cn, NL, blockIdx.y);
+  int p0, p1;
+  cn_part(NL, blockIdx.x, gridDim.x, p0, p1);
+  const CnBox none{0, 0, 0, 0};
+  float hs[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
+  double part = 0.0;
+  for (int base = p0 + warp * 16; base < p1; base += HQ_WARPS * 16) {
+    int l[2], x[2], y[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int p = min(base + g + 8 * h, NL - 1), i = p % n;
+      l[h] = p / n;
+      x[h] = i % d.nx;
+      y[h] = i / d.nx;
+    }
+    float acc[2][4];
+    cn_tile_acc(d, w, l, x, y, s.h1, s.h1, none, acc);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int p = base + g + 8 * h;
+      const bool on = p < p1;
+      uint32_t bits = 0;
+      float sum = 0.f;
+#pragma unroll
+      for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int c = 8 * nt + 2 * t + e;
+          const float a = acc[nt][2 * h + e] + w.b2[c], h2 = on ? fmaxf(a, 0.f) : 0.f;
+          if (a > 0.f) bits |= 1u << c;
+          hs[nt][e] += h2;
+          sum = fmaf(h2, w.wh[c], fmaf(h2, w.wl[c], sum));
+        }
+      bits |= __shfl_xor_sync(HQ_FULL, bits, 1);
+      bits |= __shfl_xor_sync(HQ_FULL, bits, 2);
+      sum += __shfl_xor_sync(HQ_FULL, sum, 1);
+      sum += __shfl_xor_sync(HQ_FULL, sum, 2);
+      if (on && t == 0) {
+        s.mask[p] = (uint16_t)bits;
+        part += (double)sum;
+      }
+    }
+  }
+#pragma unroll
+  for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+#pragma unroll
+      for (int o = 4; o < 32; o <<= 1) hs[nt][e] += __shfl_xor_sync(HQ_FULL, hs[nt][e], o);
+      if (g == 0) ch[warp][8 * nt + 2 * t + e] = hs[nt][e];
+    }
+  part = block_sum(part, red);  // (its barriers cover ch)
+  if (threadIdx.x < CN_C) {
     float a = 0.f;
-    for (int t = 0; t < CN_T; ++t) a += s.w[CN_W3 + t * CN_C + tid];
-    s.w3s[tid] = a;
+    for (int k = 0; k < HQ_WARPS; ++k) a += ch[k][threadIdx.x];
+    s.hs[blockIdx.x * CN_C + threadIdx.x] = a;
   }
-  float* A1 = cn.tr + (size_t)blockIdx.x * 3 * NL * CN_C;  // layer-1 activations
-  float* A2 = A1 + (size_t)NL * CN_C;                      // layer-2 activations, then dL/da2
-  float* D1 = A2 + (size_t)NL * CN_C;                      // dL/da1
-  // owned entries: W2 pairs (tap, in) q0 = tid, q1 = tid + 256 (< 432), 16 outputs each;
-  // W1 pairs (tap, out) the same indices; b2 / b1 channel (tid - 176) for 176 <= tid < 192;
-  // W3 channel tid (< 16, same for every tap); b3 by thread 16.
-  float g2a[CN_C], g2b[CN_C], g1a = 0.f, g1b = 0.f, gb = 0.f, gb1 = 0.f, g3 = 0.f;
+  if (threadIdx.x == 0) s.f[blockIdx.x] = part + (double)(p1 - p0) * (double)w.b3;
+}
+
+// Backward pass of the round's samples (grid: parts x samples).  With m(p)[co] the masks, s = dL/dF and
+// w = sum_t W3[t]:  gW2[t][ci][co] = s w[co] sum_p h1(p + t)[ci] m(p)[co];
+// d1(q)[ci] = [h1(q)[ci] > 0] s sum_t sum_co (W2[t][ci][co] w[co]) m(q - t)[co];  gW1[t][co] = sum_p d1(p)[co] z(p + t).
+// Blocks of 128 points share a table of their 27 neighbours (without it, integer divisions and the latency of
+// the loads behind them were most of 169 us for 32 samples of 8x8, L = 40).  A warp owns taps warp, warp + 8, ... of
+// gW2: per 16 points the masks are the left operand of all of them and the layer-1 fragments, transposed in registers,
+// the right ones.  d1 goes through shared memory to gW1, whose (tap, channel) entries are owned by threads.
+// Partials are written in the first round and added to later.
+constexpr int kCnBlk = 128, kCnLd = kCnBlk + 4;
+constexpr int CN_WT = CN_T * 3 * 2 * 32;  // fragments of W2 w, three terms
+constexpr int kCnOwn = (CN_T + HQ_WARPS - 1) / HQ_WARPS;
+
+__host__ __device__ inline size_t cn_back_smem_bytes() {
+  return cn_smem_bytes() + sizeof(uint2) * CN_WT + sizeof(float) * kCnLd * (CN_T + CN_C) + sizeof(int) * kCnBlk * CN_T;
+}
+
+__global__ void __launch_bounds__(HQ_THREADS) cnn_backward_kernel(Dev d, CnnState cn, const double* ys, const int* idx,
+                                                                  int B, int parts2, int first, double* Fb,
+                                                                  float* partials) {
+  extern __shared__ __align__(16) char craw[];
+  __shared__ float sw[2][CN_C];
+  __shared__ int cnt[CN_C];
+  const CnSm w = cn_setup<false>(cn.wbf, craw);
+  uint2* wt = reinterpret_cast<uint2*>(craw + cn_smem_bytes());
+  float* zn = reinterpret_cast<float*>(wt + CN_WT);  // [27][kCnLd] inputs at p + t
+  float* ds = zn + kCnLd * CN_T;                     // [16][kCnLd] d1 / s
+  int* nb = reinterpret_cast<int*>(ds + kCnLd * CN_C);  // [27][kCnBlk] places of p + t
+  const int n = d.n, L = d.L, NL = n * L, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  const int a = blockIdx.y, parts = gridDim.x;
+  const CnSample s = cn_sample(cn, NL, a);
+  int p0, p1;
+  cn_part(NL, blockIdx.x, parts, p0, p1);
+  double F = 0.0;
+  for (int k = 0; k < parts2; ++k) F += s.f[k];
+  if (tid == 0 && blockIdx.x == 0) Fb[a] = F;
+  // s and s w[co] as two floats, so that a gradient entry is rounded once
+  const double sd = 2.0 * (F - ys[idx[a]]) / B;
+  const float sg = (float)sd, sl = (float)(sd - (double)sg);
+  auto scaled = [&](float v) { return fmaf(sg, v, sl * v); };
+  if (tid < CN_C) {
+    const double v = sd * ((double)w.wh[tid] + (double)w.wl[tid]);
+    sw[0][tid] = (float)v;
+    sw[1][tid] = (float)(v - (double)(float)v);
+    cnt[tid] = 0;
+  }
+  // right fragments of (W2[t] w)^T: k = co, column ci
+  for (int e = tid; e < CN_T * 2 * 32; e += HQ_THREADS) {
+    const int ln = e & 31, nt = (e >> 5) & 1, tap = e >> 6, gg = ln >> 2, tt = ln & 3, ci = 8 * nt + gg;
+    auto v = [&](int co) { return bf16_to_float(cn.wbf[CN_W2 + tap * CN_C * CN_C + ci * CN_C + co]) * (w.wh[co] + w.wl[co]); };
+    const uint4 x = cn_split(v(2 * tt), v(2 * tt + 1)), y = cn_split(v(2 * tt + 8), v(2 * tt + 9));
+    wt[((tap * 3 + 0) * 2 + nt) * 32 + ln] = make_uint2(x.x, y.x);
+    wt[((tap * 3 + 1) * 2 + nt) * 32 + ln] = make_uint2(x.y, y.y);
+    wt[((tap * 3 + 2) * 2 + nt) * 32 + ln] = make_uint2(x.z, y.z);
+  }
+  // channels c, c + 1 of a mask, and channel c of two masks, as bfloat16 pairs of 0 and 1
+  auto cols = [](uint32_t m, int c) { return ((m >> c) & 1u) * 0x3f80u | ((m >> (c + 1)) & 1u) * 0x3f800000u; };
+  auto pair = [](uint32_t m0, uint32_t m1, int c) { return ((m0 >> c) & 1u) * 0x3f80u | ((m1 >> c) & 1u) * 0x3f800000u; };
+  float acc2[kCnOwn][2][4], low2[kCnOwn][2][4], rest2[kCnOwn][2][4];
 #pragma unroll
-  for (int c = 0; c < CN_C; ++c) g2a[c] = g2b[c] = 0.f;
-  const int q0 = tid, q1 = tid + HQ_THREADS;
-  const bool has1 = q1 < CN_T * CN_C;
-  for (int a = blockIdx.x; a < B; a += gridDim.x) {
-    const double* X = Xs + (size_t)idx[a] * NL;
-    // forward
-    const double F = cn_forward_all(d, s.w, X, x0, A1, A2, s.red);
-    if (tid == 0) Fb[a] = F;
-    const float sg = (float)(2.0 * (F - ys[idx[a]]) / B);
-    // layer 3: dF/dW3[t][ci] = sum_q h2(q)[ci] for every t; dF/db3 = L N
-    float hs[CN_C];
+  for (int o = 0; o < kCnOwn; ++o)
 #pragma unroll
-    for (int c = 0; c < CN_C; ++c) hs[c] = 0.f;
-    for (int p = tid; p < NL; p += HQ_THREADS) {
-      float h[CN_C];
-      cn_load16(A2 + (size_t)p * CN_C, h);
+    for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
-      for (int c = 0; c < CN_C; ++c) hs[c] += h[c];
-    }
-#pragma unroll
-    for (int c = 0; c < CN_C; ++c) s.hs[tid * CN_C + c] = hs[c];
+      for (int k = 0; k < 4; ++k) acc2[o][nt][k] = low2[o][nt][k] = rest2[o][nt][k] = 0.f;
+  float g1[2] = {0.f, 0.f}, gb1 = 0.f;
+  int cnt2 = 0;
+#pragma unroll 1
+  for (int b0 = p0; b0 < p1; b0 += kCnBlk) {
     __syncthreads();
-    if (tid < CN_C) {
-      float t3 = 0.f;
-      for (int k = 0; k < HQ_THREADS; ++k) t3 += s.hs[k * CN_C + tid];
-      g3 += sg * t3;
-    } else if (tid == CN_C) {
-      g3 += sg * (float)NL;
-    }
-    // dL/da2 = relu'(a2) sg sum_t W3[t]  (in place)
-    for (int p = tid; p < NL; p += HQ_THREADS) {
-      float* h = A2 + (size_t)p * CN_C;
-#pragma unroll
-      for (int c = 0; c < CN_C; ++c) h[c] = (h[c] > 0.f) ? sg * s.w3s[c] : 0.f;
-    }
-    __syncthreads();
-    // W2, b2: sum_p d2(p)[co] h1(p + tap)[ci], tiles of CN_TILE points
-    for (int p0 = 0; p0 < NL; p0 += CN_TILE) {
-      for (int e = tid; e < CN_TILE * CN_T * 4; e += HQ_THREADS) {
-        const int pt = e / (CN_T * 4), t = (e / 4) % CN_T, v = e % 4, p = p0 + pt;
-        float4 val = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (p < NL) {
-          const int l = p / n, i = p % n;
-          const int ll = (l + t / 9 - 1 + d.L) % d.L, j = cn_site(d, i, (t / 3) % 3 - 1, t % 3 - 1);
-          val = reinterpret_cast<const float4*>(A1 + ((size_t)ll * n + j) * CN_C)[v];
-        }
-        reinterpret_cast<float4*>(s.nbh + ((size_t)pt * CN_T + t) * CN_C)[v] = val;
-      }
-      for (int e = tid; e < CN_TILE * CN_C; e += HQ_THREADS) {
-        const int pt = e / CN_C, p = p0 + pt;
-        s.dt[e] = (p < NL) ? A2[(size_t)p * CN_C + e % CN_C] : 0.f;
-      }
-      __syncthreads();
-      for (int pt = 0; pt < CN_TILE; ++pt) {
-        const float* dd = s.dt + pt * CN_C;
-        const float ha = s.nbh[(size_t)pt * CN_T * CN_C + q0];
-#pragma unroll
-        for (int c = 0; c < CN_C; ++c) g2a[c] = fmaf(ha, dd[c], g2a[c]);
-        if (has1) {
-          const float hb = s.nbh[(size_t)pt * CN_T * CN_C + q1];
-#pragma unroll
-          for (int c = 0; c < CN_C; ++c) g2b[c] = fmaf(hb, dd[c], g2b[c]);
-        }
-        if (tid >= 176 && tid < 192) gb += dd[tid - 176];
-      }
-      __syncthreads();
-    }
-    // dL/da1(q)[ci] = relu'(a1(q)) sum_t sum_co W2[t][ci][co] d2(q - tap_t)[co]
-    for (int p = tid; p < NL; p += HQ_THREADS) {
-      const int l = p / n, i = p % n;
-      float acc[CN_C];
-#pragma unroll
-      for (int c = 0; c < CN_C; ++c) acc[c] = 0.f;
-      for (int t = 0; t < CN_T; ++t) {
-        const int ll = (l - (t / 9 - 1) + d.L) % d.L, j = cn_site(d, i, -((t / 3) % 3 - 1), -(t % 3 - 1));
-        float dd[CN_C];
-        cn_load16(A2 + ((size_t)ll * n + j) * CN_C, dd);
-        const float* W = s.w + CN_W2 + t * CN_C * CN_C;
-#pragma unroll
-        for (int ci = 0; ci < CN_C; ++ci) {
-          float v = 0.f;
-#pragma unroll
-          for (int c = 0; c < CN_C; ++c) v = fmaf(W[ci * CN_C + c], dd[c], v);
-          acc[ci] += v;
-        }
-      }
-      float h[CN_C];
-      cn_load16(A1 + (size_t)p * CN_C, h);
-      float4* o = reinterpret_cast<float4*>(D1 + (size_t)p * CN_C);
-#pragma unroll
-      for (int q = 0; q < CN_C / 4; ++q)
-        o[q] = make_float4(h[4 * q] > 0.f ? acc[4 * q] : 0.f, h[4 * q + 1] > 0.f ? acc[4 * q + 1] : 0.f,
-                           h[4 * q + 2] > 0.f ? acc[4 * q + 2] : 0.f, h[4 * q + 3] > 0.f ? acc[4 * q + 3] : 0.f);
+    {
+      const int p = min(b0 + (tid & (kCnBlk - 1)), NL - 1), l = p / n, i = p % n, x = i % d.nx, y = i / d.nx;
+      const int t0 = tid < kCnBlk ? 0 : 14, t1 = tid < kCnBlk ? 14 : CN_T;
+      for (int tap = t0; tap < t1; ++tap)
+        nb[tap * kCnBlk + (tid & (kCnBlk - 1))] = cn_wrap(l + tap / 9 - 1, L) * n + cn_wrap(x + tap % 3 - 1, d.nx) +
+                                                  d.nx * cn_wrap(y + (tap / 3) % 3 - 1, d.ny);
     }
     __syncthreads();
-    // W1, b1: sum_p d1(p)[co] z(p + tap)
-    for (int p0 = 0; p0 < NL; p0 += CN_TILE) {
-      for (int e = tid; e < CN_TILE * CN_T; e += HQ_THREADS) {
-        const int pt = e / CN_T, t = e % CN_T, p = p0 + pt;
-        float z = 0.f;
-        if (p < NL) {
-          const int l = p / n, i = p % n;
-          const int ll = (l + t / 9 - 1 + d.L) % d.L, j = cn_site(d, i, (t / 3) % 3 - 1, t % 3 - 1);
-          z = (float)(X[(size_t)ll * n + j] - x0);
+#pragma unroll 4
+    for (int e = tid; e < CN_T * kCnBlk; e += HQ_THREADS) zn[(e / kCnBlk) * kCnLd + e % kCnBlk] = s.z[nb[e]];
+    {  // d1 / s of the warp's 16 points
+      const int pt = warp * 16 + g, base = b0 + warp * 16;
+      float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}}, rest[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+      if (base < p1) {
+#pragma unroll 9
+        for (int tap = 0; tap < CN_T; ++tap) {
+          const int* q = nb + (CN_T - 1 - tap) * kCnBlk + pt;  // p - t
+          const uint32_t m0 = s.mask[q[0]], m1 = s.mask[q[8]];
+          const uint32_t A[4] = {cols(m0, 2 * t), cols(m1, 2 * t), cols(m0, 2 * t + 8), cols(m1, 2 * t + 8)};
+#pragma unroll
+          for (int nt = 0; nt < 2; ++nt) {
+            float e[4] = {0.f, 0.f, 0.f, 0.f};
+            mma_bf16(e, A, wt[((tap * 3 + 0) * 2 + nt) * 32 + lane]);
+            mma_bf16(rest[nt], A, wt[((tap * 3 + 2) * 2 + nt) * 32 + lane]);
+            mma_bf16(rest[nt], A, wt[((tap * 3 + 1) * 2 + nt) * 32 + lane]);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) acc[nt][k] += e[k];
+          }
         }
-        s.nbh[e] = z;
       }
-      for (int e = tid; e < CN_TILE * CN_C; e += HQ_THREADS) {
-        const int pt = e / CN_C, p = p0 + pt;
-        s.dt[e] = (p < NL) ? D1[(size_t)p * CN_C + e % CN_C] : 0.f;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const bool on = base + g + 8 * h < p1;
+        const uint4* h1 = s.h1 + (size_t)min(base + g + 8 * h, NL - 1) * 8;
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt) {
+          const uint32_t hi = h1[4 * nt + t].x;  // h1 > 0 where its leading term is not zero
+          float* o = ds + (8 * nt + 2 * t) * kCnLd + pt + 8 * h;
+          o[0] = on && (hi & 0x7fffu) ? acc[nt][2 * h] + rest[nt][2 * h] : 0.f;
+          o[kCnLd] = on && (hi & 0x7fff0000u) ? acc[nt][2 * h + 1] + rest[nt][2 * h + 1] : 0.f;
+        }
       }
-      __syncthreads();
-      for (int pt = 0; pt < CN_TILE; ++pt) {
-        const float* dd = s.dt + pt * CN_C;
-        g1a = fmaf(s.nbh[pt * CN_T + q0 / CN_C], dd[q0 % CN_C], g1a);
-        if (has1) g1b = fmaf(s.nbh[pt * CN_T + q1 / CN_C], dd[q1 % CN_C], g1b);
-        if (tid >= 176 && tid < 192) gb1 += dd[tid - 176];
+    }
+    if (tid < kCnBlk) {
+      const uint32_t m = b0 + tid < p1 ? s.mask[b0 + tid] : 0u;
+#pragma unroll
+      for (int c = 0; c < CN_C; ++c) {
+        const int k = __popc(__ballot_sync(HQ_FULL, (m >> c) & 1u));
+        if (lane == c) cnt2 += k;
       }
-      __syncthreads();
+    }
+    // gW2
+    const int np = min(kCnBlk, p1 - b0);
+#pragma unroll 1
+    for (int q = 0; q < np; q += 16) {
+      uint32_t m[4];  // masks of points 2t, 2t + 1, 2t + 8, 2t + 9 (none beyond the part)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int p = b0 + q + 2 * t + (k & 1) + 8 * (k >> 1);
+        m[k] = p < p1 ? s.mask[p] : 0u;
+      }
+      const uint32_t A[4] = {pair(m[0], m[1], g), pair(m[0], m[1], g + 8), pair(m[2], m[3], g), pair(m[2], m[3], g + 8)};
+#pragma unroll
+      for (int o = 0; o < kCnOwn; ++o) {
+        const int tap = warp + HQ_WARPS * o;
+        if (tap < CN_T) {
+          const uint4* h0 = s.h1 + (size_t)nb[tap * kCnBlk + q + g] * 8;
+          const uint4* h1 = s.h1 + (size_t)nb[tap * kCnBlk + q + g + 8] * 8;
+#pragma unroll
+          for (int nt = 0; nt < 2; ++nt) {
+            const uint4 u = h0[4 * nt + t], v = h1[4 * nt + t];
+            // the leading terms' sum is nearly exact and is added with its rounding error kept; the other terms,
+            // 2^-8 of it, stay in the tensor core's accumulators
+            float e[4] = {0.f, 0.f, 0.f, 0.f};
+            mma_bf16(e, A, make_uint2(cn_trans8x8(u.x), cn_trans8x8(v.x)));
+            mma_bf16(rest2[o][nt], A, make_uint2(cn_trans8x8(u.z), cn_trans8x8(v.z)));
+            mma_bf16(rest2[o][nt], A, make_uint2(cn_trans8x8(u.y), cn_trans8x8(v.y)));
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const float x = acc2[o][nt][k], sum = x + e[k];  // neither is negative
+              low2[o][nt][k] += fminf(x, e[k]) - (sum - fmaxf(x, e[k]));
+              acc2[o][nt][k] = sum;
+            }
+          }
+        }
+      }
+    }
+    __syncthreads();
+    // gW1, gb1
+    const int n4 = (np + 3) >> 2;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int q = tid + u * HQ_THREADS;
+      if (q < CN_T * CN_C) {
+        const float4* zt = reinterpret_cast<const float4*>(zn + (q / CN_C) * kCnLd);
+        const float4* dd = reinterpret_cast<const float4*>(ds + (q % CN_C) * kCnLd);
+        float acc = 0.f;
+#pragma unroll 4
+        for (int k = 0; k < n4; ++k) {
+          const float4 x = zt[k], y = dd[k];
+          acc = fmaf(x.w, y.w, fmaf(x.z, y.z, fmaf(x.y, y.y, fmaf(x.x, y.x, acc))));
+        }
+        g1[u] += acc;
+      }
+    }
+    if (tid >= 176 && tid < 192) {
+      const float4* dd = reinterpret_cast<const float4*>(ds + (tid - 176) * kCnLd);
+      float acc = 0.f;
+#pragma unroll 4
+      for (int k = 0; k < n4; ++k) {
+        const float4 y = dd[k];
+        acc += (y.x + y.y) + (y.z + y.w);
+      }
+      gb1 += acc;
     }
   }
-  float* out = partials + (size_t)blockIdx.x * CN_WPAD;
+  if (tid < kCnBlk && lane < CN_C) atomicAdd(&cnt[lane], cnt2);  // integers: any order
+  __syncthreads();
+  float* out = partials + ((size_t)a * parts + blockIdx.x) * CN_WPAD;
+  auto put = [&](int k, float v) { out[k] = first ? v : out[k] + v; };
+  // rows co = g, g + 8; columns ci = 8 nt + 2t, + 1
 #pragma unroll
-  for (int c = 0; c < CN_C; ++c) out[CN_W2 + q0 * CN_C + c] = g2a[c];
-  if (has1) {
+  for (int o = 0; o < kCnOwn; ++o) {
+    const int tap = warp + HQ_WARPS * o;
+    if (tap < CN_T)
 #pragma unroll
-    for (int c = 0; c < CN_C; ++c) out[CN_W2 + q1 * CN_C + c] = g2b[c];
+      for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int co = g + 8 * (k >> 1), ci = 8 * nt + 2 * t + (k & 1);
+          const float v = acc2[o][nt][k], r = low2[o][nt][k] + rest2[o][nt][k];
+          put(CN_W2 + (tap * CN_C + ci) * CN_C + co, fmaf(sw[0][co], v, fmaf(sw[0][co], r, sw[1][co] * v)));
+        }
   }
-  out[CN_W1 + q0] = g1a;
-  if (has1) out[CN_W1 + q1] = g1b;
-  if (tid >= 176 && tid < 192) {
-    out[CN_B2 + tid - 176] = gb;
-    out[CN_B1 + tid - 176] = gb1;
+#pragma unroll
+  for (int u = 0; u < 2; ++u)
+    if (tid + u * HQ_THREADS < CN_T * CN_C) put(CN_W1 + tid + u * HQ_THREADS, scaled(g1[u]));
+  if (tid >= 176 && tid < 192) put(CN_B1 + tid - 176, scaled(gb1));
+  if (tid >= 192 && tid < 208) put(CN_B2 + tid - 192, fmaf(sw[0][tid - 192], (float)cnt[tid - 192], sw[1][tid - 192] * (float)cnt[tid - 192]));
+  if (tid < CN_C) {
+    float hs = 0.f;
+    for (int k = blockIdx.x; k < parts2; k += parts) hs += s.hs[k * CN_C + tid];
+    const float v = scaled(hs);
+    for (int k = 0; k < CN_T; ++k) put(CN_W3 + k * CN_C + tid, v);
+  } else if (tid == CN_C) {
+    put(CN_B3, scaled((float)(p1 - p0)));
   }
-  if (tid < CN_C)
-    for (int t = 0; t < CN_T; ++t) out[CN_W3 + t * CN_C + tid] = g3;
-  else if (tid == CN_C)
-    out[CN_B3] = g3;
 }
 
 // Sum of the per-CTA partials (fixed order) into grad; with lr > 0 an Adam step on the FP32
 // master weights and a fresh bfloat16 copy.
 __global__ void cnn_adam_kernel(CnnState cn, const float* partials, int nparts, float lr, int t_step) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= CN_NP) return;
-  float g = 0.f;
-  for (int p = 0; p < nparts; ++p) g += partials[(size_t)p * CN_WPAD + k];
+  const int k = blockIdx.x * kSumParams + threadIdx.x % kSumParams;
+  const float g = sum_partials(partials, nparts, CN_WPAD, k < CN_NP ? k : CN_NP - 1);
+  if (k >= CN_NP || threadIdx.x >= kSumParams) return;
   cn.grad[k] = g;
   if (lr > 0.f) {
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
@@ -250,14 +400,7 @@ __global__ void cnn_set_kernel(CnnState cn, const float* src) {
 }
 
 __global__ void cnn_loss_kernel(CnnState cn, const double* ys, const int* idx, int B, double scale, double* loss) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double acc = 0.0;
-    for (int a = 0; a < B; ++a) {
-      const double r = cn.Fb[a] - ys[idx[a]];
-      acc += r * r;
-    }
-    loss[0] += acc * scale;
-  }
+  squared_error(cn.Fb, ys, idx, B, scale, loss);
 }
 
 // ------------------------------------------------------------------------ launchers
@@ -278,12 +421,24 @@ cudaError_t cnn_launch_set(const CnnState& cn, const float* src_device, cudaStre
 
 cudaError_t cnn_launch_batch(const Dev& d, const CnnState& cn, const double* Xs, const double* ys, const int* idx,
                              int B, float lr, int t_step, cudaStream_t s) {
-  const int ctas = B < cn.train_ctas ? B : cn.train_ctas;
-  const size_t sb = cn_train_smem_bytes();
-  cudaError_t st = opt_in_smem((const void*)cnn_train_kernel, sb);
+  // rounds of up to train_ctas samples, each sample on as many CTAs as fill the chip (two per SM in layer 2); a
+  // part of the backward pass keeps its partial through the rounds
+  const int NL = d.n * d.L, round = B < cn.train_ctas ? B : cn.train_ctas, tiles = (NL + 15) / 16;
+  auto parts_of = [&](int ctas, int most) { return std::min(std::max(ctas / round, 1), std::min(most, tiles)); };
+  const int parts = parts_of(kCnnTrainCtas, 8), parts2 = parts_of(2 * kCnnTrainCtas, kCnnParts);
+  const size_t s1 = cn_smem_bytes(), s3 = cn_back_smem_bytes();
+  cudaError_t st = opt_in_smem((const void*)cnn_backward_kernel, s3);
   if (st != cudaSuccess) return st;
-  cnn_train_kernel<<<ctas, HQ_THREADS, sb, s>>>(d, cn, Xs, ys, idx, B, mean_field_shift(d), cn.Fb, cn.partials);
-  cnn_adam_kernel<<<(CN_NP + 255) / 256, 256, 0, s>>>(cn, cn.partials, ctas, lr, t_step);
+  const double x0 = mean_field_shift(d);
+  for (int a0 = 0; a0 < B; a0 += round) {
+    const int r = B - a0 < round ? B - a0 : round;
+    cnn_inputs_kernel<<<dim3((NL + 1023) / 1024, r), 256, 0, s>>>(d, cn, Xs, idx + a0, x0);
+    cnn_layer1_kernel<<<dim3((2 * NL + 511) / 512, r), HQ_THREADS, s1, s>>>(d, cn);
+    cnn_layer2_kernel<<<dim3(parts2, r), HQ_THREADS, s1, s>>>(d, cn);
+    cnn_backward_kernel<<<dim3(parts, r), HQ_THREADS, s3, s>>>(d, cn, ys, idx + a0, B, parts2, a0 == 0, cn.Fb + a0,
+                                                              cn.partials);
+  }
+  cnn_adam_kernel<<<(CN_NP + kSumParams - 1) / kSumParams, HQ_THREADS, 0, s>>>(cn, cn.partials, round * parts, lr, t_step);
   return cudaGetLastError();
 }
 

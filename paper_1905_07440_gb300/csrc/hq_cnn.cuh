@@ -20,104 +20,7 @@ constexpr int CN_W1 = 0, CN_B1 = CN_T * CN_C, CN_W2 = CN_B1 + CN_C, CN_B2 = CN_W
               CN_W3 = CN_B2 + CN_C, CN_B3 = CN_W3 + CN_T * CN_C, CN_NP = CN_B3 + 1;
 constexpr int CN_WPAD = (CN_NP + 3) & ~3;
 
-__device__ inline void cn_load_weights(const uint16_t* wb, float* w) {
-  for (int k = threadIdx.x; k < CN_WPAD; k += blockDim.x) w[k] = (k < CN_NP) ? bf16_to_float(wb[k]) : 0.f;
-  __syncthreads();
-}
-
-// site of (x + dx, y + dy) on the torus
-__device__ __forceinline__ int cn_site(const Dev& d, int i, int dy, int dx) {
-  const int x = i % d.nx, y = i / d.nx;
-  return (x + dx + d.nx) % d.nx + d.nx * ((y + dy + d.ny) % d.ny);
-}
-
-// ------------------------------------------------------------------ training path (FP32, a thread per point)
-// Layer-1 activations (after ReLU) at (l, i).
-__device__ __forceinline__ void cn_layer1(const Dev& d, const float* w, const double* X, double x0, int l, int i, float* out) {
-  float a[CN_C];
-#pragma unroll
-  for (int c = 0; c < CN_C; ++c) a[c] = w[CN_B1 + c];
-  for (int t = 0; t < CN_T; ++t) {
-    const int ll = (l + t / 9 - 1 + d.L) % d.L, j = cn_site(d, i, (t / 3) % 3 - 1, t % 3 - 1);
-    const float z = (float)(X[(size_t)ll * d.n + j] - x0);
-#pragma unroll
-    for (int c = 0; c < CN_C; ++c) a[c] = fmaf(z, w[CN_W1 + t * CN_C + c], a[c]);
-  }
-  float4* o = reinterpret_cast<float4*>(out);
-#pragma unroll
-  for (int q = 0; q < CN_C / 4; ++q)
-    o[q] = make_float4(fmaxf(a[4 * q], 0.f), fmaxf(a[4 * q + 1], 0.f), fmaxf(a[4 * q + 2], 0.f), fmaxf(a[4 * q + 3], 0.f));
-}
-
-__device__ __forceinline__ void cn_load16(const float* p, float* v) {
-  const float4* q = reinterpret_cast<const float4*>(p);
-#pragma unroll
-  for (int k = 0; k < CN_C / 4; ++k) {
-    const float4 f = q[k];
-    v[4 * k] = f.x;
-    v[4 * k + 1] = f.y;
-    v[4 * k + 2] = f.z;
-    v[4 * k + 3] = f.w;
-  }
-}
-
-// Layer-2 activations (after ReLU) at (l, i); h1at(ll, j) gives the 16 layer-1 values there.
-template <class H1>
-__device__ __forceinline__ void cn_layer2(const Dev& d, const float* w, int l, int i, H1 h1at, float* out) {
-  float a[CN_C];
-#pragma unroll
-  for (int c = 0; c < CN_C; ++c) a[c] = w[CN_B2 + c];
-  for (int t = 0; t < CN_T; ++t) {
-    const int ll = (l + t / 9 - 1 + d.L) % d.L, j = cn_site(d, i, (t / 3) % 3 - 1, t % 3 - 1);
-    float h[CN_C];
-    cn_load16(h1at(ll, j), h);
-    const float* W = w + CN_W2 + t * CN_C * CN_C;
-#pragma unroll
-    for (int ci = 0; ci < CN_C; ++ci)
-#pragma unroll
-      for (int c = 0; c < CN_C; ++c) a[c] = fmaf(h[ci], W[ci * CN_C + c], a[c]);
-  }
-  float4* o = reinterpret_cast<float4*>(out);
-#pragma unroll
-  for (int q = 0; q < CN_C / 4; ++q)
-    o[q] = make_float4(fmaxf(a[4 * q], 0.f), fmaxf(a[4 * q + 1], 0.f), fmaxf(a[4 * q + 2], 0.f), fmaxf(a[4 * q + 3], 0.f));
-}
-
-// Layer-3 output at (l, i); h2at(ll, j) gives the 16 layer-2 values there.
-template <class H2>
-__device__ __forceinline__ float cn_layer3(const Dev& d, const float* w, int l, int i, H2 h2at) {
-  float o = w[CN_B3];
-  for (int t = 0; t < CN_T; ++t) {
-    const int ll = (l + t / 9 - 1 + d.L) % d.L, j = cn_site(d, i, (t / 3) % 3 - 1, t % 3 - 1);
-    float h[CN_C];
-    cn_load16(h2at(ll, j), h);
-#pragma unroll
-    for (int ci = 0; ci < CN_C; ++ci) o = fmaf(h[ci], w[CN_W3 + t * CN_C + ci], o);
-  }
-  return o;
-}
-
-// F_cnn of one field configuration by the whole CTA; layer outputs go to h1 [L N][16],
-// h2 [L N][16].  Returns F in every thread.
-__device__ inline double cn_forward_all(const Dev& d, const float* w, const double* X, double x0, float* h1, float* h2,
-                                        double* red) {
-  const int n = d.n, NL = d.n * d.L;
-  for (int p = threadIdx.x; p < NL; p += blockDim.x) cn_layer1(d, w, X, x0, p / n, p % n, h1 + (size_t)p * CN_C);
-  __syncthreads();
-  auto h1at = [&](int ll, int j) { return h1 + ((size_t)ll * n + j) * CN_C; };
-  for (int p = threadIdx.x; p < NL; p += blockDim.x) cn_layer2(d, w, p / n, p % n, h1at, h2 + (size_t)p * CN_C);
-  __syncthreads();
-  auto h2at = [&](int ll, int j) { return h2 + ((size_t)ll * n + j) * CN_C; };
-  double part = 0.0;
-  for (int p = threadIdx.x; p < NL; p += blockDim.x) {
-    const float o = cn_layer3(d, w, p / n, p % n, h2at);
-    part += (double)o;
-  }
-  return block_sum(part, red);
-}
-
-// ------------------------------------------------------------------ sampling path
-// Evaluation and block-move windows on the tensor cores.  Two facts keep the work small:
+// Evaluation, block-move windows and training on the tensor cores.  Two facts keep the work small:
 //
 //   * F_cnn sums the last layer over the whole torus, so F_cnn = L N b3 + sum_q wbar . h2(q) with
 //     wbar = sum_t W3[t]: the third convolution is a dot product per point.  wbar is kept as two floats.
@@ -141,11 +44,12 @@ struct CnSm {
 constexpr int CN_FRAGS = CN_T * 2 * 32, CN_FLOATS = CN_T * CN_C + 4 * CN_C + 4;
 __host__ __device__ inline size_t cn_smem_bytes() { return sizeof(uint2) * CN_FRAGS + sizeof(float) * CN_FLOATS; }
 
-// all threads; ends with a barrier
+// all threads; ends with a barrier (kL2: with the fragments of W2)
+template <bool kL2 = true>
 __device__ inline CnSm cn_setup(const uint16_t* wb, char* mem) {
   uint2* fr = reinterpret_cast<uint2*>(mem);
   float* f = reinterpret_cast<float*>(fr + CN_FRAGS);
-  for (int e = threadIdx.x; e < CN_FRAGS; e += blockDim.x) {
+  for (int e = threadIdx.x; kL2 && e < CN_FRAGS; e += blockDim.x) {
     const int lane = e & 31, nt = (e >> 5) & 1, tap = e >> 6, g = lane >> 2, t = lane & 3;
     const uint16_t* W = wb + CN_W2 + tap * CN_C * CN_C + 8 * nt + g;
     auto w = [&](int ci) { return (uint32_t)W[ci * CN_C]; };
@@ -165,12 +69,18 @@ __device__ inline CnSm cn_setup(const uint16_t* wb, char* mem) {
   return CnSm{fr, w1, b1, b2, wh, wl, bf16_to_float(wb[CN_B3])};
 }
 
-// Two non-negative activations as packed bfloat16 pairs hi + mid + lo.
+// Two values as packed bfloat16 pairs hi + mid + lo (24 bits: exact).
 __device__ __forceinline__ uint4 cn_split(float a, float b) {
   const uint32_t h = cvt_bf16x2(a, b);
   const float ra = a - __uint_as_float(h << 16), rb = b - __uint_as_float(h & 0xffff0000u);
   const uint32_t m = cvt_bf16x2(ra, rb);
   return make_uint4(h, m, cvt_bf16x2(ra - __uint_as_float(m << 16), rb - __uint_as_float(m & 0xffff0000u)), 0u);
+}
+
+__device__ __forceinline__ uint32_t cn_trans8x8(uint32_t v) {
+  uint32_t r;
+  asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;\n" : "=r"(r) : "r"(v));
+  return r;
 }
 
 __device__ __forceinline__ int cn_wrap(int a, int n) { return a < 0 ? a + n : (a >= n ? a - n : a); }
@@ -209,12 +119,17 @@ __device__ __forceinline__ CnBox cn_box(const Dev& d, int i, int radius) {
   return CnBox{w < d.nx ? cn_wrap(x - radius, d.nx) : 0, w < d.ny ? cn_wrap(y - radius, d.ny) : 0, min(w, d.nx), min(w, d.ny)};
 }
 
-// wbar . h2 of 16 points by one warp: rows g, g + 8 are the points (l, x, y)[2].  Layer-1 values of sites in
-// `box` come from `win` ([L][box][8]), of the others from `cur` ([L][n][8]).  Every lane of a quad gets both.
-__device__ __forceinline__ void cn_tile(const Dev& d, const CnSm& w, const int (&l)[2], const int (&x)[2], const int (&y)[2],
-                                        const uint4* cur, const uint4* win, const CnBox& box, float (&s)[2]) {
+// Layer 2 before bias and ReLU for 16 points by one warp: rows g, g + 8 are the points (l, x, y)[2], acc[nt][2h + e]
+// channel 8 nt + 2t + e of row g + 8h.  Layer-1 values of sites in `box` come from `win` ([L][box][8]), of the
+// others from `cur` ([L][n][8]).
+__device__ __forceinline__ void cn_tile_acc(const Dev& d, const CnSm& w, const int (&l)[2], const int (&x)[2],
+                                            const int (&y)[2], const uint4* cur, const uint4* win, const CnBox& box,
+                                            float (&acc)[2][4]) {
   const int lane = threadIdx.x & 31, t = lane & 3;
-  float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+#pragma unroll
+  for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) acc[nt][k] = 0.f;
   // per row: site columns and rows of the three offsets, and their places in the window (-1 outside)
   int xs[2][3], ys[2][3], px[2][3], py[2][3];
 #pragma unroll
@@ -260,6 +175,14 @@ __device__ __forceinline__ void cn_tile(const Dev& d, const CnSm& w, const int (
       }
     }
   }
+}
+
+// wbar . h2 of the 16 points; every lane of a quad gets both rows' values.
+__device__ __forceinline__ void cn_tile(const Dev& d, const CnSm& w, const int (&l)[2], const int (&x)[2], const int (&y)[2],
+                                        const uint4* cur, const uint4* win, const CnBox& box, float (&s)[2]) {
+  const int t = threadIdx.x & 3;
+  float acc[2][4];
+  cn_tile_acc(d, w, l, x, y, cur, win, box, acc);
   s[0] = s[1] = 0.f;
 #pragma unroll
   for (int nt = 0; nt < 2; ++nt)

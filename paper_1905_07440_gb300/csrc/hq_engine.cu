@@ -924,7 +924,7 @@ constexpr int kNNParamsPad = (HQ_NN_PARAMS + 3) & ~3;
 constexpr int kCnnParamsPad = (HQ_CNN_PARAMS + 3) & ~3;
 
 struct NNLayout {
-  size_t wbf, master, grad, am, av, partials, fcache, fnew, X0, ld0, F0, F1, pc, Fb, loss, idx, counters, dFpath, G0, xf, xb;
+  size_t wbf, master, grad, am, av, partials, fcache, fnew, X0, ld0, F0, F1, pc, Fb, dout, loss, idx, counters, dFpath, G0, xf, xb;
   size_t cwbf, cmaster, cgrad, cam, cav, cpartials, h1c, s2c, h1p, s2p, tr, cFb, cF;
   int train_ctas;
   size_t total;
@@ -949,6 +949,7 @@ NNLayout nn_layout(const hq::Dev& d, int max_batch, int max_samples) {
   l.F1 = take(8 * C);
   l.pc = take(8 * C);
   l.Fb = take(8 * (size_t)max_batch);
+  l.dout = take(4 * (size_t)max_batch);
   l.loss = take(8);
   l.idx = take(4 * (size_t)max_samples);
   l.counters = take(8 * C * hq::kNNCounters);
@@ -964,12 +965,12 @@ NNLayout nn_layout(const hq::Dev& d, int max_batch, int max_samples) {
   l.cgrad = take(4 * PC);
   l.cam = take(4 * PC);
   l.cav = take(4 * PC);
-  l.cpartials = take(4 * PC * l.train_ctas);
+  l.cpartials = take(4 * PC * hq::kCnnTrainCtas);
   l.h1c = take(16 * C * NL * (CH / 2));
   l.s2c = take(4 * C * NL);
   l.h1p = take(16 * C * 9 * d.L * (CH / 2));
   l.s2p = take(4 * C * 25 * d.L);
-  l.tr = take(4 * (size_t)l.train_ctas * 3 * NL * CH);
+  l.tr = take((size_t)l.train_ctas * hq::cnn_sample_bytes(NL));
   l.cFb = take(8 * (size_t)max_batch);
   l.cF = take(8 * C);
   l.total = off;
@@ -1019,6 +1020,7 @@ int hq_nn_attach(hq_engine* e, void* arena, size_t bytes, int max_batch, int max
   nn.F1 = (double*)(a + l.F1);
   nn.last_pc = (double*)(a + l.pc);
   nn.Fb = (double*)(a + l.Fb);
+  nn.dout = (float*)(a + l.dout);
   nn.loss = (double*)(a + l.loss);
   nn.idx = (int*)(a + l.idx);
   nn.counters = (long long*)(a + l.counters);
@@ -1041,7 +1043,7 @@ int hq_nn_attach(hq_engine* e, void* arena, size_t bytes, int max_batch, int max
   cn.h1p = (uint4*)(a + l.h1p);
   cn.s2p = (float*)(a + l.s2p);
   cn.xf = nn.xf;
-  cn.tr = (float*)(a + l.tr);
+  cn.tr = a + l.tr;
   cn.Fb = (double*)(a + l.cFb);
   cn.F = (double*)(a + l.cF);
   e->cn_t_step = 0;

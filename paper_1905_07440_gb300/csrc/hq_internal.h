@@ -109,6 +109,7 @@ struct NNState {
   double* F1;           // [C]
   double* last_pc;      // [C]
   double* Fb;           // [max batch] minibatch F
+  float* dout;          // [max batch] dL/dF
   double* loss;         // [1] epoch loss accumulator
   int* idx;             // [max samples] minibatch order
   long long* counters;  // [C][kNNCounters]
@@ -123,7 +124,8 @@ struct NNState {
 // on the (x, y, tau) torus, summed over every point.  Window buffers hold the block-move proposal
 // around the moved site: radius 1 (layer 1) and 2 (layer 2) in the lattice, every slice.
 constexpr int kCnnC = 16;
-constexpr int kCnnTrainCtas = 152;
+constexpr int kCnnTrainCtas = 152;  // samples trained at a time, and CTAs they are shared out over
+constexpr int kCnnParts = 16;        // most CTAs of one sample
 struct CnnState {
   int on;               // parameters have been set
   uint16_t* wbf;        // bfloat16 weights used by every kernel
@@ -131,14 +133,14 @@ struct CnnState {
   float* grad;
   float* adam_m;
   float* adam_v;
-  float* partials;      // [train_ctas][padded params]
-  int train_ctas;
+  float* partials;      // [max(train_ctas, kCnnTrainCtas)][padded params]
+  int train_ctas;       // samples of a training round
   uint4* h1c;           // [C][L N][8] layer-1 activations of the current fields (split, by channel pairs)
   float* s2c;           // [C][L N] every point's share of F
   uint4* h1p;           // [C][9 L][8] proposal, window radius 1
   float* s2p;           // [C][25 L] radius 2
   float* xf;            // [C][L N] network inputs (float)(X - x0), the patch network's table
-  float* tr;            // [train_ctas][3][L N][16] training activations and gradients
+  char* tr;             // [train_ctas] scratch of a sample in training (cnn_sample_bytes)
   double* Fb;           // [max batch] minibatch F
   double* F;            // [C]
 };
@@ -180,6 +182,7 @@ cudaError_t nn_launch_inner(const Dev& d, const NNState& nn, const CnnState& cn,
                             int do_block, int use_cnn, int window, int site_window, cudaStream_t s);
 cudaError_t cnn_launch_eval(const Dev& d, const CnnState& cn, const double* X, double* F, int write_cache,
                             cudaStream_t s);
+size_t cnn_sample_bytes(size_t NL);
 cudaError_t cnn_launch_set(const CnnState& cn, const float* src_device, cudaStream_t s);
 cudaError_t cnn_launch_batch(const Dev& d, const CnnState& cn, const double* Xs, const double* ys, const int* idx,
                              int B, float lr, int t_step, cudaStream_t s);

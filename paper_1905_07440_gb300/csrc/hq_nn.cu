@@ -15,6 +15,7 @@
 // Every kernel evaluates f through nn_tile_f (hq_nn_tc.cuh: 16 patches per warp on the tensor
 // cores, bfloat16 operands, FP32 accumulation), so the inner chain and the acceptance see
 // bit-identical values of f.
+#include <cooperative_groups.h>
 #include <cstdio>
 #include "hq_cnn.cuh"
 #include "hq_device.cuh"
@@ -23,6 +24,7 @@
 #include "../../include/holstein_dqmc.h"
 
 namespace hq {
+namespace cg = cooperative_groups;
 
 // parameter layout: W1[25][64], b1[64], W2[64][64], b2[64], W3[64], b3
 constexpr int NN_IN = 25, NN_H = 64;
@@ -159,12 +161,13 @@ __device__ __forceinline__ double warp_sum_fixed(double v) {
 
 // F of one configuration by the whole CTA: warp w takes the tiles of 16 patch rows w, w + 8, ...
 // (fixed order); the patch values go to fc when fc != nullptr.  Returns F in every thread.
-__device__ inline double fc_eval_all(const Dev& d, const NNSmem& s, const NNFrags& w, const float* xf, float* fc) {
+__device__ inline double fc_eval_all(const Dev& d, const NNSmem& s, const NNFrags& w, const float* xf, float* fc,
+                                     int part_of = 0, int parts = 1) {
   const int n = d.n, NL = d.n * d.L;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, g = lane >> 2, t = lane & 3;
   double part = 0.0;
   const NNLane kin = nn_lane_inputs();
-  for (int base = warp * 16; base < NL; base += HQ_WARPS * 16) {
+  for (int base = (part_of * HQ_WARPS + warp) * 16; base < NL; base += parts * HQ_WARPS * 16) {
     float f0, f1, z[2][8];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -547,26 +550,41 @@ __global__ void __launch_bounds__(HQ_THREADS) nn_decide_kernel(Dev d, NNState nn
 // nn_batch_backward_tc_kernel, per-CTA partial gradients summed in a fixed order by the Adam
 // kernel.
 
+// A sample's rows are shared out over a cluster (88 us with one CTA per sample at 64 samples of 8x8, L = 80: 64 of
+// 152 SMs at work).  Also writes dL/dF of the sample as a float, once, where the backward kernel's FP64 division per
+// row held its warps up for a sixth of their time.
 __global__ void __launch_bounds__(HQ_THREADS) nn_batch_forward_kernel(Dev d, NNState nn, const double* Xs,
-                                                                      const int* idx, double* Fb) {
+                                                                      const double* ys, const int* idx, int B,
+                                                                      double* Fb) {
   extern __shared__ __align__(16) char nraw[];
-  const int a = blockIdx.x, n = d.n, NL = d.n * d.L;
+  __shared__ double Fpart;
+  const cg::cluster_group cl = cg::this_cluster();
+  const int parts = cl.num_blocks(), rank = cl.block_rank(), a = blockIdx.x / parts, n = d.n, NL = d.n * d.L;
   const NNSmem s = nn_carve(n, nraw);
   build_cross(d, s.nbr);
   const NNFrags w = nn_build_frags(nn.wbf, s.frag, s.tcf);  // (ends with a barrier)
   float* xa = nn.xb + (size_t)a * NL;  // read again by the backward pass
-  to_inputs(Xs + (size_t)idx[a] * NL, nn.x0, xa, NL);
-  const double F = fc_eval_all(d, s, w, xa, nullptr);
-  if (threadIdx.x == 0) Fb[a] = F;
+  const int k0 = (int)((long long)NL * rank / parts), k1 = (int)((long long)NL * (rank + 1) / parts);
+  to_inputs(Xs + (size_t)idx[a] * NL + k0, nn.x0, xa + k0, k1 - k0);
+  cl.sync();
+  const double F = fc_eval_all(d, s, w, xa, nullptr, rank, parts);
+  if (threadIdx.x == 0) Fpart = F;
+  cl.sync();
+  if (rank == 0 && threadIdx.x == 0) {
+    double sum = 0.0;
+    for (int r = 0; r < parts; ++r) sum += *cl.map_shared_rank(&Fpart, r);
+    Fb[a] = sum;
+    nn.dout[a] = (float)(2.0 * (sum - ys[idx[a]]) / B);
+  }
+  cl.sync();  // (a peer's shared memory is read up to here)
 }
 
 // Backward pass on the tensor cores (see hq_nn_tc.cuh): CTA k takes the 128-row chunks k, k +
 // grid, ... of the minibatch's rows (row R = sample a * L N + patch), warp w rows 16 w .. 16 w + 15
 // of a chunk.  Inputs come from nn.xb, written by the forward kernel.  partials[k] receives the
 // CTA's gradient (every entry written once).
-__global__ void __launch_bounds__(HQ_THREADS) nn_batch_backward_tc_kernel(Dev d, NNState nn,
-                                                                          const double* ys, const int* idx, int B,
-                                                                          const double* Fb, float* partials) {
+__global__ void __launch_bounds__(HQ_THREADS) nn_batch_backward_tc_kernel(Dev d, NNState nn, int B,
+                                                                          float* partials) {
   extern __shared__ __align__(16) char nraw[];
   const int n = d.n, NL = d.n * d.L, rows = B * NL;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, g = lane >> 2, t = lane & 3;
@@ -633,15 +651,10 @@ __global__ void __launch_bounds__(HQ_THREADS) nn_batch_backward_tc_kernel(Dev d,
       uint32_t ahi[4], alo[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const int row = g + 8 * (q & 1);
-        const int k = 16 * st + 2 * t + 8 * (q >> 1);
         split2(z[q & 1][4 * st + 2 * (q >> 1)], z[q & 1][4 * st + 2 * (q >> 1) + 1], ahi[q], alo[q]);
-        // z^T staging (rows k >= 25 are zero)
-        zh[k * TR_LD + 16 * warp + row] = (uint16_t)(ahi[q] & 0xffffu);
-        zl[k * TR_LD + 16 * warp + row] = (uint16_t)(alo[q] & 0xffffu);
-        zh[(k + 1) * TR_LD + 16 * warp + row] = (uint16_t)(ahi[q] >> 16);
-        zl[(k + 1) * TR_LD + 16 * warp + row] = (uint16_t)(alo[q] >> 16);
       }
+      store_transposed(zh + 16 * st * TR_LD + 16 * warp, ahi);  // (rows k >= 25 are zero)
+      store_transposed(zl + 16 * st * TR_LD + 16 * warp, alo);
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         const uint2 b = w.w1[(st * 8 + j) * 32 + lane];
@@ -657,14 +670,6 @@ __global__ void __launch_bounds__(HQ_THREADS) nn_batch_backward_tc_kernel(Dev d,
       acc1[j][1] += w.b1[v + 1];
       acc1[j][2] += w.b1[v];
       acc1[j][3] += w.b1[v + 1];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        uint16_t hh, hl;
-        split1(fmaxf(acc1[j][e], 0.f), hh, hl);
-        const int col = v + (e & 1), row = g + 8 * (e >> 1);
-        h1h[col * TR_LD + 16 * warp + row] = hh;
-        h1l[col * TR_LD + 16 * warp + row] = hl;
-      }
     }
 #pragma unroll
     for (int st = 0; st < 4; ++st) {
@@ -675,6 +680,8 @@ __global__ void __launch_bounds__(HQ_THREADS) nn_batch_backward_tc_kernel(Dev d,
         split2(fmaxf(acc1[j][0], 0.f), fmaxf(acc1[j][1], 0.f), ahi[2 * half], alo[2 * half]);
         split2(fmaxf(acc1[j][2], 0.f), fmaxf(acc1[j][3], 0.f), ahi[2 * half + 1], alo[2 * half + 1]);
       }
+      store_transposed(h1h + 16 * st * TR_LD + 16 * warp, ahi);
+      store_transposed(h1l + 16 * st * TR_LD + 16 * warp, alo);
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         const uint2 b = w.w2[(st * 8 + j) * 32 + lane];
@@ -688,7 +695,7 @@ __global__ void __launch_bounds__(HQ_THREADS) nn_batch_backward_tc_kernel(Dev d,
     for (int h = 0; h < 2; ++h) {
       int a, pr;
       rowpos(g + 8 * h, a, pr);
-      dout[h] = (r0 + g + 8 * h < rows) ? (float)(2.0 * (Fb[a] - ys[idx[a]]) / B) : 0.f;
+      dout[h] = (r0 + g + 8 * h < rows) ? nn.dout[a] : 0.f;
     }
     if (t == 0) cb3 += dout[0] + dout[1];
     // d2 = relu'(a2) dout W3 (in acc2), gW3 and gb2 column sums, d2 staged transposed
@@ -696,16 +703,12 @@ __global__ void __launch_bounds__(HQ_THREADS) nn_batch_backward_tc_kernel(Dev d,
     for (int j = 0; j < 8; ++j) {
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        const int u = 8 * j + 2 * t + (e & 1), row = g + 8 * (e >> 1);
+        const int u = 8 * j + 2 * t + (e & 1);
         const float a2 = acc2[j][e] + w.b2[u];
         const float dv = a2 > 0.f ? dout[e >> 1] * w.w3[u] : 0.f;
         cw3[2 * j + (e & 1)] = fmaf(fmaxf(a2, 0.f), dout[e >> 1], cw3[2 * j + (e & 1)]);
         cb2[2 * j + (e & 1)] += dv;
         acc2[j][e] = dv;
-        uint16_t hh, hl;
-        split1(dv, hh, hl);
-        d2h[u * TR_LD + 16 * warp + row] = hh;
-        d2l[u * TR_LD + 16 * warp + row] = hl;
       }
     }
     // d1 = relu'(a1) (d2 W2^T)
@@ -723,6 +726,8 @@ __global__ void __launch_bounds__(HQ_THREADS) nn_batch_backward_tc_kernel(Dev d,
         split2(acc2[j][0], acc2[j][1], ahi[2 * half], alo[2 * half]);
         split2(acc2[j][2], acc2[j][3], ahi[2 * half + 1], alo[2 * half + 1]);
       }
+      store_transposed(d2h + 16 * st * TR_LD + 16 * warp, ahi);
+      store_transposed(d2l + 16 * st * TR_LD + 16 * warp, alo);
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         const uint2 b = w2t[(st * 8 + j) * 32 + lane];
@@ -731,28 +736,30 @@ __global__ void __launch_bounds__(HQ_THREADS) nn_batch_backward_tc_kernel(Dev d,
       }
     }
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
+    for (int st = 0; st < 4; ++st) {
+      uint32_t dhi[4], dlo[4];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int v = 8 * j + 2 * t + (e & 1), row = g + 8 * (e >> 1);
-        const float dv = acc1[j][e] > 0.f ? acc3[j][e] : 0.f;
-        cb1[2 * j + (e & 1)] += dv;
-        uint16_t hh, hl;
-        split1(dv, hh, hl);
-        d1h[v * TR_LD + 16 * warp + row] = hh;
-        d1l[v * TR_LD + 16 * warp + row] = hl;
+      for (int half = 0; half < 2; ++half) {
+        const int j = 2 * st + half;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          acc3[j][e] = acc1[j][e] > 0.f ? acc3[j][e] : 0.f;
+          cb1[2 * j + (e & 1)] += acc3[j][e];
+        }
+        split2(acc3[j][0], acc3[j][1], dhi[2 * half], dlo[2 * half]);
+        split2(acc3[j][2], acc3[j][3], dhi[2 * half + 1], dlo[2 * half + 1]);
       }
+      store_transposed(d1h + 16 * st * TR_LD + 16 * warp, dhi);
+      store_transposed(d1l + 16 * st * TR_LD + 16 * warp, dlo);
     }
     __syncthreads();
     // gW2 = h1^T d2 and gW1 = z^T d1 over the chunk's 128 rows
 #pragma unroll
     for (int ks = 0; ks < TR_ROWS / 16; ++ks) {
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-        mma_tiles3(gw2[a], h1h, h1l, d2h, d2l, 16 * (warp / 2), 8 * (4 * (warp % 2) + a), 16 * ks);
-#pragma unroll
-      for (int a = 0; a < 2; ++a)
-        mma_tiles3(gw1[a], zh, zl, d1h, d1l, 16 * (warp / 4), 8 * (2 * (warp % 4) + a), 16 * ks);
+      const int m2 = 16 * (warp / 2) * TR_LD + 16 * ks, n2 = 32 * (warp % 2) * TR_LD + 16 * ks;
+      mma_tiles3<2>(gw2, h1h + m2, h1l + m2, d2h + n2, d2l + n2);
+      const int m1 = 16 * (warp / 4) * TR_LD + 16 * ks, n1 = 16 * (warp % 4) * TR_LD + 16 * ks;
+      mma_tiles3<1>(gw1, zh + m1, zl + m1, d1h + n1, d1l + n1);
     }
     __syncthreads();
   }
@@ -820,10 +827,9 @@ __global__ void __launch_bounds__(HQ_THREADS) nn_batch_backward_tc_kernel(Dev d,
 // Sum of the per-CTA partials (fixed order) into grad; with lr > 0 an Adam step on the FP32
 // master weights and a fresh bfloat16 copy.
 __global__ void nn_adam_kernel(NNState nn, const float* partials, int nparts, float lr, int t_step) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= NN_NP) return;
-  float g = 0.f;
-  for (int p = 0; p < nparts; ++p) g += partials[(size_t)p * NN_WPAD + k];
+  const int k = blockIdx.x * kSumParams + threadIdx.x % kSumParams;
+  const float g = sum_partials(partials, nparts, NN_WPAD, k < NN_NP ? k : NN_NP - 1);
+  if (k >= NN_NP || threadIdx.x >= kSumParams) return;
   nn.grad[k] = g;
   if (lr > 0.f) {
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
@@ -839,14 +845,7 @@ __global__ void nn_adam_kernel(NNState nn, const float* partials, int nparts, fl
 }
 
 __global__ void nn_loss_kernel(NNState nn, const double* ys, const int* idx, int B, double scale) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double acc = 0.0;
-    for (int a = 0; a < B; ++a) {
-      const double r = nn.Fb[a] - ys[idx[a]];
-      acc += r * r;
-    }
-    nn.loss[0] += acc * scale;
-  }
+  squared_error(nn.Fb, ys, idx, B, scale, nn.loss);
 }
 
 __global__ void nn_set_kernel(NNState nn, const float* src) {
@@ -899,19 +898,34 @@ cudaError_t nn_launch_batch(const Dev& d, const NNState& nn, const double* Xs, c
                             int B, float lr, int t_step, cudaStream_t s) {
   const size_t sf = nn_smem_bytes(d.n);
   smem_opt_in((const void*)nn_batch_forward_kernel, sf);
-  nn_batch_forward_kernel<<<B, HQ_THREADS, sf, s>>>(d, nn, Xs, idx, nn.Fb);
-  const size_t sbk = nn_train_tc_smem_bytes();
-  smem_opt_in((const void*)nn_batch_backward_tc_kernel, sbk);
-  // one wave: one CTA per SM (the kernel takes a whole SM's registers), at most kNNTrainCtas
   static int sms = 0;
   if (sms == 0) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
       sms = kNNTrainCtas;
   }
+  // as many CTAs per sample as still make one wave
+  int parts = 8;
+  while (parts > 1 && (B * parts > sms || parts * HQ_WARPS * 16 > d.n * d.L)) parts /= 2;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = parts;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(B * parts);
+  cfg.blockDim = dim3(HQ_THREADS);
+  cfg.dynamicSmemBytes = sf;
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  cudaError_t st = cudaLaunchKernelEx(&cfg, nn_batch_forward_kernel, d, nn, Xs, ys, idx, B, nn.Fb);
+  if (st != cudaSuccess) return st;
+  const size_t sbk = nn_train_tc_smem_bytes();
+  smem_opt_in((const void*)nn_batch_backward_tc_kernel, sbk);
+  // one wave: one CTA per SM (the kernel takes a whole SM's registers), at most kNNTrainCtas
   const int grid = sms < kNNTrainCtas ? sms : kNNTrainCtas;
-  nn_batch_backward_tc_kernel<<<grid, HQ_THREADS, sbk, s>>>(d, nn, ys, idx, B, nn.Fb, nn.partials);
-  nn_adam_kernel<<<(NN_NP + 255) / 256, 256, 0, s>>>(nn, nn.partials, grid, lr, t_step);
+  nn_batch_backward_tc_kernel<<<grid, HQ_THREADS, sbk, s>>>(d, nn, B, nn.partials);
+  nn_adam_kernel<<<(NN_NP + kSumParams - 1) / kSumParams, HQ_THREADS, 0, s>>>(nn, nn.partials, grid, lr, t_step);
   return cudaGetLastError();
 }
 

@@ -227,30 +227,85 @@ __host__ __device__ inline size_t nn_train_tc_smem_bytes() {
          sizeof(uint16_t) * (size_t)TR_LD * (2 * TC_H + 2 * TC_H + 2 * TC_K1 + 2 * TC_H) + sizeof(int) * 5 * 256;
 }
 
-__device__ __forceinline__ void split1(float v, uint16_t& hi, uint16_t& lo) {
-  uint32_t h, l;
-  split2(v, 0.f, h, l);
-  hi = (uint16_t)h;
-  lo = (uint16_t)l;
+// Stores a 16 x 16 left fragment (rows g, g + 8; columns 2t ..) transposed: T[column][row], row stride TR_LD.
+__device__ __forceinline__ void store_transposed(uint16_t* T, const uint32_t (&a)[4]) {
+  const int i = threadIdx.x & 31, m = i >> 3;
+  const uint32_t p = (uint32_t)__cvta_generic_to_shared(T + (8 * (m >> 1) + (i & 7)) * TR_LD + 8 * (m & 1));
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1,%2,%3,%4};\n" ::"r"(p), "r"(a[0]), "r"(a[1]),
+               "r"(a[2]), "r"(a[3])
+               : "memory");
 }
 
-__device__ __forceinline__ uint32_t ld32(const uint16_t* p) { return *reinterpret_cast<const uint32_t*>(p); }
+// Left fragment of rows m0 .. m0 + 15, or the right fragments (b0, b1 of columns 0 .. 7, then of 8 .. 15) of 16
+// columns, from a tile T[row or column][k].
+template <bool kRight>
+__device__ __forceinline__ void load_tile(uint32_t (&a)[4], const uint16_t* T) {
+  const int i = threadIdx.x & 31, m = i >> 3;
+  const int row = (i & 7) + 8 * (kRight ? m >> 1 : m & 1), col = 8 * (kRight ? m & 1 : m >> 1);
+  const uint32_t p = (uint32_t)__cvta_generic_to_shared(T + row * TR_LD + col);
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3])
+               : "r"(p)
+               : "memory");
+}
 
-// C += A B over one k-step, A from a transposed tile AT[m][k] (rows m0.., cols k0..), B from a
-// transposed tile BT[n][k]; three products hi hi, hi lo, lo hi.
-__device__ __forceinline__ void mma_tiles3(float (&c)[4], const uint16_t* ah, const uint16_t* al, const uint16_t* bh,
-                                           const uint16_t* bl, int m0, int n0, int k0) {
-  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+// C[2p], C[2p + 1] += A B over one k-step, p < P: A from a transposed tile at ah, al (16 rows), B from one at bh, bl
+// (16 P columns); three products hi hi, hi lo, lo hi.
+template <int P>
+__device__ __forceinline__ void mma_tiles3(float (*c)[4], const uint16_t* ah, const uint16_t* al, const uint16_t* bh,
+                                           const uint16_t* bl) {
   uint32_t Ah[4], Al[4];
-  const int r0 = (m0 + g) * TR_LD + k0 + 2 * t, r1 = (m0 + g + 8) * TR_LD + k0 + 2 * t;
-  Ah[0] = ld32(ah + r0); Ah[1] = ld32(ah + r1); Ah[2] = ld32(ah + r0 + 8); Ah[3] = ld32(ah + r1 + 8);
-  Al[0] = ld32(al + r0); Al[1] = ld32(al + r1); Al[2] = ld32(al + r0 + 8); Al[3] = ld32(al + r1 + 8);
-  const int q = (n0 + g) * TR_LD + k0 + 2 * t;
-  const uint2 Bh = make_uint2(ld32(bh + q), ld32(bh + q + 8));
-  const uint2 Bl = make_uint2(ld32(bl + q), ld32(bl + q + 8));
-  mma_bf16(c, Ah, Bh);
-  mma_bf16(c, Ah, Bl);
-  mma_bf16(c, Al, Bh);
+  load_tile<false>(Ah, ah);
+  load_tile<false>(Al, al);
+#pragma unroll
+  for (int p = 0; p < P; ++p) {
+    uint32_t Bh[4], Bl[4];
+    load_tile<true>(Bh, bh + 16 * p * TR_LD);
+    load_tile<true>(Bl, bl + 16 * p * TR_LD);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      mma_bf16(c[2 * p + q], Ah, make_uint2(Bh[2 * q], Bh[2 * q + 1]));
+      mma_bf16(c[2 * p + q], Ah, make_uint2(Bl[2 * q], Bl[2 * q + 1]));
+      mma_bf16(c[2 * p + q], Al, make_uint2(Bh[2 * q], Bh[2 * q + 1]));
+    }
+  }
+}
+
+// Sum of partials[.][k] over nparts rows of `stride`, by four threads of a CTA per entry (threads k, k + 64, ...):
+// compensated, in a fixed order.  Threads below kSumParams get it.
+constexpr int kSumParams = HQ_THREADS / 4;
+__device__ __forceinline__ float sum_partials(const float* partials, int nparts, int stride, int k) {
+  __shared__ float2 part[3][kSumParams];
+  const int q = threadIdx.x / kSumParams, j = threadIdx.x % kSumParams;
+  float s = 0.f, low = 0.f;
+  auto add = [&](float v) {
+    const float sum = s + v, b = sum - s;
+    low += (s - (sum - b)) + (v - b);
+    s = sum;
+  };
+  const int hi = nparts * (q + 1) / 4;
+#pragma unroll 8
+  for (int p = nparts * q / 4; p < hi; ++p) add(partials[(size_t)p * stride + k]);
+  if (q > 0) part[q - 1][j] = make_float2(s, low);
+  __syncthreads();
+  if (q == 0)
+    for (int i = 0; i < 3; ++i) {
+      low += part[i][j].y;
+      add(part[i][j].x);
+    }
+  return s + low;
+}
+
+// *loss += scale sum_a (F_a - y_a)^2 in ascending order of a (one warp)
+__device__ __forceinline__ void squared_error(const double* F, const double* ys, const int* idx, int B, double scale,
+                                              double* loss) {
+  double acc = 0.0;
+  for (int a0 = 0; a0 < B; a0 += 32) {
+    const int a = a0 + (int)(threadIdx.x & 31);
+    const double r = a < B ? F[a] - ys[idx[a]] : 0.0, v = r * r;
+    for (int k = 0; k < min(32, B - a0); ++k) acc += __shfl_sync(HQ_FULL, v, k);
+  }
+  if (threadIdx.x == 0) *loss += acc * scale;
 }
 
 }  // namespace hq

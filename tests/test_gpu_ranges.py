@@ -67,3 +67,31 @@ def test_non_finite_fields_are_reported(hq):  # noqa: F811
         obs = eng.observables()
         assert obs[0]["status"] == 0 and obs[1]["status"] == hq.HQ_ENAN
         eng.close()
+
+
+# (sides, beta, batch): tiles of 16 points with a remainder, one and several CTAs per sample, more samples
+# than are trained at a time (two rounds), blocks of 128 points with a remainder.  The convolutional gradient
+# is FP32 (sums of up to 432 products: 432 * 2^-24 = 3e-5); the patch gradient keeps 16 bits of an activation
+# and has the parity tests' tolerance.
+@pytest.mark.parametrize("nx,ny,beta,batch", [(4, 4, 0.5, 1), (6, 4, 0.7, 3), (4, 4, 0.5, 155), (10, 4, 0.6, 9), (6, 6, 1.1, 40)])
+def test_gradients_over_all_splits(hq, nx, ny, beta, batch):  # noqa: F811
+    import torch
+    from oracle import cnn, nn
+    p = HolsteinParams(nx=nx, ny=ny, beta=beta)
+    X = random_fields(p, batch, seed=5 * nx + ny, offset=-1.4)
+    y = np.linspace(-3.0, 2.0, batch)
+    eng = hq.Engine(p, 1)
+    eng.attach_network(batch, batch)
+    tp, tc = nn.init_params(2).astype(np.float32) * np.float32(3.0), cnn.init_params(3, out_scale=30.0)
+    eng.set_params(tp)
+    eng.cnn_set_params(tc)
+    Xd, yd = torch.from_numpy(X).cuda(), torch.from_numpy(y).cuda()
+    g, loss = eng.cnn_gradient(Xd, yd)
+    lref, gref = cnn.loss_and_grad(p, nn.to_bfloat16(tc.astype(np.float32)), X, y)
+    assert abs(loss - lref) <= 1e-4 * lref
+    assert np.max(np.abs(g - gref)) <= 1e-4 * np.max(np.abs(gref))
+    g, loss = eng.nn_gradient(Xd, yd)
+    lref, gref = nn.loss_and_grad(p, nn.to_bfloat16(tp), X, y)
+    assert abs(loss - lref) <= 2e-3 * lref
+    assert np.max(np.abs(g - gref)) <= 2e-3 * np.max(np.abs(gref))
+    eng.close()
