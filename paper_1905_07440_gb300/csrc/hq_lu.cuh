@@ -223,12 +223,12 @@ struct Rank16 {
 template <int LM>
 __device__ __noinline__ void oz_rank(const Rank16 q, int r0, int r1, int c0, int c1, int kb, uint2* frag, int* er) {
   oz_rank16<LM <= 8 ? 1 : 2>(q.base == 0.0, r0, r1, c0, c1, kb, frag, er, [&](int r, int k) { return q.A[(size_t)r * q.ar + (size_t)k * q.ak]; },
-            [&](int k, int c) { return q.B[(size_t)k * q.bk + (size_t)c * q.bc]; },
-            [&](int r, int c, double s0, double s1) {
-              const size_t at = (size_t)c * q.ldc + r;
-              double2 v = make_double2(0.0, 0.0);
-              if (q.base != 0.0) v = *reinterpret_cast<const double2*>(q.Cin + at);
-              *reinterpret_cast<double2*>(q.C + at) = make_double2(fma(q.sign, s0, v.x), fma(q.sign, s1, v.y));
+            [&](int k, int c) { return q.sign * q.B[(size_t)k * q.bk + (size_t)c * q.bc]; },
+            [&](int r, int c) {
+              return q.base != 0.0 ? *reinterpret_cast<const double2*>(q.Cin + (size_t)c * q.ldc + r) : make_double2(0.0, 0.0);
+            },
+            [&](int r, int c, double v0, double v1, double p0, double p1, double2 x) {
+              *reinterpret_cast<double2*>(q.C + (size_t)c * q.ldc + r) = make_double2(fma(v0, p0, x.x), fma(v1, p1, x.y));
             });
 }
 

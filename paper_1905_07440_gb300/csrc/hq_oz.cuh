@@ -315,16 +315,65 @@ __device__ __forceinline__ void oz_left_from_acc(const double (&w)[2][4], uint32
   }
 }
 
-// For the warp's 16 columns ca = c0 + g, cb = c0 + g + 8 and rows 0 .. nr - 1:
-// io(r, c, v0, v1) gets the products of rows r, r + 1 (from the staged coefficients) with the
-// column's left fragment.  NT tiles of 8 rows at a time: with two, one tile's conversions fill the gaps of the
-// other's MMA chains.
-template <int NT, class IO>
+// T as a double by integer instructions (rounded to nearest, halves away from zero).  A conversion and a DFMA hold the
+// scheduler's FP64 pipe 64 cycles each; with every second conversion of a rank update done here (about 18 instructions
+// of 2 cycles) the two pipes are about equally loaded.  16x16 local sweeps 345 -> 332 ms, 329 with three of four,
+// which costs the small class as much.
+__device__ __forceinline__ double oz_to_double(long long T) {
+  const uint32_t sgn = (uint32_t)((unsigned long long)T >> 32) & 0x80000000u;
+  const unsigned long long m = (unsigned long long)(T < 0 ? -T : T);
+  uint32_t w1 = (uint32_t)(m >> 32), w0 = (uint32_t)m;
+  int e = (1023 + 62) << 20;
+  if (w1 == 0) {
+    w1 = w0;
+    w0 = 0;
+    e -= 32 << 20;
+  }
+  const int c = __clz((int)w1);
+  w1 = __funnelshift_l(w0, w1, c);
+  w0 <<= c;
+  const unsigned long long r = (((unsigned long long)w1 << 32 | w0) >> 11) + ((w0 >> 10) & 1u);
+  const uint32_t nh = (uint32_t)(r >> 32) + e - ((uint32_t)c << 20);
+  return __hiloint2double((int)(w1 == 0 ? 0u : nh | sgn), (int)r);
+}
+
+// 2^x with oz_scale's limits: zero below the normal range, infinity above it and for a marked line.
+__device__ __forceinline__ double oz_pow2(int x) {
+  return __hiloint2double((int)((unsigned)min(max(x + 1023, 0), 2047) << 20), 0);
+}
+
+// For the warp's 16 columns ca = c0 + g, cb = c0 + g + 8 and rows 0 .. nr - 1: io(r, c, v0, v1, p0, p1, old) gets the
+// products v0 p0, v1 p1 (p powers of two) of rows r, r + 1 (from the staged coefficients) with the column's left
+// fragment, and old = ld(r, c), the entries that they are added to: one DFMA each, where scaling the products first
+// would put twelve more instructions on the integer pipe.  NT tiles of 8 rows at a time: with two, one tile's conversions fill the gaps of
+// the other's MMA chains.  With kAhead the next tiles' entries are fetched before this one's MMAs: N = 256 reads
+// them from L2 or beyond (16x16 block moves 145 -> 139 ms, weights' stacks 66 -> 64 ms); the small class has no registers
+// to spare for it and its matrices stay in L1 (8x8 block moves 202 -> 206 ms with it).
+template <int NT, bool kAhead, class LD, class IO>
 __device__ __forceinline__ void oz_apply_rows(const uint2* frag, const int* er, int nr, const uint32_t (&a)[4][kOzDigits],
-                                              const int (&E)[2], int ca, int cb, int cend, IO io) {
+                                              const int (&E)[2], int ca, int cb, int cend, LD ld, IO io) {
   const int lane = threadIdx.x & 31, t = lane & 3;
+  double2 old[NT][2];
+  auto fetch = [&](int tile) {
+#pragma unroll
+    for (int j = 0; j < NT; ++j) {
+      const int r = 8 * (tile + j) + 2 * t;
+      if (r < nr && ca < cend) old[j][0] = ld(r, ca);
+      if (r < nr && cb < cend) old[j][1] = ld(r, cb);
+    }
+  };
+  if (kAhead) fetch(0);
 #pragma unroll 1
   for (int tile = 0; 8 * tile < nr; tile += NT) {
+    double2 now[NT][2];
+    if (kAhead) {
+#pragma unroll
+      for (int j = 0; j < NT; ++j) {
+        now[j][0] = old[j][0];
+        now[j][1] = old[j][1];
+      }
+      fetch(tile + NT);
+    }
     long long T[NT][4];
 #pragma unroll
     for (int j = 0; j < NT; ++j) {
@@ -339,9 +388,11 @@ __device__ __forceinline__ void oz_apply_rows(const uint2* frag, const int* er, 
       if (r < nr) {
         const int E0 = er[r], E1 = er[r + 1];
         if (ca < cend)
-          io(r, ca, oz_scale((double)T[j][0], oz_expo<kOzP>(E0, E[0])), oz_scale((double)T[j][1], oz_expo<kOzP>(E1, E[0])));
+          io(r, ca, (double)T[j][0], oz_to_double(T[j][1]), oz_pow2(oz_expo<kOzP>(E0, E[0])), oz_pow2(oz_expo<kOzP>(E1, E[0])),
+             kAhead ? now[j][0] : ld(r, ca));
         if (cb < cend)
-          io(r, cb, oz_scale((double)T[j][2], oz_expo<kOzP>(E0, E[1])), oz_scale((double)T[j][3], oz_expo<kOzP>(E1, E[1])));
+          io(r, cb, (double)T[j][2], oz_to_double(T[j][3]), oz_pow2(oz_expo<kOzP>(E0, E[1])), oz_pow2(oz_expo<kOzP>(E1, E[1])),
+             kAhead ? now[j][1] : ld(r, cb));
       }
     }
   }
@@ -349,12 +400,12 @@ __device__ __forceinline__ void oz_apply_rows(const uint2* frag, const int* er, 
 
 // (The callers keep to few instances with runtime strides: a chunk of the chain runs through all of this
 // code once per factorisation step, and what is instantiated twice is fetched twice.)
-// out(r, c, s0, s1): s = sum_k A(r, k) B(k, c) for r0 <= r < r1, c0 <= c < c1 and kb <= 16 terms; fa, fb
-// values.  Reads of fa and fb must not overlap what `out` writes, except that with one_part (a warp
+// out(r, c, v0, v1, p0, p1, old): v p = sum_k A(r, k) B(k, c) for r0 <= r < r1, c0 <= c < c1 and kb <= 16 terms; fa, fb
+// values, old = ld(r, c).  Reads of fa and fb must not overlap what `out` writes, except that with one_part (a warp
 // owns its columns whole) `out` may overwrite the column entries that fb reads.  Ends with a barrier.
-template <int NT, class FA, class FB, class OUT>
+template <int NT, class FA, class FB, class LD, class OUT>
 __device__ __forceinline__ void oz_rank16(bool one_part, int r0, int r1, int c0, int c1, int kb, uint2* frag, int* er,
-                                          FA fa, FB fb, OUT out) {
+                                          FA fa, FB fb, LD ld, OUT out) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int nr = r1 - r0;
   oz_stage_rows(frag, er, nr, kb, [&](int r, int k) { return fa(r0 + r, k); });
@@ -377,8 +428,11 @@ __device__ __forceinline__ void oz_rank16(bool one_part, int r0, int r1, int c0,
     uint32_t a[4][kOzDigits];
     int E[2];
     oz_left_from_acc(w, a, E);
-    oz_apply_rows<NT>(frag + (size_t)(rb >> 3) * kOzDigits * 32, er + rb, min(rp, nr - rb), a, E, ca, cb, c1,
-                  [&](int r, int c, double s0, double s1) { out(r0 + rb + r, c, s0, s1); });
+    oz_apply_rows<NT, (NT > 1)>(frag + (size_t)(rb >> 3) * kOzDigits * 32, er + rb, min(rp, nr - rb), a, E, ca, cb, c1,
+                                [&](int r, int c) { return ld(r0 + rb + r, c); },
+                                [&](int r, int c, double v0, double v1, double p0, double p1, double2 old) {
+                                  out(r0 + rb + r, c, v0, v1, p0, p1, old);
+                                });
   }
   __syncthreads();
 }

@@ -159,12 +159,20 @@ __device__ __noinline__ void oz_wy_apply(bool trans, const double* V, int ld, in
       // W^T: sums over up to 256 rows fit one accumulator, because |v|^2 < 16 bounds the sum by
       // 4 sqrt(n) times the column's largest entry
       long long Tw[2][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}};
+      RowPair nx[4];
+      auto fetch = [&](int r) {  // a step ahead in the wide class
+        const RowPair z0{0.0, 0.0};
+        nx[0] = r < nr ? load_pair(pa + r) : z0;
+        nx[1] = r < nr ? load_pair(pb + r) : z0;
+        nx[2] = r + 8 < nr ? load_pair(pa + r + 8) : z0;
+        nx[3] = r + 8 < nr ? load_pair(pb + r + 8) : z0;
+      };
+      if (LM > 8) fetch(2 * t);
 #pragma unroll 1
       for (int ks = 0; ks < nk; ++ks) {
-        const int r = 16 * ks + 2 * t;
-        const RowPair z0{0.0, 0.0};
-        const RowPair x0 = r < nr ? load_pair(pa + r) : z0, x1 = r < nr ? load_pair(pb + r) : z0;
-        const RowPair x2 = r + 8 < nr ? load_pair(pa + r + 8) : z0, x3 = r + 8 < nr ? load_pair(pb + r + 8) : z0;
+        if (LM <= 8) fetch(16 * ks + 2 * t);
+        const RowPair x0 = nx[0], x1 = nx[1], x2 = nx[2], x3 = nx[3];
+        if (LM > 8) fetch(16 * (ks + 1) + 2 * t);
         oz_split<kOzP>(x0.v0, x0.v1, E[0], E[0], a[0]);
         oz_split<kOzP>(x1.v0, x1.v1, E[1], E[1], a[1]);
         oz_split<kOzP>(x2.v0, x2.v1, E[0], E[0], a[2]);
@@ -194,12 +202,12 @@ __device__ __noinline__ void oz_wy_apply(bool trans, const double* V, int ld, in
     }
     if (parts > 1) __syncthreads();  // W of every warp is formed before rows change
     if (work && rb < nr)
-      oz_apply_rows<kTiles>(vn + (size_t)(rb >> 3) * kOzDigits * 32, z.er + rb, min(rp, nr - rb), a, E, ca, cb, cend,
-                    [&](int r, int c, double s0, double s1) {
-                      double* p = A + (size_t)c * ld + j0 + rb + r;
-                      const RowPair x = load_pair(p);
-                      store_pair(p, x.v0 - s0, x.v1 - s1);
-                    });
+      oz_apply_rows<kTiles, (kTiles > 1)>(
+          vn + (size_t)(rb >> 3) * kOzDigits * 32, z.er + rb, min(rp, nr - rb), a, E, ca, cb, cend,
+          [&](int r, int c) { return *reinterpret_cast<const double2*>(A + (size_t)c * ld + j0 + rb + r); },
+          [&](int r, int c, double v0, double v1, double p0, double p1, double2 x) {
+            store_pair(A + (size_t)c * ld + j0 + rb + r, fma(-v0, p0, x.x), fma(-v1, p1, x.y));
+          });
   }
   __syncthreads();
 }
@@ -341,10 +349,9 @@ __device__ __noinline__ void oz_flush(double* G, const double* A, const double* 
     else
       oz_rank16<2>(false, 0, n, 0, n, kb, z.frag, z.er, [&](int r, int k) { return A[(m0 + k) * n + r]; },
                 [&](int k, int c) { return B[(m0 + k) * n + c]; },
-                [&](int r, int c, double s0, double s1) {
-                  double* p = G + c * n + r;
-                  const RowPair x = load_pair(p);
-                  store_pair(p, x.v0 + s0, x.v1 + s1);
+                [&](int r, int c) { return *reinterpret_cast<const double2*>(G + c * n + r); },
+                [&](int r, int c, double v0, double v1, double p0, double p1, double2 x) {
+                  store_pair(G + c * n + r, fma(v0, p0, x.x), fma(v1, p1, x.y));
                 });
   }
 }
