@@ -28,9 +28,9 @@ constexpr int CN_WPAD = (CN_NP + 3) & ~3;
 //     and layer 2 within 2 of its site (every slice), no outputs beyond.
 //   * Layer 2 (27 taps x 16 x 16) runs as m16n8k16 MMAs, 16 points per warp.  Weights are bfloat16
 //     already; a layer-1 value is split into three bfloat16 terms (24 bits: exact), once when it is
-//     written, and stored as fragments' register pairs: uint4 (hi, mid, lo, 0) per two channels.  Each
-//     tap's three products are added to the FP32 sums with FADDs, so no rounding of the tensor core's
-//     own accumulation carries over from tap to tap.
+//     written, and stored as fragments' register pairs: uint4 (hi, mid, lo, 0) per two channels.  The tensor
+//     core truncates its sums, which would bias F: a tap's leading products, nearly exact within 24 bits, are
+//     added to the FP32 sums with FADDs, and only the other terms, 2^-8 of them, stay in its accumulators.
 //
 // Every path computes a point through cn_tile in the same order, so a value recomputed in a window
 // equals the cached one bit for bit.  (The scalar form took 600 thousand cycles per block move at 8x8,
@@ -126,10 +126,11 @@ __device__ __forceinline__ void cn_tile_acc(const Dev& d, const CnSm& w, const i
                                             const int (&y)[2], const uint4* cur, const uint4* win, const CnBox& box,
                                             float (&acc)[2][4]) {
   const int lane = threadIdx.x & 31, t = lane & 3;
+  float rest[2][4];
 #pragma unroll
   for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
-    for (int k = 0; k < 4; ++k) acc[nt][k] = 0.f;
+    for (int k = 0; k < 4; ++k) acc[nt][k] = rest[nt][k] = 0.f;
   // per row: site columns and rows of the three offsets, and their places in the window (-1 outside)
   int xs[2][3], ys[2][3], px[2][3], py[2][3];
 #pragma unroll
@@ -167,14 +168,18 @@ __device__ __forceinline__ void cn_tile_acc(const Dev& d, const CnSm& w, const i
       for (int nt = 0; nt < 2; ++nt) {
         const uint2 b = w.w2[((9 * dl + q) * 2 + nt) * 32 + lane];
         float e[4] = {0.f, 0.f, 0.f, 0.f};
-        mma_bf16(e, lo, b);
-        mma_bf16(e, mid, b);
         mma_bf16(e, hi, b);
+        mma_bf16(rest[nt], lo, b);
+        mma_bf16(rest[nt], mid, b);
 #pragma unroll
         for (int k = 0; k < 4; ++k) acc[nt][k] += e[k];
       }
     }
   }
+#pragma unroll
+  for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) acc[nt][k] += rest[nt][k];
 }
 
 // wbar . h2 of the 16 points; every lane of a quad gets both rows' values.
