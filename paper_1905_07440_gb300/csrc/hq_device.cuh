@@ -1,9 +1,7 @@
-// Device building blocks of the Holstein DQMC engine (FP64, one CTA per Markov chain).
-//
-// Every routine is called by all HQ_THREADS threads of a CTA and works on column-major
-// n x n matrices (element (r, c) at c*ld + r) that live in global memory (L1/L2 cached).
-// The FP64 pipe is narrow on GB300 (about 1/74 of the FP32 rate): contractions run on the
-// tensor cores (hq_oz.cuh), panels on the integer pipe (hq_panel.cuh).
+// Device building blocks of the Holstein DQMC engine (one CTA per Markov chain): sums, bounded
+// waits, random numbers, section counters.  Matrices are column-major n x n (element (r, c) at c*ld + r) in
+// global memory (L1/L2 cached).  The FP64 pipe is narrow on GB300 (about 1/74 of the FP32 rate):
+// contractions run on the tensor cores (hq_oz.cuh), panels in registers (hq_panel.cuh, hq_lu.cuh).
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>

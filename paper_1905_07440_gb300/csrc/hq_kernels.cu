@@ -1,4 +1,5 @@
-// Kernels of the Holstein DQMC engine: one CTA per Markov chain, FP64 throughout.
+// Kernels of the Holstein DQMC engine: one CTA per Markov chain, FP64 results; contractions on the tensor
+// cores (hq_oz_linalg.cuh), FP64 only in chains, ratios and sums.
 //
 //   stack_build   fields -> left UDV stack of B_L..B_{b+1} at every restabilisation
 //                 boundary b, fresh G_0 and log|det M|           (DQMC section: M = I + B_L..B_1)
