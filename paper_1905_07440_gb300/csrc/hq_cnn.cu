@@ -84,64 +84,74 @@ __device__ __forceinline__ void cn_part(int NL, int part, int parts, int& p0, in
   p1 = min((int)((long long)tiles * (part + 1) / parts) * 16, NL);
 }
 
-// Layer 2 of the round's samples: masks, channel sums and shares of F (grid: parts x samples).
+// Layer 2 of the round's samples: masks, channel sums and shares of F (grid: parts x samples), a point per thread in
+// FP32.  F enters the gradient as F - y, and the tensor core's truncation biases F by about 2e-8 of itself (three
+// terms, leading products apart), which the residuals' cancellation made 5e-7 of a gradient; FMAs round to nearest.
+// (With MMAs the gradient of 32 samples of 8x8, L = 40 took 196 us, with this 303, at the start 1713.)
+__host__ __device__ inline size_t cn_layer2_smem_bytes() { return cn_smem_bytes() + sizeof(float) * CN_T * CN_C * CN_C; }
+
 __global__ void __launch_bounds__(HQ_THREADS, 2) cnn_layer2_kernel(Dev d, CnnState cn) {
   extern __shared__ __align__(16) char craw[];
   __shared__ double red[HQ_WARPS];
   __shared__ float ch[HQ_WARPS][CN_C];
-  const CnSm w = cn_setup(cn.wbf, craw);
-  const int n = d.n, NL = d.n * d.L, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  float* W2 = reinterpret_cast<float*>(craw + cn_smem_bytes());  // [27][16][16]
+  for (int e = threadIdx.x; e < CN_T * CN_C * CN_C; e += HQ_THREADS) W2[e] = bf16_to_float(cn.wbf[CN_W2 + e]);
+  const CnSm w = cn_setup<false>(cn.wbf, craw);  // (ends with a barrier)
+  const int n = d.n, NL = d.n * d.L, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const CnSample s = cn_sample(cn, NL, blockIdx.y);
   int p0, p1;
   cn_part(NL, blockIdx.x, gridDim.x, p0, p1);
-  const CnBox none{0, 0, 0, 0};
-  float hs[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
+  float hs[CN_C];
+#pragma unroll
+  for (int c = 0; c < CN_C; ++c) hs[c] = 0.f;
   double part = 0.0;
-  for (int base = p0 + warp * 16; base < p1; base += HQ_WARPS * 16) {
-    int l[2], x[2], y[2];
+  for (int p = p0 + threadIdx.x; p < p1; p += HQ_THREADS) {
+    const int l = p / n, i = p % n, x = i % d.nx, y = i / d.nx;
+    float acc[CN_C];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int p = min(base + g + 8 * h, NL - 1), i = p % n;
-      l[h] = p / n;
-      x[h] = i % d.nx;
-      y[h] = i / d.nx;
-    }
-    float acc[2][4];
-    cn_tile_acc(d, w, l, x, y, s.h1, s.h1, none, acc);
+    for (int c = 0; c < CN_C; ++c) acc[c] = 0.f;
+#pragma unroll 1
+    for (int tap = 0; tap < CN_T; ++tap) {
+      const int j = cn_wrap(l + tap / 9 - 1, d.L) * n + cn_wrap(x + tap % 3 - 1, d.nx) + d.nx * cn_wrap(y + (tap / 3) % 3 - 1, d.ny);
+      const uint4* h = s.h1 + (size_t)j * 8;
+      const float4* W = reinterpret_cast<const float4*>(W2 + tap * CN_C * CN_C);
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int p = base + g + 8 * h;
-      const bool on = p < p1;
-      uint32_t bits = 0;
-      float sum = 0.f;
+      for (int k = 0; k < CN_C / 2; ++k) {
+        const uint4 u = h[k];
+        const float v[2] = {__uint_as_float(u.x << 16) + (__uint_as_float(u.y << 16) + __uint_as_float(u.z << 16)),
+                            __uint_as_float(u.x & 0xffff0000u) +
+                                (__uint_as_float(u.y & 0xffff0000u) + __uint_as_float(u.z & 0xffff0000u))};
 #pragma unroll
-      for (int nt = 0; nt < 2; ++nt)
+        for (int e = 0; e < 2; ++e)
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const int c = 8 * nt + 2 * t + e;
-          const float a = acc[nt][2 * h + e] + w.b2[c], h2 = on ? fmaxf(a, 0.f) : 0.f;
-          if (a > 0.f) bits |= 1u << c;
-          hs[nt][e] += h2;
-          sum = fmaf(h2, w.wh[c], fmaf(h2, w.wl[c], sum));
-        }
-      bits |= __shfl_xor_sync(HQ_FULL, bits, 1);
-      bits |= __shfl_xor_sync(HQ_FULL, bits, 2);
-      sum += __shfl_xor_sync(HQ_FULL, sum, 1);
-      sum += __shfl_xor_sync(HQ_FULL, sum, 2);
-      if (on && t == 0) {
-        s.mask[p] = (uint16_t)bits;
-        part += (double)sum;
+          for (int q = 0; q < CN_C / 4; ++q) {
+            const float4 f = W[(2 * k + e) * (CN_C / 4) + q];
+            acc[4 * q] = fmaf(v[e], f.x, acc[4 * q]);
+            acc[4 * q + 1] = fmaf(v[e], f.y, acc[4 * q + 1]);
+            acc[4 * q + 2] = fmaf(v[e], f.z, acc[4 * q + 2]);
+            acc[4 * q + 3] = fmaf(v[e], f.w, acc[4 * q + 3]);
+          }
       }
     }
+    uint32_t bits = 0;
+    float sum = 0.f, low = 0.f;
+#pragma unroll
+    for (int c = 0; c < CN_C; ++c) {
+      const float a = acc[c] + w.b2[c], h2 = fmaxf(a, 0.f);
+      if (a > 0.f) bits |= 1u << c;
+      hs[c] += h2;
+      sum = fmaf(h2, w.wh[c], sum);
+      low = fmaf(h2, w.wl[c], low);
+    }
+    s.mask[p] = (uint16_t)bits;
+    part += (double)(sum + low);
   }
 #pragma unroll
-  for (int nt = 0; nt < 2; ++nt)
+  for (int c = 0; c < CN_C; ++c) {
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-#pragma unroll
-      for (int o = 4; o < 32; o <<= 1) hs[nt][e] += __shfl_xor_sync(HQ_FULL, hs[nt][e], o);
-      if (g == 0) ch[warp][8 * nt + 2 * t + e] = hs[nt][e];
-    }
+    for (int o = 1; o < 32; o <<= 1) hs[c] += __shfl_xor_sync(HQ_FULL, hs[c], o);
+    if (lane == 0) ch[warp][c] = hs[c];
+  }
   part = block_sum(part, red);  // (its barriers cover ch)
   if (threadIdx.x < CN_C) {
     float a = 0.f;
@@ -421,12 +431,12 @@ cudaError_t cnn_launch_set(const CnnState& cn, const float* src_device, cudaStre
 
 cudaError_t cnn_launch_batch(const Dev& d, const CnnState& cn, const double* Xs, const double* ys, const int* idx,
                              int B, float lr, int t_step, cudaStream_t s) {
-  // rounds of up to train_ctas samples, each sample on as many CTAs as fill the chip (two per SM in layer 2); a
+  // rounds of up to train_ctas samples, each sample on as many CTAs as fill the chip (in layer 2 a CTA per 256 points); a
   // part of the backward pass keeps its partial through the rounds
   const int NL = d.n * d.L, round = B < cn.train_ctas ? B : cn.train_ctas, tiles = (NL + 15) / 16;
   auto parts_of = [&](int ctas, int most) { return std::min(std::max(ctas / round, 1), std::min(most, tiles)); };
-  const int parts = parts_of(kCnnTrainCtas, 8), parts2 = parts_of(2 * kCnnTrainCtas, kCnnParts);
-  const size_t s1 = cn_smem_bytes(), s3 = cn_back_smem_bytes();
+  const int parts = parts_of(kCnnTrainCtas, 8), parts2 = std::min((NL + HQ_THREADS - 1) / HQ_THREADS, kCnnParts);
+  const size_t s1 = cn_smem_bytes(), s2 = cn_layer2_smem_bytes(), s3 = cn_back_smem_bytes();
   cudaError_t st = opt_in_smem((const void*)cnn_backward_kernel, s3);
   if (st != cudaSuccess) return st;
   const double x0 = mean_field_shift(d);
@@ -434,7 +444,7 @@ cudaError_t cnn_launch_batch(const Dev& d, const CnnState& cn, const double* Xs,
     const int r = B - a0 < round ? B - a0 : round;
     cnn_inputs_kernel<<<dim3((NL + 1023) / 1024, r), 256, 0, s>>>(d, cn, Xs, idx + a0, x0);
     cnn_layer1_kernel<<<dim3((2 * NL + 511) / 512, r), HQ_THREADS, s1, s>>>(d, cn);
-    cnn_layer2_kernel<<<dim3(parts2, r), HQ_THREADS, s1, s>>>(d, cn);
+    cnn_layer2_kernel<<<dim3(parts2, r), HQ_THREADS, s2, s>>>(d, cn);
     cnn_backward_kernel<<<dim3(parts, r), HQ_THREADS, s3, s>>>(d, cn, ys, idx + a0, B, parts2, a0 == 0, cn.Fb + a0,
                                                               cn.partials);
   }
