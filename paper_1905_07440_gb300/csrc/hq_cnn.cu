@@ -5,7 +5,7 @@
 // squared error, as for the patch network.  Because F_cnn is a plain sum of the last layer,
 // dF/d(layer-2 output at any point) is the same vector sum_t W3[t][.], so the error behind layer 2
 // is a mask times a constant: both contractions with it (the gradient of W2 over points, the error of
-// layer 1 over channels) are MMAs with an exact 0/1 operand.  Every sample is shared out over
+// layer 1 over channels) are MMAs with an exact 0/1 operand; layer 2 itself runs in FP32 FMAs.  Every sample is shared out over
 // several CTAs; sums run in a fixed order and the per-CTA partials are added in a fixed order by the
 // Adam kernel, so training is deterministic.
 #include <algorithm>

@@ -20,7 +20,7 @@ constexpr int CN_W1 = 0, CN_B1 = CN_T * CN_C, CN_W2 = CN_B1 + CN_C, CN_B2 = CN_W
               CN_W3 = CN_B2 + CN_C, CN_B3 = CN_W3 + CN_T * CN_C, CN_NP = CN_B3 + 1;
 constexpr int CN_WPAD = (CN_NP + 3) & ~3;
 
-// Evaluation, block-move windows and training on the tensor cores.  Two facts keep the work small:
+// Evaluation and block-move windows on the tensor cores (training: hq_cnn.cu).  Two facts keep the work small:
 //
 //   * F_cnn sums the last layer over the whole torus, so F_cnn = L N b3 + sum_q wbar . h2(q) with
 //     wbar = sum_t W3[t]: the third convolution is a dot product per point.  wbar is kept as two floats.
