@@ -108,7 +108,8 @@ __device__ __noinline__ void panel_house(double* Q, double* V, int ld, int n, in
       }
       const double d = p[0];
       const double Sj = __shfl_sync(HQ_FULL, d, 4);
-      const double a = ps->a[warp][((lane >> 4) & 1) | ((lane >> 2) & 2)];  // (ordered by the shuffles above)
+      __syncwarp();  // lane j's entries (shuffles order no memory)
+      const double a = ps->a[warp][((lane >> 4) & 1) | ((lane >> 2) & 2)];
       const int hs = __double2hiint(Sj), es = (hs >> 20) - 1023, h = es >> 1;
       const bool zero = (hs & 0x7fffffff) == 0;
       // s = S / 4^h in [1, 4); the scalars are in units of 2^h of column j
