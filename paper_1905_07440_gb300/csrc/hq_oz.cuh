@@ -26,6 +26,7 @@
 // that uses it is NaN, so that the checks on G and log|det| see it as before.
 #pragma once
 #include <cstdint>
+#include <type_traits>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include "hq_device.cuh"
@@ -196,18 +197,33 @@ __device__ inline void oz_line_bounds(bool along_k, int lines, int K, int* e, F 
   __syncthreads();
 }
 
+// v 2^x, any v
+__device__ __forceinline__ double oz_scale_any(double v, int x) {
+  return oz_abs_hi(v) >= 0x7ff00000u ? v : oz_scale(v, x);
+}
+
 // -------------------------------------------------------------------- staging
+// Exponents of the terms of a sum: term k of the left operand is taken times 2^sk(k), of the right one times 2^-sk(k),
+// by moving the exponents of the splits (a bound below 128 would not shift a zero out).
+struct OzNoShift {};
+template <class SK>
+__device__ __forceinline__ int oz_shift_at(const SK& sk, int k, int K) { return k < K ? sk(k) : 0; }
+__device__ __forceinline__ int oz_shift_at(const OzNoShift&, int, int) { return 0; }
+template <class SK>
+__device__ __forceinline__ int oz_shifted(int E, int shift) { return std::is_same<SK, OzNoShift>::value ? E : max(E + shift, 128); }
+
 // Right-operand fragments of nk k-steps x nt tiles of 8 lines: frag[((ks nt + tile) 6 + digit) 32 + lane],
-// line = 8 tile + g, k = 16 ks + 2t (+1, +8, +9).  f(line, k): value; eb(line): bound.
-template <int P, class F, class EB>
-__device__ __forceinline__ void oz_stage(uint2* frag, int k0, int nk, int nt, F f, EB eb) {
+// line = 8 tile + g, k = 16 ks + 2t (+1, +8, +9).  f(line, k): value; eb(line): bound of the values 2^sk(k), k < K.
+template <int P, class F, class EB, class SK = OzNoShift>
+__device__ __forceinline__ void oz_stage(uint2* frag, int k0, int nk, int nt, F f, EB eb, SK sk = SK(), int K = 0) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   for (int it = threadIdx.x >> 5; it < (nk - k0) * nt; it += HQ_WARPS) {
     const int ks = k0 + it / nt, tile = it % nt, line = 8 * tile + g, k = 16 * ks + 2 * t;
     const int E = eb(line);
     uint32_t x[kOzDigits], y[kOzDigits];
-    oz_split<P>(f(line, k), f(line, k + 1), E, E, x);
-    oz_split<P>(f(line, k + 8), f(line, k + 9), E, E, y);
+    auto e = [&](int kk) { return oz_shifted<SK>(E, -oz_shift_at(sk, kk, K)); };
+    oz_split<P>(f(line, k), f(line, k + 1), e(k), e(k + 1), x);
+    oz_split<P>(f(line, k + 8), f(line, k + 9), e(k + 8), e(k + 9), y);
     uint2* o = frag + (size_t)(ks * nt + tile) * kOzDigits * 32 + lane;
 #pragma unroll
     for (int d = 0; d < kOzDigits; ++d) o[d * 32] = make_uint2(x[d], y[d]);
@@ -219,10 +235,11 @@ __device__ __forceinline__ void oz_stage(uint2* frag, int k0, int nk, int nt, F 
 // fa(r, k), fb(k, c) values (asked only inside the ranges), ea(r), eb(c) bounds.  Row blocks of RB
 // rows of A are split once into shared-memory fragments (all K terms); a warp then takes 16
 // columns x 8 NT rows, splitting its columns of B in registers, so no other barrier is needed.
-// kTri: A(r, k) = 0 for k < r (the sum starts at the row block's first row).
-template <int NT, bool kWide, bool kTri, class FA, class EA, class FB, class EB, class OUT>
+// kTri: A(r, k) = 0 for k < r (the sum starts at the row block's first row).  sk(k), k < K: exponent that moves from B's
+// terms to A's (the bounds are those of A(r, k) 2^sk(k) and B(k, c) 2^-sk(k)).
+template <int NT, bool kWide, bool kTri, class FA, class EA, class FB, class EB, class OUT, class SK = OzNoShift>
 __device__ __forceinline__ void oz_gemm(int M, int N, int K, int RB, uint2* frag, FA fa, EA ea, FB fb, EB eb,
-                                        OUT out) {
+                                        OUT out, SK sk = SK()) {
   constexpr int P = kOzP;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int nk = (K + 15) >> 4, ncg = (N + 15) >> 4, nt = RB >> 3;
@@ -231,7 +248,7 @@ __device__ __forceinline__ void oz_gemm(int M, int N, int K, int RB, uint2* frag
     __syncthreads();
     oz_stage<P>(frag, k0, nk, nt,
                 [&](int line, int k) { return (r0 + line < M && k < K) ? fa(r0 + line, k) : 0.0; },
-                [&](int line) { return r0 + line < M ? ea(r0 + line) : 128; });
+                [&](int line) { return r0 + line < M ? ea(r0 + line) : 128; }, sk, K);
     __syncthreads();
     const int nh = (min(RB, M - r0) + 8 * NT - 1) / (8 * NT);
     for (int unit = warp; unit < ncg * nh; unit += HQ_WARPS) {
@@ -247,11 +264,13 @@ __device__ __forceinline__ void oz_gemm(int M, int N, int K, int RB, uint2* frag
       for (int ks = k0; ks < nk; ++ks) {
         const int k = 16 * ks + 2 * t;
         auto get = [&](int kk, int c) { return (kk < K && c < N) ? fb(kk, c) : 0.0; };
+        const int s0 = oz_shift_at(sk, k, K), s1 = oz_shift_at(sk, k + 1, K), s8 = oz_shift_at(sk, k + 8, K),
+                  s9 = oz_shift_at(sk, k + 9, K);
         uint32_t a[4][kOzDigits];
-        oz_split<P>(get(k, ca), get(k + 1, ca), Ea, Ea, a[0]);
-        oz_split<P>(get(k, cb), get(k + 1, cb), Eb, Eb, a[1]);
-        oz_split<P>(get(k + 8, ca), get(k + 9, ca), Ea, Ea, a[2]);
-        oz_split<P>(get(k + 8, cb), get(k + 9, cb), Eb, Eb, a[3]);
+        oz_split<P>(get(k, ca), get(k + 1, ca), oz_shifted<SK>(Ea, s0), oz_shifted<SK>(Ea, s1), a[0]);
+        oz_split<P>(get(k, cb), get(k + 1, cb), oz_shifted<SK>(Eb, s0), oz_shifted<SK>(Eb, s1), a[1]);
+        oz_split<P>(get(k + 8, ca), get(k + 9, ca), oz_shifted<SK>(Ea, s8), oz_shifted<SK>(Ea, s9), a[2]);
+        oz_split<P>(get(k + 8, cb), get(k + 9, cb), oz_shifted<SK>(Eb, s8), oz_shifted<SK>(Eb, s9), a[3]);
 #pragma unroll
         for (int j = 0; j < NT; ++j) {
           const uint2* fr = frag + (size_t)(ks * nt + part * NT + j) * kOzDigits * 32 + lane;

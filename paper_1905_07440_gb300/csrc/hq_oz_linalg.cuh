@@ -250,17 +250,30 @@ __device__ inline void oz_form_q(const double* V, int ld, int n, double* U, cons
     oz_wy_apply<LM>(false, V, ld, n, j0, min(j0 + 16, n), z.tall + (j0 >> 4) * 256, U, j0, n, z);
 }
 
-// Tout = D^-1 R (rows of Tprev in pivot order): T' Tprev with T' = D^-1 R Pi^T.
+// Tout = D^-1 R (rows of Tprev in pivot order): T' Tprev with T' = D^-1 R Pi^T.  The rows of Tprev differ in size, and
+// R(r, k) makes up for it: with one exponent per line the small rows would keep few bits of the digits, where a
+// sum of FP64 products keeps all (G of an 8x8 lattice at beta = 16, charge-ordered: error 2e-14 against 5e-15; with a
+// site lowered by 6: 4e-10 against 1e-12).  So the terms of the sum are scaled to rows of Tprev in 1/2 .. 1.
 template <int LM, bool kWide>
 __device__ __noinline__ void oz_t_product(const double* P, int n, const int* perm, const double* rinv,
                                           const double* Tprev, double* Tout, const OzScratch& z) {
   auto fr = [&](int r, int k) { return k >= r ? P[(size_t)k * n + r] * rinv[r] : 0.0; };
-  oz_line_bounds(false, n, n, z.er, fr);
-  oz_line_bounds(true, n, n, z.ec, [&](int c, int k) { return Tprev[(size_t)c * n + k]; });
+  int* se = z.ev;  // exponents of the rows of Tprev, in the end in pivot order (the reflectors' bounds are done with)
+  const int tid = threadIdx.x;  // n <= HQ_THREADS
+  oz_line_bounds(false, n, n, se, [&](int k, int c) { return Tprev[(size_t)c * n + k]; });
+  if (tid < n) se[tid] = se[tid] == kOzBad ? 0 : se[tid] - 1023;
+  __syncthreads();
+  oz_line_bounds(true, n, n, z.ec, [&](int c, int k) { return oz_scale_any(Tprev[(size_t)c * n + k], -se[k]); });
+  const int mine = tid < n ? se[perm[tid]] : 0;
+  __syncthreads();
+  if (tid < n) se[tid] = mine;
+  __syncthreads();
+  oz_line_bounds(false, n, n, z.er, [&](int r, int k) { return oz_scale_any(fr(r, k), se[k]); });
   oz_gemm<LM <= 8 ? 2 : 4, kWide, true>(
       n, n, n, oz_rows(n), z.frag, fr, [&](int r) { return z.er[r]; },
       [&](int k, int c) { return Tprev[(size_t)c * n + perm[k]]; }, [&](int c) { return z.ec[c]; },
-      [&](int r, int c, double v0, double v1) { store_pair(Tout + (size_t)c * n + r, v0, v1); });
+      [&](int r, int c, double v0, double v1) { store_pair(Tout + (size_t)c * n + r, v0, v1); },
+      [&](int k) { return se[k]; });
 }
 
 template <int LM>
