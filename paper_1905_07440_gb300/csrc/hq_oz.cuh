@@ -23,7 +23,7 @@
 // staging their digits through shared-memory descriptors would cost more than the MMAs.
 //
 // Non-finite values: a line with a NaN or infinity gets the exponent kOzBad, and every result
-// that uses it is NaN, so that the checks on G and log|det| see it as before.
+// that uses it is NaN or infinite, so that the checks on G and log|det| see it.
 #pragma once
 #include <cstdint>
 #include <type_traits>
@@ -137,7 +137,7 @@ __device__ __forceinline__ void oz_mma_wide(const uint32_t (&a)[4][kOzDigits], B
   }
 }
 
-// v 2^x by an integer add to the exponent; zero below the normal range, NaN for a marked line.
+// v 2^x for a finite v by an integer add to the exponent; zero below the normal range, NaN for a marked line.
 __device__ __forceinline__ double oz_scale(double v, int x) {
   const int hi = __double2hiint(v), e0 = (hi >> 20) & 0x7ff, e = e0 + x;
   int nh = hi + (int)((unsigned)x << 20);

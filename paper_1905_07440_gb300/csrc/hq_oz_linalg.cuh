@@ -3,6 +3,7 @@
 // aligned), one CTA per matrix.  What stays on the FP64 pipe is O(n^2) or narrow: panels of 16
 // columns, 16 x 16 triangles, scalings.
 #pragma once
+#include <climits>
 #include "hq_device.cuh"
 #include "hq_oz.cuh"
 #include "hq_lu.cuh"
@@ -58,9 +59,32 @@ constexpr int kTiny = 16;
 // one-time ordering gives the graded R that the UDV decomposition needs, without per-step
 // pivot searches and norm downdates.
 
+// Ordering key of a squared norm a 4^e: the IEEE bit pattern, which orders positive doubles exactly like their values,
+// with the exponent counted from 0 and free to leave its eleven bits downwards.
+__device__ __forceinline__ long long norm_key(double a, int e) {
+  return __double_as_longlong(a) - (1023ll << 52) + (long long)min(2 * e, 2036) * (1ll << 52);
+}
+
+// The key of a column whose squares leave the normal range (norms outside 2^-450 .. 2^511), by a group of 4 lanes: the
+// column is summed scaled by its largest entry.  Zero columns come last, columns with a non-finite value first.
+__device__ __noinline__ long long scaled_norm_key(const double* col, int n) {
+  const int sub = threadIdx.x & 3;
+  uint32_t top = 0;
+  for (int r = sub; r < n; r += 4) top = max(top, oz_abs_hi(col[r]));
+  top = max(top, __shfl_xor_sync(HQ_FULL, top, 1));
+  top = max(top, __shfl_xor_sync(HQ_FULL, top, 2));
+  const int e = (int)(top >> 20) - 1023;
+  double b = 0.0;
+  for (int r = sub; r < n; r += 4) {
+    const double v = shift_exponent(col[r], -e);
+    b = fma(v, v, b);
+  }
+  b = group_sum<4>(b);
+  return e == kPanelBad ? LLONG_MAX : e == kPanelZero ? LLONG_MIN : norm_key(b, e);
+}
+
 // Q <- columns of P ordered by decreasing norm (stable: ties keep index order); perm records the order.
-// Norms are compared through their IEEE bit patterns, which order non-negative doubles exactly like their
-// values.  norm2: n doubles of scratch.
+// norm2: n doubles of scratch.
 __device__ inline void prepivot(const double* P, double* Q, int ld, int n, const QrScratch& s, double* norm2) {
   const int g = threadIdx.x >> 2, sub = threadIdx.x & 3;
   for (int base = 0; base < n; base += HQ_THREADS / 4) {
@@ -71,7 +95,14 @@ __device__ inline void prepivot(const double* P, double* Q, int ld, int n, const
       for (int r = sub; r < n; r += 4) a = fma(col[r], col[r], a);
     }
     a = group_sum<4>(a);
-    if (c < n && sub == 0) norm2[c] = a;
+    const int f = __double2hiint(a) >> 20;
+    const bool out = c < n && (f < 1023 - 900 || f >= 0x7ff);
+    long long key = norm_key(a, 0);
+    if (__any_sync(HQ_FULL, out)) {
+      const long long k = scaled_norm_key(P + (size_t)min(c, n - 1) * ld, n);
+      if (out) key = k;
+    }
+    if (c < n && sub == 0) norm2[c] = __longlong_as_double(key);
   }
   __syncthreads();
   for (int c = threadIdx.x; c < n; c += HQ_THREADS) {
@@ -97,10 +128,10 @@ __device__ __noinline__ void oz_panel(double* Q, double* V, int ld, int n, int j
                                       const OzScratch& z) {
   PanelShared* ps = reinterpret_cast<PanelShared*>(z.frag);
   const int m = n - j0;
-  if (m <= 32) panel_house<LM, 1>(Q, V, ld, n, j0, kb, ps, tau, z.ev);
-  else if (LM <= 8 || m <= 64) panel_house<LM, 2>(Q, V, ld, n, j0, kb, ps, tau, z.ev);  // LM <= 8: n <= 64
-  else if (m <= 128) panel_house<LM, LM <= 8 ? 2 : 4>(Q, V, ld, n, j0, kb, ps, tau, z.ev);
-  else panel_house<LM, LM <= 8 ? 2 : 8>(Q, V, ld, n, j0, kb, ps, tau, z.ev);
+  if (m <= 32) panel_house<LM, 1>(Q, V, ld, n, j0, kb, ps, tau, z.ev, z.er);
+  else if (LM <= 8 || m <= 64) panel_house<LM, 2>(Q, V, ld, n, j0, kb, ps, tau, z.ev, z.er);  // LM <= 8: n <= 64
+  else if (m <= 128) panel_house<LM, LM <= 8 ? 2 : 4>(Q, V, ld, n, j0, kb, ps, tau, z.ev, z.er);
+  else panel_house<LM, LM <= 8 ? 2 : 8>(Q, V, ld, n, j0, kb, ps, tau, z.ev, z.er);
   stage_panel(z.frag, V, ld, n, j0, kb, z.ev);
   // the sums go behind the fragments, where the block application stages T
   const int nk = (m + 15) >> 4;

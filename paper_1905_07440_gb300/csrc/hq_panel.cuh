@@ -11,6 +11,11 @@
 //     values over 32 lanes in eight adds, fewer as columns finish), so no partial sums cross warps.
 //   * 1 / norm and 2 / v^T v come from single-precision seeds with one third-order step each; factors
 //     of two are exponent adds.
+//   * Squares and products of columns have to stay normal numbers.  They do for largest entries of 2^-200 .. 2^200 and
+//     residuals with squared norms of 2^-512 .. 2^512 (sampling at beta = 16: 2^-100 .. 2^100); the first column
+//     outside, a zero or a non-finite one included, and those behind it go through a second form of the loop, in which a
+//     column is passed on scaled by its largest entry: norms of 1e-308 to 1e308.  (Scaling in every step costs block
+//     moves 2 % at 8x8 and 3 % at 16x16, a second pass over the sums inside the step 3 to 4 %.)
 //   * The loop over the columns is rolled; a warp's columns rotate through the registers so that its
 //     next one is x[.][0] and the finished ones are at the end, where the loops skip them.
 //
@@ -39,20 +44,39 @@ constexpr int kPanelWarps = 4;  // one per scheduler
 struct PanelShared {
   double col[2][256];
   double a[kPanelWarps][4];
+  int e[2];             // scales of the columns: col 2^e is the column
+  int out[kPanelWarps];  // a column of the warp is outside the range
 };
 
-// v 2^k for a v that is zero or stays in the normal range
+// Exponents of a column with a non-finite value and of a zero (or subnormal) one, as its largest entry gives them.
+constexpr int kPanelBad = 1024, kPanelZero = -1023;
+
+// v 2^k for results below 2^1024: zero below the normal range, infinities and NaN as they are
 __device__ __forceinline__ double shift_exponent(double v, int k) {
-  const int hi = __double2hiint(v);
-  return __hiloint2double((hi & 0x7fffffff) == 0 ? hi : hi + (int)((unsigned)k << 20), __double2loint(v));
+  const int hi = __double2hiint(v), f = (hi >> 20) & 0x7ff;
+  const bool zero = f == 0 || f + k <= 0;
+  return f == 0x7ff ? v
+                    : __hiloint2double(zero ? hi & (int)0x80000000 : hi + (int)((unsigned)k << 20), zero ? 0 : __double2loint(v));
 }
 
-// Columns j0 .. j0 + kb - 1 (kb <= 16), rows j0 .. n - 1 of Q.  Writes R (rows j0 .. j0 + c of column
+// Exponent of the largest of a warp's values c(r), rows r > 0 and, with r = 0, lanes from `first` on.
+template <int RPL, class F>
+__device__ __forceinline__ int column_exponent(int first, F c) {
+  uint32_t top = 0;
+#pragma unroll
+  for (int r = 0; r < RPL; ++r)
+    if (r > 0 || (int)(threadIdx.x & 31) >= first) top = max(top, oz_abs_hi(c(r)));
+  return (int)(__reduce_max_sync(HQ_FULL, top) >> 20) - 1023;
+}
+
+// Columns j0 + c0 .. j0 + kb - 1 (kb <= 16) of a panel with rows j0 .. n - 1 of Q.  Writes R (rows j0 .. j0 + c of column
 // j0 + c) to Q, the reflector vectors (norms of 1 to 4; H = I - tau v v^T) to the same columns of V with zeros
-// above, their bounds to ev[j0 ..], and tau.  Ends with a barrier.
-template <int LM, int RPL>
-__device__ __noinline__ void panel_house(double* Q, double* V, int ld, int n, int j0, int kb, PanelShared* ps,
-                                         double* tau, int* ev) {
+// above, their bounds to ev[j0 ..], and tau.  Without kScaled it stops before the first column outside the range, with
+// all columns behind it updated in Q, and *done counts the columns finished.  From a column with a non-finite
+// value on, R, V and tau are NaN (the bound kOzBad).  Ends with a barrier.
+template <int LM, int RPL, bool kScaled>
+__device__ __noinline__ void panel_columns(double* Q, double* V, int ld, int n, int j0, int c0, int kb, PanelShared* ps,
+                                           double* tau, int* ev, int* done_out) {
   constexpr int kThreads = 32 * kPanelWarps;
   const int m = n - j0, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (warp < kPanelWarps) {
@@ -61,24 +85,47 @@ __device__ __noinline__ void panel_house(double* Q, double* V, int ld, int n, in
     for (int r = 0; r < RPL; ++r)
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const int c = 4 * i + warp, row = lane + 32 * r;
+        const int c = 4 * (i + (c0 >> 2)) + warp, row = lane + 32 * r;
         x[r][i] = (row < m && c < kb) ? Q[(size_t)(j0 + c) * ld + j0 + row] : 0.0;
       }
-    if (warp == 0) {
+    // column j (`next`: the warp's second one in its registers) to the other warps
+    auto publish = [&](int j, bool next) {
+      auto c = [&](int r) { return next ? x[r][1] : x[r][0]; };
+      if (kScaled) {
+        const int e = column_exponent<RPL>(j, c);
 #pragma unroll
-      for (int r = 0; r < RPL; ++r) ps->col[0][lane + 32 * r] = x[r][0];
+        for (int r = 0; r < RPL; ++r) ps->col[j & 1][lane + 32 * r] = shift_exponent(c(r), -e);
+        if (lane == 0) ps->e[j & 1] = e;
+      } else {
+#pragma unroll
+        for (int r = 0; r < RPL; ++r) ps->col[j & 1][lane + 32 * r] = c(r);
+      }
+    };
+    if (!kScaled) {
+      bool out = false;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int e = column_exponent<RPL>(0, [&](int r) { return x[r][i]; });
+        out = out || (4 * i + warp < kb && (e < -200 || e > 200));
+      }
+      if (lane == 0) ps->out[warp] = out;
     }
+    if (warp == (c0 & 3)) publish(c0, false);
     bar_warps(kThreads);
+    int j = c0;
+    if (!kScaled && (ps->out[0] | ps->out[1] | ps->out[2] | ps->out[3])) j = kb;  // (leaves *done at 0)
+    int finished = j == kb ? 0 : kb;
 #pragma unroll 1
-    for (int j = 0; j < kb; ++j) {
+    for (; j < kb; ++j) {
       // x[.][i] is column 4 (i + done) + warp; the warp's columns after j are entries first .. left - 1
       const int jw = j & 3, done = j >> 2, left = 4 - done, first = warp <= jw ? 1 : 0;
       double xj[RPL], p[5];
 #pragma unroll
       for (int r = 0; r < RPL; ++r) xj[r] = ps->col[j & 1][lane + 32 * r];
       const double al0 = __shfl_sync(HQ_FULL, xj[0], j);
-      double keep = xj[0];                // rows above j hold entries of R
-      if (lane < j) xj[0] = 0.0;
+      if (lane < j) xj[0] = 0.0;  // rows above j hold entries of R
+      const int ej = kScaled ? ps->e[j & 1] : 0;
+      const bool zero = kScaled && ej == kPanelZero, bad = kScaled && ej == kPanelBad;
       if (lane == j) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) ps->a[warp][i] = x[0][i];
@@ -111,8 +158,11 @@ __device__ __noinline__ void panel_house(double* Q, double* V, int ld, int n, in
       __syncwarp();  // lane j's entries (shuffles order no memory)
       const double a = ps->a[warp][((lane >> 4) & 1) | ((lane >> 2) & 2)];
       const int hs = __double2hiint(Sj), es = (hs >> 20) - 1023, h = es >> 1;
-      const bool zero = (hs & 0x7fffffff) == 0;
-      // s = S / 4^h in [1, 4); the scalars are in units of 2^h of column j
+      if (!kScaled && (unsigned)(es + 512) >= 1024u) {  // the same in every warp
+        finished = j;
+        break;
+      }
+      // s = S / 4^h in [1, 4); the scalars are in units of 2^h of the column as it was passed on
       const double s = zero ? 1.0 : __hiloint2double((hs & 0xfffff) | ((1023 + (es & 1)) << 20), __double2loint(Sj));
       const float sf = __uint_as_float((uint32_t)__double2hiint(s) * 8u - ((1023u - 127u) << 23) +
                                        ((uint32_t)__double2loint(s) >> 29));
@@ -132,8 +182,11 @@ __device__ __noinline__ void panel_house(double* Q, double* V, int ld, int n, in
       const double wc = fma(neg ? -nrm : nrm, a, shift_exponent(d, -h));  // v^T x_c
       const double e2 = fma(-td, g0, 1.0);
       const double gam = fma(g0, fma(e2, e2, e2), g0);  // 2 / v^T v
-      const double phi = zero ? 0.0 : shift_exponent(gam * wc, -h);
-      const double beta = zero ? 0.0 : shift_exponent(neg ? nrm : -nrm, h);
+      const double nan = __hiloint2double(0x7ff80000, 0);
+      // (gam is 1/16 to 1, the norm 1 to 2: normal numbers with these h)
+      auto units = [&](double v, int k) { return __hiloint2double(__double2hiint(v) + k * (1 << 20), __double2loint(v)); };
+      const double phi = bad ? nan : zero ? 0.0 : units(gam, -h) * wc;
+      const double beta = zero ? 0.0 : units(neg ? nrm : -nrm, h);
       if (lane == j) xj[0] = al0 - beta;
 #pragma unroll
       for (int i = 0; i < 4; ++i)
@@ -143,21 +196,20 @@ __device__ __noinline__ void panel_house(double* Q, double* V, int ld, int n, in
           for (int r = 0; r < RPL; ++r) x[r][i] = fma(f, xj[r], x[r][i]);
         }
       // the next column goes out before this one's records
-      if (j + 1 < kb && warp == ((j + 1) & 3)) {
-        const bool turned = jw == 3;  // warp 0 takes its next column
-#pragma unroll
-        for (int r = 0; r < RPL; ++r) ps->col[(j + 1) & 1][lane + 32 * r] = turned ? x[r][1] : x[r][0];
-      }
+      if (j + 1 < kb && warp == ((j + 1) & 3)) publish(j + 1, jw == 3);  // (warp 0 takes its next one)
       if (warp == jw) {
 #pragma unroll
         for (int r = 0; r < RPL; ++r) {
           const int row = lane + 32 * r;
-          if (row < m) V[(size_t)(j0 + j) * ld + j0 + row] = zero ? 0.0 : oz_scale(xj[r], -h);
+          if (row < m) V[(size_t)(j0 + j) * ld + j0 + row] = zero ? 0.0 : oz_scale(xj[r], bad ? kOzBad : -h);
         }
-        if (lane <= j && lane < m) Q[(size_t)(j0 + j) * ld + j0 + lane] = lane == j ? (zero ? al0 : beta) : keep;
+        // x[0][0] holds the column's entries of R above row j, and entry j before the reflection
+        if (lane <= j && lane < m)
+          Q[(size_t)(j0 + j) * ld + j0 + lane] =
+              lane < j || zero ? x[0][0] : kScaled ? oz_scale(beta, bad ? kOzBad : ej) : beta;
         if (lane == 0) {
-          tau[j] = zero ? 0.0 : gam;
-          ev[j0 + j] = zero ? kOzUnit : oz_bound(oz_abs_hi(aa + nrm));
+          tau[j] = bad ? nan : zero ? 0.0 : gam;
+          ev[j0 + j] = bad ? kOzBad : zero ? kOzUnit : oz_bound(oz_abs_hi(aa + nrm));
         }
       }
       if (jw == 3) {
@@ -169,8 +221,33 @@ __device__ __noinline__ void panel_house(double* Q, double* V, int ld, int n, in
       }
       bar_warps(kThreads);
     }
+    if (!kScaled) {
+      if (finished < kb) {  // what is left of the columns behind, for the second form
+#pragma unroll 1
+        for (int i = 0; i < 4; ++i) {
+          const int c = 4 * ((finished >> 2) + i) + warp;
+#pragma unroll
+          for (int r = 0; r < RPL; ++r) {
+            const int row = lane + 32 * r;
+            if (c >= finished && c < kb && row < m) Q[(size_t)(j0 + c) * ld + j0 + row] = x[r][0];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) x[r][k] = x[r][k + 1];
+          }
+        }
+      }
+      if (tid == 0) *done_out = finished;
+    }
   }
   __syncthreads();
+}
+
+// A panel's columns (as panel_columns).  done: an int of shared memory that the panel's fragments do not cover.
+template <int LM, int RPL>
+__device__ __forceinline__ void panel_house(double* Q, double* V, int ld, int n, int j0, int kb, PanelShared* ps, double* tau,
+                                            int* ev, int* done) {
+  panel_columns<LM, RPL, false>(Q, V, ld, n, j0, 0, kb, ps, tau, ev, done);
+  const int c0 = *done;
+  if (c0 < kb) panel_columns<LM, RPL, true>(Q, V, ld, n, j0, c0, kb, ps, tau, ev, nullptr);
 }
 
 // Right-operand fragments of V's panel with the rows as terms (fragment order of oz_stage, 2 tiles of 8
