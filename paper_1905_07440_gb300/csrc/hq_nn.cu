@@ -89,12 +89,13 @@ __device__ __forceinline__ void bar_arrive(int id, int threads) {
 }
 
 // sum over the warp of (double)a - (double)b: a 64-bit integer sum in units of 2^-57 of the largest term
-// (a dependent FP64 instruction takes 64 cycles here, an integer shuffle-and-add about 35).
+// (a dependent FP64 instruction takes 64 cycles here, an integer shuffle-and-add about 35).  Infinite terms are summed
+// in FP64: a patch value of minus infinity has to reject its move.
 __device__ __forceinline__ double warp_sum_diff(float a, float b) {
   const uint32_t ua = __float_as_uint(a), ub = __float_as_uint(b);
   const uint32_t top = __reduce_max_sync(HQ_FULL, max(ua & 0x7fffffffu, ub & 0x7fffffffu));
   const int E = (int)(top >> 23);
-  if (E == 255) return __longlong_as_double(0x7ff8000000000000ll);
+  if (E == 255) return warp_sum((double)a - (double)b);
   auto fix = [&](uint32_t u) {
     const int e = (int)((u >> 23) & 0xffu);
     const long long m = e ? (long long)((((unsigned long long)((u & 0x7fffffu) | 0x800000u)) << 33) >> min(E - e, 63)) : 0ll;
