@@ -19,7 +19,7 @@ static_assert(CN_NP == HQ_CNN_PARAMS, "parameter count");
 
 // ------------------------------------------------------------------------ evaluation
 // F_cnn of every chain (grid = chains); refreshes the chain's caches and network inputs.
-__global__ void __launch_bounds__(HQ_THREADS, 2) cnn_eval_kernel(Dev d, CnnState cn, const double* Xall, double* Fout,
+__global__ void __launch_bounds__(HQ_THREADS, 2) cnn_eval_kernel(const __grid_constant__ Dev d, CnnState cn, const double* Xall, double* Fout,
                                                                  double x0) {
   extern __shared__ __align__(16) char craw[];
   __shared__ double red[HQ_WARPS];
@@ -28,7 +28,7 @@ __global__ void __launch_bounds__(HQ_THREADS, 2) cnn_eval_kernel(Dev d, CnnState
   float* xf = cn.xf + (size_t)c * NL;
   for (int k = threadIdx.x; k < NL; k += HQ_THREADS) xf[k] = (float)(X[k] - x0);
   const CnSm w = cn_setup(cn.wbf, craw);  // (ends with a barrier)
-  const double F = cn_refresh(d, w, xf, cn.h1c + (size_t)c * NL * 8, cn.s2c + (size_t)c * NL, red);
+  const double F = cn_refresh(d, w, xf, cn.h1c + (size_t)c * NL * 4, cn.s2c + (size_t)c * NL, red);
   if (threadIdx.x == 0) Fout[c] = F;
 }
 
@@ -73,7 +73,10 @@ __global__ void __launch_bounds__(HQ_THREADS) cnn_layer1_kernel(Dev d, CnnState 
   const CnSample s = cn_sample(cn, NL, blockIdx.y);
   for (int e = blockIdx.x * HQ_THREADS + threadIdx.x; e < 2 * NL; e += gridDim.x * HQ_THREADS) {
     const int p = e >> 1, l = p / n, i = p % n;
-    cn_point1(d, w, l, i % d.nx, i / d.nx, e & 1, [&](int ll, int j) { return s.z[ll * n + j]; }, s.h1 + (size_t)p * 8);
+    float a[8];
+    cn_point1(d, w, l, i % d.nx, i / d.nx, e & 1, [&](int ll, int j) { return s.z[ll * n + j]; }, a);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) s.h1[(size_t)p * 8 + 4 * (e & 1) + c] = cn_split(a[2 * c], a[2 * c + 1]);
   }
 }
 
@@ -88,15 +91,11 @@ __device__ __forceinline__ void cn_part(int NL, int part, int parts, int& p0, in
 // FP32.  F enters the gradient as F - y, and the tensor core's truncation biases F by about 2e-8 of itself (three
 // terms, leading products apart), which the residuals' cancellation made 5e-7 of a gradient; FMAs round to nearest.
 // (With MMAs the gradient of 32 samples of 8x8, L = 40 took 196 us, with this 303, at the start 1713.)
-__host__ __device__ inline size_t cn_layer2_smem_bytes() { return cn_smem_bytes() + sizeof(float) * CN_T * CN_C * CN_C; }
-
 __global__ void __launch_bounds__(HQ_THREADS, 2) cnn_layer2_kernel(Dev d, CnnState cn) {
   extern __shared__ __align__(16) char craw[];
   __shared__ double red[HQ_WARPS];
   __shared__ float ch[HQ_WARPS][CN_C];
-  float* W2 = reinterpret_cast<float*>(craw + cn_smem_bytes());  // [27][16][16]
-  for (int e = threadIdx.x; e < CN_T * CN_C * CN_C; e += HQ_THREADS) W2[e] = bf16_to_float(cn.wbf[CN_W2 + e]);
-  const CnSm w = cn_setup<false>(cn.wbf, craw);  // (ends with a barrier)
+  const CnSm w = cn_setup(cn.wbf, craw);  // (ends with a barrier)
   const int n = d.n, NL = d.n * d.L, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const CnSample s = cn_sample(cn, NL, blockIdx.y);
   int p0, p1;
@@ -114,7 +113,7 @@ __global__ void __launch_bounds__(HQ_THREADS, 2) cnn_layer2_kernel(Dev d, CnnSta
     for (int tap = 0; tap < CN_T; ++tap) {
       const int j = cn_wrap(l + tap / 9 - 1, d.L) * n + cn_wrap(x + tap % 3 - 1, d.nx) + d.nx * cn_wrap(y + (tap / 3) % 3 - 1, d.ny);
       const uint4* h = s.h1 + (size_t)j * 8;
-      const float4* W = reinterpret_cast<const float4*>(W2 + tap * CN_C * CN_C);
+      const float4* W = w.w2 + tap * CN_C * (CN_C / 4);
 #pragma unroll
       for (int k = 0; k < CN_C / 2; ++k) {
         const uint4 u = h[k];
@@ -174,7 +173,7 @@ constexpr int CN_WT = CN_T * 3 * 2 * 32;  // fragments of W2 w, three terms
 constexpr int kCnOwn = (CN_T + HQ_WARPS - 1) / HQ_WARPS;
 
 __host__ __device__ inline size_t cn_back_smem_bytes() {
-  return cn_smem_bytes() + sizeof(uint2) * CN_WT + sizeof(float) * kCnLd * (CN_T + CN_C) + sizeof(int) * kCnBlk * CN_T;
+  return cn_smem_bytes(false) + sizeof(uint2) * CN_WT + sizeof(float) * kCnLd * (CN_T + CN_C) + sizeof(int) * kCnBlk * CN_T;
 }
 
 __global__ void __launch_bounds__(HQ_THREADS) cnn_backward_kernel(Dev d, CnnState cn, const double* ys, const int* idx,
@@ -184,7 +183,7 @@ __global__ void __launch_bounds__(HQ_THREADS) cnn_backward_kernel(Dev d, CnnStat
   __shared__ float sw[2][CN_C];
   __shared__ int cnt[CN_C];
   const CnSm w = cn_setup<false>(cn.wbf, craw);
-  uint2* wt = reinterpret_cast<uint2*>(craw + cn_smem_bytes());
+  uint2* wt = reinterpret_cast<uint2*>(craw + cn_smem_bytes(false));
   float* zn = reinterpret_cast<float*>(wt + CN_WT);  // [27][kCnLd] inputs at p + t
   float* ds = zn + kCnLd * CN_T;                     // [16][kCnLd] d1 / s
   int* nb = reinterpret_cast<int*>(ds + kCnLd * CN_C);  // [27][kCnBlk] places of p + t
@@ -418,7 +417,7 @@ static double mean_field_shift(const Dev& d) { return -d.g / (d.mass * d.omega *
 
 cudaError_t cnn_launch_eval(const Dev& d, const CnnState& cn, const double* X, double* F, int /*write_cache*/,
                             cudaStream_t s) {
-  const size_t sb = cn_smem_bytes();
+  const size_t sb = cn_smem_bytes(true);
   opt_in_smem((const void*)cnn_eval_kernel, sb);
   cnn_eval_kernel<<<d.n_chains, HQ_THREADS, sb, s>>>(d, cn, X, F, mean_field_shift(d));
   return cudaGetLastError();
@@ -436,7 +435,7 @@ cudaError_t cnn_launch_batch(const Dev& d, const CnnState& cn, const double* Xs,
   const int NL = d.n * d.L, round = B < cn.train_ctas ? B : cn.train_ctas, tiles = (NL + 15) / 16;
   auto parts_of = [&](int ctas, int most) { return std::min(std::max(ctas / round, 1), std::min(most, tiles)); };
   const int parts = parts_of(kCnnTrainCtas, 8), parts2 = std::min((NL + HQ_THREADS - 1) / HQ_THREADS, kCnnParts);
-  const size_t s1 = cn_smem_bytes(), s2 = cn_layer2_smem_bytes(), s3 = cn_back_smem_bytes();
+  const size_t s1 = cn_smem_bytes(false), s2 = cn_smem_bytes(true), s3 = cn_back_smem_bytes();
   cudaError_t st = opt_in_smem((const void*)cnn_backward_kernel, s3);
   if (st != cudaSuccess) return st;
   const double x0 = mean_field_shift(d);

@@ -966,9 +966,9 @@ NNLayout nn_layout(const hq::Dev& d, int max_batch, int max_samples) {
   l.cam = take(4 * PC);
   l.cav = take(4 * PC);
   l.cpartials = take(4 * PC * hq::kCnnTrainCtas);
-  l.h1c = take(16 * C * NL * (CH / 2));
+  l.h1c = take(4 * C * NL * CH);
   l.s2c = take(4 * C * NL);
-  l.h1p = take(16 * C * 9 * d.L * (CH / 2));
+  l.h1p = take(4 * C * 9 * d.L * CH);
   l.s2p = take(4 * C * 25 * d.L);
   l.tr = take((size_t)l.train_ctas * hq::cnn_sample_bytes(NL));
   l.cFb = take(8 * (size_t)max_batch);
@@ -1038,9 +1038,9 @@ int hq_nn_attach(hq_engine* e, void* arena, size_t bytes, int max_batch, int max
   cn.adam_v = (float*)(a + l.cav);
   cn.partials = (float*)(a + l.cpartials);
   cn.train_ctas = l.train_ctas;
-  cn.h1c = (uint4*)(a + l.h1c);
+  cn.h1c = (float4*)(a + l.h1c);
   cn.s2c = (float*)(a + l.s2c);
-  cn.h1p = (uint4*)(a + l.h1p);
+  cn.h1p = (float4*)(a + l.h1p);
   cn.s2p = (float*)(a + l.s2p);
   cn.xf = nn.xf;
   cn.tr = a + l.tr;

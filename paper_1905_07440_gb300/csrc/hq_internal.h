@@ -135,9 +135,9 @@ struct CnnState {
   float* adam_v;
   float* partials;      // [max(train_ctas, kCnnTrainCtas)][padded params]
   int train_ctas;       // samples of a training round
-  uint4* h1c;           // [C][L N][8] layer-1 activations of the current fields (split, by channel pairs)
+  float4* h1c;          // [C][4][L N] layer-1 activations of the current fields, by channel quads
   float* s2c;           // [C][L N] every point's share of F
-  uint4* h1p;           // [C][9 L][8] proposal, window radius 1
+  float4* h1p;          // [C][9 L][4] those that a proposal has replaced, window radius 1
   float* s2p;           // [C][25 L] radius 2
   float* xf;            // [C][L N] network inputs (float)(X - x0), the patch network's table
   char* tr;             // [train_ctas] scratch of a sample in training (cnn_sample_bytes)

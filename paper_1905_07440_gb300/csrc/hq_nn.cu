@@ -56,7 +56,7 @@ __host__ __device__ inline size_t nn_smem_bytes(int n, bool with_cnn = false) {
   size_t b = sizeof(uint2) * TC_FRAGS + sizeof(double) * (HQ_WARPS + 3 * (size_t)n + NN_GROUPS + 8) +
              sizeof(float) * (TC_FLOATS + 32 + 128 + (size_t)n) + sizeof(int) * (4 + 5 * (size_t)n);
   b = (b + 15) & ~(size_t)15;
-  if (with_cnn) b += cn_smem_bytes();
+  if (with_cnn) b += cn_smem_bytes(true);
   return b;
 }
 
@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(HQ_THREADS) nn_eval_kernel(Dev d, NNState nn, 
 // The caches of the current fields (fc; with use_cnn also the convolutional activations) are
 // valid on entry; with use_cnn each network's cache is rebuilt before its part when the other
 // part has changed the fields.
-__global__ void __launch_bounds__(HQ_THREADS, 2) nn_inner_kernel(Dev d, NNState nn, CnnState cn, int n_inner,
+__global__ void __launch_bounds__(HQ_THREADS, 2) nn_inner_kernel(const __grid_constant__ Dev d, NNState nn, CnnState cn, int n_inner,
                                                               int do_local, int do_block, int use_cnn, int window,
                                                               int site_window) {
   extern __shared__ __align__(16) char nraw[];
@@ -238,9 +238,9 @@ __global__ void __launch_bounds__(HQ_THREADS, 2) nn_inner_kernel(Dev d, NNState 
   float* fc = nn.fcache + (size_t)c * NL;
   float* fnew = nn.fnew + (size_t)c * 6 * L;
   float* xsh = fnew + 5 * L;  // inputs of the moved site's proposed values (block moves)
-  uint4* h1c = cn.h1c + (size_t)c * NL * 8;
+  float4* h1c = cn.h1c + (size_t)c * NL * 4;
   float* s2c = cn.s2c + (size_t)c * NL;
-  uint4* h1p = cn.h1p + (size_t)c * 9 * L * 8;
+  float4* h1p = cn.h1p + (size_t)c * 9 * L * 4;
   float* s2p = cn.s2p + (size_t)c * 25 * L;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, g = lane >> 2, t = lane & 3;
   const uint32_t* id = d.cid + 4 * (size_t)c;
@@ -486,13 +486,13 @@ __global__ void __launch_bounds__(HQ_THREADS, 2) nn_inner_kernel(Dev d, NNState 
             xf[(size_t)sl * n + i] = net_input(v, nn.x0);
           }
           if (use_cnn) {
-            cn_block_commit(d, i, h1c, s2c, h1p, s2p);
             fc_stale = true;
           } else {
             for (int q = threadIdx.x; q < 5 * L; q += HQ_THREADS)
               fc[(q / 5) * n + s.nbr[5 * i + opposite(q % 5)]] = fnew[q];
           }
         }
+        if (use_cnn) cn_block_end(d, i, s.scal[0] != 0.0, h1c, s2c, h1p, s2p);
         __syncthreads();
       }
     }
