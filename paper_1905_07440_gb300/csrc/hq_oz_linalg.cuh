@@ -67,7 +67,7 @@ __device__ __forceinline__ long long norm_key(double a, int e) {
 
 // The key of a column whose squares leave the normal range (norms outside 2^-450 .. 2^511), by a group of 4 lanes: the
 // column is summed scaled by its largest entry.  Zero columns come last, columns with a non-finite value first.
-__device__ __noinline__ long long scaled_norm_key(const double* col, int n) {
+static __device__ __noinline__ long long scaled_norm_key(const double* col, int n) {
   const int sub = threadIdx.x & 3;
   uint32_t top = 0;
   for (int r = sub; r < n; r += 4) top = max(top, oz_abs_hi(col[r]));

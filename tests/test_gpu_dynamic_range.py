@@ -7,7 +7,7 @@ The oracle's pivoted QR scales its norms: on the shapes below its two orders of 
 import numpy as np
 import pytest
 
-from tests.test_gpu_parity import G_ATOL, LD_RTOL, hq  # noqa: F401
+from tests.test_gpu_parity import G_ATOL, LD_RTOL, check_against_oracle, hq  # noqa: F401
 from workloads import HolsteinParams, initial_fields, ordered_fields
 
 pytestmark = pytest.mark.gpu
@@ -38,6 +38,13 @@ def test_norms_beyond_the_range_of_their_squares(hq, nx, ny, beta, n_wrap, shift
     out = torch.empty(1, dtype=torch.float64, device="cuda")
     hq.logdet_noalloc(p, torch.from_numpy(X).cuda(), out)
     assert abs(out.item() - ld_ref) <= LD_RTOL * abs(ld_ref)
+
+
+@pytest.mark.parametrize("local,method", [(True, 1), (False, 1), (False, 2)])
+def test_sweeps_beyond_the_range_of_the_squares(hq, local, method):  # noqa: F811
+    """Moves, two-sided G and block determinants where the chain's norms pass 1e+-166: the oracle's decisions."""
+    p = HolsteinParams(nx=4, ny=4, beta=90.0, seed=21, block_method=method)
+    check_against_oracle(hq, p, ordered_fields(p, 1, 0.9), 1, local=local, global_=not local)
 
 
 def test_norms_beyond_64_bits_are_reported(hq):  # noqa: F811
