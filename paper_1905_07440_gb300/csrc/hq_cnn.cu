@@ -18,7 +18,8 @@ namespace hq {
 static_assert(CN_NP == HQ_CNN_PARAMS, "parameter count");
 
 // ------------------------------------------------------------------------ evaluation
-// F_cnn of every chain (grid = chains); refreshes the chain's caches and network inputs.
+// F_cnn of every chain (grid = chains).  The chain's caches and its input table (the patch network's too) become those of
+// Xall, so this is called on the current fields only.
 __global__ void __launch_bounds__(HQ_THREADS, 2) cnn_eval_kernel(const __grid_constant__ Dev d, CnnState cn, const double* Xall, double* Fout,
                                                                  double x0) {
   extern __shared__ __align__(16) char craw[];
@@ -415,8 +416,7 @@ __global__ void cnn_loss_kernel(CnnState cn, const double* ys, const int* idx, i
 // ------------------------------------------------------------------------ launchers
 static double mean_field_shift(const Dev& d) { return -d.g / (d.mass * d.omega * d.omega); }
 
-cudaError_t cnn_launch_eval(const Dev& d, const CnnState& cn, const double* X, double* F, int /*write_cache*/,
-                            cudaStream_t s) {
+cudaError_t cnn_launch_eval(const Dev& d, const CnnState& cn, const double* X, double* F, cudaStream_t s) {
   const size_t sb = cn_smem_bytes(true);
   opt_in_smem((const void*)cnn_eval_kernel, sb);
   cnn_eval_kernel<<<d.n_chains, HQ_THREADS, sb, s>>>(d, cn, X, F, mean_field_shift(d));

@@ -1193,7 +1193,7 @@ int hq_cumulative_sweep(hq_engine* e, int n_steps, int n_inner, unsigned flags) 
     {
       PhaseTimer pt(e, 6, use_cnn ? 2 : 1);
       rc = rc ? rc : cuda_check(e, hq::nn_launch_eval(d, e->nn, d.X, e->nn.F0, 1, e->stream), "nn eval F0");
-      if (use_cnn) rc = rc ? rc : cuda_check(e, hq::cnn_launch_eval(d, e->cn, d.X, e->cn.F, 1, e->stream), "cnn eval");
+      if (use_cnn) rc = rc ? rc : cuda_check(e, hq::cnn_launch_eval(d, e->cn, d.X, e->cn.F, e->stream), "cnn eval");
     }
     {
       PhaseTimer pt(e, 7, 1);
@@ -1288,7 +1288,7 @@ int hq_cnn_eval(hq_engine* e, double* F_host) {
   if (rc) return rc;
   if (!F_host) return HQ_EINVAL;
   if (!e->cn.on) return set_err(e, HQ_EINVAL, "no convolutional parameters (hq_cnn_set_params)");
-  rc = cuda_check(e, hq::cnn_launch_eval(e->d, e->cn, e->d.X, e->cn.F, 1, e->stream), "cnn eval");
+  rc = cuda_check(e, hq::cnn_launch_eval(e->d, e->cn, e->d.X, e->cn.F, e->stream), "cnn eval");
   rc = rc ? rc : cuda_check(e, cudaMemcpyAsync(F_host, e->cn.F, sizeof(double) * e->d.n_chains,
                                                cudaMemcpyDeviceToHost, e->stream), "cnn eval copy");
   return rc ? rc : cuda_check(e, cudaStreamSynchronize(e->stream), "cnn eval sync");

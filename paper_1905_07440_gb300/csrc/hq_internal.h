@@ -180,8 +180,7 @@ cudaError_t nn_launch_loss(const NNState& nn, const double* ys, const int* idx, 
 // site_window > 0 block moves to `site_window` consecutive sites, from random starts per step.
 cudaError_t nn_launch_inner(const Dev& d, const NNState& nn, const CnnState& cn, int n_inner, int do_local,
                             int do_block, int use_cnn, int window, int site_window, cudaStream_t s);
-cudaError_t cnn_launch_eval(const Dev& d, const CnnState& cn, const double* X, double* F, int write_cache,
-                            cudaStream_t s);
+cudaError_t cnn_launch_eval(const Dev& d, const CnnState& cn, const double* X, double* F, cudaStream_t s);
 size_t cnn_sample_bytes(size_t NL);
 cudaError_t cnn_launch_set(const CnnState& cn, const float* src_device, cudaStream_t s);
 cudaError_t cnn_launch_batch(const Dev& d, const CnnState& cn, const double* Xs, const double* ys, const int* idx,
