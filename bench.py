@@ -106,6 +106,31 @@ def split_boundary(p):
     return (q // 2) * p.n_wrap if q >= 2 else 0
 
 
+def roofline_fields(achieved, dfma):
+    """Denominators of an FP64 rate whose contractions run as digit products on the tensor cores: 21 half-precision
+    products to one FP64 multiply-add, at the measured bf16 burst rate.  The panels' scalar FP64 work, which is what
+    the kernels wait for, has the DFMA probe of the same run beside it."""
+    path = os.path.join(ROOT, "MEASURED_PEAKS.json")
+    bf16 = 1900.0
+    if os.path.exists(path):
+        with open(path) as f:
+            bf16 = json.load(f)["bf16_tflops"]
+    peak = bf16 / 21.0
+    return {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+            "frac": achieved / peak if achieved else None, "fp64_dfma_tflops": dfma,
+            "times_fp64_dfma": achieved / dfma if achieved else None,
+            "peak_source": "bf16 burst %.0f TFLOP/s (%s) / 21 digit products; fp64_dfma_tflops: probe measured in this run"
+                           % (bf16, "measured" if os.path.exists(path) else "fallback")}
+
+
+def source_hash():
+    """Hash of all device sources: a traffic record holds for the sources it was taken with."""
+    import hashlib
+    src = os.path.join(ROOT, "paper_1905_07440_gb300", "csrc")
+    names = sorted(f for f in os.listdir(src) if f.endswith((".cu", ".cuh", ".h")))
+    return hashlib.sha256(b"".join(open(os.path.join(src, f), "rb").read() for f in names)).hexdigest()[:16]
+
+
 def flops_split_halves(p):
     """FP64 flops of one chain in the two-half log|det M| launch: the slices above the
     boundary m (top down, chunks of n_wrap from the top) and below it (right factors)."""
@@ -440,8 +465,7 @@ def run_ours(args):
     if n_l:
         fl_l = chains * flops_local_phase(params, acc_l0)
         per_sweep_s = ms_l / 1e3 / args.steps
-        roof_local = {"bound": "alu", "kernel": "local_phase_kernel", "achieved": fl_l / per_sweep_s / 1e12,
-                      "peak": peak, "unit": "TFLOP/s", "frac": fl_l / per_sweep_s / 1e12 / peak,
+        roof_local = {"kernel": "local_phase_kernel", **roofline_fields(fl_l / per_sweep_s / 1e12, peak),
                       "flops_per_sweep": fl_l, "launches_per_sweep": n_l / args.steps,
                       "ms_per_sweep": ms_l / args.steps}
     gpu_launches = sum(n for _, n in phases.values())
@@ -460,12 +484,9 @@ def run_ours(args):
     traffic = None
     tr_path = os.path.join(ROOT, "profiles", f"traffic_global_phase_{args.workload}.json")
     if dom == "block_moves" and os.path.exists(tr_path):
-        import hashlib
         with open(tr_path) as f:
             tr = json.load(f)
-        src = b"".join(open(os.path.join(ROOT, "paper_1905_07440_gb300", "csrc", x), "rb").read()
-                       for x in ("hq_kernels.cu", "hq_device.cuh"))
-        if hashlib.sha256(src).hexdigest()[:16] == tr["source_hash"] and chains == workload_params(args.workload)[1]:
+        if source_hash() == tr["source_hash"] and chains == workload_params(args.workload)[1]:
             traffic = tr["dram_bytes_per_launch"]
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
@@ -479,10 +500,8 @@ def run_ours(args):
                    "l2": "flushed (512 MB write) before every timed sweep; flush outside the events"},
         "e2e": {"value": e2e, "unit": UNIT, "h2d_bytes_per_step": xbytes, "d2h_bytes_per_step": xbytes + obs_bytes},
         "gpu_launches": gpu_launches,
-        "roofline": {"bound": "alu", "kernel": kernel_names[dom], "achieved": achieved, "peak": peak,
-                     "unit": "TFLOP/s", "frac": (achieved / peak) if achieved else None, "traffic": traffic,
+        "roofline": {"kernel": kernel_names[dom], **roofline_fields(achieved, peak), "traffic": traffic,
                      "traffic_source": "ncu dram__bytes_read.sum + dram__bytes_write.sum, profiles/" + os.path.basename(tr_path),
-                     "peak_source": "FP64 DFMA probe measured in this run (hq_fp64_peak_tflops)",
                      "flops_per_launch": fl, "ms_per_launch": per_launch_s * 1e3,
                      "share": ms / total_ms if total_ms else None},
         "roofline_local": roof_local,
@@ -730,12 +749,9 @@ def run_headline(args):
     traffic, tr_src = None, None
     tr_path = os.path.join(ROOT, "profiles", f"traffic_{kernel_names.get(dom, dom)}_largest.json")
     if os.path.exists(tr_path) and C == workloads.LARGEST_RUN["n_chains"]:
-        import hashlib
         with open(tr_path) as f:
             tr = json.load(f)
-        src = b"".join(open(os.path.join(ROOT, "paper_1905_07440_gb300", "csrc", x), "rb").read()
-                       for x in ("hq_kernels.cu", "hq_device.cuh"))
-        if hashlib.sha256(src).hexdigest()[:16] == tr["source_hash"]:
+        if source_hash() == tr["source_hash"]:
             traffic, tr_src = tr["dram_bytes_per_launch"], "profiles/" + os.path.basename(tr_path)
     xbytes = 8 * C * big.n_slices * big.n_sites
     e2e = C * world * args.e2e_steps / t_e2e / (2.0 * tau["s_cdw"])
@@ -787,11 +803,9 @@ def run_headline(args):
                 "note": "per step: fields in from pinned host memory (state rebuilt), one cumulative step, fields "
                         "and observables out"},
         "gpu_launches": sum(n for _, n in phases.values()) + K,
-        "roofline": {"bound": "alu", "kernel": kernel_names.get(dom, dom), "achieved": achieved, "peak": peak,
-                     "unit": "TFLOP/s", "frac": (achieved / peak) if achieved else None, "traffic": traffic,
+        "roofline": {"kernel": kernel_names.get(dom, dom), **roofline_fields(achieved, peak), "traffic": traffic,
                      "traffic_source": tr_src,
-                     "peak_source": "FP64 DFMA probe measured in this run (hq_fp64_peak_tflops)",
-                     "frac_vs_cublas_dgemm": (achieved / dgemm) if (achieved and dgemm) else None,
+                     "times_cublas_dgemm": (achieved / dgemm) if (achieved and dgemm) else None,
                      "cublas_dgemm_tflops": dgemm, "flops_per_launch": fl, "ms_per_launch": per_launch_s * 1e3,
                      "share": ms / total_ms if total_ms else None},
         "phases_ms_per_step": {k: v[0] / K for k, v in phases.items() if v[1]},
@@ -860,11 +874,10 @@ def measure_batched(args, hq, dev, stream, world, first, peak, dgemm, steps=5, w
     fl_l = chains * flops_local_phase(params, acc_l)
     return {"workload": "batched plain DQMC 8x8 beta=8 L=80", "chains_per_rank": chains,
             "value": chains * world * steps / t_dev, "unit": UNIT, "ms_per_sweep": t_dev * 1e3 / steps,
-            "roofline_block_moves": {"kernel": "global_phase_kernel", "achieved": achieved, "peak": peak,
-                                     "frac": achieved / peak if achieved else None,
-                                     "frac_vs_cublas_dgemm": achieved / dgemm if achieved else None},
-            "roofline_local_phase": {"kernel": "local_phase_kernel", "achieved": fl_l / (ms_l / 1e3 / steps) / 1e12,
-                                     "frac": fl_l / (ms_l / 1e3 / steps) / 1e12 / peak},
+            "roofline_block_moves": {"kernel": "global_phase_kernel", **roofline_fields(achieved, peak),
+                                     "times_cublas_dgemm": achieved / dgemm if achieved else None},
+            "roofline_local_phase": {"kernel": "local_phase_kernel",
+                                     **roofline_fields(fl_l / (ms_l / 1e3 / steps) / 1e12, peak)},
             "phases_ms_per_sweep": {k: v[0] / steps for k, v in phases.items() if v[1]}}
 
 
