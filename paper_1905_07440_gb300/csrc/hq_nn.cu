@@ -12,9 +12,9 @@
 // periodic convolutional action F_cnn in place of F (hq_cnn.cuh).  Each move is reversible for
 // its own weight, so p_c = exp(2 dlog|det M| - 2 sum of the accepted moves' network changes)
 // (the phonon action cancels; for one network the sum telescopes to F(X') - F(X)).
-// Every kernel evaluates f through nn_tile_f (hq_nn_tc.cuh: 16 patches per warp on the tensor
-// cores, bfloat16 operands, FP32 accumulation), so the inner chain and the acceptance see
-// bit-identical values of f.
+// Every evaluation of f runs nn_layer1, nn_layer2 and nn_layer3 (hq_nn_tc.cuh: 16 patches per tile on the
+// tensor cores, bfloat16 operands, FP32 accumulation) with the sums of an entry in the same order, in one warp
+// (nn_tile_f) or shared by two (local moves), so the inner chain and the acceptance see bit-identical values of f.
 #include <cooperative_groups.h>
 #include <cstdio>
 #include "hq_cnn.cuh"
@@ -217,7 +217,8 @@ __global__ void __launch_bounds__(HQ_THREADS) nn_eval_kernel(Dev d, NNState nn, 
 // cumulative accept needs a reversible proposal; so each step draws a direction (second
 // uniform of the step's Philox block, tag 4): forward (l, i ascending, then block moves i
 // ascending) or the exact reverse of that sequence, with probability 1/2 each.  The accepted
-// moves' dF are summed (thread 0, fixed order) into nn.dFpath for the cumulative accept.
+// moves' dF are summed in their order (local moves by warp 1, block moves by thread 0) into nn.dFpath for the
+// cumulative accept.
 // The caches of the current fields (fc; with use_cnn also the convolutional activations) are
 // valid on entry; with use_cnn each network's cache is rebuilt before its part when the other
 // part has changed the fields.

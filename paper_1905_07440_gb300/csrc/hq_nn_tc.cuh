@@ -7,8 +7,8 @@
 // layers see the FP32 operand to about 2^-17 relative instead of bfloat16's 2^-9.  Layer 3 (64
 // -> 1) is a per-row dot product in FP32.
 //
-// Every evaluation of f in the library goes through nn_tile_f with the same instruction
-// sequence, and each output row of an mma depends only on its own A row, so a patch gets
+// Every evaluation of f in the library goes through nn_layer1, nn_layer2 and nn_layer3 with the same
+// sequence of operations per entry, and each output row of an mma depends only on its own A row, so a patch gets
 // bit-identical f wherever it sits in a tile: the inner chain's changes of F and the cached
 // patch values agree exactly, which the exactness of the cumulative accept relies on.
 //

@@ -1,6 +1,6 @@
 // FP64 matrix products on the tensor cores (error-free splitting into FP16 digits).
 //
-// GB300 issues about 1.65 DFMA per clock and SM, but 1024 FP16 multiply-adds with FP32
+// GB300 issues about 1.65 DFMA per clock and SM, but 870 FP16 multiply-adds with FP32
 // accumulation through mma.sync.m16n8k16 (measured: 550 TFLOP/s against 1.06).  So the
 // contractions of the engine run as sums of exact digit products (the splitting of Ozaki, Ogita,
 // Oishi and Rump, Numer. Algorithms 59 (2012), with fixed-point digits):
@@ -15,7 +15,9 @@
 //     when all digits are extreme and then lose units that weigh 2^-58 of 2^(ea+eb).
 //   * S_0 .. S_4 (+ S_5 / 1024) are added up in 64-bit integers, converted once and scaled by
 //     the exponents.  The digit pairs left out (i + j > 5) and the last integer digit weigh about
-//     2^-56 of the largest |a| |b| of the sum, against 2^-53 per operation of a DFMA chain.
+//     2^-56 of the largest |a| |b| of the sum, against 2^-53 per operation of a DFMA chain.  Where a line's terms
+//     differ in size and the other factor's make up for it, a DFMA chain keeps the small ones' bits and this does
+//     not, unless the terms are scaled (oz_gemm's sk, oz_t_product).
 //
 // The splits run on the integer pipe (about 27 instructions per value), so a product costs about
 // as much as its operands' splits plus 1/16 of the DFMA time.  tcgen05 is not used: operands

@@ -22,7 +22,7 @@
 // 33 FP64 instructions per step at m = 64.  Measured for 64 x 16 (256 x 16), cycles: column by column with
 // two warp reductions per step 82 (145) thousand; rows spread over the warps 67 (146); 64-bit integers with
 // 128-bit dot products 62 (130).  Whole QR of n = 64 (256), thousand cycles: rows spread over the warps 375 (3760),
-// this form 310 (2840).
+// this form 329 (2890).
 #pragma once
 #include "hq_device.cuh"
 #include "hq_oz.cuh"
